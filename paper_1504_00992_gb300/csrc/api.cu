@@ -475,7 +475,8 @@ static int plan_handle(tebd_s* h, int n_chains, const tebd_desc_t* descs, Handle
   lay_plan.sweep_off = off; off += ALIGN;
   lay_plan.tcerr_off = off; off += ALIGN;
   lay_plan.queue_off = off; off += ALIGN;
-  lay_plan.op_off = off; off += align_up(sizeof(cplx) * 64 * 64) + ALIGN;
+  // an operator, then its expectation value and the partial sums of it
+  lay_plan.op_off = off; off += align_up(sizeof(cplx) * 64 * 64) + align_up(sizeof(cplx) * (1 + EX_PARTS));
   // problems of each parity, chain-major, and their waves under the budget
   const size_t budget = d0.workspace_budget;
   size_t ws_max = 0;
@@ -1164,7 +1165,8 @@ extern "C" int tebd_expect(tebd_t h, int site, const double* op, double* out) {
   if (site < 0 || site >= C.N || !op || !out) { h->err.set(TEBD_EINVAL, "bad site or NULL pointer"); return h->err.code; }
   const int d = C.d[site];
   CU_OR(h, cudaMemcpyAsync(h->op_dev, op, sizeof(cplx) * d * d, cudaMemcpyHostToDevice, h->stream));
-  CU_OR(h, launch_expect(C.dev, site, h->op_dev, d, h->out_dev, h->stream));
+  CU_OR(h, launch_expect(C.dev, site, (int64_t)C.cap_ext[site] * C.cap_ext[site + 1], h->op_dev, d,
+                         h->out_dev + 1, h->out_dev, h->stream));
   CU_OR(h, cudaMemcpyAsync(out, h->out_dev, sizeof(cplx), cudaMemcpyDeviceToHost, h->stream));
   return tebd_check_status(h);
 }

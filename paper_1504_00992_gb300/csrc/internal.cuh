@@ -193,7 +193,10 @@ cudaError_t launch_rebuild(const Dims* dims, const ProbPtr* ptrs, int batch, dou
 cudaError_t launch_wacc(const Dims* dims, const ProbPtr* ptrs, const double* wout, int batch, double* wacc,
                         cudaStream_t st);
 cudaError_t launch_sweep_tick(uint64_t* sweep_dev, cudaStream_t st);
-cudaError_t launch_expect(const ChainDev& ch, int site, const cplx* op, int d, cplx* out, cudaStream_t st);
+// elems: the capacity of the site's bond pair; part: scratch of EX_PARTS numbers
+enum { EX_PARTS = 304 };
+cudaError_t launch_expect(const ChainDev& ch, int site, int64_t elems, const cplx* op, int d, cplx* part, cplx* out,
+                          cudaStream_t st);
 
 // --- persistent fused bond update (fused.cu) -------------------------------
 // Bonds of a wave whose capacities satisfy fused_fits can be updated by one
