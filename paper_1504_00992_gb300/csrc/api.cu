@@ -172,6 +172,7 @@ struct Wave {
   MixedKnobs mk{0, 0, 0, 0};  // launch choices of the mixed form (TF32 handles)
   float tune_ms[2] = {0.f, 0.f};  // tuner timings of the staged and fused RRSVD (0: not timed)
   MixedSizes ms{};  // TF32 handles: the wave's FP32 arrays at its capacities
+  size_t dp = 0;    // FP64 handles: bytes of the digit-split products' scratch (0: no bond of the wave takes them)
 };
 
 struct ParitySet {
@@ -186,6 +187,7 @@ struct ParitySet {
 struct HandlePlan {
   size_t one_off = 0, st_off = 0, wacc_off = 0, sweep_off = 0, tcerr_off = 0, op_off = 0, wout_off = 0, queue_off = 0;
   size_t desc_off = 0, desc_per = 0, ws_off = 0, mixed_off = 0, total = 0;
+  size_t dp_limit = 0;  // bound of a wave's digit-split scratch (beyond one bond's own)
   std::vector<WsLayout> lay[2];
   int max_batch = 0;
 };
@@ -210,7 +212,7 @@ struct tebd_s {
   uint64_t* sweep_dev = nullptr;
   int* queue = nullptr;        // work counter of the persistent fused launch
   int* tcerr = nullptr;        // tensor-core wait timeout flag (TF32 handles)
-  char* mixed = nullptr;       // FP32 arrays of the current wave (TF32 handles)
+  char* mixed = nullptr;       // FP32 arrays of the current wave (TF32 handles), or the digit-split scratch (FP64)
   cplx* op_dev = nullptr;
   cplx* out_dev = nullptr;
   double* one_lam = nullptr;
@@ -322,6 +324,12 @@ static int tune_wave(tebd_s* h, const ParitySet& ps, Wave& w, cudaStream_t st, D
   // fused kernel, on synthetic theta at the capacity sizes (the two give the
   // same results; the data only sets the QR and Jacobi work)
   if (fused_mode == 0 && fused_fits(w.cap)) {
+    DpScratch dp;
+    if (w.dp) {  // the staged launches as enqueue_sweep makes them
+      dp = dp_carve(h->mixed, w.cap, w.count, h->plan.dp_limit, h->tcerr);
+      for (Dims& D : hd) D.dig = dp_rule(D.m, D.n, D.l) ? 1 : 0;
+      if (cudaMemcpy(scratch_dims, hd.data(), sizeof(Dims) * w.count, cudaMemcpyHostToDevice) != cudaSuccess) return -1;
+    }
     if (launch_tune_theta(scratch_dims, ps.ptrs + w.first, w.count, st) != cudaSuccess) return -1;
     float ms[2] = {1e30f, 1e30f};
     for (int variant = 0; variant < 2; ++variant)
@@ -329,7 +337,7 @@ static int tune_wave(tebd_s* h, const ParitySet& ps, Wave& w, cudaStream_t st, D
         cudaEventRecord(e0, st);
         const cudaError_t e =
             variant == 0 ? run_rrsvd(scratch_dims, ps.ptrs + w.first, w.count, w.cap, h->q, h->seed, 0, 0, -1,
-                                     h->status, st, h->sweep_dev, w.tiles)
+                                     h->status, st, h->sweep_dev, w.tiles, w.dp ? &dp : nullptr)
                          : launch_bond_fused(ps.ptrs + w.first, nullptr, scratch_dims, w.count, p_os, h->q, h->seed,
                                              h->sweep_dev, h->cutoff, nullptr, h->status, h->queue, st);
         if (e != cudaSuccess) return -1;
@@ -479,6 +487,8 @@ static int plan_handle(tebd_s* h, int n_chains, const tebd_desc_t* descs, Handle
   lay_plan.op_off = off; off += align_up(sizeof(cplx) * 64 * 64) + align_up(sizeof(cplx) * (1 + EX_PARTS));
   // problems of each parity, chain-major, and their waves under the budget
   const size_t budget = d0.workspace_budget;
+  // the digit-split scratch: a quarter of a budget at most (or what one bond needs)
+  lay_plan.dp_limit = budget > 0 ? std::min((size_t)DP_LIMIT, budget / 4) : (size_t)DP_LIMIT;
   size_t ws_max = 0;
   std::vector<WsLayout>* lay = lay_plan.lay;
   std::vector<size_t> pbytes[2];
@@ -492,6 +502,16 @@ static int plan_handle(tebd_s* h, int n_chains, const tebd_desc_t* descs, Handle
     kc = std::min(C.cap_ext[b + 1], std::min(mc, nc));
     lc = std::min(kc + h->p, std::min(mc, nc));
   };
+  // FP64 handles with large bonds take the digit-split products; a fused
+  // choice other than 0 asks for the persistent launch's own summation order
+  bool digits = false;
+  if (!tf32 && d0.fused == 0)
+    for (const ChainH& C : h->ch)
+      for (int b = 0; b < C.N - 1; ++b) {
+        int mc, nc, kc, lc;
+        bond_caps(C, b, mc, nc, kc, lc);
+        digits = digits || dp_handle_rule(mc, nc, lc);
+      }
   for (int par = 0; par < 2; ++par) {
     ParitySet& ps = h->par[par];
     for (int c = 0; c < n_chains; ++c) {
@@ -562,6 +582,12 @@ static int plan_handle(tebd_s* h, int n_chains, const tebd_desc_t* descs, Handle
         wv.ms = mixed_sizes(wv.cap.m, wv.cap.n, wv.cap.k, wv.cap.l, bf16, &wv.cap);
         mixed_max = std::max(mixed_max, mixed_bytes(wv.ms, wv.count));
       }
+    else if (digits)
+      for (Wave& wv : ps.waves)
+        if (dp_rule(wv.cap.m, wv.cap.n, wv.cap.l)) {
+          wv.dp = dp_bytes(wv.cap, wv.count, lay_plan.dp_limit);
+          mixed_max = std::max(mixed_max, wv.dp);
+        }
   }
   lay_plan.wout_off = off; off += align_up(sizeof(double) * std::max(1, max_batch));
   lay_plan.desc_off = off;
@@ -599,14 +625,13 @@ extern "C" int tebd_plan_query(int n_chains, const tebd_desc_t* descs, size_t* a
 static bool bind_arena(tebd_s* h) {
   const HandlePlan& L = h->plan;
   char* A = h->arena;
-  const bool tf32 = prec_mixed(h->precision);
   h->one_lam = (double*)(A + L.one_off);
   h->status = (int*)(A + L.st_off);
   h->wacc = (double*)(A + L.wacc_off);
   h->sweep_dev = (uint64_t*)(A + L.sweep_off);
   h->queue = (int*)(A + L.queue_off);
-  h->tcerr = tf32 ? (int*)(A + L.tcerr_off) : nullptr;
-  h->mixed = tf32 ? A + L.mixed_off : nullptr;
+  h->tcerr = (int*)(A + L.tcerr_off);
+  h->mixed = A + L.mixed_off;
   h->op_dev = (cplx*)(A + L.op_off);
   h->out_dev = (cplx*)(A + L.op_off + align_up(sizeof(cplx) * 64 * 64));
   h->wout = (double*)(A + L.wout_off);
@@ -721,6 +746,7 @@ extern "C" int tebd_create_multi(int n_chains, const tebd_desc_t* descs, tebd_t*
     for (int par = 0; par < 2; ++par)
       for (const Wave& w : h->par[par].waves)
         if (mixed_prepare(w.cap) != cudaSuccess) { cudaGetLastError(); tebd_free(h); return TEBD_ECUDA; }
+  else if (oz_prepare() != cudaSuccess || cholqr_prepare() != cudaSuccess) { cudaGetLastError(); tebd_free(h); return TEBD_ECUDA; }
   if (fused_prepare() != cudaSuccess) { cudaGetLastError(); tebd_free(h); return TEBD_ECUDA; }
   if (!bind_arena(h)) { tebd_free(h); return TEBD_ECUDA; }
   // every chain starts in |0...0>
@@ -1054,6 +1080,14 @@ extern "C" int tebd_set_gates(tebd_t h, int parity, const double* gates) {
   return TEBD_OK;
 }
 
+// The staged RRSVD of one wave of an FP64 handle.
+static cudaError_t wave_rrsvd(tebd_t h, const Wave& w, const Dims* dims, const ProbPtr* ptrs, cudaStream_t st) {
+  DpScratch dp;
+  if (w.dp) dp = dp_carve(h->mixed, w.cap, w.count, h->plan.dp_limit, h->tcerr);
+  return run_rrsvd(dims, ptrs, w.count, w.cap, h->q, h->seed, 0, 0, -1, h->status, st, h->sweep_dev,
+                   w.tiles[0] != 0 ? w.tiles : nullptr, w.dp ? &dp : nullptr);
+}
+
 // The launch sequence of one sweep: per wave, sizes -> theta -> RRSVD ->
 // rebuild -> weights; then the device sweep counter advances.
 static cudaError_t enqueue_sweep(tebd_t h, int parity) {
@@ -1061,7 +1095,6 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
   for (const Wave& w : ps.waves) {
     Dims* dims = ps.dims + w.first;
     ProbPtr* ptrs = ps.ptrs + w.first;
-    const bool tuned = w.tiles[0] != 0;
     cudaError_t e;
     if (w.fused) {
       // the whole update of every bond of the wave in one persistent launch
@@ -1071,7 +1104,7 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
       if ((e = launch_wacc(dims, ptrs, h->wout + w.first, w.count, h->wacc, h->stream)) != cudaSuccess) return e;
       continue;
     }
-    if ((e = launch_plan(ptrs, dims, w.count, h->p, h->stream)) != cudaSuccess) return e;
+    if ((e = launch_plan(ptrs, dims, w.count, h->p, h->stream, w.dp > 0)) != cudaSuccess) return e;
     if (prec_mixed(h->precision)) {
       // bonds of large local dimensions: contraction and gate as GEMMs, on
       // the tensor cores from digit splits or in double-float arithmetic
@@ -1096,8 +1129,7 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
       if ((e = run_rrsvd_mixed(dims, ptrs, w.count, w.cap, mp, h->q, h->seed, 0, 0, -1, h->status, h->tcerr,
                                h->stream, h->sweep_dev, &w.mk, h->precision == TEBD_PREC_BF16)) != cudaSuccess)
         return e;
-    } else if ((e = run_rrsvd(dims, ptrs, w.count, w.cap, h->q, h->seed, 0, 0, -1, h->status, h->stream,
-                              h->sweep_dev, tuned ? w.tiles : nullptr)) != cudaSuccess) {
+    } else if ((e = wave_rrsvd(h, w, dims, ptrs, h->stream)) != cudaSuccess) {
       return e;
     }
     if ((e = launch_rebuild(dims, ptrs, w.count, h->cutoff, h->wout + w.first, h->status, h->stream)) != cudaSuccess)
@@ -1429,14 +1461,12 @@ extern "C" int tebd_backward(tebd_t h, int site, const double* op, double* dgate
         Dims* dims = ps.dims + w.first;
         ProbPtr* ptrs = ps.ptrs + w.first;
         AdjPtr* adj = h->adj_dev[ck.parity] + w.first;
-        const bool tuned = w.tiles[0] != 0;
-        if (launch_plan(ptrs, dims, w.count, h->p, st) != cudaSuccess ||
+        if (launch_plan(ptrs, dims, w.count, h->p, st, w.dp > 0) != cudaSuccess ||
             launch_theta(dims, ptrs, w.count, w.cap, st, 1) != cudaSuccess ||
             launch_adj_keep_theta(dims, ptrs, adj, w.count, st) != cudaSuccess ||
             launch_theta(dims, ptrs, w.count, w.cap, st) != cudaSuccess ||
             launch_gate_gemm(dims, ptrs, w.count, w.cap, st) != cudaSuccess ||
-            run_rrsvd(dims, ptrs, w.count, w.cap, h->q, h->seed, 0, 0, -1, h->status, st, h->sweep_dev,
-                      tuned ? w.tiles : nullptr) != cudaSuccess ||
+            wave_rrsvd(h, w, dims, ptrs, st) != cudaSuccess ||
             launch_rebuild(dims, ptrs, w.count, h->cutoff, h->wout + w.first, h->status, st) != cudaSuccess ||
             launch_adj_bond(dims, ptrs, adj, w.count, region, region + rbytes, ck.buf, h->cutoff, 1e-24, 1e-24,
                             st) != cudaSuccess ||
@@ -1492,7 +1522,8 @@ struct rrsvd_plan_s {
   ProbPtr* ptrs = nullptr;
   int* status = nullptr;
   int* tcerr = nullptr;
-  size_t mixed_off = 0;  // start of the mixed-precision arrays in the workspace
+  size_t mixed_off = 0;  // start of the mixed-precision arrays (or of the FP64 form's digit-split scratch) in the workspace
+  int dig = 0;           // FP64: the products and QRs run from digit splits (dp_rule)
   MixedSizes ms{};
   // accuracy check (Alg. 2); check_r == 0: fixed rank
   int check_r = 0, l_max = 0, rounds = 0, k0 = 0, l0 = 0;
@@ -1523,9 +1554,9 @@ struct rrsvd_plan_s {
 namespace tg {
 __global__ void k_rrsvd_bind(ProbPtr* ptrs, int batch, char* ws, size_t per, WsLayout lay, const cplx* theta,
                              size_t theta_stride, cplx* U, size_t U_stride, cplx* Vh, size_t V_stride, Dims* dims,
-                             int dims_m, int dims_n, int dims_k, int dims_l, int* status) {
+                             int dims_m, int dims_n, int dims_k, int dims_l, int dig, int* status) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (dims_m > 0 && p == 0) *status = 0;
+  if (status && p == 0) *status = 0;
   if (p >= batch) return;
   ProbPtr P;
   memset(&P, 0, sizeof P);
@@ -1537,7 +1568,7 @@ __global__ void k_rrsvd_bind(ProbPtr* ptrs, int batch, char* ws, size_t per, WsL
   if (dims_m > 0) {
     Dims D;
     memset(&D, 0, sizeof D);
-    D.m = dims_m; D.n = dims_n; D.k = dims_k; D.l = dims_l; D.bond = 0; D.active = 1;
+    D.m = dims_m; D.n = dims_n; D.k = dims_k; D.l = dims_l; D.bond = 0; D.active = 1; D.dig = dig;
     dims[p] = D;
   }
 }
@@ -1575,6 +1606,15 @@ extern "C" int rrsvd_plan_create_ex(int m, int n, int k_max, int p, int q, int b
     P->ms = mixed_sizes(m, n, P->k, P->l, precision == TEBD_PREC_BF16);
     P->mixed_off = P->ws_bytes;
     P->ws_bytes += mixed_bytes(P->ms, batch);
+  } else if (dp_rule(m, n, P->l)) {
+    P->dig = 1;
+    P->mixed_off = align_up(P->ws_bytes);
+    P->ws_bytes = P->mixed_off + dp_bytes(P->cap, batch, DP_LIMIT);
+    if (oz_prepare() != cudaSuccess || cholqr_prepare() != cudaSuccess) {
+      cudaGetLastError();
+      delete P;
+      return TEBD_ECUDA;
+    }
   }
   const size_t meta = align_up(sizeof(Dims) * batch) + align_up(sizeof(ProbPtr) * batch) + 2 * ALIGN;
   if (fault_take(TEBD_FAULT_ALLOC) || cudaMalloc(&P->meta, meta) != cudaSuccess) {
@@ -1590,7 +1630,7 @@ extern "C" int rrsvd_plan_create_ex(int m, int n, int k_max, int p, int q, int b
   for (int i = 0; i < batch; ++i) {
     Dims& D = hd[i];
     memset(&D, 0, sizeof D);
-    D.m = m; D.n = n; D.k = P->k; D.l = P->l; D.bond = 0; D.active = 1;
+    D.m = m; D.n = n; D.k = P->k; D.l = P->l; D.bond = 0; D.active = 1; D.dig = P->dig;
   }
   if (cudaMemcpy(P->dims, hd.data(), sizeof(Dims) * batch, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(P->status, 0, 2 * ALIGN) != cudaSuccess) {
@@ -1651,6 +1691,16 @@ extern "C" int rrsvd_plan_dims(rrsvd_plan_t P, int* k, int* l) {
   return TEBD_OK;
 }
 
+// Whether an FP64 plan's launches take the digit-split products: where its
+// sizes do, unless GEMM tiles were forced (rrsvd_plan_set_tuning) or tuned to
+// be faster.
+static int plan_digits(rrsvd_plan_t P) {
+  if (!P->dig) return 0;
+  for (int t : P->tiles)
+    if (P->tuned && t) return 0;
+  return 1;
+}
+
 // The fixed-rank truncation of instances z0 .. z0 + cnt - 1 of a bound plan
 // (k_rrsvd_bind has run): sigma, Vh, w and rank point at instance z0's
 // entries.  Sub-batches of one plan may run concurrently on different streams.
@@ -1665,8 +1715,11 @@ static cudaError_t exec_range(rrsvd_plan_t P, int z0, int cnt, int64_t chain0, d
     e = run_rrsvd_mixed(dims, ptrs, cnt, P->cap, mp, P->q, P->seed, 0, chain0 + z0, 1, P->status, P->tcerr, st,
                         nullptr, &kn, P->precision == TEBD_PREC_BF16);
   } else {
+    DpScratch dp;
+    const bool dig = plan_digits(P);
+    if (dig) dp = dp_carve((char*)workspace + P->mixed_off, P->cap, P->batch, DP_LIMIT, P->tcerr);
     e = run_rrsvd(dims, ptrs, cnt, P->cap, P->q, P->seed, 0, chain0 + z0, 1, P->status, st, nullptr,
-                  P->tuned ? P->tiles : nullptr);
+                  P->tuned ? P->tiles : nullptr, dig ? &dp : nullptr);
   }
   if (e != cudaSuccess) return e;
   return launch_rrsvd_finalize(dims, ptrs, cnt, P->cap, 1e-14, sigma, Vh, w, rank, P->status, st);
@@ -1686,10 +1739,12 @@ extern "C" int rrsvd_execute(rrsvd_plan_t P, const double* theta, int64_t chain0
   const bool checked = P->check_r > 0;
   {
   ProfScope ps("k_rrsvd_bind", st);
+  // (a checked plan's descriptors are written by launch_checked_init)
   k_rrsvd_bind<<<(P->batch + 127) / 128, 128, 0, st>>>(P->ptrs, P->batch, (char*)workspace, P->per, P->lay,
                                                      (const cplx*)theta, (size_t)P->m * P->n,
                                                      checked ? nullptr : (cplx*)U, (size_t)P->m * P->k, (cplx*)Vh,
-                                                     (size_t)P->k * P->n, nullptr, 0, 0, 0, 0, nullptr);
+                                                     (size_t)P->k * P->n, P->dims, checked ? 0 : P->m, P->n, P->k,
+                                                     P->l, plan_digits(P), nullptr);
   }
   CU_OR(P, cudaGetLastError());
   if (checked) {
@@ -1697,9 +1752,12 @@ extern "C" int rrsvd_execute(rrsvd_plan_t P, const double* theta, int64_t chain0
     memset(&t, 0, sizeof t);
     t.m = P->m; t.n = P->n; t.k = P->k0; t.l = P->l0; t.active = 1; t.r = P->check_r;
     t.chk = (P->l0 + P->check_r <= P->l_max) ? 1 : 0;
+    t.dig = P->dig;
+    DpScratch dp;
+    if (P->dig) dp = dp_carve((char*)workspace + P->mixed_off, P->cap, P->batch, DP_LIMIT, P->tcerr);
     CU_OR(P, launch_checked_init(P->dims, P->batch, t, st));
     CU_OR(P, run_rrsvd_checked(P->dims, P->ptrs, P->batch, P->cap, P->q, P->rounds, P->eps, P->l_max, P->p, P->seed,
-                               chain0, P->status, st));
+                               chain0, P->status, st, P->dig ? &dp : nullptr));
     CU_OR(P, launch_finalize_checked(P->dims, P->ptrs, P->batch, P->k, 1e-14, sigma, U, w, rank, nullptr, P->status,
                                      st));
     return TEBD_OK;
@@ -1787,14 +1845,14 @@ extern "C" int rrsvd_execute_host(rrsvd_plan_t P, const double* theta, int64_t c
       k_rrsvd_bind<<<(P->batch + 127) / 128, 128, 0, st>>>(P->ptrs, P->batch, (char*)d_ws, P->per, P->lay,
                                                          (const cplx*)d_th, (size_t)P->m * P->n,
                                                          U ? (cplx*)d_u : nullptr, (size_t)P->m * P->k,
-                                                         Vh ? (cplx*)d_v : nullptr, (size_t)P->k * P->n, nullptr, 0,
-                                                         0, 0, 0, nullptr);
+                                                         Vh ? (cplx*)d_v : nullptr, (size_t)P->k * P->n, P->dims,
+                                                         P->m, P->n, P->k, P->l, 0, nullptr);
       CU_OR(P, cudaGetLastError());
     }
     CU_OR(P, cudaEventRecord(P->hev[nch], st));
     MixedKnobs kc = P->mk;
-    if (kc.qrbh == 0) kc.qrbh = qr_multi_chosen(QR_BH, P->cap, P->batch, 0) ? 2 : 3;
-    if (kc.jac == 0) kc.jac = jacobi_cluster_chosen(P->cap, P->batch, 0) ? 2 : 3;
+    kc.qrbh = mixed_qrbh(kc, P->cap, P->batch);
+    kc.jac = mixed_jac(kc, P->cap, P->batch);
     const size_t mn = (size_t)P->m * P->n, mk = (size_t)P->m * P->k, kn = (size_t)P->k * P->n;
     const int per = (P->batch + nch - 1) / nch;
     for (int i = 0; i < nch; ++i) {
@@ -1924,7 +1982,7 @@ extern "C" int rrsvd_plan_autotune(rrsvd_plan_t P, const double* theta, void* wo
   cudaStream_t st = (cudaStream_t)stream;
   k_rrsvd_bind<<<(P->batch + 127) / 128, 128, 0, st>>>(P->ptrs, P->batch, (char*)workspace, P->per, P->lay,
                                                      (const cplx*)theta, (size_t)P->m * P->n, nullptr, 0, nullptr, 0,
-                                                     nullptr, 0, 0, 0, 0, nullptr);
+                                                     P->dims, P->m, P->n, P->k, P->l, 0, nullptr);
   CU_OR(P, cudaGetLastError());
   if (prec_mixed(P->precision)) {
     const MixedPtrs mp = mixed_carve((char*)workspace + P->mixed_off, P->ms, P->batch);
@@ -1958,6 +2016,28 @@ extern "C" int rrsvd_plan_autotune(rrsvd_plan_t P, const double* theta, void* wo
         cudaEventElapsedTime(&t, e0, e1);
         if (t < best) { best = t; P->tiles[stage] = tile; }
       }
+    }
+    if (P->dig) {
+      // the whole truncation with these tiles against the digit-split
+      // products, which run where no tile is set
+      DpScratch dp = dp_carve((char*)workspace + P->mixed_off, P->cap, P->batch, DP_LIMIT, P->tcerr);
+      float ms[2] = {0.f, 0.f};
+      for (int v = 0; v < 2; ++v) {
+        k_rrsvd_bind<<<(P->batch + 127) / 128, 128, 0, st>>>(P->ptrs, P->batch, (char*)workspace, P->per, P->lay,
+                                                           (const cplx*)theta, (size_t)P->m * P->n, nullptr, 0,
+                                                           nullptr, 0, P->dims, P->m, P->n, P->k, P->l, v, nullptr);
+        for (int r = 0; r < 2; ++r) {  // the first run warms up
+          cudaEventRecord(e0, st);
+          const cudaError_t e = run_rrsvd(P->dims, P->ptrs, P->batch, P->cap, P->q, P->seed, 0, 0, 1, P->status, st,
+                                          nullptr, v ? nullptr : P->tiles, v ? &dp : nullptr);
+          cudaEventRecord(e1, st);
+          cudaEventSynchronize(e1);
+          cudaEventElapsedTime(&ms[v], e0, e1);
+          if (e != cudaSuccess) ms[v] = 1e30f;
+        }
+      }
+      if (ms[1] <= ms[0])
+        for (int& t : P->tiles) t = 0;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

@@ -15,6 +15,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "mixed.cuh"
 #include "profiler.cuh"
 
 namespace tg {
@@ -85,7 +86,8 @@ __global__ void __launch_bounds__(256) k_check_decide(Dims* dims, const ProbPtr*
 
 cudaError_t run_accuracy_check(const Dims* dims_mut, const ProbPtr* ptrs, int batch, const Caps& cap, int rounds,
                                double eps, int l_max, int p, uint64_t seed, uint64_t sweep, int64_t chain0,
-                               int chain_stride, cudaStream_t st) {
+                               int chain_stride, cudaStream_t st, const DpScratch* dp, int final_basis) {
+  const DpPath P{dims_mut, ptrs, batch, cap, dp, st, nullptr};
   Dims* dims = const_cast<Dims*>(dims_mut);
   for (int t = 0; t < rounds; ++t) {
     {
@@ -98,39 +100,45 @@ cudaError_t run_accuracy_check(const Dims* dims_mut, const ProbPtr* ptrs, int ba
       if (e != cudaSuccess) return e;
     }
     cudaError_t e;
-    if ((e = launch_zgemm(G_PR, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;  // Br = A Omega_r
-    if ((e = launch_zgemm(G_PQ, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;  // C1 = Q^H Br
-    if ((e = launch_zgemm(G_PD, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;  // Dr = Q C1
+    if ((e = P.gemm(G_PR)) != cudaSuccess) return e;  // Br = A Omega_r
+    if ((e = P.gemm(G_PQ)) != cudaSuccess) return e;  // C1 = Q^H Br
+    if ((e = P.gemm(G_PD)) != cudaSuccess) return e;  // Dr = Q C1
     {
       ProfScope ps("k_check_decide", st);
       k_check_decide<<<batch, 256, 0, st>>>(dims, ptrs, eps, l_max, p);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = launch_qr(QR_Y, dims, ptrs, batch, st, 1)) != cudaSuccess) return e;  // [Q | Br] = Q' R'
+    // [Q | Br] = Q' R' (a basis no power round follows stays with Householder)
+    e = (dp && !final_basis) ? P.qr(QR_Y, DPQ_CHECK) : launch_qr(QR_Y, dims, ptrs, batch, st, QRS_QFLAG);
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
 cudaError_t run_rrsvd_checked(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int q, int rounds,
                               double eps, int l_max, int p, uint64_t seed, int64_t chain0, int* status,
-                              cudaStream_t st) {
+                              cudaStream_t st, const DpScratch* dp) {
+  const DpPath P{dims, ptrs, batch, cap, dp, st, nullptr};
   cudaError_t e;
   if ((e = launch_omega(dims, ptrs, batch, cap, seed, 0, chain0, 1, st)) != cudaSuccess) return e;
-  if ((e = launch_zgemm(G_Y0, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-  if ((e = launch_qr_sized(QR_Y, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-  if ((e = run_accuracy_check(dims, ptrs, batch, cap, rounds, eps, l_max, p, seed, 0, chain0, 1, st)) != cudaSuccess)
+  if ((e = dp_begin(P)) != cudaSuccess) return e;
+  if ((e = P.gemm(G_Y0)) != cudaSuccess) return e;
+  // the residuals of the check need an orthonormal basis
+  if ((e = P.qr(QR_Y, q == 0 ? DPQ_LAST0 : DPQ_FIRST_LD)) != cudaSuccess) return e;
+  if ((e = run_accuracy_check(dims, ptrs, batch, cap, rounds, eps, l_max, p, seed, 0, chain0, 1, st, dp, q == 0)) !=
+      cudaSuccess)
     return e;
   for (int j = 0; j < q; ++j) {
-    if ((e = launch_zgemm(G_YT, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-    if ((e = launch_qr_sized(QR_YT, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-    if ((e = launch_zgemm(G_Y, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-    if ((e = launch_qr_sized(QR_Y, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
+    if ((e = P.gemm(G_YT)) != cudaSuccess) return e;
+    if ((e = P.qr(QR_YT, DPQ_MID)) != cudaSuccess) return e;
+    if ((e = P.gemm(G_Y)) != cudaSuccess) return e;
+    if ((e = P.qr(QR_Y, j + 1 == q ? DPQ_LAST : DPQ_MID)) != cudaSuccess) return e;
   }
-  if ((e = launch_zgemm(G_BH, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-  if ((e = launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
+  if ((e = P.gemm(G_BH)) != cudaSuccess) return e;
+  if ((e = P.qr(QR_BH, DPQ_LAST)) != cudaSuccess) return e;
   if ((e = launch_jacobi_sized(dims, ptrs, batch, cap, status, st)) != cudaSuccess) return e;
-  if ((e = launch_zgemm(G_U, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
-  if ((e = launch_zgemm(G_V, dims, ptrs, batch, cap, st)) != cudaSuccess) return e;
+  if ((e = P.gemm(G_U)) != cudaSuccess) return e;
+  if ((e = P.gemm(G_V)) != cudaSuccess) return e;
   return launch_frob2(dims, ptrs, batch, st);
 }
 

@@ -28,6 +28,8 @@
 namespace tg {
 
 static const double CQ_PIVOT = 1e-10;
+// the same bound for the scaled Gram matrix of the digit-split form (2^-30: kappa(B S) ~ 3e4)
+static const float CQ_MIN_PIVOT = 9.3132257461547852e-10f;
 
 // Cholesky G = R^H R of the l x l Hermitian matrix in P.R (upper triangle,
 // column-major, in place), then J = R^-1 (upper triangular, zero below).  One
@@ -278,12 +280,20 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_inv_sm(Dims* dims, const Pr
   }
 }
 
+// the kernel of the digit-split form below
+template <bool SM>
+__global__ void k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass, int passes, float min_pivot,
+                          float again, int cond);
+
 cudaError_t cholqr_prepare() {
   static int done = 0;
   if (!done) {
     const cudaError_t e =
         cudaFuncSetAttribute(k_chol_inv_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs_smem_bytes(CS_MAXL));
     if (e != cudaSuccess) return e;
+    const cudaError_t e2 =
+        cudaFuncSetAttribute(k_chol_eq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs_smem_bytes(CS_MAXL));
+    if (e2 != cudaSuccess) return e2;
     done = 1;
   }
   return cudaSuccess;
@@ -309,10 +319,12 @@ static cudaError_t chol_inv(Dims* dims, const ProbPtr* ptrs, int batch, int lcap
 
 cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
                           const OzScratch* oz, int* err) {
-  auto gemm = [&](int stage) {
-    return oz ? launch_oz_stage(stage, dims, ptrs, batch, cap, *oz, err, st)
-              : launch_zgemm_df(stage, dims, ptrs, batch, cap, st);
-  };
+  if (oz) {
+    CQ_TRY(run_cholqr(1, 2, CQ_LOWDIN, CQ_MIN_PIVOT, dims, ptrs, batch, cap, *oz, batch, 0, err, st));
+    CQ_TRY(launch_oz_stage(G_X, dims, ptrs, batch, cap, *oz, err, st, DPC_OK));  // X = B Qb = Rb^H
+    return launch_qr_rest(QR_BH, dims, ptrs, batch, cap, st, QRS_CF);
+  }
+  auto gemm = [&](int stage) { return launch_zgemm_df(stage, dims, ptrs, batch, cap, st); };
   CQ_TRY(gemm(G_G1));                          // G1 = B B^H
   CQ_TRY(chol_inv(dims, ptrs, batch, cap.l, 0, st));  // R1, J = R1^-1
   CQ_TRY(gemm(G_Q1));                          // Q1 = B^H R1^-1
@@ -321,7 +333,403 @@ cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps
   CQ_TRY(gemm(G_QB));                          // Qb = Q1 R2^-1
   CQ_TRY(gemm(G_X));                           // X = B Qb = Rb^H
   // ill-conditioned instances: Householder QR of B^H (overwrites X and Qb)
-  return launch_qr(QR_BH, dims, ptrs, batch, st, 1);
+  return launch_qr(QR_BH, dims, ptrs, batch, st, QRS_QFLAG);
+}
+
+// ---------------------------------------------------------------------------
+// Cholesky QR from digit-split products: Y into Q (m rows), or Yt into Qt (n).
+//
+// One pass is G = X^H X (56-bit digit products), the Cholesky factor R of the
+// scaled S G S and its inverse in double-float arithmetic (k_chol_eq), and
+// Q = (X S) R^-1 (digit products), with S the powers of two that bring the
+// columns of X to norms in [1, 2).  The scaling takes out the grading of the
+// columns that a power round leaves (Y = A Q~ with Q~ near the singular
+// vectors: kappa(Y) up to 1/eps, kappa(Y S) of 3 to 1000, measured on CPU
+// emulations of decaying spectra down to 1e-16), so one pass is enough there.
+// Y0 = A Omega is as ill-conditioned as A itself: a pivot below CE_PIVOT adds
+// the shift CE_SHIFT to the diagonal and asks for another pass (shifted
+// Cholesky QR: Fukaya, Kannan, Nakatsukasa, Yamamoto, Yanagisawa, SIAM J. Sci.
+// Comput. 42, 2020); each shifted pass brings directions of relative size
+// below sqrt(CE_SHIFT) up by 1/sqrt(CE_SHIFT) ~ 2e5, so three passes take
+// rounding-level directions to O(1).
+//
+// Q's range: the product with R^-1 is rounded to ~2^-56 kappa(X S) of a unit
+// column, so the last basis before the projection and the QR of B^H ask for
+// pivots above their min_pivot (kappa ~ 100: 1e-15, Householder's level),
+// and the basis is then made orthonormal to FP64 by the symmetric correction
+// Q (I + E)^-1/2, E = Q^H Q - I formed from digits (k_lowdin64).  Problems
+// that miss a bound have cf set and are left to the Householder QR.
+// ---------------------------------------------------------------------------
+static const float CE_PIVOT = 5.8207660913467407e-11f;  // 2^-34: above the double-float rounding of a pivot
+static const float CE_SHIFT = 2.9103830456733704e-11f;  // 2^-35
+static const float CE_AGAIN = 1.4901161193847656e-08f;  // 2^-26: below it another pass, where one is left
+static const float CE_AGAIN_LD = 6.103515625e-05f;      // 2^-14: the same before the symmetric correction
+
+enum { CE_THREADS = 512, CE_MAXL = 512 };
+
+// x 2^k by the exponent bits (x = 0 and results below the normal range: 0)
+__device__ __forceinline__ double ce_scale(double x, int k) {
+  const long long u = __double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7FF) + k;
+  return (((u >> 52) & 0x7FF) == 0 || e <= 0) ? 0.0 : __longlong_as_double(u + ((long long)k << 52));
+}
+
+__device__ __forceinline__ bool ce_takes(const Dims& D, int pass, int cond) {
+  if (!D.active) return false;
+  if ((cond & DPC_QFLAG) && !D.qflag) return false;
+  if ((cond & DPC_DIG) && !D.dig) return false;
+  return pass == 0 || (D.cq >= pass && !D.cf);
+}
+
+// S, R and R^-1 of the Gram matrix in P.R (full, column-major): sigma = S,
+// J = R^-1 (upper triangular, zero below).  The triangle lives packed in
+// shared memory (SM), or in place in P.R's upper half (the lower half keeps G
+// for a second attempt with the shift).
+template <bool SM>
+__global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass,
+                                                        int passes, float min_pivot, float again, int cond) {
+  extern __shared__ __align__(16) unsigned char ce_raw[];
+  __shared__ double s_diag[CE_MAXL];
+  __shared__ int s_exp[CE_MAXL];
+  __shared__ float2 s_inv;
+  __shared__ int s_state;  // 0 factored, 1 a pivot below the bound, 2 not a Gram matrix
+  __shared__ float s_min;
+  const int p = blockIdx.x;
+  const Dims D = dims[p];
+  if (!ce_takes(D, pass, cond)) return;
+  const ProbPtr P = ptrs[p];
+  const int L = D.l, tid = threadIdx.x;
+  cplx* G = P.R;
+  cplx* J = P.J;
+  float4* Tg = reinterpret_cast<float4*>(P.R);
+  float4* Ts = reinterpret_cast<float4*>(ce_raw);
+  float4* tmp = SM ? Ts + (size_t)L * (L + 1) / 2 : Ts;  // L
+  auto T = [&](int r, int c) -> float4& { return SM ? Ts[cs_at(r, c)] : Tg[(size_t)c * L + r]; };
+  if (tid == 0) s_state = 0;
+  __syncthreads();
+  for (int c = tid; c < L; c += CE_THREADS) {
+    const double d = G[(size_t)c * L + c].x;
+    const int e = (int)(((unsigned long long)__double_as_longlong(d) >> 52) & 0x7FF);
+    if (!(d > 0.0) || e == 0 || e == 0x7FF) s_state = 2;
+    s_diag[c] = d;
+    s_exp[c] = -((e - 1023) >> 1);
+  }
+  __syncthreads();
+  bool shifted = false;
+  for (int attempt = 0; s_state != 2 && attempt < 2; ++attempt) {
+    shifted = attempt == 1;
+    for (int e = tid; e < L * L; e += CE_THREADS) {
+      const int r = e % L, c = e / L;
+      if (r > c) continue;
+      const int k = s_exp[r] + s_exp[c];
+      cplx v;
+      if (r == c) {
+        v = cmk(s_diag[c], 0.0);
+      } else {
+        const cplx w = G[(size_t)r * L + c];  // the lower triangle: conj of (r, c)
+        v = cmk(w.x, -w.y);
+      }
+      float4 t = cs_split(cmk(ce_scale(v.x, k), ce_scale(v.y, k)));
+      if (r == c && shifted) {
+        float h = t.x, l = t.y;
+        two_sum(t.x, CE_SHIFT, h, l);
+        l += t.y;
+        fast2(h, l);
+        t.x = h;
+        t.y = l;
+      }
+      T(r, c) = t;
+    }
+    if (tid == 0) {
+      s_state = 0;
+      s_min = 4.f;
+    }
+    __syncthreads();
+    const float bound = fmaxf(CE_PIVOT, min_pivot) * (shifted ? 0.25f : 1.f);
+    for (int j = 0; j < L; ++j) {
+      if (tid == 0) {
+        const float4 dd = T(j, j);
+        const dfl d{dd.x, dd.y};
+        if (!(d.h > bound) || !isfinite(d.h)) {
+          s_state = isfinite(d.h) ? 1 : 2;
+        } else {
+          const dfl r = dsqrt(d);
+          const dfl inv = drecip(r);
+          T(j, j) = make_float4(r.h, r.l, 0.f, 0.f);
+          s_inv = make_float2(inv.h, inv.l);
+          s_min = fminf(s_min, d.h);
+        }
+      }
+      __syncthreads();
+      if (s_state) break;
+      const dfl inv{s_inv.x, s_inv.y};
+      for (int c = j + 1 + tid; c < L; c += CE_THREADS) {
+        const float4 v = T(j, c);
+        const dfl re = dmul(dfl{v.x, v.y}, inv), im = dmul(dfl{v.z, v.w}, inv);
+        T(j, c) = make_float4(re.h, re.l, im.h, im.l);
+      }
+      __syncthreads();
+      const int w = L - j - 1, j1 = j + 1;
+      for (int e = tid; e < w * (w + 1) / 2; e += CE_THREADS) {
+        int a, b;
+        cs_pair(e, a, b);
+        const int c1 = j1 + a, c2 = j1 + b;
+        const float4 x = T(j, c1), y = T(j, c2);
+        float4& g = T(c1, c2);
+        float rh = g.x, rl = g.y, ih = g.z, il = g.w;
+        dfx_dd(rh, rl, -x.x, -x.y, y.x, y.y);
+        dfx_dd(rh, rl, -x.z, -x.w, y.z, y.w);
+        dfx_dd(ih, il, -x.x, -x.y, y.z, y.w);
+        dfx_dd(ih, il, x.z, x.w, y.x, y.y);
+        fast2(rh, rl);
+        fast2(ih, il);
+        g = make_float4(rh, rl, ih, il);
+      }
+      __syncthreads();
+    }
+    // a pivot below the bound: once more with the shift, where the caller takes one
+    const bool retry = s_state == 1 && attempt == 0 && min_pivot == 0.f;
+    __syncthreads();
+    if (!retry) break;
+  }
+  const bool fail = s_state != 0 || (shifted && pass + 1 == passes);
+  const bool more = !fail && (shifted || (s_min < again && pass + 1 < passes));
+  if (tid == 0) {
+    dims[p].cf = fail ? 1 : 0;
+    dims[p].cq = more ? pass + 1 : pass;
+  }
+  if (fail) {  // an identity factor: the products in between stay finite
+    for (int e = tid; e < L * L; e += CE_THREADS) J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
+    for (int c = tid; c < L; c += CE_THREADS) P.sigma[c] = 1.0;
+    return;
+  }
+  // R^-1 in place, column by column: X[0:j, j] = -X[j][j] X[0:j, 0:j] R[0:j, j].
+  // Four lanes per row: the dot products of a column are up to j long.
+  const int quad = tid >> 2, ql = tid & 3;
+  for (int j = 0; j < L; ++j) {
+    for (int r0 = 0; r0 < j; r0 += CE_THREADS / 4) {
+      const int r = r0 + quad;
+      float sh = 0.f, sl = 0.f, th = 0.f, tl = 0.f;
+      if (r < j)
+        for (int k = r + ql; k < j; k += 4) {
+          const float4 x = T(r, k), u = T(k, j);
+          dfx_dd(sh, sl, x.x, x.y, u.x, u.y);
+          dfx_dd(sh, sl, -x.z, -x.w, u.z, u.w);
+          dfx_dd(th, tl, x.x, x.y, u.z, u.w);
+          dfx_dd(th, tl, x.z, x.w, u.x, u.y);
+        }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        const dfl a = dadd(dfl{sh, sl}, dfl{__shfl_xor_sync(0xffffffffu, sh, o), __shfl_xor_sync(0xffffffffu, sl, o)});
+        const dfl b = dadd(dfl{th, tl}, dfl{__shfl_xor_sync(0xffffffffu, th, o), __shfl_xor_sync(0xffffffffu, tl, o)});
+        sh = a.h;
+        sl = a.l;
+        th = b.h;
+        tl = b.l;
+      }
+      if (r < j && ql == 0) tmp[r] = make_float4(sh, sl, th, tl);
+    }
+    __syncthreads();
+    const float4 djj = T(j, j);
+    const dfl dj = drecip(dfl{djj.x, djj.y});
+    __syncthreads();
+    for (int r = tid; r <= j; r += CE_THREADS) {
+      if (r == j) {
+        T(j, j) = make_float4(dj.h, dj.l, 0.f, 0.f);
+      } else {
+        const float4 v = tmp[r];
+        const dfl re = dmul(dfl{v.x, v.y}, dneg(dj)), im = dmul(dfl{v.z, v.w}, dneg(dj));
+        T(r, j) = make_float4(re.h, re.l, im.h, im.l);
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < L * L; e += CE_THREADS) {
+    const int r = e % L, c = e / L;
+    cplx v = cmk(0.0, 0.0);
+    if (r <= c) {
+      const float4 t = T(r, c);
+      v = cmk((double)t.x + (double)t.y, (double)t.z + (double)t.w);
+    }
+    J[e] = v;
+  }
+  for (int c = tid; c < L; c += CE_THREADS) P.sigma[c] = ce_scale(1.0, s_exp[c]);
+}
+
+// Column phases of the Householder QR.  The Cholesky QR has a positive
+// diagonal of R; the Householder QR of this library (alpha = -e^{i arg x0}
+// ||x||) multiplies column j of Q by -e^{-i phi_j}, phi_j the phase of the
+// leading entry of column j when reflector j is formed.  These phases come
+// from a modified LU of Q's leading l x l block (Ballard, Demmel, Grigori,
+// Jacquelin, Knight, Nguyen, Solomonik, IPDPS 2014): at step j the entry
+// x = M[j][j] of the Schur complement gives s = -x / |x|, M[j][j] - s is the
+// pivot (of modulus at least 1) and the trailing block is eliminated as
+// usual.  The singular vectors then keep the phases they have when the
+// Householder QR factors the basis.  Double-float, the block in P.J; the
+// phases conj(s) go to P.Jk.
+__global__ void __launch_bounds__(CE_THREADS) k_hh_phase(const Dims* __restrict__ dims,
+                                                         const ProbPtr* __restrict__ ptrs, int side, int cond) {
+  __shared__ float4 s_col[CE_MAXL];  // the multipliers of column j
+  const int p = blockIdx.x;
+  const Dims D = dims[p];
+  if (!ce_takes(D, 0, cond) || D.cf) return;
+  const ProbPtr P = ptrs[p];
+  const int L = D.l, ld = side == 0 ? D.m : D.n, tid = threadIdx.x;
+  const cplx* Q = side == 0 ? P.Q : P.Qt;
+  float4* M = reinterpret_cast<float4*>(P.J);  // column-major L x L
+  for (int e = tid; e < L * L; e += CE_THREADS) M[e] = cs_split(Q[(size_t)(e / L) * ld + e % L]);
+  __syncthreads();
+  for (int j = 0; j < L; ++j) {
+    const float4 x = M[(size_t)j * L + j];
+    // s = -x / |x| (1 for an entry negligible against the unit column)
+    const dfl a2 = dadd(dmul(dfl{x.x, x.y}, dfl{x.x, x.y}), dmul(dfl{x.z, x.w}, dfl{x.z, x.w}));
+    dfl sr{-1.f, 0.f}, si{0.f, 0.f};
+    if (a2.h > 1e-30f) {
+      const dfl ia = drecip(dsqrt(a2));
+      sr = dneg(dmul(dfl{x.x, x.y}, ia));
+      si = dneg(dmul(dfl{x.z, x.w}, ia));
+    }
+    if (tid == 0) {
+      double re = (double)sr.h + (double)sr.l, im = (double)si.h + (double)si.l;
+      const double f = 1.0 / sqrt(fma(re, re, im * im));  // unit modulus to FP64
+      P.Jk[j] = cmk(re * f, -im * f);
+    }
+    // 1 / (x - s)
+    const dfl pr = dadd(dfl{x.x, x.y}, dneg(sr)), pi = dadd(dfl{x.z, x.w}, dneg(si));
+    const dfl id = drecip(dadd(dmul(pr, pr), dmul(pi, pi)));
+    const dfl ir = dmul(pr, id), ii = dneg(dmul(pi, id));
+    for (int r = j + 1 + tid; r < L; r += CE_THREADS) {
+      const float4 v = M[(size_t)j * L + r];
+      const dfl a{v.x, v.y}, b{v.z, v.w};
+      const dfl re = dadd(dmul(a, ir), dneg(dmul(b, ii))), im = dadd(dmul(a, ii), dmul(b, ir));
+      s_col[r] = make_float4(re.h, re.l, im.h, im.l);
+    }
+    __syncthreads();
+    const int w = L - j - 1;
+    for (int e = tid; e < w * w; e += CE_THREADS) {
+      const int r = j + 1 + e % w, c = j + 1 + e / w;
+      const float4 u = s_col[r], v = M[(size_t)c * L + j];
+      float4& g = M[(size_t)c * L + r];
+      float rh = g.x, rl = g.y, ih = g.z, il = g.w;
+      dfx_dd(rh, rl, -u.x, -u.y, v.x, v.y);
+      dfx_dd(rh, rl, u.z, u.w, v.z, v.w);
+      dfx_dd(ih, il, -u.x, -u.y, v.z, v.w);
+      dfx_dd(ih, il, -u.z, -u.w, v.x, v.y);
+      fast2(rh, rl);
+      fast2(ih, il);
+      g = make_float4(rh, rl, ih, il);
+    }
+    __syncthreads();
+  }
+}
+
+// J = (I + E)^-1/2 = I - E/2 + 3 E^2/8 to FP64 from G = I + E in P.R, for
+// l max|E| <= 3e-6 (the next term is below 1e-17); S = 1.  E^2 enters at the
+// level of 1e-12 at most, so it is formed in FP32, and not at all where it is
+// below FP64's resolution.  phases: column j also takes k_hh_phase's phase.
+__global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __restrict__ ptrs, int cond,
+                                                  int phases) {
+  __shared__ float red[16];
+  const int p = blockIdx.x;
+  const Dims D = dims[p];
+  if (!ce_takes(D, 0, cond) || D.cf) return;
+  const ProbPtr P = ptrs[p];
+  const int L = D.l, tid = threadIdx.x;
+  const cplx* G = P.R;
+  float mx = 0.f;
+  for (int e = tid; e < L * L; e += 512) {
+    const cplx g = G[e];
+    const double re = (e / L == e % L) ? g.x - 1.0 : g.x;
+    const float m = fmaxf(fabsf((float)re), fabsf((float)g.y));
+    mx = (m > mx || m != m) ? m : mx;  // NaN sticks
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float y = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = (y > mx || y != y) ? y : mx;
+  }
+  if ((tid & 31) == 0) red[tid >> 5] = mx;
+  __syncthreads();
+  mx = 0.f;
+  for (int w = 0; w < 16; ++w) mx = (red[w] > mx || red[w] != red[w]) ? red[w] : mx;
+  const bool ok = mx * (float)L <= 3e-6f;
+  if (!ok && tid == 0) dims[p].cf = 1;
+  const bool square = mx > 1e-9f;
+  for (int e = tid; e < L * L; e += 512) {
+    const int a = e % L, b = e / L;
+    const cplx g = G[e];
+    cplx t = cmk(a == b ? 1.0 : 0.0, 0.0);
+    if (ok) {
+      t = cmk(a == b ? 1.0 - 0.5 * (g.x - 1.0) : -0.5 * g.x, -0.5 * g.y);
+      if (square) {
+        float sx = 0.f, sy = 0.f;
+        for (int k = 0; k < L; ++k) {
+          const cplx u = G[(size_t)k * L + a], v = G[(size_t)b * L + k];
+          const float ux = (float)(k == a ? u.x - 1.0 : u.x), uy = (float)u.y;
+          const float vx = (float)(k == b ? v.x - 1.0 : v.x), vy = (float)v.y;
+          sx = fmaf(ux, vx, fmaf(-uy, vy, sx));
+          sy = fmaf(ux, vy, fmaf(uy, vx, sy));
+        }
+        t.x += 0.375 * (double)sx;
+        t.y += 0.375 * (double)sy;
+      }
+    }
+    P.J[e] = phases ? cmul(t, P.Jk[b]) : t;
+  }
+  for (int c = tid; c < L; c += 512) P.sigma[c] = 1.0;
+}
+
+static size_t ce_smem_bytes(int L) { return L <= CS_MAXL ? cs_smem_bytes(L) : sizeof(float4) * (size_t)L; }
+
+cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* dims, const ProbPtr* ptrs, int batch,
+                       const Caps& cap, const OzScratch& oz, int chunk, int cond, int* err, cudaStream_t st) {
+  auto prod = [&](int stage, int c) {
+    return launch_oz_range(stage, dims, ptrs, batch, cap, oz, chunk, c, err, st);
+  };
+  CQ_TRY(cholqr_prepare());
+  const int g0 = side == 0 ? G_CYG : G_CTG, q0 = side == 0 ? G_CYQ : G_CTQ;
+  const int g1 = side == 0 ? G_CQG : G_CRG, q1 = side == 0 ? G_CQQ : G_CRQ;
+  for (int pass = 0; pass < passes; ++pass) {
+    const int in_pass = cond | (pass << DPC_PASS);
+    CQ_TRY(prod(pass ? g1 : g0, in_pass | (pass ? DPC_OK : 0)));
+    {
+      ProfScope ps("k_chol_inv", st);
+      const float mp = pass == 0 ? min_pivot : 0.f, again = lowdin ? CE_AGAIN_LD : CE_AGAIN;
+      if (cap.l <= CS_MAXL)
+        k_chol_eq<true><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond);
+      else
+        k_chol_eq<false><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond);
+      CQ_TRY(cudaGetLastError());
+    }
+    CQ_TRY(prod(pass ? q1 : q0, in_pass | DPC_OK));
+  }
+  if (!lowdin) return cudaSuccess;
+  if (lowdin == CQ_PHASES) {
+    ProfScope ps("k_hh_phase", st);
+    k_hh_phase<<<batch, CE_THREADS, 0, st>>>(dims, ptrs, side, cond);
+    CQ_TRY(cudaGetLastError());
+  }
+  CQ_TRY(prod(g1, cond | DPC_OK));
+  {
+    ProfScope ps("k_lowdin", st);
+    k_lowdin64<<<batch, 512, 0, st>>>(dims, ptrs, cond, lowdin == CQ_PHASES);
+    CQ_TRY(cudaGetLastError());
+  }
+  return prod(q1, cond | DPC_OK);
+}
+
+cudaError_t DpPath::qr(int stage, int kind) const {
+  if (!dp || kind == DPQ_LAST0) return launch_qr_sized(stage, dims, ptrs, batch, cap, st);
+  const int side = stage == QR_Y ? 0 : 1;
+  const int check = kind == DPQ_CHECK ? DPC_QFLAG : 0;
+  const bool first = kind == DPQ_FIRST || kind == DPQ_FIRST_LD;
+  const int passes = first ? 3 : (kind == DPQ_CHECK ? 2 : 1);
+  const int lowdin = kind == DPQ_LAST ? CQ_PHASES : (kind == DPQ_CHECK || kind == DPQ_FIRST_LD ? CQ_LOWDIN : 0);
+  const float min_pivot = first ? 0.f : (kind == DPQ_LAST ? CE_AGAIN_LD : CE_PIVOT);
+  CQ_TRY(run_cholqr(side, passes, lowdin, min_pivot, const_cast<Dims*>(dims), ptrs, batch, cap, dp->oz, dp->chunk,
+                    DPC_DIG | check, dp->err, st));
+  if (stage == QR_BH) CQ_TRY(launch_dp_stage(G_X, *this, DPC_DIG | DPC_OK));  // X = B Qb = Rb^H
+  return launch_qr_rest(stage, dims, ptrs, batch, cap, st, check ? QRS_QFLAG_REST : QRS_REST);
 }
 
 }  // namespace tg

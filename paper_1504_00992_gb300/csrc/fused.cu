@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2) k_bond_fused(const ProbPtr* 
     if (p >= batch) break;
     const ProbPtr& P = ptrs[p];  // read through L1 where used: not held in registers
     const bool whole = dims_in == nullptr;
-    const Dims D = whole ? plan_dev(P, p_os) : dims_in[p];
+    const Dims D = whole ? plan_dev(P, p_os, 0) : dims_in[p];
     if (whole && tid == 0) dims[p] = D;  // read by the discarded-weight accumulation
     if (!D.active) continue;
     // theta~ = gate (lam Gamma lam Gamma lam), block by block

@@ -25,7 +25,18 @@ struct Dims {
   int r;           // accuracy check: probes per round (0 = no check)
   int chk;         // accuracy check still running for this problem
   int qflag;       // this round extended the basis: re-orthonormalise it
+  int dig;         // FP64 form: this problem's products and QRs run from digit splits (dp_rule)
+  int cq;          // Cholesky QR: the last pass this problem takes part in
+  int cf;          // Cholesky QR: given up, the Householder QR factors it
 };
+
+// Sizes from which the FP64 form's products and QRs run on the tensor cores
+// from digit splits (oz_proj.cu, cholqr.cu).
+__host__ __device__ inline bool dp_rule(int m, int n, int l) { return l >= 40 && m >= 128 && n >= 128; }
+// A chain handle makes those launches when some bond's capacities are of this
+// size (its smaller bonds of dp_rule's sizes then take them too): the ~80
+// launches of a wave cost ~0.2 ms also while the bonds are still small.
+inline bool dp_handle_rule(int m, int n, int l) { return dp_rule(m, n, l) && (long long)m * n >= 192 * 192; }
 
 struct ProbPtr {
   // operands of the theta contraction (TEBD only)
@@ -76,7 +87,12 @@ enum GemmStage { G_Y0 = 0, G_YT = 1, G_Y = 2, G_BH = 3, G_U = 4, G_V = 5,
                  // Cholesky QR of B^H (the mixed form, cholqr.cu): G1 = B B^H into R,
                  // Q1 = B^H R1^-1 into omega, G2 = Q1^H Q1 into R, Qb = Q1 R2^-1 into Qt,
                  // X = B Qb (= Rb^H) into R; the inverse factors come in J
-                 G_G1 = 9, G_Q1 = 10, G_G2 = 11, G_QB = 12, G_X = 13 };
+                 G_G1 = 9, G_Q1 = 10, G_G2 = 11, G_QB = 12, G_X = 13,
+                 // Cholesky QR of Y into Q (m rows; run_cholqr): G = Y^H Y, Q = (Y S) J,
+                 // G = Q^H Q, Q = (Q S) J, with S the column scales in sigma ...
+                 G_CYG = 14, G_CYQ = 15, G_CQG = 16, G_CQQ = 17,
+                 // ... and of Yt into Qt (n rows)
+                 G_CTG = 18, G_CTQ = 19, G_CRG = 20, G_CRQ = 21 };
 // QR stages: which buffer is factored and where Q goes.
 enum QrStage { QR_Y = 0, QR_YT = 1, QR_BH = 2 };
 
@@ -96,8 +112,16 @@ cudaError_t launch_omega(const Dims* dims, const ProbPtr* ptrs, int batch, const
                          const uint64_t* sweep_dev = nullptr);
 cudaError_t launch_zgemm(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
                          cudaStream_t st);
+// which problems a launch of the one-CTA QR factors: all, those with qflag,
+// those the digit-split Cholesky QR does not (not dig, or cf), or those with cf
+enum { QRS_ALL = 0, QRS_QFLAG = 1, QRS_REST = 2, QRS_QFLAG_REST = 3, QRS_CF = 4 };
+__host__ __device__ inline bool qr_takes(const Dims& D, int which) {
+  if ((which & QRS_QFLAG) && !D.qflag) return false;
+  if ((which & QRS_REST) && D.dig && !D.cf) return false;
+  return !((which & QRS_CF) && !D.cf);
+}
 cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, cudaStream_t st,
-                      int only_flagged = 0);
+                      int which = QRS_ALL);
 // the same, spread over many CTAs per instance (qr_multi.cu) when the batch
 // is a few tall matrices (cap.m or cap.n rows, cap.l columns); every
 // instance's R and J buffers must hold at least qr_multi_scratch_r(l) and
@@ -105,7 +129,10 @@ cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batc
 // force: 0 the size rule, 1 the one-CTA kernel, 2 the many-CTA form wherever
 // its structure allows (the autotuner's choices)
 cudaError_t launch_qr_sized(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
-                           cudaStream_t st, int force = 0);
+                           cudaStream_t st, int force = 0, int which = QRS_ALL);
+// the problems the Cholesky QR left: one CTA each, or the many-CTA form for large ones
+cudaError_t launch_qr_rest(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
+                           cudaStream_t st, int which);
 // true when launch_qr_sized(stage, ..., force) runs the many-CTA form
 bool qr_multi_chosen(int stage, const Caps& cap, int batch, int force);
 size_t qr_multi_scratch_r(int l);
@@ -144,21 +171,25 @@ cudaError_t launch_theta_df(const Dims* dims, const ProbPtr* ptrs, int batch, co
 cudaError_t launch_rrsvd_finalize(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, double cutoff,
                                   double* sigma, double* Vh, double* w, int* rank, int* status, cudaStream_t st);
 
+// Scratch of the FP64 form's digit-split products (mixed.cuh); with it, the
+// problems whose Dims::dig is set take them.
+struct DpScratch;
 // the whole RRSVD from theta to (sigma, Jk, Wk, U, V): Alg. 1 + steps i-iii
 cudaError_t run_rrsvd(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int q, uint64_t seed,
                       uint64_t sweep, int64_t chain0, int chain_stride, int* status, cudaStream_t st,
-                      const uint64_t* sweep_dev = nullptr, const int* tiles = nullptr);
+                      const uint64_t* sweep_dev = nullptr, const int* tiles = nullptr,
+                      const DpScratch* dp = nullptr);
 
 // Accuracy check (Alg. 2) rounds between the first basis of Alg. 1 and the power
 // iterations: rounds = host bound on the number of rounds; l grows on the
 // device; eps the threshold; stream-1 Philox probes.
 cudaError_t run_accuracy_check(const Dims* dims_mut, const ProbPtr* ptrs, int batch, const Caps& cap, int rounds,
                                double eps, int l_max, int p, uint64_t seed, uint64_t sweep, int64_t chain0,
-                               int chain_stride, cudaStream_t st);
+                               int chain_stride, cudaStream_t st, const DpScratch* dp = nullptr, int final_basis = 0);
 // the whole fixed-precision RRSVD (Alg. 1 + Alg. 2 + steps i-iii), FP64
 cudaError_t run_rrsvd_checked(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int q, int rounds,
                               double eps, int l_max, int p, uint64_t seed, int64_t chain0, int* status,
-                              cudaStream_t st);
+                              cudaStream_t st, const DpScratch* dp = nullptr);
 
 cudaError_t launch_finalize_checked(const Dims* dims, const ProbPtr* ptrs, int batch, int kcap, double cutoff,
                                     double* sigma, double* Uout, double* w, int* rank, int* lw, int* status,
@@ -185,7 +216,8 @@ struct ChainDev {
 };
 
 // per-bond sizes of a wave of problems from the current bond dimensions
-cudaError_t launch_plan(const ProbPtr* ptrs, Dims* dims, int batch, int p, cudaStream_t st);
+// (digits: bonds of the sizes of dp_rule get Dims::dig)
+cudaError_t launch_plan(const ProbPtr* ptrs, Dims* dims, int batch, int p, cudaStream_t st, int digits = 0);
 // truncation, renormalisation and Gamma rebuild; w of problem i goes to wout[i]
 cudaError_t launch_rebuild(const Dims* dims, const ProbPtr* ptrs, int batch, double cutoff, double* wout,
                            int* status, cudaStream_t st);

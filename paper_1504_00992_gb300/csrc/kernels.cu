@@ -14,6 +14,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "mixed.cuh"
 #include "profiler.cuh"
 #include "dfsplit.cuh"
 #include "stages.cuh"
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(256) k_zgemm(const Dims* __restrict__ dims, co
   __shared__ cplx Bs[ZG_TK][T + 1];
   const int p = blockIdx.z;
   const Dims D = dims[p];
-  if (!D.active) return;
+  if (!D.active || D.dig) return;  // dig: oz_proj.cu forms this product
   if ((STAGE == G_PR || STAGE == G_PQ || STAGE == G_PD) && !D.chk) return;
   const GemmOp g = gemm_of<STAGE>(D, ptrs[p]);
   const int tm = blockIdx.y * T, tn = blockIdx.x * T;
@@ -276,27 +277,27 @@ cudaError_t launch_zgemm(int stage, const Dims* dims, const ProbPtr* ptrs, int b
 
 template <int QS>
 __global__ void __launch_bounds__(QR_THREADS) k_qr(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
-                                            int only_flagged) {
+                                            int which) {
   __shared__ double red[32];
   __shared__ double tau[QR_MAXL];
   __shared__ cplx alph[QR_MAXL];
   const int p = blockIdx.x;
   const Dims D = dims[p];
   if (!D.active) return;
-  if (only_flagged && !D.qflag) return;
+  if (!qr_takes(D, which)) return;
   qr_dev<QS>(D, ptrs[p], red, tau, alph);
 }
 
 cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, cudaStream_t st,
-                      int only_flagged) {
+                      int which) {
   ProfScope ps("k_qr", st);
   // batches of four matrices per SM or more: 256-thread CTAs, four per SM,
   // so that one matrix's per-column barriers overlap with the others' work
   const int nt = batch >= 4 * 152 ? 256 : QR_THREADS;
   switch (stage) {
-    case QR_Y: k_qr<QR_Y><<<batch, nt, 0, st>>>(dims, ptrs, only_flagged); break;
-    case QR_YT: k_qr<QR_YT><<<batch, nt, 0, st>>>(dims, ptrs, only_flagged); break;
-    case QR_BH: k_qr<QR_BH><<<batch, nt, 0, st>>>(dims, ptrs, only_flagged); break;
+    case QR_Y: k_qr<QR_Y><<<batch, nt, 0, st>>>(dims, ptrs, which); break;
+    case QR_YT: k_qr<QR_YT><<<batch, nt, 0, st>>>(dims, ptrs, which); break;
+    case QR_BH: k_qr<QR_BH><<<batch, nt, 0, st>>>(dims, ptrs, which); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -435,22 +436,26 @@ cudaError_t launch_rrsvd_finalize(const Dims* dims, const ProbPtr* ptrs, int bat
 
 cudaError_t run_rrsvd(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int q, uint64_t seed,
                       uint64_t sweep, int64_t chain0, int chain_stride, int* status, cudaStream_t st,
-                      const uint64_t* sweep_dev, const int* tiles) {
-  auto T = [&](int stage) { return tiles ? tiles[stage] : 0; };
+                      const uint64_t* sweep_dev, const int* tiles, const DpScratch* dp) {
+  // with scratch for them, the problems of dp_rule's sizes take every product
+  // and QR from digit splits (a forced GEMM tile keeps all on the FP64 pipe);
+  // the launches of the others skip them
+  const DpPath P{dims, ptrs, batch, cap, dp, st, tiles};
   TG_TRY(launch_omega(dims, ptrs, batch, cap, seed, sweep, chain0, chain_stride, st, sweep_dev));
-  TG_TRY(launch_zgemm_tile(G_Y0, T(G_Y0), dims, ptrs, batch, cap, st));  // Y0 = A Omega
-  TG_TRY(launch_qr_sized(QR_Y, dims, ptrs, batch, cap, st));              // Y0 = Q0 R0
+  TG_TRY(dp_begin(P));
+  TG_TRY(P.gemm(G_Y0));                              // Y0 = A Omega
+  TG_TRY(P.qr(QR_Y, q == 0 ? DPQ_LAST0 : DPQ_FIRST));  // Y0 = Q0 R0
   for (int j = 0; j < q; ++j) {
-    TG_TRY(launch_zgemm_tile(G_YT, T(G_YT), dims, ptrs, batch, cap, st)); // Y~ = A^H Q
-    TG_TRY(launch_qr_sized(QR_YT, dims, ptrs, batch, cap, st));           // Y~ = Q~ R~
-    TG_TRY(launch_zgemm_tile(G_Y, T(G_Y), dims, ptrs, batch, cap, st));   // Y = A Q~
-    TG_TRY(launch_qr_sized(QR_Y, dims, ptrs, batch, cap, st));            // Y = Q R
+    TG_TRY(P.gemm(G_YT));                            // Y~ = A^H Q
+    TG_TRY(P.qr(QR_YT, DPQ_MID));                    // Y~ = Q~ R~
+    TG_TRY(P.gemm(G_Y));                             // Y = A Q~
+    TG_TRY(P.qr(QR_Y, j + 1 == q ? DPQ_LAST : DPQ_MID));  // Y = Q R
   }
-  TG_TRY(launch_zgemm_tile(G_BH, T(G_BH), dims, ptrs, batch, cap, st));   // B^H = A^H Q
-  TG_TRY(launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st));             // B^H = Qb Rb
-  TG_TRY(launch_jacobi_sized(dims, ptrs, batch, cap, status, st));        // Rb^H J = W S
-  TG_TRY(launch_zgemm_tile(G_U, T(G_U), dims, ptrs, batch, cap, st));     // U = Q J_k
-  TG_TRY(launch_zgemm_tile(G_V, T(G_V), dims, ptrs, batch, cap, st));     // V = Qb W_k  (stored as V^H)
+  TG_TRY(P.gemm(G_BH));                              // B^H = A^H Q
+  TG_TRY(P.qr(QR_BH, DPQ_LAST));                     // B^H = Qb Rb
+  TG_TRY(launch_jacobi_sized(dims, ptrs, batch, cap, status, st));  // Rb^H J = W S
+  TG_TRY(P.gemm(G_U));                               // U = Q J_k
+  TG_TRY(P.gemm(G_V));                               // V = Qb W_k  (stored as V^H)
   TG_TRY(launch_frob2(dims, ptrs, batch, st));
   return cudaSuccess;
 }

@@ -59,7 +59,10 @@ __device__ __forceinline__ float tf32_rna(float x) {
 //     remainder;
 //   BF16 copies of both (the BF16 form's products before the refinement
 //     round), when thf_b / tha_b are set;
-//   the tile partial sums of ||theta||_F^2 (double-float, then FP64).
+//   the tile partial sums of ||theta||_F^2 (double-float, then FP64);
+//   the largest exponent of every column (bsc, zero before), which the digits
+//   of theta are scaled by (a pass of its own over theta took 1.5 ms of the
+//   152 x 2000 x 2000 step).
 // The tiles cover the zero padding of every copy.
 // ---------------------------------------------------------------------------
 // double-float pair sum (Knuth's TwoSum on the high words)
@@ -75,6 +78,7 @@ __device__ __forceinline__ void df_add2(float& h, float& l, float oh, float ol) 
 __global__ void __launch_bounds__(256) k_conv_theta(const MixedPtrs mp, const Dims* __restrict__ dims,
                                                     const ProbPtr* __restrict__ ptrs, int mc, int nc, int K1, int K2,
                                                     int want_lo, int K1b, int K2b) {
+  __shared__ int emax[32];  // largest biased exponents of the tile's columns (the digits' scales)
   __shared__ float2 tile[32][33];  // TF32 hi and remainder computed once per element
   __shared__ float2 tlo[32][33];
   __shared__ unsigned tb16[32][33];  // BF16 (Re, Im) pairs of the BF16 copies
@@ -93,10 +97,14 @@ __global__ void __launch_bounds__(256) k_conv_theta(const MixedPtrs mp, const Di
   unsigned* ab = mp.tha_b ? reinterpret_cast<unsigned*>(mp.tha_b + (size_t)z * nc * K2b) : nullptr;
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  if (ty == 0) emax[tx] = 0;
+  __syncthreads();
+  int ex = 0;
   float sh = 0.f, sl = 0.f;  // double-float sum of |theta|^2 over this thread's elements
   for (int i = ty; i < 32; i += 8) {
     const int r = r0 + i, c = c0 + tx;
     const cplx v = (r < m && c < n) ? th[(int64_t)r * n + c] : cmk(0.0, 0.0);
+    ex = max(ex, max(oz_exp(v.x), oz_exp(v.y)));
     float xh, xl, yh, yl;
     split_bits(v.x, xh, xl);
     split_bits(v.y, yh, yl);
@@ -127,7 +135,9 @@ __global__ void __launch_bounds__(256) k_conv_theta(const MixedPtrs mp, const Di
     red[2 * ty] = sh;
     red[2 * ty + 1] = sl;
   }
+  atomicMax(&emax[tx], ex);
   __syncthreads();
+  if (ty == 1 && c0 + tx < n && r0 < m) atomicMax(&mp.bsc[(size_t)z * nc + c0 + tx], emax[tx]);
   if (threadIdx.x == 0) {
     float h = red[0], l = red[1];
     for (int w = 1; w < 8; ++w) df_add2(h, l, red[2 * w], red[2 * w + 1]);
@@ -473,9 +483,9 @@ MixedSizes mixed_sizes(int m, int n, int k, int l, int bf16, const Caps* gate) {
   s.df = (size_t)l * l * sizeof(float2);
   // the projection runs on the tensor cores from BF16 digits (oz_proj.cu)
   s.bd = oz_digits_bytes(n, m);
-  s.bsc = oz_scales_bytes(n, m);
-  s.ad = oz_digits_bytes(l, m);
-  s.asc = oz_scales_bytes(l, m);
+  s.bsc = oz_scales_bytes(n);
+  s.ad = oz_digits_q_bytes(l, m);
+  s.asc = oz_scales_bytes(l);
   s.thfb = s.bf16 ? (size_t)m * s.K1b * 2 : 0;
   s.thab = s.bf16 ? (size_t)n * s.K2b * 2 : 0;
   s.btb = s.bf16 ? (size_t)s.Np * (s.K1b > s.K2b ? s.K1b : s.K2b) * 2 : 0;
@@ -528,16 +538,16 @@ MixedPtrs mixed_carve(char* base, const MixedSizes& s, int batch) {
   p.qscr = s.qs ? (float2*)(base + o) : nullptr;
   o += up256(s.qs * batch);
   p.bd = (uint16_t*)(base + o); o += up256(s.bd * batch);
-  p.bsc = (float*)(base + o); o += up256(s.bsc * batch);
+  p.bsc = (int*)(base + o); o += up256(s.bsc * batch);
   p.ad = (uint16_t*)(base + o); o += up256(s.ad * batch);
-  p.asc = (float*)(base + o); o += up256(s.asc * batch);
+  p.asc = (int*)(base + o); o += up256(s.asc * batch);
   p.thf_b = s.bf16 ? (uint16_t*)(base + o) : nullptr; o += up256(s.thfb * batch);
   p.tha_b = s.bf16 ? (uint16_t*)(base + o) : nullptr; o += up256(s.thab * batch);
   p.bt_b = s.bf16 ? (uint16_t*)(base + o) : nullptr; o += up256(s.btb * batch);
   p.gad = (uint16_t*)(base + o); o += up256(s.gad * batch);
-  p.gas = (float*)(base + o); o += up256(s.gas * batch);
+  p.gas = (int*)(base + o); o += up256(s.gas * batch);
   p.gbd = (uint16_t*)(base + o); o += up256(s.gbd * batch);
-  p.gbs = (float*)(base + o); o += up256(s.gbs * batch);
+  p.gbs = (int*)(base + o); o += up256(s.gbs * batch);
   return p;
 }
 
@@ -675,6 +685,24 @@ cudaError_t mixed_prepare(const Caps& cap) {
   return qr_blocked_prepare(cap.m, cap.n, cap.l);
 }
 
+// The QR of B^H where no choice is set.  On the tensor cores the Cholesky QR
+// (with Householder per ill-conditioned instance) also takes the few tall
+// matrices the many-CTA FP64 Householder ran before: 8 x 2000 x 120 in 1.3 ms
+// against 21 ms, 16 x 7700 x 262 in 5 ms against 28 ms.
+int mixed_qrbh(const MixedKnobs& kn, const Caps& cap, int batch) {
+  if (kn.qrbh) return kn.qrbh;
+  const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));
+  return tc || !qr_multi_chosen(QR_BH, cap, batch, 0) ? 3 : 2;
+}
+
+// The Jacobi SVD where no choice is set: double-float on one CTA, or for a few
+// wide instances FP64 over a cluster (l = 120: 10 ms for up to 152 instances
+// on one CTA each, 14 ms for 16 on clusters; l = 262: ~100 ms against 21 ms).
+int mixed_jac(const MixedKnobs& kn, const Caps& cap, int batch) {
+  if (kn.jac) return kn.jac;
+  return cap.l > 160 && jacobi_cluster_chosen(cap, batch, 0) ? 2 : 3;
+}
+
 cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, const MixedPtrs& mp,
                             int q, uint64_t seed, uint64_t sweep, int64_t chain0, int chain_stride, int* status,
                             int* err, cudaStream_t st, const uint64_t* sweep_dev, const MixedKnobs* knobs,
@@ -691,6 +719,7 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
     ProfScope ps("k_conv_theta", st);
     // padded extents (>= n, >= m) of every copy written
     const int cext = (bf && s.K1b > s.K1 ? s.K1b : s.K1) / 2, rext = (bf && s.K2b > s.K2 ? s.K2b : s.K2) / 2;
+    MX_TRY(cudaMemsetAsync(mp.bsc, 0, s.bsc * batch, st));
     MixedPtrs mq = mp;
     if (!bf) mq.thf_b = mq.tha_b = nullptr;
     const dim3 grid((cext + 31) / 32, (rext + 31) / 32, batch);  // grid.x * grid.y <= s.ntile
@@ -746,28 +775,31 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   // every basis they pass fits it.
   if (!reorth_fits(m, l)) return cudaErrorInvalidValue;
   MX_TRY(qr_f32(mp.Yf, mp.Qf, m, l, batch, mp, s, dims, 0, st, kn.qr_threads));
-  // digits of Q_f once: the Gram of the re-orthonormalisation and the
-  // projection B^H = A^H Q both take them
-  MX_TRY(launch_oz_digits_qf(dims, mp.Qf, mp.ad, mp.asc, m, l, batch, st));
-  MX_TRY(launch_oz_gram(dims, ptrs, mp.ad, mp.asc, m, l, batch, err, st));
-  MX_TRY(launch_reorth(mp.Qf, mp.Df, dims, ptrs, m, l, batch, status, st));
-  MX_TRY(launch_proj_oz(dims, ptrs, mp.Qf, mp.Df, mp.ad, mp.asc, mp.bd, mp.bsc, m, n, l, batch, err, st,
-                        true));  // B^H = A^H Q
-  // QR of B^H: Cholesky QR where the one-CTA Householder would run (it falls
-  // back to Householder per ill-conditioned instance), else the size rule
   // the FP64-accurate products after the projection: tensor cores from digit
   // splits, or double-float GEMMs on the CUDA cores
   const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));
   const OzScratch oz{mp.gad, mp.gas, mp.gbd, mp.gbs};
-  if (kn.qrbh == 3 || (kn.qrbh == 0 && !qr_multi_chosen(QR_BH, cap, batch, 0)))
+  // digits of Q_f once: the Gram of the re-orthonormalisation and the
+  // projection A^H Q_f both take them
+  MX_TRY(launch_oz_digits_qf(dims, ptrs, mp.Qf, mp.ad, mp.asc, m, l, batch, st));
+  MX_TRY(launch_oz_gram(dims, ptrs, mp.ad, mp.asc, m, l, batch, err, st));
+  MX_TRY(launch_reorth(mp.Qf, mp.Df, dims, ptrs, m, l, batch, status, st, !tc));
+  MX_TRY(launch_proj_oz(dims, ptrs, mp.ad, mp.asc, mp.bd, mp.bsc, m, n, l, batch, err, st));  // A^H Q_f
+  // QR of it (mixed_qrbh); then Rb^H of B^H = A^H Q_f (I + D) is (I + D) times what it gives (folding
+  // I + D into the n x l and m x l matrices instead took 6.3 ms of the 92 ms
+  // step of 152 x 2000 x 2000, folding it into the small ones 0.2 ms)
+  if (mixed_qrbh(kn, cap, batch) == 3)
     MX_TRY(run_cholqr_bh(const_cast<Dims*>(dims), ptrs, batch, cap, st, tc ? &oz : nullptr, err));
   else
-    MX_TRY(launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st, kn.qrbh));
+    MX_TRY(launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st, mixed_qrbh(kn, cap, batch)));
+  MX_TRY(launch_fold_small(mp.Df, dims, ptrs, l, k, batch, 0, st));
   // Jacobi SVD: double-float one-CTA kernel unless the cluster form is chosen
-  if (kn.jac == 3 || (kn.jac == 0 && !jacobi_cluster_chosen(cap, batch, 0)))
+  const int jac = mixed_jac(kn, cap, batch);
+  if (jac == 3)
     MX_TRY(launch_jacobi_df(dims, ptrs, batch, cap.l, status, st));
   else
-    MX_TRY(launch_jacobi_sized(dims, ptrs, batch, cap, status, st, kn.jac));
+    MX_TRY(launch_jacobi_sized(dims, ptrs, batch, cap, status, st, jac));
+  if (tc) MX_TRY(launch_fold_small(mp.Df, dims, ptrs, l, k, batch, 1, st));  // U = Q_f (I + D) J_k
   for (int stage : {G_U, G_V})
     MX_TRY(tc ? launch_oz_stage(stage, dims, ptrs, batch, cap, oz, err, st)
               : launch_zgemm_df(stage, dims, ptrs, batch, cap, st));

@@ -16,7 +16,7 @@ struct MixedSizes {
   int Np;        // 2l rounded up to 16: rows of Bt (tensor-core N)
   int BN;        // tensor-core tile width, min(Np, 256)
   size_t thf, tha, bt, yf, ytf, df;  // bytes per instance
-  size_t bd, bsc, ad, asc;  // BF16 digits and block scales of theta and of Q_f^H (tensor-core projection)
+  size_t bd, bsc, ad, asc;  // BF16 digits and row exponents of theta and of Q_f^H (tensor-core projection)
   size_t thfb, thab, btb;   // BF16 copies of theta, theta^H and Bt (bf16 only)
   size_t gad, gas, gbd, gbs;  // digit scratch of the other tensor-core products (oz_stage_bytes)
   size_t qs;     // bytes per instance of the many-CTA FP32 QR's scratch (0: not used)
@@ -37,16 +37,16 @@ struct MixedPtrs {
   float2* Qtf;
   float2* Df;     // l x l correction of the re-orthonormalisation
   uint16_t* bd;   // digits of theta for the tensor-core projection (oz_proj.cu)
-  float* bsc;     // their block scales
+  int* bsc;       // their rows' largest exponents
   uint16_t* ad;   // digits of Q_f^H
-  float* asc;
+  int* asc;
   uint16_t* thf_b;  // m x K1b BF16 theta (bf16 form), or null
   uint16_t* tha_b;  // n x K2b BF16 theta^H
   uint16_t* bt_b;   // Np x max(K1b, K2b) BF16 right operand
   uint16_t* gad;  // digit scratch of the Cholesky QR and U / V products (OzScratch)
-  float* gas;
+  int* gas;
   uint16_t* gbd;
-  float* gbs;
+  int* gbs;
   double* tpart;  // ntile partial sums of |theta|^2 per instance
   float2* qscr;   // scratch of the many-CTA FP32 QR (qs bytes per instance), or null
 };
@@ -75,31 +75,35 @@ bool qr_multi_f32_fits(int M, int L);
 size_t qr_multi_f32_scratch(int M, int L);
 cudaError_t launch_qr_multi_f32(float2* A, float2* Q, float2* scr, size_t stride, int M, int L, int batch,
                                 cudaStream_t st, const Dims* dims = nullptr, int use_n = 0);
-// Q_f (FP32, M x L) -> ptrs[z].Q (FP64) orthonormal to ~1e-13, spanning
-// range(Q_f), from E = Q_f^H Q_f - I already in ptrs[z].R (launch_oz_gram);
-// usable when reorth_fits(M, L).
+// The correction D of the re-orthonormalisation Q = Q_f (I + D) (FP64
+// orthonormal to ~1e-13, spanning range(Q_f)) from E = Q_f^H Q_f - I already in
+// ptrs[z].R (launch_oz_gram); with fold, Q itself into ptrs[z].Q; usable when
+// reorth_fits(M, L).
 bool reorth_fits(int M, int L);
 cudaError_t launch_reorth(const float2* Qf, float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int M, int L,
-                          int batch, int* status, cudaStream_t st);
-// B^H <- B^H (I + D) in place on ptrs[z].Yt (qr_blocked.cu).
-cudaError_t launch_fold_bh(const float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int n, int l, int batch,
-                           cudaStream_t st);
+                          int batch, int* status, cudaStream_t st, bool fold);
+// X <- (I + D) X on the l x l matrix ptrs[z].R (jk = 0: Rb^H of B^H = A^H Q_f
+// (I + D) from that of A^H Q_f) or the l x k ptrs[z].Jk (jk = 1: the left
+// factors of U = Q_f (I + D) J_k).
+cudaError_t launch_fold_small(const float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int l, int k, int batch,
+                              int jk, cudaStream_t st);
 
-// B^H = A^H Q_f (I + D) into ptrs[z].Yt on the tensor cores from BF16 digits
-// (oz_proj.cu): launch_oz_digits_theta once theta is in place, launch_proj_oz
-// after launch_reorth.  Arrays at capacities m x n (theta) and m x l (Q_f).
+// A^H Q_f into ptrs[z].Yt on the tensor cores from BF16 digits (oz_proj.cu):
+// launch_oz_digits_theta once theta is in place, launch_oz_digits_qf, then
+// launch_proj_oz.  Arrays at capacities m x n (theta) and m x l (Q_f).
 int oz_kpad(int m);
 size_t oz_digits_bytes(int rows, int m);
-size_t oz_scales_bytes(int rows, int m);
+size_t oz_digits_q_bytes(int rows, int m);  // of the FP32 basis (four digits)
+size_t oz_scales_bytes(int rows);
 cudaError_t oz_prepare();
 // The other FP64-accurate products on the tensor cores (GemmStage G_G1 ..
 // G_X of the Cholesky QR, G_U, G_V): digit scratch of both operands, sized
 // by oz_stage_bytes for the capacities, reused by every stage.
 struct OzScratch {
   uint16_t* ad;
-  float* as;
+  int* as;
   uint16_t* bd;
-  float* bs;
+  int* bs;
 };
 struct OzStageBytes {
   size_t ad, as, bd, bs;  // per instance
@@ -113,10 +117,62 @@ OzStageBytes oz_stage_bytes(int m, int n, int k, int l, const Caps* gate = nullp
 enum { OZ_THETA_STAGE = 102, OZ_GATE_STAGE = 103 };
 bool oz_gate_rule(const Caps& cap);
 cudaError_t launch_oz_stage(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
-                            const OzScratch& sc, int* err, cudaStream_t st);
+                            const OzScratch& sc, int* err, cudaStream_t st, int cond = 0);
 // the size rule of MixedKnobs::dfg: the tensor-core products for bonds whose
 // products are deep and wide enough to fill the digit-pair pipeline
 bool oz_stage_rule(const Caps& cap);
+
+// --- the FP64 form on the tensor cores -------------------------------------
+// Scratch of its digit-split products: theta's digits in both directions
+// (tr: its rows, tc: its columns) and those of the other operands, for
+// `chunk` problems at a time.  all: every problem of the batch has its theta
+// digits (made once per truncation); otherwise tr and tc are one buffer,
+// filled before each product for a chunk of problems.
+struct DpScratch {
+  OzScratch oz;
+  uint16_t *tr, *tc;
+  int *er, *ec;
+  int chunk, all;
+  int* err;  // tensor-core wait timeout flag
+};
+// Bytes for `batch` problems of capacities cap, at most `limit` or what one problem needs.
+size_t dp_bytes(const Caps& cap, int batch, size_t limit);
+DpScratch dp_carve(char* base, const Caps& cap, int batch, size_t limit, int* err);
+enum : size_t { DP_LIMIT = (size_t)6 << 30 };  // the FP64 form's scratch: enough to fill the GPU with large problems
+
+// Which QR of Alg. 1 a launch is: the first (of A Omega, as ill-conditioned as
+// A), a middle one, the last before the projection (or of B^H), or the first
+// when it is the last too.
+// (FIRST_LD, CHECK: the bases of the accuracy check, orthonormal to FP64)
+enum { DPQ_FIRST = 0, DPQ_MID = 1, DPQ_LAST = 2, DPQ_LAST0 = 3, DPQ_CHECK = 4, DPQ_FIRST_LD = 5 };
+
+// One truncation's launches: products and QRs on whichever path takes each problem.
+struct DpPath {
+  const Dims* dims;
+  const ProbPtr* ptrs;
+  int batch;
+  const Caps& cap;
+  const DpScratch* dp;
+  cudaStream_t st;
+  const int* tiles;
+  cudaError_t gemm(int stage) const;
+  cudaError_t qr(int stage, int kind) const;
+};
+cudaError_t dp_begin(const DpPath& p);  // theta's digits, when they are kept
+// one digit-split product of the problems selected by cond: bits, and from
+// bit 8 up the pass of a Cholesky QR (the problems that take part in it)
+enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_PASS = 8 };
+cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
+// Cholesky QR of Y into Q (side 0) or Yt into Qt (side 1) (cholqr.cu): up to
+// `passes` passes, then, with lowdin, the symmetric orthonormalisation to
+// FP64 (CQ_PHASES: with the column phases of the Householder QR);
+// min_pivot: the smallest pivot of the scaled Gram matrix accepted in a first
+// pass (0: any, by shifted passes).  Problems given up have cf set.
+enum { CQ_LOWDIN = 1, CQ_PHASES = 2 };
+cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* dims, const ProbPtr* ptrs, int batch,
+                       const Caps& cap, const OzScratch& oz, int chunk, int cond, int* err, cudaStream_t st);
+cudaError_t launch_oz_range(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
+                            const OzScratch& sc, int chunk, int cond, int* err, cudaStream_t st);
 
 // Cholesky QR (two passes) of B^H for well-conditioned instances, Householder
 // for the others (cholqr.cu); writes dims[p].qflag.  oz: the products on the
@@ -125,18 +181,19 @@ bool oz_stage_rule(const Caps& cap);
 cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
                           const OzScratch* oz, int* err);
 cudaError_t cholqr_prepare();
-cudaError_t launch_oz_digits_theta(const Dims* dims, const ProbPtr* ptrs, uint16_t* Bd, float* Bs, int m, int n,
+cudaError_t launch_oz_digits_theta(const Dims* dims, const ProbPtr* ptrs, uint16_t* Bd, int* Bs, int m, int n,
                                    int batch, cudaStream_t st);
-// (digits_done: Q_f's digits already in Ad / As from launch_oz_digits_qf)
-cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const float2* Qf, const float2* Dbuf,
-                           uint16_t* Ad, float* As, const uint16_t* Bd, const float* Bs, int m, int n, int l, int batch,
-                           int* err, cudaStream_t st, bool digits_done = false);
-// Digits of conj(Q_f) (the projection's left operand) into Ad / As, and the
+// (Q_f's digits in Ad / As from launch_oz_digits_qf)
+cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const int* As,
+                           const uint16_t* Bd, const int* Bs, int m, int n, int l, int batch, int* err,
+                           cudaStream_t st);
+// Digits of Q_f (the projection's left operand, conjugated by the MMAs; Q_f's
+// entries are rounded to what its four digits hold) into Ad / As, and the
 // Gram matrix E = Q_f^H Q_f - I of the re-orthonormalisation from them into
 // ptrs[z].R (l x l column-major), FP64-accurate, on the tensor cores.
-cudaError_t launch_oz_digits_qf(const Dims* dims, const float2* Qf, uint16_t* Ad, float* As, int m, int l, int batch,
+cudaError_t launch_oz_digits_qf(const Dims* dims, const ProbPtr* ptrs, float2* Qf, uint16_t* Ad, int* As, int m, int l, int batch,
                                 cudaStream_t st);
-cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const float* As, int m, int l,
+cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const int* As, int m, int l,
                            int batch, int* err, cudaStream_t st);
 
 // Launch choices of the mixed form that the autotuner may override (0 keeps
@@ -154,6 +211,11 @@ cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t
 struct MixedKnobs {
   int tc_half, qr_threads, qrbh, jac, dfg;
 };
+
+// The choices a launch on `batch` problems of capacities cap makes (a set knob,
+// or the size rule): the QR of B^H (1, 2 or 3) and the Jacobi SVD.
+int mixed_qrbh(const MixedKnobs& kn, const Caps& cap, int batch);
+int mixed_jac(const MixedKnobs& kn, const Caps& cap, int batch);
 
 // Everything that must happen outside a stream capture before
 // run_rrsvd_mixed runs on capacities `cap` (shared-memory limits, the

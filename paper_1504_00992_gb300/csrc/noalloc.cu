@@ -95,7 +95,7 @@ extern "C" int rrsvd_execute_noalloc(int m, int n, int k_max, int p, int q, int 
     ProfScope ps("k_rrsvd_bind", st);
     k_rrsvd_bind<<<(batch + 127) / 128, 128, 0, st>>>(ptrs, batch, ws, lay.total, lay, (const cplx*)theta,
                                                        (size_t)m * n, (cplx*)U, (size_t)m * k, (cplx*)Vh,
-                                                       (size_t)k * n, dims, m, n, k, l, status);
+                                                       (size_t)k * n, dims, m, n, k, l, 0, status);
   }
   if (cudaGetLastError() != cudaSuccess) return TEBD_ECUDA;
   Caps cap;

@@ -2,39 +2,45 @@
 //
 // The step B = Q^H A of Section IV (after Alg. 1), in the mixed form with the
 // FP32 basis Q_f and its re-orthonormalisation Q = Q_f (I + D): C = Q_f^H A
-// (l x n) is formed from error-free slices of both operands, then
-// B^H = C^H (I + D) (the fold of qr_blocked.cu).
+// (l x n) is formed from error-free slices of both operands; the factor I + D
+// is applied to the l x l matrices after it (launch_fold_small, qr_blocked.cu).
 //
 // Slices (Ozaki's error-free splitting; Ozaki, Ogita, Oishi, Rump, Numer.
-// Algorithms 59, 2012): within each block of OZ_KB consecutive k, every row i
-// of Q_f^H and every column j of A is scaled by a power of two s so that the
-// block's entries x satisfy |x| < s 2^8, and x / s is cut into OZ_S = 6
-// signed 8-bit digits d_1 .. d_6 (x = s (d_1 + d_2 2^-8 + ... ), truncated
-// after 48 bits).  Digit t is stored as the BF16 number d_t 2^-8(t-1) (exact:
-// 8 significant bits).  A product of digits t and u is then an integer times
-// 2^-8(t+u-2) below 2^16 in that unit, and the tensor core sums them in FP32
-// exactly as long as each sum stays below 2^24 units.  Per block of
-// OZ_DRAIN = 32 k, with 2 real products per digit pair and k for C_r or C_i:
-//   level 2 (t + u = 2): one digit pair, 64 products: exact;
-//   level 3: two pairs, 128 products; level 4: three pairs, 192 products;
-//   level 5: four pairs, 256 products (< 2^23.99 units): all exact;
-//   levels 6 and 7: five and six pairs, rounded in FP32 (each rounding 2^-56
-//   of the level-2 sum or less); digit pairs with t + u > 7 are dropped
-//   (2^-48 relative).
-// Each block therefore runs into twelve accumulators in tensor memory (C_r
-// and C_i at levels 2 .. 7), which the epilogue warps read after every block,
-// scale by the two block scales and add into double-float (FP32 pair) sums in
-// registers.  Measured on 40-bit digits with levels 4 .. 6 in one
-// inexact group: ~3e-10 relative (some 10^4 roundings of 2^-40 per output of
-// a 2000-deep product add up like a random walk); with level 4 exact, 1.4e-11
-// (the 40-bit truncation of the digits).  With 48-bit digits and levels 2 .. 5
-// exact the roundings left are 2^-56 (levels 6+) and 2^-48 (combining the
-// levels once per block): FP64-accurate, like the double-float path it
-// replaces (~1e-14).
+// Algorithms 59, 2012): every row i of the left operand and every column j of
+// the right one is scaled by its own power of two (the exponent of its
+// largest entry over all k) to a 56-bit integer N, |N| <= 2^55, rounded to
+// nearest, and N is cut into OZ_S = 7 balanced base-256 digits, |d_t| <= 128
+// (N = sum_t d_t 256^(7-t)), each an exact BF16 number.  A product of two
+// digits is an integer of at most 2^14, and level L = t + u of the digit
+// pairs sums at most L - 1 pairs x 2 real products x k of them, so over
+// OZ_DRAIN = 64 k every level up to 8 stays below 128 * 7 * 2^14 < 2^24: the
+// tensor core's FP32 sums are exact integers.  The epilogue reads the
+// fourteen accumulators (C_r and C_i at levels 2 .. 8) after every 64 k and
+// adds them exactly: levels 2 .. 6 into one 64-bit integer, levels 7 and 8
+// (2^-40 and 2^-48 of the leading level) into one FP32 number.  The scales
+// are applied once at the end.  What is lost is the rounding of the operands
+// (2^-56 of a row's largest entry) and the digit pairs with t + u > 8
+// (2^-56 of the largest product, random signs): on a CPU emulation 1.8e-16
+// relative at K = 64 and 3e-16 at K = 2000 for Gaussian or orthonormal
+// operands, against 3e-16 and 1.5e-15 of FP64 multiply-adds in order; rows
+// graded over 2^-46 give 1.4e-15 against 2e-15.  Six digits would give
+// 4e-14 to 8e-14, eight would cost 36 digit pairs instead of 28 for accuracy
+// FP64 results cannot hold.
+//
+// What bounds it.  An MMA of M = 128 costs ~130 cycles whatever its N up to 256
+// (timed with every N set to 32: 10% less), so the 28 MMAs of a k step of 16
+// are ~3600 cycles, and the 72 KB of digits of a k step take about as long at
+// the 38 GB/s per SM the copies reach alone.  Tensor memory holds no wider
+// tile than 32 columns of fourteen sums.  At 16 x 2000 x 2000 x 120 a product
+// takes 1.6 ms (38 TFLOP/s FP64-equivalent; the FP64 pipe 54 ms), the read-out
+// of the accumulators (which nothing overlaps) 0.35 ms of it.  Tried and not
+// kept: reading out C_r while C_i is filled (stages held longer: 15% slower),
+// clusters sharing the left operand by multicast (same time), TMA tiles (32-
+// byte rows: 10% slower).
 //
 // Complex products: C_r = Ar Br - Ai Bi, C_i = Ar Bi + Ai Br with Ar, Ai the
-// digits of Re and Im of Q_f^H (the conjugate folded in) and Br, Bi those of
-// A; the minus sign is the MMA's negate-A bit.
+// digits of Re and Im of the left operand and Br, Bi those of the right one;
+// minus signs, and the conjugate of either operand, are the MMA's negate-A bit.
 //
 // The same kernel serves the other FP64-accurate products of the mixed form
 // (k_oz_gemm<stage>): the Cholesky QR of B^H (Gram matrices B B^H and
@@ -44,19 +50,18 @@
 // digits, and a conjugated left operand flips the negate bits of the MMAs
 // that take its imaginary digits instead of negating them.
 //
-// Kernel structure (one CTA = 128 rows of C (l) x OZ_BN = 32 columns (n), all
-// k): warp 0 lane 0 streams the digit tiles of each 16-deep k step with 5-D
-// TMA loads (k, row, digit, re/im, instance; 32-byte swizzle) into a ring of
-// OZ_STAGES stages; warp 1 lane 0 issues 24 tcgen05.mma.kind::f16 per k step:
-// the digit planes u = 1 .. 6 of a part of A's side lie one after another in
-// shared memory and the accumulators of levels 2 .. 7 one after another in
-// tensor memory, so digit t of the other operand times planes 1 .. 7 - t is
-// one MMA of N = 32 (7 - t) into the accumulators of levels t + 1 .. 7 (six
-// MMAs per real product instead of 21 small ones); warps 2 .. 17 read the
-// accumulators after each k block (warp w reads TMEM lanes 32 (w % 4) .. +31
-// and a quarter of the columns) and keep the double-float sums.  Every mbarrier wait is
-// bounded; on expiry the kernel raises *err, waits for its own copies and
-// MMAs, and frees its tensor memory.
+// Kernel structure (one CTA = 128 rows of C x OZ_BN = 32 columns, all k):
+// warp 0 streams the digit planes of each 16-deep k step with bulk copies
+// (the digit arrays are stored step by step, swizzled for the MMAs) into a
+// ring of stages; warp 1 issues 28 tcgen05.mma.kind::f16 per k step:
+// the digit planes u = 1 .. 7 of a part of B's side lie one after another in
+// shared memory and the accumulators of levels 2 .. 8 one after another in
+// tensor memory, so digit t of the other operand times planes 1 .. 8 - t is
+// one MMA of N = 32 (8 - t) into the accumulators of levels t + 1 .. 8; warps
+// 2 .. 17 read the accumulators after each 64 k (warp w reads TMEM lanes
+// 32 (w % 4) .. +31 and a quarter of the columns) and keep the sums.  Every
+// mbarrier wait is bounded; on expiry the kernel raises *err, waits for its
+// own copies and MMAs, and frees its tensor memory.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -76,177 +81,90 @@
 namespace tg {
 
 enum {
-  OZ_S = 6,        // digits per operand
-  OZ_KB = 64,      // k per block of the digit scales
-  OZ_DRAIN = 32,   // k per exact accumulation (the accumulators are read and cleared after each)
+  OZ_S = 7,        // digits per operand
+  OZ_KB = 64,      // k padding of the digit arrays
   OZ_KS = 16,      // k per MMA / TMA stage
   OZ_BM = 128,     // rows of C per CTA (TMEM lanes)
   OZ_BN = 32,      // columns of C per CTA
-  OZ_STAGES = 3,
+  OZ_DRAIN = 64,   // k per exact accumulation (the accumulators are read and cleared after each)
+  OZ_SQ = 4,       // digits of the FP32 basis Q_f
   OZ_EPI_WARPS = 16,  // four per TMEM lane quadrant, 8 columns each
   OZ_THREADS = 64 + 32 * OZ_EPI_WARPS,
-  OZ_NGRP = OZ_S,  // accumulators per part: levels 2 .. 7
-  OZ_TMEM_COLS = 512  // twelve 32-column accumulators, rounded up to a power of two
+  OZ_NGRP = OZ_S,  // accumulators per part: levels 2 .. 8
+  OZ_TMEM_COLS = 512,  // fourteen 32-column accumulators, rounded up to a power of two
+  OZ_FLUSH = 256,  // blocks after which the integer sums move to FP64 (level 2: below 2^53 per block)
+  OZ_SELF_K = 512  // depths up to this: the digit kernels find a row's largest exponent themselves
 };
 
-static const uint32_t OZ_A_TILE = OZ_BM * OZ_KS * 2;  // one digit tile of Q_f^H: 4 KB
-static const uint32_t OZ_B_TILE = OZ_BN * OZ_KS * 2;  // one digit tile of A: 1.5 KB
-static const uint32_t OZ_A_STAGE = 2 * OZ_S * OZ_A_TILE;
-static const uint32_t OZ_B_STAGE = 2 * OZ_S * OZ_B_TILE;
-
+static const uint32_t OZ_A_TILE = OZ_BM * OZ_KS * 2;  // one digit tile of the left operand: 4 KB
+static const uint32_t OZ_B_TILE = OZ_BN * OZ_KS * 2;  // one digit tile of the right operand: 1 KB
 
 // ---------------------------------------------------------------------------
-// Digits.  An FP64 or FP32 value and the block's largest biased exponent E
-// give a 48-bit fixed-point magnitude N (x = +-N 2^(E - bias - mantissa - 5)
-// for FP64), cut into six 8-bit digits, each stored as the BF16 number
-// +-d_t 2^-8(t-1) (bit pattern built from FP32 arithmetic that is exact).
+// Digits of one value relative to its row's largest biased FP64 exponent E:
+// N = rint(x 2^(54 - (E - 1023))) with integer operations only (the FP64 pipe
+// runs at 1/64 of the FP32 rate), then balanced base-256 digits: adding 128
+// to each of the six lower digits makes them plain bytes.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint16_t oz_bf16_digit(unsigned d, int t, bool neg) {
-  const float f = (float)d * __uint_as_float((unsigned)(127 - 8 * t) << 23);  // d 2^-8t, exact
-  const unsigned u = __float_as_uint(f) >> 16;
-  return (uint16_t)(u | (neg && d ? 0x8000u : 0u));
-}
-
-// 48-bit magnitude of an FP64 value relative to block exponent E (biased).
-__device__ __forceinline__ uint64_t oz_n48_f64(double x, int E) {
+__device__ __forceinline__ int64_t oz_fix(double x, int E) {
   const uint64_t u = (uint64_t)__double_as_longlong(x);
   const int e = (int)((u >> 52) & 0x7FF);
-  if (e == 0 || e == 0x7FF) return 0;  // zero, subnormal (negligible), non-finite (flagged elsewhere)
-  const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = E - e + 5;  // >= 5
-  return sh >= 64 ? 0 : (m >> sh);
+  if (e == 0 || e == 0x7FF) return 0;
+  const int64_t m = (int64_t)((u & 0xFFFFFFFFFFFFFull) | (1ull << 52));
+  const int sh = E - e - 2;  // x = m 2^(e - 1075), N = m 2^-sh; sh >= -2
+  const int64_t n = sh <= 0 ? (m << (-sh)) : (sh >= 56 ? 0 : ((m + (1ll << (sh - 1))) >> sh));
+  return (u >> 63) ? -n : n;
 }
-
-__device__ __forceinline__ uint64_t oz_n48_f32(float x, int E) {
+// N = rint(x 2^(30 - (E - 1023))) of an FP32 value, |N| < 2^31 (E the row's largest exponent)
+__device__ __forceinline__ int64_t oz_fix31(float x, int E) {
   const unsigned u = __float_as_uint(x);
   const int e = (int)((u >> 23) & 0xFF);
   if (e == 0 || e == 0xFF) return 0;
-  const uint64_t m = (uint64_t)((u & 0x7FFFFFu) | 0x800000u);
-  const int sh = e - E + 24;  // <= 24
-  return sh >= 0 ? (m << sh) : ((-sh) >= 64 ? 0 : (m >> (-sh)));
+  const int m = (int)((u & 0x7FFFFFu) | 0x800000u);
+  const int sh = E - (e - 127 + 1023) - 7;  // x = m 2^(e - 150), N = m 2^-sh; sh >= -7
+  const int n = sh <= 0 ? (m << (-sh)) : (sh >= 26 ? 0 : ((m + (1 << (sh - 1))) >> sh));
+  return (u >> 31) ? -n : n;
 }
 
-// Scale 2^(E - off) as an FP32 number, or 0 when it is below the normal range
-// (the whole block is then negligible and its digits are zero).
-__device__ __forceinline__ float oz_scale(int E, int off) {
-  const int b = E - off + 127;
-  return (b >= 1 && b <= 254) ? __uint_as_float((unsigned)b << 23) : 0.f;
-}
-
-// ---------------------------------------------------------------------------
-// Digits of A (theta, m x n row-major FP64 per instance) into
-// Bd[z][reim][t][j][k] (k contiguous, Kp per row, rows nc) and block scales
-// Bs[z][kb][j].  A CTA takes 64 k x 16 j; rows past the instance's (m, n)
-// become zero digits.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_oz_digits_theta(const Dims* __restrict__ dims,
-                                                         const ProbPtr* __restrict__ ptrs, uint16_t* Bd, float* Bs,
-                                                         int nc, int Kp) {
-  __shared__ int emax[16][17];
-  __shared__ uint16_t dig[2 * OZ_S][16][OZ_KB + 2];  // [reim t][j][k]
-  const int z = blockIdx.z;
-  const Dims D = dims[z];
-  if (!D.active) return;
-  const int m = D.m, n = D.n;
-  const cplx* th = ptrs[z].theta;
-  const int k0 = blockIdx.y * OZ_KB, j0 = blockIdx.x * 16;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int j = j0 + tx;
-  cplx v[4];
-  int e = 0;
+// The NS digits of four values of 8 NS bits as packed BF16 quadruples (planes t = 1 .. NS).
+template <int NS>
+__device__ __forceinline__ void oz_digits4(const int64_t n[4], uint2 d[NS]) {
+  const float bias = 8388608.f + 128.f;
+  uint64_t m[4];
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int k = k0 + ty + 16 * s;
-    v[s] = (k < m && j < n) ? th[(int64_t)k * n + j] : cmk(0.0, 0.0);
-    const uint64_t ur = (uint64_t)__double_as_longlong(v[s].x), ui = (uint64_t)__double_as_longlong(v[s].y);
-    const int er = (int)((ur >> 52) & 0x7FF), ei = (int)((ui >> 52) & 0x7FF);
-    e = max(e, max(er == 0x7FF ? 0 : er, ei == 0x7FF ? 0 : ei));
-  }
-  emax[ty][tx] = e;
-  __syncthreads();
-  int E = 0;
+  for (int q = 0; q < 4; ++q) m[q] = (uint64_t)n[q] + (0x0000808080808080ull >> (8 * (OZ_S - NS)));
 #pragma unroll
-  for (int s = 0; s < 16; ++s) E = max(E, emax[s][tx]);
-  const float sc = oz_scale(E, 1030);  // x = sum_t digit_t * 2^(E - 1030)
-  const bool live = sc != 0.f;
+  for (int t = 0; t < NS; ++t) {
+    unsigned f[4];
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int k = ty + 16 * s;
-    const uint64_t nr = live ? oz_n48_f64(v[s].x, E) : 0, ni = live ? oz_n48_f64(v[s].y, E) : 0;
-    const bool sr = v[s].x < 0.0, si = v[s].y < 0.0;
-#pragma unroll
-    for (int t = 0; t < OZ_S; ++t) {
-      dig[t][tx][k] = oz_bf16_digit((unsigned)((nr >> (40 - 8 * t)) & 0xFF), t, sr);
-      dig[OZ_S + t][tx][k] = oz_bf16_digit((unsigned)((ni >> (40 - 8 * t)) & 0xFF), t, si);
+    for (int q = 0; q < 4; ++q) {
+      if (t == 0)
+        f[q] = __float_as_uint((float)(int)((int64_t)m[q] >> (8 * (NS - 1))));
+      else
+        f[q] = __float_as_uint(__uint_as_float(0x4B000000u | (unsigned)((m[q] >> (8 * (NS - 1 - t))) & 0xFF)) - bias);
     }
-  }
-  if (ty == 0 && j < nc) Bs[((size_t)z * (Kp / OZ_KB) + blockIdx.y) * nc + j] = live ? sc : 0.f;
-  __syncthreads();
-  // rows (reim t, j) of 64 k = 128 bytes each: 8 threads per row, 16 bytes each
-  uint16_t* base = Bd + (size_t)z * 2 * OZ_S * nc * Kp;
-  for (int w = threadIdx.x; w < 2 * OZ_S * 16 * 8; w += 256) {
-    const int q = w & 7, row = w >> 3, jj = row & 15, rt = row >> 4;
-    if (j0 + jj >= nc) continue;
-    const uint16_t* src = &dig[rt][jj][q * 8];
-    uint4 pk;
-    pk.x = (unsigned)src[0] | ((unsigned)src[1] << 16);
-    pk.y = (unsigned)src[2] | ((unsigned)src[3] << 16);
-    pk.z = (unsigned)src[4] | ((unsigned)src[5] << 16);
-    pk.w = (unsigned)src[6] | ((unsigned)src[7] << 16);
-    *reinterpret_cast<uint4*>(base + ((size_t)rt * nc + j0 + jj) * Kp + k0 + q * 8) = pk;
+    d[t].x = __byte_perm(f[0], f[1], 0x7632);  // the upper halves: exact BF16 numbers
+    d[t].y = __byte_perm(f[2], f[3], 0x7632);
   }
 }
 
-// Digits of Q_f^H (Q_f m x l column-major FP32 complex per instance, capacity
-// mc x lc) into Ad[z][reim][t][i][k] and scales As[z][kb][i]: one warp per
-// (i, k block), two k per lane; Im negated (the conjugate).
-__global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ dims, const float2* __restrict__ Qf,
-                                                     uint16_t* Ad, float* As, int mc, int lc, int Kp) {
-  const int z = blockIdx.y;
-  const Dims D = dims[z];
-  if (!D.active) return;
-  const int nkb = Kp / OZ_KB;
-  const int lane = threadIdx.x & 31;
-  const int wid = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (wid >= lc * nkb) return;
-  const int i = wid / nkb, kb = wid % nkb;
-  const int k = kb * OZ_KB + 2 * lane;
-  float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-  if (i < D.l) {
-    const float2* q = Qf + (size_t)z * mc * lc + (size_t)i * mc;
-    if (k < D.m) a = q[k];
-    if (k + 1 < D.m) b = q[k + 1];
-  }
-  auto ex = [](float x) {
-    const int e = (int)((__float_as_uint(x) >> 23) & 0xFF);
-    return e == 0xFF ? 0 : e;
-  };
-  int E = max(max(ex(a.x), ex(a.y)), max(ex(b.x), ex(b.y)));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-  const float sc = oz_scale(E, 134);  // x = sum_t digit_t * 2^(E - 134)
-  const bool live = sc != 0.f;
-  uint16_t* base = Ad + (size_t)z * 2 * OZ_S * lc * Kp;
-  const float re[2] = {a.x, b.x}, im[2] = {-a.y, -b.y};
-#pragma unroll
-  for (int t = 0; t < OZ_S; ++t) {
-    uint16_t dr[2], di[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint64_t nr = live ? oz_n48_f32(re[h], E) : 0, ni = live ? oz_n48_f32(im[h], E) : 0;
-      dr[h] = oz_bf16_digit((unsigned)((nr >> (40 - 8 * t)) & 0xFF), t, re[h] < 0.f);
-      di[h] = oz_bf16_digit((unsigned)((ni >> (40 - 8 * t)) & 0xFF), t, im[h] < 0.f);
-    }
-    *reinterpret_cast<unsigned*>(base + ((size_t)t * lc + i) * Kp + k) = (unsigned)dr[0] | ((unsigned)dr[1] << 16);
-    *reinterpret_cast<unsigned*>(base + ((size_t)(OZ_S + t) * lc + i) * Kp + k) =
-        (unsigned)di[0] | ((unsigned)di[1] << 16);
-  }
-  if (lane == 0) As[((size_t)z * nkb + kb) * lc + i] = live ? sc : 0.f;
+// Where a digit lives: [z][k step][plane][row][16 k], 32 bytes per row and
+// step, so that the rows of a tile are one run per plane (a bulk copy each)
+// and lie in shared memory as the MMA's 32-byte swizzle wants them: the two
+// 16-byte halves of a row trade places where bit 2 of the row is set.
+// Offset in digits of the half `ch` (k 8 ch .. 8 ch + 7) of k step ks.
+template <int NS>
+__device__ __forceinline__ size_t oz_at(int ks, int plane, int row, int ch, int rc) {
+  return (((size_t)ks * (2 * NS) + plane) * rc + row) * OZ_KS + 8 * (ch ^ ((row >> 2) & 1));
+}
+
+// Scale of a row in the product: 2^(E - 1023 - 22); zero for a zero row.
+__device__ __forceinline__ double oz_scale(int E) {
+  return E > 22 ? __longlong_as_double((long long)(E - 22) << 52) : 0.0;
 }
 
 // ---------------------------------------------------------------------------
 // Stages.  OZ_PROJ is the projection C = Q_f^H A (l x n, K = m), written as
-// B^H = C^H into Yt; the others are the GemmStage products of stages.cuh,
+// C^H = A^H Q_f into Yt; the others are the GemmStage products of stages.cuh,
 // C = op(A) op(B) with op(A) conjugated where StageFlags says so and C
 // stored conjugated for G_V.
 // ---------------------------------------------------------------------------
@@ -287,12 +205,19 @@ __device__ __forceinline__ OzOp oz_op(const Dims& D, const ProbPtr& P) {
 
 template <int ST>
 struct OzConj {
-  // the projection and the Gram fold conj(Q_f) into Q_f's digits; the Gram
-  // multiplies them by their own conjugate
   static constexpr bool own = ST < OZ_PROJ;  // a GemmStage of stages.cuh
-  static constexpr bool A = own && StageFlags<ST>::conjA;
-  static constexpr bool B = ST == OZ_GRAM;
+  static constexpr bool A = ST == OZ_PROJ || ST == OZ_GRAM || (own && StageFlags<ST>::conjA);  // Q_f^H
   static constexpr bool C = ST == OZ_PROJ || (own && StageFlags<ST>::conjC);
+};
+
+// Digits of each operand and the ring of stages of a product.
+template <int ST>
+struct OzGeo {
+  static constexpr int SA = (ST == OZ_PROJ || ST == OZ_GRAM) ? OZ_SQ : OZ_S;
+  static constexpr int SB = ST == OZ_GRAM ? OZ_SQ : OZ_S;
+  static constexpr uint32_t A_STAGE = 2 * SA * OZ_A_TILE, B_STAGE = 2 * SB * OZ_B_TILE;
+  static constexpr int STAGES = SA == OZ_S ? 3 : 4;
+  static constexpr size_t smem = 1024 + (size_t)STAGES * (A_STAGE + B_STAGE) + (2 * STAGES + 3) * 8 + 16;
 };
 
 // The stages that skip a bond: the contraction and gate GEMMs run only for
@@ -300,6 +225,16 @@ struct OzConj {
 template <int ST>
 __device__ __forceinline__ bool oz_skip(const ProbPtr& P) {
   return (ST == OZ_THETA || ST == OZ_GATE) && P.Cpre == nullptr;
+}
+
+// Whether a launch's condition bits take a problem.
+__device__ __forceinline__ bool oz_takes(const Dims& D, int cond) {
+  if ((cond >> DPC_PASS) > 0 && D.cq < (cond >> DPC_PASS)) return false;
+  if ((cond & DPC_OK) && D.cf) return false;
+  if ((cond & DPC_QFLAG) && !D.qflag) return false;
+  if ((cond & DPC_DIG) && !D.dig) return false;
+  if ((cond & DPC_CHK) && !D.chk) return false;
+  return true;
 }
 
 // Element (i, j) of C into its destination.
@@ -324,9 +259,10 @@ __device__ __forceinline__ void oz_store(const Dims& D, const ProbPtr& P, const 
 template <int ST, int SIDE>
 struct OzSrc {  // a GemmStage: strided operand of the stage table
   const cplx* X;
+  const double* scale;
   int64_t rs, ks;
   int rows, K;
-  __device__ OzSrc(const Dims& D, const ProbPtr& P) {
+  __device__ OzSrc(const Dims& D, const ProbPtr& P) : scale(P.sigma) {
     const GemmOp g = gemm_of<ST>(D, P);
     rows = SIDE == 0 ? g.M : g.N;
     K = g.K;
@@ -335,7 +271,19 @@ struct OzSrc {  // a GemmStage: strided operand of the stage table
     ks = SIDE == 0 ? g.acs : g.brs;
   }
   __device__ bool rows_contig() const { return rs == 1; }
-  __device__ cplx at(int r, int k) const { return X[(int64_t)r * rs + (int64_t)k * ks]; }
+  __device__ cplx at(int r, int k) const {
+    const cplx v = X[(int64_t)r * rs + (int64_t)k * ks];
+    if constexpr (SIDE == 0 && StageFlags<ST>::scaleA) return cscale(v, scale[k]);
+    return v;
+  }
+};
+template <>
+struct OzSrc<OZ_PROJ, 1> {  // the columns of theta
+  const cplx* X;
+  int rows, K;
+  __device__ OzSrc(const Dims& D, const ProbPtr& P) : X(P.theta), rows(D.n), K(D.m) {}
+  __device__ bool rows_contig() const { return true; }
+  __device__ cplx at(int r, int k) const { return X[(int64_t)k * rows + r]; }
 };
 template <int SIDE>
 struct OzSrc<OZ_THETA, SIDE> {  // A = Gamma_l (rows (i, alpha)), B = lam_m Gamma_r (columns (j, beta))
@@ -373,69 +321,203 @@ struct OzSrc<OZ_GATE, SIDE> {  // A = the gate (rows (i, j)), B = the (i', j') x
   }
 };
 
-// Digits of a stage operand in its K-major view: SIDE 0 the rows i of op(A)
-// (element A[i ars + k acs], not conjugated: the MMAs conjugate), SIDE 1 the
-// columns j of op(B) (element B[k brs + j bcs]); into Xd[z][reim][t][row][k]
-// (rows rc, Kp per row) and scales Xs[z][kb][row].  A CTA takes 16 rows x 64
-// k; rows and k past the instance's own extents become zero digits.
+// Largest biased exponent of every row of a stage operand into Es[z][row]
+// (zero before the launch; a maximum does not depend on the order of the
+// atomics).  A CTA takes 16 rows x OZ_MAX_K k.
+enum { OZ_MAX_K = 512 };
+
 template <int ST, int SIDE>
-__global__ void __launch_bounds__(256) k_oz_digits_op(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
-                                                      uint16_t* Xd, float* Xs, int rc, int Kp) {
-  __shared__ cplx tile[16][OZ_KB + 1];
-  __shared__ uint16_t dig[2 * OZ_S][16][OZ_KB + 2];  // [reim t][row][k]
+__global__ void __launch_bounds__(256) k_oz_max(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
+                                                int* Es, int rc, int cond) {
+  __shared__ int emax[16];
   const int z = blockIdx.z;
   const Dims D = dims[z];
-  if (!D.active || oz_skip<ST>(ptrs[z])) return;
+  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(ptrs[z])) return;
+  const OzSrc<ST, SIDE> src(D, ptrs[z]);
+  const int r0 = blockIdx.x * 16, k0 = blockIdx.y * OZ_MAX_K, k1 = min(src.K, k0 + OZ_MAX_K);
+  if (r0 >= src.rows || k0 >= src.K) return;  // uniform over the block
+  const int tid = threadIdx.x;
+  if (tid < 16) emax[tid] = 0;
+  __syncthreads();
+  const bool rowc = src.rows_contig();
+  int E = 0;
+  int r;
+  if (rowc) {
+    r = tid & 15;
+    if (r0 + r < src.rows)
+      for (int k = k0 + (tid >> 4); k < k1; k += 16) {
+        const cplx v = src.at(r0 + r, k);
+        E = max(E, max(oz_exp(v.x), oz_exp(v.y)));
+      }
+  } else {
+    r = tid >> 4;
+    if (r0 + r < src.rows)
+      for (int k = k0 + (tid & 15); k < k1; k += 16) {
+        const cplx v = src.at(r0 + r, k);
+        E = max(E, max(oz_exp(v.x), oz_exp(v.y)));
+      }
+  }
+  atomicMax(&emax[r], E);
+  __syncthreads();
+  if (tid < 16 && r0 + tid < src.rows) atomicMax(&Es[(size_t)z * rc + r0 + tid], emax[tid]);
+}
+
+// Digits of a stage operand in its K-major view: SIDE 0 the rows i of op(A)
+// (element A[i ars + k acs], not conjugated: the MMAs conjugate), SIDE 1 the
+// columns j of op(B) (element B[k brs + j bcs]); into Xd (oz_at; rows rc, Kp / 16 k steps).  SELF: the CTA takes 16 rows and all k, finds their
+// largest exponents itself (a second read of at most OZ_SELF_K k, from L2)
+// and stores them; otherwise it takes 16 rows x 64 k and reads them from Es.
+// Rows and k past the instance's own extents become zero digits.
+struct OzDigSmem {
+  cplx tile[16][OZ_KB + 1];
+  __align__(16) uint16_t dig[2 * OZ_S][16][OZ_KB + 8];  // [reim t][row][k]
+  int emax[16];
+};
+
+template <int ST, int SIDE, bool SELF>
+__device__ __forceinline__ void oz_digits_block(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
+                                                uint16_t* Xd, int* Es, int rc, int Kp, int cond, OzDigSmem& sm) {
+  auto& tile = sm.tile;
+  auto& dig = sm.dig;
+  auto& emax = sm.emax;
+  const int z = blockIdx.z;
+  const Dims D = dims[z];
+  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(ptrs[z])) return;
   const OzSrc<ST, SIDE> src(D, ptrs[z]);
   const int rows = src.rows, K = src.K;
   const bool rowc = src.rows_contig();
-  const int r0 = blockIdx.x * 16, k0 = blockIdx.y * OZ_KB;
+  const int r0 = blockIdx.x * 16;
   const int tid = threadIdx.x;
-  for (int e = tid; e < 16 * OZ_KB; e += 256) {
-    int r, k;  // consecutive threads along the unit-stride direction
-    if (rowc) { r = e & 15; k = e >> 4; } else { k = e & (OZ_KB - 1); r = e >> 6; }
-    const int gr = r0 + r, gk = k0 + k;
-    tile[r][k] = (gr < rows && gk < K) ? src.at(gr, gk) : cmk(0.0, 0.0);
-  }
-  __syncthreads();
   const int r = tid >> 4, pq = tid & 15;  // 16 threads per row, 4 k each
-  cplx v[4];
   int E = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    v[q] = tile[r][pq * 4 + q];
-    const uint64_t ur = (uint64_t)__double_as_longlong(v[q].x), ui = (uint64_t)__double_as_longlong(v[q].y);
-    const int er = (int)((ur >> 52) & 0x7FF), ei = (int)((ui >> 52) & 0x7FF);
-    E = max(E, max(er == 0x7FF ? 0 : er, ei == 0x7FF ? 0 : ei));
+  if (SELF) {
+    if (tid < 16) emax[tid] = 0;
+    __syncthreads();
+    const int lr = rowc ? (tid & 15) : (tid >> 4);
+    int e = 0;
+    if (r0 + lr < rows)
+      for (int k = rowc ? (tid >> 4) : (tid & 15); k < K; k += 16) {
+        const cplx v = src.at(r0 + lr, k);
+        e = max(e, max(oz_exp(v.x), oz_exp(v.y)));
+      }
+    atomicMax(&emax[lr], e);
+    __syncthreads();
+    E = emax[r];
+    if (pq == 0 && r0 + r < rc) Es[(size_t)z * rc + r0 + r] = E;
+  } else {
+    E = (r0 + r < rc) ? Es[(size_t)z * rc + r0 + r] : 0;
   }
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));  // within the row's 16 lanes
-  const float sc = oz_scale(E, 1030);
-  const bool live = sc != 0.f;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int k = pq * 4 + q;
-    const uint64_t nr = live ? oz_n48_f64(v[q].x, E) : 0, ni = live ? oz_n48_f64(v[q].y, E) : 0;
-    const bool sr = v[q].x < 0.0, si = v[q].y < 0.0;
-#pragma unroll
-    for (int t = 0; t < OZ_S; ++t) {
-      dig[t][r][k] = oz_bf16_digit((unsigned)((nr >> (40 - 8 * t)) & 0xFF), t, sr);
-      dig[OZ_S + t][r][k] = oz_bf16_digit((unsigned)((ni >> (40 - 8 * t)) & 0xFF), t, si);
-    }
-  }
-  if (pq == 0 && r0 + r < rc) Xs[((size_t)z * (Kp / OZ_KB) + blockIdx.y) * rc + r0 + r] = live ? sc : 0.f;
-  __syncthreads();
   uint16_t* base = Xd + (size_t)z * 2 * OZ_S * rc * Kp;
-  for (int w = tid; w < 2 * OZ_S * 16 * 8; w += 256) {
-    const int q = w & 7, row = w >> 3, rr = row & 15, rt = row >> 4;
-    if (r0 + rr >= rc) continue;
-    const uint16_t* src = &dig[rt][rr][q * 8];
-    uint4 pk;
-    pk.x = (unsigned)src[0] | ((unsigned)src[1] << 16);
-    pk.y = (unsigned)src[2] | ((unsigned)src[3] << 16);
-    pk.z = (unsigned)src[4] | ((unsigned)src[5] << 16);
-    pk.w = (unsigned)src[6] | ((unsigned)src[7] << 16);
-    *reinterpret_cast<uint4*>(base + ((size_t)rt * rc + r0 + rr) * Kp + k0 + q * 8) = pk;
+  // whole blocks of 64 k the GEMM reads: zero digits past K within the last
+  const int kend = min(Kp, ((K + OZ_KB - 1) / OZ_KB) * OZ_KB);
+  for (int k0 = SELF ? 0 : (int)blockIdx.y * OZ_KB; k0 < kend; k0 += SELF ? OZ_KB : kend) {
+    for (int e = tid; e < 16 * OZ_KB; e += 256) {
+      int tr, k;  // consecutive threads along the unit-stride direction
+      if (rowc) { tr = e & 15; k = e >> 4; } else { k = e & (OZ_KB - 1); tr = e >> 6; }
+      const int gr = r0 + tr, gk = k0 + k;
+      tile[tr][k] = (gr < rows && gk < K) ? src.at(gr, gk) : cmk(0.0, 0.0);
+    }
+    __syncthreads();
+    int64_t nr[4], ni[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const cplx v = tile[r][pq * 4 + q];
+      nr[q] = oz_fix(v.x, E);
+      ni[q] = oz_fix(v.y, E);
+    }
+    uint2 d[OZ_S];
+    oz_digits4<OZ_S>(nr, d);
+#pragma unroll
+    for (int t = 0; t < OZ_S; ++t) *reinterpret_cast<uint2*>(&dig[t][r][pq * 4]) = d[t];
+    oz_digits4<OZ_S>(ni, d);
+#pragma unroll
+    for (int t = 0; t < OZ_S; ++t) *reinterpret_cast<uint2*>(&dig[OZ_S + t][r][pq * 4]) = d[t];
+    __syncthreads();
+    // (k step, plane, row, half) of 16 bytes each: 512-byte runs of 16 rows
+    for (int w = tid; w < 2 * OZ_S * 16 * 8; w += 256) {
+      const int ch = w & 1, rr = (w >> 1) & 15, t = w >> 5;  // t = plane + 14 k step
+      const int plane = t % (2 * OZ_S), ks = t / (2 * OZ_S);
+      if (r0 + rr >= rc) continue;
+      *reinterpret_cast<uint4*>(base + oz_at<OZ_S>((k0 >> 4) + ks, plane, r0 + rr, ch, rc)) =
+          *reinterpret_cast<const uint4*>(&dig[plane][rr][16 * ks + 8 * ch]);
+    }
+    if (SELF) __syncthreads();
+  }
+}
+
+template <int ST, int SIDE, bool SELF>
+__global__ void __launch_bounds__(256) k_oz_digits_op(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
+                                                      uint16_t* Xd, int* Es, int rc, int Kp, int cond) {
+  __shared__ OzDigSmem sm;
+  oz_digits_block<ST, SIDE, SELF>(dims, ptrs, Xd, Es, rc, Kp, cond, sm);
+}
+
+// Both operands of a product in one launch (depths up to OZ_SELF_K).
+template <int ST>
+__global__ void __launch_bounds__(256) k_oz_digits_two(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
+                                                       uint16_t* Ad, int* As, int ac, uint16_t* Bd, int* Bs, int bc,
+                                                       int Kp, int cond) {
+  __shared__ OzDigSmem sm;
+  if (blockIdx.y == 0) {
+    if ((int)blockIdx.x * 16 < ac) oz_digits_block<ST, 0, true>(dims, ptrs, Ad, As, ac, Kp, cond, sm);
+  } else {
+    if ((int)blockIdx.x * 16 < bc) oz_digits_block<ST, 1, true>(dims, ptrs, Bd, Bs, bc, Kp, cond, sm);
+  }
+}
+
+// Digits of Q_f (m x l column-major FP32 complex per instance, capacity
+// mc x lc) into Ad (oz_at) and Es[z][i]: one warp per column.  An FP32 column
+// is four digits: its entries are rounded to multiples of 2^-31 of the power
+// of two above the largest one, in place, so that every later use of Q_f sees
+// the numbers the digits hold exactly (entries above 2^-8 of the largest one
+// keep all their 24 bits).  Against seven digits the projection loads 47 KB
+// instead of 72 KB per k step and runs 22 digit pairs instead of 28.  The same
+// numbers go to P.Q in FP64, the left operand of U = Q_f (I + D) J_k.
+__global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ dims,
+                                                     const ProbPtr* __restrict__ ptrs, float2* __restrict__ Qf,
+                                                     uint16_t* Ad, int* Es, int mc, int lc, int Kp) {
+  const int z = blockIdx.y;
+  const Dims D = dims[z];
+  if (!D.active) return;
+  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= lc) return;
+  const int K = i < D.l ? D.m : 0;
+  float2* q = Qf + (size_t)z * mc * lc + (size_t)i * mc;
+  cplx* Qd = ptrs[z].Q + (size_t)i * D.m;  // (i < D.l where it is written)
+  int E = 0;
+  for (int k = lane; k < K; k += 32) {
+    const float2 v = q[k];
+    E = max(E, max(oz_exp(v.x), oz_exp(v.y)));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+  if (lane == 0) Es[(size_t)z * lc + i] = E;
+  // x = N 2^(E - 1023 - 30), the scale as an FP32 number (a Q_f column has unit norm: E far from its ends)
+  const float unit = __uint_as_float((unsigned)max(1, min(254, E - 1023 - 30 + 127)) << 23);
+  uint16_t* base = Ad + (size_t)z * 2 * OZ_SQ * lc * Kp;
+  const int kend = min(Kp, ((D.m + OZ_KB - 1) / OZ_KB) * OZ_KB);
+  for (int k = 4 * lane; k < kend; k += 128) {
+    int64_t nr[4], ni[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float2 v = (k + u < K) ? q[k + u] : make_float2(0.f, 0.f);
+      nr[u] = oz_fix31(v.x, E);
+      ni[u] = oz_fix31(v.y, E);
+      if (k + u < K) {
+        const float2 r = make_float2((float)(int)nr[u] * unit, (float)(int)ni[u] * unit);
+        q[k + u] = r;
+        Qd[k + u] = cmk((double)r.x, (double)r.y);
+      }
+    }
+    uint2 d[OZ_SQ];
+    uint16_t* at = base + oz_at<OZ_SQ>(k >> 4, 0, i, (k >> 3) & 1, lc) + (k & 4);
+    oz_digits4<OZ_SQ>(nr, d);
+#pragma unroll
+    for (int t = 0; t < OZ_SQ; ++t) *reinterpret_cast<uint2*>(at + (size_t)t * lc * OZ_KS) = d[t];
+    oz_digits4<OZ_SQ>(ni, d);
+#pragma unroll
+    for (int t = 0; t < OZ_SQ; ++t) *reinterpret_cast<uint2*>(at + (size_t)(OZ_SQ + t) * lc * OZ_KS) = d[t];
   }
 }
 
@@ -443,32 +525,30 @@ __global__ void __launch_bounds__(256) k_oz_digits_op(const Dims* __restrict__ d
 // The digit-pair GEMM.
 // ---------------------------------------------------------------------------
 struct OzArgs {
+  const uint16_t* Ad;  // digits of both operands (oz_at)
+  const uint16_t* Bd;
   int lc, nc, Kp;      // capacities: rows of C, columns of C, padded k
-  const float* As;     // [z][kb][i]
-  const float* Bs;     // [z][kb][j]
+  const int* As;       // [z][i] largest biased exponents of the left operand's rows
+  const int* Bs;       // [z][j]
   int* err;
   uint32_t poll_limit;
   int stall;
+  int cond;            // which problems the launch takes (DPC_*)
 };
 
-__device__ __forceinline__ void oz_tma_load_5d(void* dst, const CUtensorMap* tm, int c0, int c1, int c4, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
-      "%6}], [%7];" ::"r"(tc_smem_u32(dst)),
-      "l"((uint64_t)tm), "r"(c0), "r"(c1), "r"(0), "r"(0), "r"(c4), "r"(tc_smem_u32(bar))
-      : "memory");
+__device__ __forceinline__ void oz_bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   tc_smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(tc_smem_u32(bar))
+               : "memory");
 }
 
-// K-major, 32-byte swizzle: 8-row atoms of 256 bytes (stride byte offset 256).
-__device__ __forceinline__ uint64_t oz_desc_sw32(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;            // leading byte offset (unused: one atom along k)
-  d |= (uint64_t)(256 >> 4) << 32;   // stride byte offset
-  d |= (uint64_t)1 << 46;            // version
-  d |= (uint64_t)6 << 61;            // 32-byte swizzle
-  return d;
-}
+// Shared-memory descriptor, K-major, 32-byte swizzle: 8-row atoms of 256
+// bytes (stride byte offset 256).  The low word holds the address (in units
+// of 16 bytes; the offsets below stay inside its 14 bits) and the leading
+// byte offset (unused: one atom along k); the high word is a constant.
+enum : uint32_t { OZ_DESC_HI = (256u >> 4) | (1u << 14) | (6u << 29) };  // stride, version, 32-byte swizzle
+__device__ __forceinline__ uint32_t oz_desc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
 
 // kind::f16 instruction descriptor: D = F32, A = B = BF16, K-major, M x N.
 __host__ __device__ constexpr uint32_t oz_idesc(int M, int N, bool negA) {
@@ -476,12 +556,18 @@ __host__ __device__ constexpr uint32_t oz_idesc(int M, int N, bool negA) {
          ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void oz_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// One MMA by the lane with leader != 0 (the warp runs the issue loop uniformly:
+// descriptors then stay in uniform registers).
+__device__ __forceinline__ void oz_mma(uint32_t leader, uint32_t d, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                       uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "setp.ne.b32 q, %0, 0;\n\t"
+      "mov.b64 a, {%2, %6};\n\t"
+      "mov.b64 b, {%3, %6};\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %4, p;\n\t}\n" ::"r"(leader),
+      "r"(d), "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"((uint32_t)OZ_DESC_HI)
       : "memory");
 }
 
@@ -502,45 +588,47 @@ __device__ __forceinline__ bool oz_warp_wait(uint64_t* bar, uint32_t parity, uin
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
-// four consecutive accumulator columns of this warp's 32 lanes
-__device__ __forceinline__ void oz_ld4(uint32_t taddr, float* v) {
-  uint32_t r0, r1, r2, r3;
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(taddr)
-               : "memory");
+// two consecutive accumulator columns of this warp's 32 lanes
+__device__ __forceinline__ void oz_ld2(uint32_t taddr, float* v) {
+  uint32_t r0, r1;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(taddr) : "memory");
   v[0] = __uint_as_float(r0);
   v[1] = __uint_as_float(r1);
-  v[2] = __uint_as_float(r2);
-  v[3] = __uint_as_float(r3);
 }
 
-// acc (h, l) += s (hs, ls), then renormalised
-__device__ __forceinline__ void oz_df_add(float& h, float& l, float hs, float ls) {
-  float t, e;
-  two_sum(h, hs, t, e);
-  e += l + ls;
-  h = t + e;
-  l = e - (h - t);
+// (hi, lo) += the seven level sums v[0], v[1], ... (levels 2 .. 8): hi counts
+// units of level 6, lo (FP32) units of level 8.  Levels 2 and 3 (below 2^22)
+// become integers by adding 1.5 2^23, the others by conversion.
+__device__ __forceinline__ void oz_add_levels(int64_t& hi, float& lo, const float (*v)[2], int q) {
+  const float magic = 12582912.f;  // 1.5 2^23: the low bits of the sum are the integer
+  const unsigned mb = 0x4B400000u;
+  const int i01 = (int)(__float_as_uint(v[0][q] + magic) * 256u + __float_as_uint(v[1][q] + magic) - mb * 257u);
+  const int i2 = __float2int_rn(v[2][q]), i3 = __float2int_rn(v[3][q]), i4 = __float2int_rn(v[4][q]);
+  hi += (int64_t)i01 * 16777216;
+  hi += (int64_t)i2 * 65536;
+  hi += (int64_t)i3 * 256;
+  hi += i4;
+  lo += fmaf(v[5][q], 256.f, v[6][q]);
 }
 
 template <int ST>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs, OzArgs a) {
+    k_oz_gemm(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs, OzArgs a) {
+  typedef OzGeo<ST> Geo;
+  constexpr int SA = Geo::SA, SB = Geo::SB, STAGES = Geo::STAGES;
   extern __shared__ __align__(1024) uint8_t oz_smem_raw[];
   const int z = blockIdx.z;
   const Dims D = dims[z];
   const int i0 = blockIdx.y * OZ_BM, j0 = blockIdx.x * OZ_BN;
-  if (!D.active || oz_skip<ST>(ptrs[z])) return;
+  if (!D.active || !oz_takes(D, a.cond) || oz_skip<ST>(ptrs[z])) return;
   const OzOp op = oz_op<ST>(D, ptrs[z]);
   if (i0 >= op.M || j0 >= op.N) return;  // uniform: before any barrier or allocation
   uint8_t* smem = (uint8_t*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
-  uint8_t* sB = smem + OZ_STAGES * OZ_A_STAGE;
-  uint64_t* full = (uint64_t*)(sB + OZ_STAGES * OZ_B_STAGE);
-  uint64_t* empty = full + OZ_STAGES;
-  uint64_t* accf = empty + OZ_STAGES;
+  uint8_t* sB = smem + STAGES * Geo::A_STAGE;
+  uint64_t* full = (uint64_t*)(sB + STAGES * Geo::B_STAGE);
+  uint64_t* empty = full + STAGES;
+  uint64_t* accf = empty + STAGES;
   uint64_t* accfree = accf + 1;
   uint64_t* drain = accfree + 1;
   uint32_t* tmem_holder = (uint32_t*)(drain + 1);
@@ -548,8 +636,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nks = (min(op.K, a.Kp) + OZ_KS - 1) / OZ_KS;  // k steps of this instance
-  const int nkb = (nks + (OZ_DRAIN / OZ_KS) - 1) / (OZ_DRAIN / OZ_KS);  // exact accumulation blocks
-  const int iters = nkb * (OZ_DRAIN / OZ_KS);  // whole blocks (zero digits past m)
+  const int nkb = (nks + OZ_DRAIN / OZ_KS - 1) / (OZ_DRAIN / OZ_KS);  // exact accumulation blocks
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem_u32(tmem_holder)),
@@ -558,7 +645,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 32) {
-    for (int s = 0; s < OZ_STAGES; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       tc_mbar_init(&full[s], 1);
       tc_mbar_init(&empty[s], 1);
     }
@@ -574,80 +661,98 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   const uint32_t tmem = *tmem_holder;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- producer
-      int issued = 0;
-      for (int it = 0; it < (a.stall ? 0 : iters); ++it) {
-        const int s = it % OZ_STAGES;
-        const uint32_t r = (uint32_t)(it / OZ_STAGES);
-        if (it >= OZ_STAGES && !tc_mbar_wait(&empty[s], (r & 1u) ^ 1u, a.poll_limit, a.err, abort_flag)) break;
-        tc_mbar_expect_tx(&full[s], OZ_A_STAGE + OZ_B_STAGE);
-        oz_tma_load_5d(sA + s * OZ_A_STAGE, &tmA, it * OZ_KS, i0, z, &full[s]);
-        oz_tma_load_5d(sB + s * OZ_B_STAGE, &tmB, it * OZ_KS, j0, z, &full[s]);
-        issued = it + 1;
-      }
-      if (*abort_flag) {  // every copy issued lands before the teardown
-        for (int it = (issued > OZ_STAGES ? issued - OZ_STAGES : 0); it < issued; ++it)
-          for (uint32_t i = 0; i < (1u << 22); ++i)
-            if (tc_mbar_try_wait(&full[it % OZ_STAGES], (uint32_t)(it / OZ_STAGES) & 1u)) break;
-      }
+    // ---- producer: per k step one bulk copy per plane and operand (lanes
+    // 0 .. 2 SA - 1 the left operand's, the next 2 SB the right one's); rows past the
+    // arrays' own are not copied, and what those rows of the tile hold only
+    // reaches outputs that are not stored.
+    const bool isA = lane < 2 * SA;
+    const int plane = isA ? lane : lane - 2 * SA, row0 = isA ? i0 : j0, rc = isA ? a.lc : a.nc;
+    const int na = min((int)OZ_BM, a.lc - i0), nb = min((int)OZ_BN, a.nc - j0);  // rows copied
+    const uint32_t bytes = (uint32_t)(isA ? na : nb) * (OZ_KS * 2);
+    const uint16_t* src = (isA ? a.Ad : a.Bd) + (size_t)z * (isA ? 2 * SA : 2 * SB) * rc * a.Kp + ((size_t)plane * rc + row0) * OZ_KS;
+    const size_t step = (size_t)(isA ? 2 * SA : 2 * SB) * rc * OZ_KS;
+    uint8_t* dst = (isA ? sA : sB) + (size_t)plane * (isA ? OZ_A_TILE : OZ_B_TILE);
+    const uint32_t stage = isA ? Geo::A_STAGE : Geo::B_STAGE;
+    int issued = 0;
+    bool ok = true;
+    for (int it = 0; it < (a.stall ? 0 : nks); ++it) {
+      const int s = it % STAGES;
+      const uint32_t r = (uint32_t)(it / STAGES);
+      if (it >= STAGES && !(ok = oz_warp_wait(&empty[s], (r & 1u) ^ 1u, a.poll_limit, a.err, abort_flag))) break;
+      if (lane == 0) tc_mbar_expect_tx(&full[s], (uint32_t)(na * SA + nb * SB) * (2 * OZ_KS * 2));
+      __syncwarp();
+      if (lane < 2 * (SA + SB)) oz_bulk_load(dst + (size_t)s * stage, src + (size_t)it * step, bytes, &full[s]);
+      issued = it + 1;
+    }
+    if (lane == 0 && *abort_flag) {  // every copy issued lands before the teardown
+      for (int it = (issued > STAGES ? issued - STAGES : 0); it < issued; ++it)
+        for (uint32_t i = 0; i < (1u << 22); ++i)
+          if (tc_mbar_try_wait(&full[it % STAGES], (uint32_t)(it / STAGES) & 1u)) break;
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- MMA issuer: per k step the 21 digit pairs (t, u) with t + u <= 7,
-      // as six MMAs per real product
-      bool ok = true;
-      int issued_mma = 0;
-      for (int kb = 0; kb < nkb && ok; ++kb) {
-        if (kb > 0 && !tc_mbar_wait(accfree, (uint32_t)(kb - 1) & 1u, a.poll_limit, a.err, abort_flag)) {
-          ok = false;
-          break;
-        }
+    // ---- MMA issuer: per k step the digit pairs (t, u) with t + u <= 8, as
+    // one MMA per digit t of A and real product; all lanes run the loop, lane
+    // 0 issues
+    const uint32_t leader = lane == 0 ? 1u : 0u;
+    const uint32_t a0 = oz_desc_lo(tc_smem_u32(sA)), b0 = oz_desc_lo(tc_smem_u32(sB));
+    bool ok = true;
+    int issued_mma = 0, s = 0, it = 0;
+    uint32_t ph = 0;
+    for (int kb = 0; kb < nkb && ok; ++kb) {
+      if (kb > 0 && !(ok = oz_warp_wait(accfree, (uint32_t)(kb - 1) & 1u, a.poll_limit, a.err, abort_flag))) break;
+      for (int ks = 0; ks < OZ_DRAIN / OZ_KS && it < nks; ++ks, ++it) {
+        if (!(ok = oz_warp_wait(&full[s], ph, a.poll_limit, a.err, abort_flag))) break;
         tc_fence_after();
-        for (int ks = 0; ks < OZ_DRAIN / OZ_KS; ++ks) {
-          const int it = kb * (OZ_DRAIN / OZ_KS) + ks;
-          const int s = it % OZ_STAGES;
-          if (!tc_mbar_wait(&full[s], (uint32_t)(it / OZ_STAGES) & 1u, a.poll_limit, a.err, abort_flag)) {
-            ok = false;
-            break;
+        const uint32_t as = a0 + (uint32_t)s * (Geo::A_STAGE >> 4), br = b0 + (uint32_t)s * (Geo::B_STAGE >> 4);
+        const uint32_t bi = br + SB * (OZ_B_TILE >> 4);
+        const uint32_t first = ks == 0 ? 0u : 1u;
+        // digit t of A times planes u = 1 .. min(SB, 8 - t) of B (adjacent in
+        // shared memory) into the accumulators of levels t + 1 .. (adjacent in
+        // tensor memory).  The t = 1 MMAs of a block's first k step start the
+        // sums of the levels they cover; with SB < 7 the levels above SB + 1
+        // start with the first larger t that reaches them
+#pragma unroll
+        for (int t = 1; t <= SA; ++t) {
+          constexpr bool cA = OzConj<ST>::A;  // a conjugated left operand: C_r = Ar Br + Ai Bi, C_i = Ar Bi - Ai Br
+          const int nu = SB < OZ_S + 1 - t ? SB : OZ_S + 1 - t;
+          const uint32_t ar = as + (t - 1) * (OZ_A_TILE >> 4), ai = as + (SA + t - 1) * (OZ_A_TILE >> 4);
+          const uint32_t dr = tmem + (uint32_t)(OZ_BN * (t - 1)), di = dr + (uint32_t)(OZ_BN * OZ_NGRP);
+          // planes 1 .. nu - 1 reach levels earlier digits t have started (t > 1);
+          // the last plane of a short right operand opens a new level
+          const bool opens = t > 1 && SB < OZ_S + 1 - (t - 1) && nu == SB;
+          const int n0 = opens ? nu - 1 : nu;
+          const uint32_t acc0 = t == 1 ? first : 1u;
+          const uint32_t ip = oz_idesc(OZ_BM, OZ_BN * n0, false), in = oz_idesc(OZ_BM, OZ_BN * n0, true);
+          oz_mma(leader, dr, ar, br, ip, acc0);                         // C_r += Ar Br
+          oz_mma(leader, dr, ai, bi, cA ? ip : in, 1u);                 // C_r -= Ai Bi
+          oz_mma(leader, di, ar, bi, ip, acc0);                         // C_i += Ar Bi
+          oz_mma(leader, di, ai, br, cA ? in : ip, 1u);                 // C_i += Ai Br
+          if (opens) {
+            const uint32_t jp = oz_idesc(OZ_BM, OZ_BN, false), jn = oz_idesc(OZ_BM, OZ_BN, true);
+            const uint32_t off = (uint32_t)(OZ_BN * n0), bo = n0 * (OZ_B_TILE >> 4);
+            oz_mma(leader, dr + off, ar, br + bo, jp, first);
+            oz_mma(leader, dr + off, ai, bi + bo, cA ? jp : jn, 1u);
+            oz_mma(leader, di + off, ar, bi + bo, jp, first);
+            oz_mma(leader, di + off, ai, br + bo, cA ? jn : jp, 1u);
           }
-          tc_fence_after();
-          const uint32_t abase = tc_smem_u32(sA + s * OZ_A_STAGE), bbase = tc_smem_u32(sB + s * OZ_B_STAGE);
-          // digit t of A times planes u = 1 .. 7 - t of B (adjacent in shared
-          // memory) into the accumulators of levels t + 1 .. 7 (adjacent in
-          // tensor memory); the t = 1 MMAs of a block's first k step cover
-          // every level and start the block's sums
-          const uint64_t br = oz_desc_sw32(bbase), bi = oz_desc_sw32(bbase + OZ_S * OZ_B_TILE);
-#pragma unroll 1
-          for (int t = 1; t <= OZ_S; ++t) {
-            const int N = OZ_BN * (OZ_S + 1 - t);
-            const uint32_t ip = oz_idesc(OZ_BM, N, false), in = oz_idesc(OZ_BM, N, true);
-            const uint32_t acc0 = (ks == 0 && t == 1) ? 0u : 1u;
-            const uint32_t dr = tmem + (uint32_t)(OZ_BN * (t - 1)), di = tmem + (uint32_t)(OZ_BN * (OZ_NGRP + t - 1));
-            const uint64_t ar = oz_desc_sw32(abase + (0 * OZ_S + t - 1) * OZ_A_TILE);
-            const uint64_t ai = oz_desc_sw32(abase + (1 * OZ_S + t - 1) * OZ_A_TILE);
-            // signs of a conjugated operand: C_r = Ar Br - sA sB Ai Bi,
-            // C_i = sB Ar Bi + sA Ai Br with s = -1 for a conjugated side
-            constexpr bool cA = OzConj<ST>::A, cB = OzConj<ST>::B;
-            oz_mma(dr, ar, br, ip, acc0);                         // C_r += Ar Br
-            oz_mma(dr, ai, bi, (cA != cB) ? ip : in, 1u);         // C_r -= Ai Bi
-            oz_mma(di, ar, bi, cB ? in : ip, acc0);               // C_i += Ar Bi
-            oz_mma(di, ai, br, cA ? in : ip, 1u);                 // C_i += Ai Br
-          }
-          oz_commit(&empty[s]);  // the stage is free once these MMAs have read it
-          issued_mma = it + 1;
         }
-        if (!ok) break;
-        oz_commit(accf);  // block kb's sums are ready
+        if (leader) oz_commit(&empty[s]);  // the stage is free once these MMAs have read it
+        issued_mma = 1;
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        if (issued_mma > 0) {  // the MMAs issued read shared memory and write the tensor memory freed below
-          oz_commit(drain);
-          for (uint32_t i = 0; i < a.poll_limit; ++i)
-            if (tc_mbar_try_wait(drain, 0)) break;
-        }
+      if (!ok) break;
+      if (leader) oz_commit(accf);  // block kb's sums are ready
+    }
+    if (!ok && leader) {
+      *abort_flag = 1;
+      if (issued_mma > 0) {  // the MMAs issued read shared memory and write the tensor memory freed below
+        oz_commit(drain);
+        for (uint32_t i = 0; i < a.poll_limit; ++i)
+          if (tc_mbar_try_wait(drain, 0)) break;
       }
     }
     __syncwarp();
@@ -656,53 +761,64 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int ew = warp - 2, quad = warp & 3, part = ew >> 2;
     const int i = i0 + 32 * quad + lane;  // row of C
     const int jq = j0 + 8 * part;         // first column of this warp
-    const int nkbt = a.Kp / OZ_KB;        // k blocks of the scale arrays
-    float hr[8], lr[8], hi[8], li[8];      // double-float sums (Re, Im) of 8 columns
+    int64_t hr[8], hi[8];  // sums (Re, Im) of 8 columns in units of level 6
+    float lr[8], li[8];    // levels 7 and 8, in units of level 8
+    volatile double ext[16];  // what OZ_FLUSH blocks moved out of hr, hi (depths above 64 OZ_FLUSH only)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) hr[c] = lr[c] = hi[c] = li[c] = 0.f;
+    for (int c = 0; c < 8; ++c) {
+      hr[c] = hi[c] = 0;
+      lr[c] = li[c] = 0.f;
+    }
+    const bool deep = nkb > OZ_FLUSH;
+    if (deep)
+      for (int c = 0; c < 16; ++c) ext[c] = 0.0;
     bool ok = true;
+    const uint32_t lanes = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(8 * part);
     for (int kb = 0; kb < nkb; ++kb) {
-      // the block scales first: their loads overlap the wait for the MMAs
-      const int sb = kb / (OZ_KB / OZ_DRAIN);  // the scale block holding this accumulation block
-      const float sa = (i < a.lc) ? a.As[((size_t)z * nkbt + sb) * a.lc + i] : 0.f;
-      const float* sbp = a.Bs + ((size_t)z * nkbt + sb) * a.nc;
-      float sbv[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) sbv[c] = (jq + c < a.nc) ? __ldg(sbp + jq + c) : 0.f;
-      ok = oz_warp_wait(accf, (uint32_t)kb & 1u, a.poll_limit, a.err, abort_flag);
-      if (!ok) break;
+      if (!(ok = oz_warp_wait(accf, (uint32_t)kb & 1u, a.poll_limit, a.err, abort_flag))) break;
       tc_fence_after();
-      const uint32_t lanes = (uint32_t)(32 * quad) << 16;
 #pragma unroll
-      for (int c4 = 0; c4 < 8; c4 += 4) {  // four columns of every accumulator per load
-        float v[2 * OZ_NGRP][4];
+      for (int c2 = 0; c2 < 8; c2 += 2) {  // two columns of every accumulator per load
+        float v[2 * OZ_NGRP][2];
 #pragma unroll
-        for (int g = 0; g < 2 * OZ_NGRP; ++g) oz_ld4(tmem + lanes + (uint32_t)(OZ_BN * g + 8 * part + c4), v[g]);
+        for (int g = 0; g < 2 * OZ_NGRP; ++g) oz_ld2(lanes + (uint32_t)(OZ_BN * g + c2), v[g]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (c2 == 6) {  // everything is in registers: the accumulators may be overwritten
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) oz_arrive(accfree);
+        }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float sc = sa * sbv[c4 + q];
-          // levels 2, 3, 4 exactly into (s, e + e2), levels 5, 6, 7 into the low part
-          float s, e, s2, e2;
-          two_sum(v[0][q], v[1][q], s, e);
-          two_sum(s, v[2][q], s2, e2);
-          float lo = (e + e2) + (v[3][q] + (v[4][q] + v[5][q]));
-          oz_df_add(hr[c4 + q], lr[c4 + q], s2 * sc, lo * sc);
-          two_sum(v[6][q], v[7][q], s, e);
-          two_sum(s, v[8][q], s2, e2);
-          lo = (e + e2) + (v[9][q] + (v[10][q] + v[11][q]));
-          oz_df_add(hi[c4 + q], li[c4 + q], s2 * sc, lo * sc);
+        for (int q = 0; q < 2; ++q) {
+          oz_add_levels(hr[c2 + q], lr[c2 + q], v, q);
+          oz_add_levels(hi[c2 + q], li[c2 + q], v + OZ_NGRP, q);
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) oz_arrive(accfree);  // the accumulators may be overwritten
+      if (deep && (kb % OZ_FLUSH) == OZ_FLUSH - 1) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          ext[c] = ext[c] + (double)hr[c];
+          ext[8 + c] = ext[8 + c] + (double)hi[c];
+          hr[c] = hi[c] = 0;
+        }
+      }
     }
     if (ok && i < op.M) {
+      // (the digits of a short operand are those of N 2^24, its integer in the units of a full one)
+      const double sa = oz_scale(a.As[(size_t)z * a.lc + i]);
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const int j = jq + c;
-        if (j < op.N) oz_store<ST>(D, ptrs[z], op, i, j, (double)hr[c] + (double)lr[c], (double)hi[c] + (double)li[c]);
+        if (j < op.N) {
+          const double sc = sa * oz_scale(a.Bs[(size_t)z * a.nc + j]);
+          double re = fma((double)lr[c], 1.52587890625e-5, (double)hr[c]);  // level 8 = 2^-16 of level 6
+          double im = fma((double)li[c], 1.52587890625e-5, (double)hi[c]);
+          if (deep) {
+            re += ext[c];
+            im += ext[8 + c];
+          }
+          oz_store<ST>(D, ptrs[z], op, i, j, re * sc, im * sc);
+        }
       }
     }
   }
@@ -715,61 +831,38 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   }
 }
 
-static size_t oz_smem_bytes() { return 1024 + (size_t)OZ_STAGES * (OZ_A_STAGE + OZ_B_STAGE) + (2 * OZ_STAGES + 3) * 8 + 16; }
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-typedef CUresult (*OzEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static OzEncodeFn oz_encode_fn() {
-  static std::mutex mu;
-  static OzEncodeFn fn = nullptr;
-  std::lock_guard<std::mutex> g(mu);
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (OzEncodeFn)p;
-  }
-  return fn;
-}
-
-// 5-D map over digit arrays [z][reim][t][row][k] (BF16): box 16 k x box_rows
-// rows x all digits x both parts x one instance, 32-byte swizzle.
-static bool oz_make_map(CUtensorMap* m, const uint16_t* base, int Kp, int rows, int batch, int box_rows) {
-  OzEncodeFn enc = oz_encode_fn();
-  if (!enc) return false;
-  cuuint64_t dims[5] = {(cuuint64_t)Kp, (cuuint64_t)rows, (cuuint64_t)OZ_S, 2, (cuuint64_t)batch};
-  const cuuint64_t rb = (cuuint64_t)Kp * 2;
-  cuuint64_t strides[4] = {rb, rb * rows, rb * rows * OZ_S, rb * rows * OZ_S * 2};
-  cuuint32_t box[5] = {(cuuint32_t)OZ_KS, (cuuint32_t)box_rows, (cuuint32_t)OZ_S, 2, 1};
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)base, dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 int oz_kpad(int m) { return ((m + OZ_KB - 1) / OZ_KB) * OZ_KB; }
 
 size_t oz_digits_bytes(int rows, int m) { return (size_t)2 * OZ_S * rows * oz_kpad(m) * sizeof(uint16_t); }
-size_t oz_scales_bytes(int rows, int m) { return (size_t)(oz_kpad(m) / OZ_KB) * rows * sizeof(float); }
+size_t oz_digits_q_bytes(int rows, int m) { return (size_t)2 * OZ_SQ * rows * oz_kpad(m) * sizeof(uint16_t); }
+size_t oz_scales_bytes(int rows) { return (size_t)rows * sizeof(int); }
+
+template <int ST>
+static cudaError_t oz_launch(int Mc, int Nc, int batch, const Dims* dims, const ProbPtr* ptrs, const OzArgs& oa,
+                             cudaStream_t st) {
+  k_oz_gemm<ST><<<dim3((Nc + OZ_BN - 1) / OZ_BN, (Mc + OZ_BM - 1) / OZ_BM, batch), OZ_THREADS, OzGeo<ST>::smem, st>>>(
+      dims, ptrs, oa);
+  return cudaGetLastError();
+}
 
 template <int ST>
 static cudaError_t oz_attr() {
-  return cudaFuncSetAttribute(k_oz_gemm<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_smem_bytes());
+  return cudaFuncSetAttribute(k_oz_gemm<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OzGeo<ST>::smem);
 }
 
 cudaError_t oz_prepare() {
-  if (!oz_encode_fn()) return cudaErrorNotSupported;
   static int done = 0;
   if (!done) {
-    const cudaError_t es[] = {oz_attr<OZ_PROJ>(), oz_attr<OZ_GRAM>(), oz_attr<G_G1>(), oz_attr<G_Q1>(), oz_attr<G_G2>(),
-                              oz_attr<G_QB>(),    oz_attr<G_X>(),  oz_attr<G_U>(),  oz_attr<G_V>(),
-                              oz_attr<OZ_THETA>(), oz_attr<OZ_GATE>()};
+    const cudaError_t es[] = {
+        oz_attr<OZ_PROJ>(), oz_attr<OZ_GRAM>(), oz_attr<OZ_THETA>(), oz_attr<OZ_GATE>(), oz_attr<G_X>(),
+        oz_attr<G_U>(),     oz_attr<G_V>(),     oz_attr<G_Y0>(),     oz_attr<G_Y>(),     oz_attr<G_YT>(),
+        oz_attr<G_BH>(),    oz_attr<G_PR>(),    oz_attr<G_PQ>(),     oz_attr<G_PD>(),    oz_attr<G_CYG>(),
+        oz_attr<G_CYQ>(),   oz_attr<G_CQG>(),   oz_attr<G_CQQ>(),    oz_attr<G_CTG>(),   oz_attr<G_CTQ>(),
+        oz_attr<G_CRG>(),   oz_attr<G_CRQ>()};
     for (cudaError_t e : es)
       if (e != cudaSuccess) return e;
     done = 1;
@@ -780,8 +873,15 @@ cudaError_t oz_prepare() {
 // Capacities (rows of C, columns of C, depth) of a stage's product.
 static void oz_stage_caps(int stage, const Caps& c, int& Mc, int& Nc, int& Kc) {
   switch (stage) {
-    case G_G1: case G_G2: case G_X: Mc = c.l; Nc = c.l; Kc = c.n; break;
-    case G_Q1: case G_QB: Mc = c.n; Nc = c.l; Kc = c.l; break;
+    case G_Y0: case G_Y: Mc = c.m; Nc = c.l; Kc = c.n; break;
+    case G_YT: case G_BH: Mc = c.n; Nc = c.l; Kc = c.m; break;
+    case G_PR: Mc = c.m; Nc = c.r; Kc = c.n; break;
+    case G_PQ: Mc = c.l; Nc = c.r; Kc = c.m; break;
+    case G_PD: Mc = c.m; Nc = c.r; Kc = c.l; break;
+    case G_CYG: case G_CQG: Mc = c.l; Nc = c.l; Kc = c.m; break;
+    case G_CYQ: case G_CQQ: Mc = c.m; Nc = c.l; Kc = c.l; break;
+    case G_CTG: case G_CRG: case G_X: Mc = c.l; Nc = c.l; Kc = c.n; break;
+    case G_CTQ: case G_CRQ: Mc = c.n; Nc = c.l; Kc = c.l; break;
     case G_U: Mc = c.m; Nc = c.k; Kc = c.l; break;
     case OZ_THETA: Mc = c.m; Nc = c.n; Kc = c.cm; break;  // K = chi_m, at most its bond's capacity
     case OZ_GATE: Mc = c.dl * c.dr; Nc = c.cl * c.cr; Kc = c.dl * c.dr; break;
@@ -791,15 +891,15 @@ static void oz_stage_caps(int stage, const Caps& c, int& Mc, int& Nc, int& Kc) {
 
 bool oz_stage_rule(const Caps& cap) { return cap.l >= 48 && (cap.m >= 256 || cap.n >= 256); }
 
-static const int OZ_STAGE_LIST[] = {G_G1, G_Q1, G_G2, G_QB, G_X, G_U, G_V};
+static const int OZ_STAGE_LIST[] = {G_CTG, G_CTQ, G_X, G_U, G_V};
 
 static void oz_grow(OzStageBytes& b, int stage, const Caps& c) {
   int Mc, Nc, Kc;
   oz_stage_caps(stage, c, Mc, Nc, Kc);
   b.ad = std::max(b.ad, oz_digits_bytes(Mc, Kc));
-  b.as = std::max(b.as, oz_scales_bytes(Mc, Kc));
+  b.as = std::max(b.as, oz_scales_bytes(Mc));
   b.bd = std::max(b.bd, oz_digits_bytes(Nc, Kc));
-  b.bs = std::max(b.bs, oz_scales_bytes(Nc, Kc));
+  b.bs = std::max(b.bs, oz_scales_bytes(Nc));
 }
 
 OzStageBytes oz_stage_bytes(int m, int n, int k, int l, const Caps* gate) {
@@ -816,93 +916,256 @@ OzStageBytes oz_stage_bytes(int m, int n, int k, int l, const Caps* gate) {
 
 bool oz_gate_rule(const Caps& cap) { return cap.dl * cap.dr >= GATE_GEMM_MIN; }
 
-template <int ST>
-static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch, int Mc, int Nc, int Kc,
-                                const OzScratch& sc, int* err, cudaStream_t st) {
-  const int Kp = oz_kpad(Kc);
-  // G1 and G2 multiply an operand by its own adjoint: one set of digits
-  const bool same = ST == G_G1 || ST == G_G2;
-  {
-    ProfScope ps("k_oz_digits[op]", st);
-    k_oz_digits_op<ST, 0><<<dim3((Mc + 15) / 16, Kp / OZ_KB, batch), 256, 0, st>>>(dims, ptrs, sc.ad, sc.as, Mc, Kp);
-    if (!same)
-      k_oz_digits_op<ST, 1><<<dim3((Nc + 15) / 16, Kp / OZ_KB, batch), 256, 0, st>>>(dims, ptrs, sc.bd, sc.bs, Nc,
-                                                                                      Kp);
-    const cudaError_t e = cudaGetLastError();
+// Digits and exponents of one operand (rows rc, padded depth Kp).
+template <int ST, int SIDE>
+static cudaError_t oz_digits(const Dims* dims, const ProbPtr* ptrs, int batch, int rc, int Kp, uint16_t* Xd, int* Es,
+                             int cond, cudaStream_t st, const char* label = "k_oz_digits[op]") {
+  ProfScope ps(label, st);
+  if (Kp <= OZ_SELF_K) {
+    k_oz_digits_op<ST, SIDE, true><<<dim3((rc + 15) / 16, 1, batch), 256, 0, st>>>(dims, ptrs, Xd, Es, rc, Kp, cond);
+  } else {
+    const cudaError_t e = cudaMemsetAsync(Es, 0, sizeof(int) * (size_t)rc * batch, st);
     if (e != cudaSuccess) return e;
+    k_oz_max<ST, SIDE><<<dim3((rc + 15) / 16, (Kp + OZ_MAX_K - 1) / OZ_MAX_K, batch), 256, 0, st>>>(dims, ptrs, Es,
+                                                                                                   rc, cond);
+    k_oz_digits_op<ST, SIDE, false><<<dim3((rc + 15) / 16, Kp / OZ_KB, batch), 256, 0, st>>>(dims, ptrs, Xd, Es, rc,
+                                                                                             Kp, cond);
   }
-  CUtensorMap ta, tb;
-  if (!oz_make_map(&ta, sc.ad, Kp, Mc, batch, OZ_BM) || !oz_make_map(&tb, same ? sc.ad : sc.bd, Kp, Nc, batch, OZ_BN))
-    return cudaErrorInvalidValue;
-  OzArgs oa;
-  oa.lc = Mc;
-  oa.nc = Nc;
-  oa.Kp = Kp;
-  oa.As = sc.as;
-  oa.Bs = same ? sc.as : sc.bs;
-  oa.err = err;
-  oa.poll_limit = 1u << 24;
-  oa.stall = 0;
-  ProfScope ps(ST == G_U || ST == G_V ? "k_oz_gemm[uv]"
-               : ST == OZ_THETA          ? "k_oz_gemm[theta]"
-               : ST == OZ_GATE           ? "k_oz_gemm[gate]"
-                                         : "k_oz_gemm[cholqr]",
-               st);
-  k_oz_gemm<ST><<<dim3((Nc + OZ_BN - 1) / OZ_BN, (Mc + OZ_BM - 1) / OZ_BM, batch), OZ_THREADS, oz_smem_bytes(), st>>>(
-      ta, tb, dims, ptrs, oa);
   return cudaGetLastError();
 }
 
+// One product; pre: the left operand's digits where they are already made
+// (theta's), else they go to the scratch.
+template <int ST>
+static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch, int Mc, int Nc, int Kc,
+                                const OzScratch& sc, int cond, int* err, cudaStream_t st,
+                                const uint16_t* pre = nullptr, const int* pre_es = nullptr) {
+  const int Kp = oz_kpad(Kc);
+  // an operand times its own adjoint: one set of digits
+  constexpr bool same = ST == G_G1 || ST == G_G2 || ST == G_CYG || ST == G_CQG || ST == G_CTG || ST == G_CRG;
+  cudaError_t e = cudaSuccess;
+  if (!same && !pre && Kp <= OZ_SELF_K) {
+    if constexpr (!same) {
+      ProfScope ps("k_oz_digits[op]", st);
+      k_oz_digits_two<ST><<<dim3((std::max(Mc, Nc) + 15) / 16, 2, batch), 256, 0, st>>>(dims, ptrs, sc.ad, sc.as, Mc,
+                                                                                        sc.bd, sc.bs, Nc, Kp, cond);
+      e = cudaGetLastError();
+    }
+  } else {
+    if (!pre) e = oz_digits<ST, 0>(dims, ptrs, batch, Mc, Kp, sc.ad, sc.as, cond, st);
+    if constexpr (!same)
+      if (e == cudaSuccess) e = oz_digits<ST, 1>(dims, ptrs, batch, Nc, Kp, sc.bd, sc.bs, cond, st);
+  }
+  if (e != cudaSuccess) return e;
+  const uint16_t* ad = pre ? pre : sc.ad;
+  OzArgs oa;
+  oa.Ad = ad;
+  oa.Bd = same ? ad : sc.bd;
+  oa.lc = Mc;
+  oa.nc = Nc;
+  oa.Kp = Kp;
+  oa.As = pre ? pre_es : sc.as;
+  oa.Bs = same ? oa.As : sc.bs;
+  oa.err = err;
+  oa.poll_limit = 1u << 24;
+  oa.stall = 0;
+  oa.cond = cond;
+  ProfScope ps(ST == G_U || ST == G_V ? "k_oz_gemm[uv]"
+               : ST == OZ_THETA          ? "k_oz_gemm[theta]"
+               : ST == OZ_GATE           ? "k_oz_gemm[gate]"
+               : ST <= G_BH || (ST >= G_PR && ST <= G_PD) ? "k_oz_gemm[sketch]"
+                                         : "k_oz_gemm[cholqr]",
+               st);
+  return oz_launch<ST>(Mc, Nc, batch, dims, ptrs, oa, st);
+}
+
 cudaError_t launch_oz_stage(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
-                            const OzScratch& sc, int* err, cudaStream_t st) {
+                            const OzScratch& sc, int* err, cudaStream_t st, int cond) {
   const cudaError_t e = oz_prepare();
   if (e != cudaSuccess) return e;
   int Mc, Nc, Kc;
   oz_stage_caps(stage, cap, Mc, Nc, Kc);
+#define OZ_CASE(S) \
+  case S: return oz_stage_run<S>(dims, ptrs, batch, Mc, Nc, Kc, sc, cond, err, st)
   switch (stage) {
     case OZ_THETA:
-      if (!oz_gate_rule(cap)) return cudaSuccess;
-      return oz_stage_run<OZ_THETA>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
     case OZ_GATE:
       if (!oz_gate_rule(cap)) return cudaSuccess;
-      return oz_stage_run<OZ_GATE>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_G1: return oz_stage_run<G_G1>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_Q1: return oz_stage_run<G_Q1>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_G2: return oz_stage_run<G_G2>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_QB: return oz_stage_run<G_QB>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_X: return oz_stage_run<G_X>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_U: return oz_stage_run<G_U>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
-    case G_V: return oz_stage_run<G_V>(dims, ptrs, batch, Mc, Nc, Kc, sc, err, st);
+      return stage == OZ_THETA ? oz_stage_run<OZ_THETA>(dims, ptrs, batch, Mc, Nc, Kc, sc, cond, err, st)
+                               : oz_stage_run<OZ_GATE>(dims, ptrs, batch, Mc, Nc, Kc, sc, cond, err, st);
+    OZ_CASE(G_X);
+    OZ_CASE(G_U);
+    OZ_CASE(G_V);
+    OZ_CASE(G_PQ);
+    OZ_CASE(G_PD);
+    OZ_CASE(G_CYG);
+    OZ_CASE(G_CYQ);
+    OZ_CASE(G_CQG);
+    OZ_CASE(G_CQQ);
+    OZ_CASE(G_CTG);
+    OZ_CASE(G_CTQ);
+    OZ_CASE(G_CRG);
+    OZ_CASE(G_CRQ);
     default: return cudaErrorInvalidValue;
   }
+#undef OZ_CASE
 }
 
-cudaError_t launch_oz_digits_theta(const Dims* dims, const ProbPtr* ptrs, uint16_t* Bd, float* Bs, int m, int n,
+// The same for a batch in runs of `chunk` problems, which share the scratch.
+cudaError_t launch_oz_range(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
+                            const OzScratch& sc, int chunk, int cond, int* err, cudaStream_t st) {
+  for (int z = 0; z < batch; z += chunk) {
+    const cudaError_t e = launch_oz_stage(stage, dims + z, ptrs + z, std::min(chunk, batch - z), cap, sc, err, st, cond);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 form's products with theta.
+// ---------------------------------------------------------------------------
+struct DpLayout {
+  size_t tr, tc, er, ec, ad, as, bd, bs;  // bytes per problem
+  size_t per(bool both) const { return (both ? tr + tc : std::max(tr, tc)) + er + ec + ad + as + bd + bs; }
+};
+
+static DpLayout dp_layout(const Caps& c) {
+  DpLayout d;
+  const int mx = std::max(c.m, c.n), w = std::max(c.l, std::max(c.k, c.r));
+  d.tr = oz_digits_bytes(c.m, c.n);
+  d.tc = oz_digits_bytes(c.n, c.m);
+  d.er = oz_scales_bytes(c.m);
+  d.ec = oz_scales_bytes(c.n);
+  // left operands: l or mx rows, depths mx or l; right ones: w rows
+  d.ad = std::max(oz_digits_bytes(c.l, mx), oz_digits_bytes(mx, c.l));
+  d.as = oz_scales_bytes(std::max(mx, c.l));
+  d.bd = std::max(oz_digits_bytes(w, mx), oz_digits_bytes(w, c.l));
+  d.bs = oz_scales_bytes(w);
+  return d;
+}
+
+static size_t dp_up(size_t x) { return (x + 255) & ~(size_t)255; }
+
+static int dp_chunk(const DpLayout& d, int batch, size_t limit, int* all) {
+  *all = d.per(true) * batch <= limit;
+  if (*all) return batch;
+  const size_t c = limit / d.per(false);
+  return c < 1 ? 1 : (c < (size_t)batch ? (int)c : batch);
+}
+
+size_t dp_bytes(const Caps& cap, int batch, size_t limit) {
+  const DpLayout d = dp_layout(cap);
+  int all;
+  const size_t c = dp_chunk(d, batch, limit, &all);
+  return (all ? dp_up(d.tr * c) + dp_up(d.tc * c) : dp_up(std::max(d.tr, d.tc) * c)) + dp_up(d.er * c) +
+         dp_up(d.ec * c) + dp_up(d.ad * c) + dp_up(d.as * c) + dp_up(d.bd * c) + dp_up(d.bs * c);
+}
+
+DpScratch dp_carve(char* base, const Caps& cap, int batch, size_t limit, int* err) {
+  const DpLayout d = dp_layout(cap);
+  DpScratch s;
+  s.chunk = dp_chunk(d, batch, limit, &s.all);
+  s.err = err;
+  const size_t c = s.chunk;
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    char* q = base + o;
+    o += dp_up(bytes * c);
+    return q;
+  };
+  if (s.all) {
+    s.tr = (uint16_t*)take(d.tr);
+    s.tc = (uint16_t*)take(d.tc);
+  } else {
+    s.tr = s.tc = (uint16_t*)take(std::max(d.tr, d.tc));
+  }
+  s.er = (int*)take(d.er);
+  s.ec = (int*)take(d.ec);
+  s.oz.ad = (uint16_t*)take(d.ad);
+  s.oz.as = (int*)take(d.as);
+  s.oz.bd = (uint16_t*)take(d.bd);
+  s.oz.bs = (int*)take(d.bs);
+  return s;
+}
+
+// theta's digits: rows (for Y = A X) or columns (for A^H Q)
+static cudaError_t dp_theta(const DpPath& p, int z, int cnt, bool rows) {
+  return rows ? oz_digits<G_Y, 0>(p.dims + z, p.ptrs + z, cnt, p.cap.m, oz_kpad(p.cap.n), p.dp->tr, p.dp->er, DPC_DIG,
+                                  p.st, "k_oz_digits[theta]")
+              : oz_digits<G_YT, 0>(p.dims + z, p.ptrs + z, cnt, p.cap.n, oz_kpad(p.cap.m), p.dp->tc, p.dp->ec, DPC_DIG,
+                                   p.st, "k_oz_digits[theta]");
+}
+
+cudaError_t dp_begin(const DpPath& p) {
+  if (!p.dp || !p.dp->all) return cudaSuccess;
+  cudaError_t e = dp_theta(p, 0, p.batch, true);
+  return e == cudaSuccess ? dp_theta(p, 0, p.batch, false) : e;
+}
+
+cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond) {
+  const DpScratch& s = *p.dp;
+  if (stage != G_Y0 && stage != G_Y && stage != G_YT && stage != G_BH && stage != G_PR)
+    return launch_oz_range(stage, p.dims, p.ptrs, p.batch, p.cap, s.oz, s.chunk, cond, s.err, p.st);
+  cudaError_t e = oz_prepare();
+  if (e != cudaSuccess) return e;
+  const bool rows = stage != G_YT && stage != G_BH;
+  int Mc, Nc, Kc;
+  oz_stage_caps(stage, p.cap, Mc, Nc, Kc);
+  for (int z = 0; z < p.batch; z += s.chunk) {
+    const int cnt = std::min(s.chunk, p.batch - z);
+    if (!s.all && (e = dp_theta(p, z, cnt, rows)) != cudaSuccess) return e;
+    const uint16_t* pre = rows ? s.tr : s.tc;
+    const int* es = rows ? s.er : s.ec;
+    const Dims* dm = p.dims + z;
+    const ProbPtr* pp = p.ptrs + z;
+    switch (stage) {
+      case G_Y0: e = oz_stage_run<G_Y0>(dm, pp, cnt, Mc, Nc, Kc, s.oz, cond, s.err, p.st, pre, es); break;
+      case G_Y: e = oz_stage_run<G_Y>(dm, pp, cnt, Mc, Nc, Kc, s.oz, cond, s.err, p.st, pre, es); break;
+      case G_PR: e = oz_stage_run<G_PR>(dm, pp, cnt, Mc, Nc, Kc, s.oz, cond, s.err, p.st, pre, es); break;
+      case G_YT: e = oz_stage_run<G_YT>(dm, pp, cnt, Mc, Nc, Kc, s.oz, cond, s.err, p.st, pre, es); break;
+      default: e = oz_stage_run<G_BH>(dm, pp, cnt, Mc, Nc, Kc, s.oz, cond, s.err, p.st, pre, es); break;
+    }
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t DpPath::gemm(int stage) const {
+  const int tile = (tiles && stage <= G_V) ? tiles[stage] : 0;
+  if (dp) {
+    const int chk = (stage >= G_PR && stage <= G_PD) ? DPC_CHK : 0;
+    const cudaError_t e = launch_dp_stage(stage, *this, DPC_DIG | chk);
+    if (e != cudaSuccess) return e;
+    if (dp_rule(cap.m, cap.n, cap.l) && cap.cm == 0) return cudaSuccess;  // a plan: every problem has the same sizes
+  }
+  return launch_zgemm_tile(stage, tile, dims, ptrs, batch, cap, st);
+}
+
+cudaError_t launch_oz_digits_theta(const Dims* dims, const ProbPtr* ptrs, uint16_t* Bd, int* Bs, int m, int n,
                                    int batch, cudaStream_t st) {
+  // the columns' exponents are in Bs (k_conv_theta)
   ProfScope ps("k_oz_digits[theta]", st);
   const int Kp = oz_kpad(m);
-  k_oz_digits_theta<<<dim3((n + 15) / 16, Kp / OZ_KB, batch), 256, 0, st>>>(dims, ptrs, Bd, Bs, n, Kp);
+  k_oz_digits_op<OZ_PROJ, 1, false><<<dim3((n + 15) / 16, Kp / OZ_KB, batch), 256, 0, st>>>(dims, ptrs, Bd, Bs, n, Kp,
+                                                                                            0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_oz_digits_qf(const Dims* dims, const float2* Qf, uint16_t* Ad, float* As, int m, int l, int batch,
+cudaError_t launch_oz_digits_qf(const Dims* dims, const ProbPtr* ptrs, float2* Qf, uint16_t* Ad, int* As, int m, int l, int batch,
                                 cudaStream_t st) {
   const int Kp = oz_kpad(m);
   ProfScope ps("k_oz_digits[q]", st);
-  const int warps = l * (Kp / OZ_KB);
-  k_oz_digits_q<<<dim3((warps + 7) / 8, batch), 256, 0, st>>>(dims, Qf, Ad, As, m, l, Kp);
+  k_oz_digits_q<<<dim3((l + 7) / 8, batch), 256, 0, st>>>(dims, ptrs, Qf, Ad, As, m, l, Kp);
   return cudaGetLastError();
 }
 
-cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const float* As, int m, int l,
+cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const int* As, int m, int l,
                            int batch, int* err, cudaStream_t st) {
   const cudaError_t e = oz_prepare();
   if (e != cudaSuccess) return e;
   const int Kp = oz_kpad(m);
-  CUtensorMap ta, tb;
-  if (!oz_make_map(&ta, Ad, Kp, l, batch, OZ_BM) || !oz_make_map(&tb, Ad, Kp, l, batch, OZ_BN))
-    return cudaErrorInvalidValue;
   OzArgs oa;
+  oa.Ad = oa.Bd = Ad;
   oa.lc = l;
   oa.nc = l;
   oa.Kp = Kp;
@@ -911,27 +1174,20 @@ cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t
   oa.err = err;
   oa.poll_limit = 1u << 24;
   oa.stall = 0;
+  oa.cond = 0;
   ProfScope ps("k_oz_gemm[gram]", st);
-  k_oz_gemm<OZ_GRAM><<<dim3((l + OZ_BN - 1) / OZ_BN, (l + OZ_BM - 1) / OZ_BM, batch), OZ_THREADS, oz_smem_bytes(),
-                       st>>>(ta, tb, dims, ptrs, oa);
-  return cudaGetLastError();
+  return oz_launch<OZ_GRAM>(l, l, batch, dims, ptrs, oa, st);
 }
 
-cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const float2* Qf, const float2* Dbuf,
-                           uint16_t* Ad, float* As, const uint16_t* Bd, const float* Bs, int m, int n, int l, int batch,
-                           int* err, cudaStream_t st, bool digits_done) {
+cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const int* As, const uint16_t* Bd, const int* Bs, int m, int n, int l, int batch,
+                           int* err, cudaStream_t st) {
   const int Kp = oz_kpad(m);
-  if (!digits_done) {
-    cudaError_t e = launch_oz_digits_qf(dims, Qf, Ad, As, m, l, batch, st);
-    if (e != cudaSuccess) return e;
-  }
   {
     cudaError_t e = oz_prepare();
     if (e != cudaSuccess) return e;
-    CUtensorMap ta, tb;
-    if (!oz_make_map(&ta, Ad, Kp, l, batch, OZ_BM) || !oz_make_map(&tb, Bd, Kp, n, batch, OZ_BN))
-      return cudaErrorInvalidValue;
     OzArgs oa;
+    oa.Ad = Ad;
+    oa.Bd = Bd;
     oa.lc = l;
     oa.nc = n;
     oa.Kp = Kp;
@@ -944,13 +1200,11 @@ cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const float2* 
     const bool stall = cap_st == cudaStreamCaptureStatusNone && fault_take(TEBD_FAULT_TC_STALL);
     oa.poll_limit = stall ? (1u << 12) : (1u << 24);
     oa.stall = stall ? 1 : 0;
+    oa.cond = 0;
     ProfScope ps("k_oz_proj[project]", st);
-    k_oz_gemm<OZ_PROJ><<<dim3((n + OZ_BN - 1) / OZ_BN, (l + OZ_BM - 1) / OZ_BM, batch), OZ_THREADS, oz_smem_bytes(),
-                         st>>>(ta, tb, dims, ptrs, oa);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    e = oz_launch<OZ_PROJ>(l, n, batch, dims, ptrs, oa, st);
+    return e;
   }
-  return launch_fold_bh(Dbuf, dims, ptrs, n, l, batch, st);
 }
 
 }  // namespace tg

@@ -460,7 +460,7 @@ static cudaError_t ensure_smem(K kernel, size_t bytes, size_t* done) {
 
 // Shared-memory limits set so far, per kernel (one record each, shared by the
 // launchers and qr_blocked_prepare so that a limit is never lowered).
-static size_t g_attr_qr = 0, g_attr_qr256 = 0, g_attr_ld = 0, g_attr_fold[2][2] = {{0, 0}, {0, 0}};
+static size_t g_attr_qr = 0, g_attr_qr256 = 0, g_attr_ld = 0, g_attr_fold[2] = {0, 0};
 
 // Batches of many small matrices take smaller CTAs when several fit an SM
 // (registers: 128 per thread; shared memory): the per-column barriers of one
@@ -544,15 +544,14 @@ __global__ void __launch_bounds__(512) k_lowdin(const Dims* __restrict__ dims, c
   }
 }
 
-// Out = X + X D with the small correction X D in FP32 (|D| ~ 1e-6, so its
-// relative FP32 error costs ~1e-13 absolute): Q = Q_f (I + D) from the FP32
-// Q_f (capacity Mc x Lc per instance) into ptrs[z].Q (D.m x D.l, compact), or,
-// in place, B^H = (A^H Q_f)(I + D) on ptrs[z].Yt (D.n x D.l, compact).  RPL
+// Q = Q_f + Q_f D with the small correction Q_f D in FP32 (|D| ~ 1e-6, so its
+// relative FP32 error costs ~1e-13 absolute) from the FP32 Q_f (capacity
+// Mc x Lc per instance) into ptrs[z].Q (D.m x D.l, compact).  RPL
 // rows per lane (32 RPL rows per CTA), staged column-major in shared memory
 // as FP32; warp w owns the columns c = w (mod 8).
 enum { QF_MAXL = 144, QF_MAXCPW = QF_MAXL / 8 };
 
-template <bool FROM_F32, int RPL>
+template <int RPL>
 __global__ void __launch_bounds__(256) k_fold(const float2* __restrict__ Qf, const float2* __restrict__ Dbase,
                                               const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs, int Mc,
                                               int Lc) {
@@ -561,27 +560,20 @@ __global__ void __launch_bounds__(256) k_fold(const float2* __restrict__ Qf, con
   const int z = blockIdx.y;
   const Dims Dm = dims[z];
   if (!Dm.active) return;
-  const int M = FROM_F32 ? Dm.m : Dm.n, L = Dm.l;
+  const int M = Dm.m, L = Dm.l;
   const int r0 = blockIdx.x * ROWS;
   if (r0 >= M) return;
   float2* Ds = reinterpret_cast<float2*>(qf_raw);  // L x L column-major
   float2* Qs = Ds + ((L * L + 1) & ~1);            // ROWS x L column-major (16-byte aligned)
-  const float2* q = FROM_F32 ? Qf + (size_t)z * Mc * Lc : nullptr;
-  cplx* X = FROM_F32 ? ptrs[z].Q : ptrs[z].Yt;  // output (and FP64 source when !FROM_F32), ld M
+  const float2* q = Qf + (size_t)z * Mc * Lc;
+  cplx* X = ptrs[z].Q;  // ld M
   const float2* D = Dbase + (size_t)z * Lc * Lc;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int e = tid; e < L * L; e += 256) Ds[e] = D[e];
   for (int e = tid; e < ROWS * L; e += 256) {
     const int c = e / ROWS, r = e % ROWS;
     float2 v = make_float2(0.f, 0.f);
-    if (r0 + r < M) {
-      if (FROM_F32) {
-        v = q[(size_t)c * Mc + r0 + r];
-      } else {
-        const cplx x = X[(size_t)c * M + r0 + r];
-        v = make_float2((float)x.x, (float)x.y);
-      }
-    }
+    if (r0 + r < M) v = q[(size_t)c * Mc + r0 + r];
     Qs[e] = v;
   }
   __syncthreads();
@@ -620,13 +612,8 @@ __global__ void __launch_bounds__(256) k_fold(const float2* __restrict__ Qf, con
     for (int j = 0; j < QF_MAXCPW; ++j) {
       const int c = warp + 8 * j;
       if (c < L) {
-        cplx b;
-        if (FROM_F32) {
-          const float2 f = Qs[c * ROWS + r];
-          b = cmk((double)f.x, (double)f.y);
-        } else {
-          b = X[(size_t)c * M + r0 + r];
-        }
+        const float2 f = Qs[c * ROWS + r];
+        const cplx b = cmk((double)f.x, (double)f.y);
         X[(size_t)c * M + r0 + r] = cmk(b.x + (double)acc[i][j].x, b.y + (double)acc[i][j].y);
       }
     }
@@ -634,19 +621,18 @@ __global__ void __launch_bounds__(256) k_fold(const float2* __restrict__ Qf, con
 }
 
 // batch == 0 only raises the shared-memory limit.
-template <bool FROM_F32>
 static cudaError_t launch_fold(const float2* Qf, const float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int Mc,
                                int Lc, int batch, cudaStream_t st) {
   if (Lc <= 128) {
     const size_t sm = sizeof(float2) * ((size_t)((Lc * Lc + 1) & ~1) + 64 * (size_t)Lc);
-    cudaError_t e = ensure_smem(k_fold<FROM_F32, 2>, sm, &g_attr_fold[FROM_F32][1]);
+    cudaError_t e = ensure_smem(k_fold<2>, sm, &g_attr_fold[1]);
     if (e != cudaSuccess || batch == 0) return e;
-    k_fold<FROM_F32, 2><<<dim3((Mc + 63) / 64, batch), 256, sm, st>>>(Qf, Dbuf, dims, ptrs, Mc, Lc);
+    k_fold<2><<<dim3((Mc + 63) / 64, batch), 256, sm, st>>>(Qf, Dbuf, dims, ptrs, Mc, Lc);
   } else {
     const size_t sm = sizeof(float2) * ((size_t)((Lc * Lc + 1) & ~1) + 32 * (size_t)Lc);
-    cudaError_t e = ensure_smem(k_fold<FROM_F32, 1>, sm, &g_attr_fold[FROM_F32][0]);
+    cudaError_t e = ensure_smem(k_fold<1>, sm, &g_attr_fold[0]);
     if (e != cudaSuccess || batch == 0) return e;
-    k_fold<FROM_F32, 1><<<dim3((Mc + 31) / 32, batch), 256, sm, st>>>(Qf, Dbuf, dims, ptrs, Mc, Lc);
+    k_fold<1><<<dim3((Mc + 31) / 32, batch), 256, sm, st>>>(Qf, Dbuf, dims, ptrs, Mc, Lc);
   }
   return cudaGetLastError();
 }
@@ -658,9 +644,7 @@ static cudaError_t launch_fold(const float2* Qf, const float2* Dbuf, const Dims*
 // its upper triangle in FP64 and staged as FP32, 32-deep K slices).
 // k_fold_big: one CTA per 32 rows holding its rows of X (all L columns, FP32)
 // in shared memory; each warp computes 16 output columns at a time with D
-// read through L1 (every lane of a warp reads the same D element).  Out of
-// place for Q; for B^H the rows are staged before any is overwritten, and a
-// CTA owns whole rows, so the in-place update is safe.
+// read through L1 (every lane of a warp reads the same D element).
 // ---------------------------------------------------------------------------
 enum { QF_MAXL_BIG = 512, QFB_ROWS = 32, QFB_CW = 16 };
 
@@ -735,7 +719,6 @@ __global__ void __launch_bounds__(256) k_lowdin_big(const Dims* __restrict__ dim
     }
 }
 
-template <bool FROM_F32>
 __global__ void __launch_bounds__(256) k_fold_big(const float2* __restrict__ Qf, const float2* __restrict__ Dbase,
                                                   const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
                                                   int Mc, int Lc) {
@@ -743,25 +726,18 @@ __global__ void __launch_bounds__(256) k_fold_big(const float2* __restrict__ Qf,
   const int z = blockIdx.y;
   const Dims Dm = dims[z];
   if (!Dm.active) return;
-  const int M = FROM_F32 ? Dm.m : Dm.n, L = Dm.l;
+  const int M = Dm.m, L = Dm.l;
   const int r0 = blockIdx.x * QFB_ROWS;
   if (r0 >= M) return;
   float2* Xs = reinterpret_cast<float2*>(qfb_raw);  // QFB_ROWS x L column-major
-  const float2* q = FROM_F32 ? Qf + (size_t)z * Mc * Lc : nullptr;
-  cplx* X = FROM_F32 ? ptrs[z].Q : ptrs[z].Yt;  // output (and FP64 source when !FROM_F32), ld M
+  const float2* q = Qf + (size_t)z * Mc * Lc;
+  cplx* X = ptrs[z].Q;  // ld M
   const float2* D = Dbase + (size_t)z * Lc * Lc;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int e = tid; e < QFB_ROWS * L; e += 256) {
     const int c = e / QFB_ROWS, r = e % QFB_ROWS;
     float2 v = make_float2(0.f, 0.f);
-    if (r0 + r < M) {
-      if (FROM_F32) {
-        v = q[(size_t)c * Mc + r0 + r];
-      } else {
-        const cplx x = X[(size_t)c * M + r0 + r];
-        v = make_float2((float)x.x, (float)x.y);
-      }
-    }
+    if (r0 + r < M) v = q[(size_t)c * Mc + r0 + r];
     Xs[e] = v;
   }
   __syncthreads();
@@ -786,13 +762,8 @@ __global__ void __launch_bounds__(256) k_fold_big(const float2* __restrict__ Qf,
       for (int j = 0; j < QFB_CW; ++j) {
         const int c = cb + j;
         if (c < L) {
-          cplx b;
-          if (FROM_F32) {
-            const float2 f = Xs[c * QFB_ROWS + lane];
-            b = cmk((double)f.x, (double)f.y);
-          } else {
-            b = X[(size_t)c * M + r];
-          }
+          const float2 f = Xs[c * QFB_ROWS + lane];
+          const cplx b = cmk((double)f.x, (double)f.y);
           X[(size_t)c * M + r] = cmk(b.x + (double)acc[j].x, b.y + (double)acc[j].y);
         }
       }
@@ -800,16 +771,15 @@ __global__ void __launch_bounds__(256) k_fold_big(const float2* __restrict__ Qf,
   }
 }
 
-static size_t g_attr_foldbig[2] = {0, 0};
+static size_t g_attr_foldbig = 0;
 
 // batch == 0 only raises the shared-memory limit.
-template <bool FROM_F32>
 static cudaError_t launch_fold_big(const float2* Qf, const float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int Mc,
                                    int Lc, int batch, cudaStream_t st) {
   const size_t sm = sizeof(float2) * (size_t)QFB_ROWS * Lc;
-  cudaError_t e = ensure_smem(k_fold_big<FROM_F32>, sm, &g_attr_foldbig[FROM_F32]);
+  cudaError_t e = ensure_smem(k_fold_big, sm, &g_attr_foldbig);
   if (e != cudaSuccess || batch == 0) return e;
-  k_fold_big<FROM_F32><<<dim3((Mc + QFB_ROWS - 1) / QFB_ROWS, batch), 256, sm, st>>>(Qf, Dbuf, dims, ptrs, Mc, Lc);
+  k_fold_big<<<dim3((Mc + QFB_ROWS - 1) / QFB_ROWS, batch), 256, sm, st>>>(Qf, Dbuf, dims, ptrs, Mc, Lc);
   return cudaGetLastError();
 }
 
@@ -824,11 +794,9 @@ cudaError_t qr_blocked_prepare(int M, int N, int L) {
   if (e == cudaSuccess && qr128 <= 56 * 1024) e = ensure_smem(k_qr_blk_f32<128>, qr128, &g_attr_qr128);
   if (e == cudaSuccess && L <= QF_MAXL) {
     e = ensure_smem(k_lowdin, sizeof(float2) * (size_t)L * L, &g_attr_ld);
-    if (e == cudaSuccess) e = launch_fold<true>(nullptr, nullptr, nullptr, nullptr, M, L, 0, nullptr);
-    if (e == cudaSuccess) e = launch_fold<false>(nullptr, nullptr, nullptr, nullptr, N, L, 0, nullptr);
+    if (e == cudaSuccess) e = launch_fold(nullptr, nullptr, nullptr, nullptr, M, L, 0, nullptr);
   } else if (e == cudaSuccess && L <= QF_MAXL_BIG) {
-    e = launch_fold_big<true>(nullptr, nullptr, nullptr, nullptr, M, L, 0, nullptr);
-    if (e == cudaSuccess) e = launch_fold_big<false>(nullptr, nullptr, nullptr, nullptr, N, L, 0, nullptr);
+    e = launch_fold_big(nullptr, nullptr, nullptr, nullptr, M, L, 0, nullptr);
   }
   return e;
 }
@@ -836,7 +804,7 @@ cudaError_t qr_blocked_prepare(int M, int N, int L) {
 bool reorth_fits(int M, int L) { return M >= L && L <= QF_MAXL_BIG; }
 
 cudaError_t launch_reorth(const float2* Qf, float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int M, int L,
-                          int batch, int* status, cudaStream_t st) {
+                          int batch, int* status, cudaStream_t st, bool fold) {
   const int nt = (L + 31) / 32;
   if (L > QF_MAXL) {
     {
@@ -845,8 +813,9 @@ cudaError_t launch_reorth(const float2* Qf, float2* Dbuf, const Dims* dims, cons
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
+    if (!fold) return cudaSuccess;
     ProfScope ps("k_fold[q]", st);
-    return launch_fold_big<true>(Qf, Dbuf, dims, ptrs, M, L, batch, st);
+    return launch_fold_big(Qf, Dbuf, dims, ptrs, M, L, batch, st);
   }
   const size_t sm_l = sizeof(float2) * (size_t)L * L;
   cudaError_t e0 = ensure_smem(k_lowdin, sm_l, &g_attr_ld);
@@ -857,16 +826,51 @@ cudaError_t launch_reorth(const float2* Qf, float2* Dbuf, const Dims* dims, cons
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
+  if (!fold) return cudaSuccess;
   ProfScope ps("k_fold[q]", st);
-  return launch_fold<true>(Qf, Dbuf, dims, ptrs, M, L, batch, st);
+  return launch_fold(Qf, Dbuf, dims, ptrs, M, L, batch, st);
 }
 
-// B^H <- B^H (I + D) in place on ptrs[z].Yt (D.n x D.l column-major).
-cudaError_t launch_fold_bh(const float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int n, int l, int batch,
-                           cudaStream_t st) {
-  ProfScope ps("k_fold[bh]", st);
-  if (l > QF_MAXL) return launch_fold_big<false>(nullptr, Dbuf, dims, ptrs, n, l, batch, st);
-  return launch_fold<false>(nullptr, Dbuf, dims, ptrs, n, l, batch, st);
+// X <- X + D X for the small FP64 matrices after the projection (the l x l Rb^H
+// or the l x k J_k, column-major with l rows; |D| ~ 1e-6, its product in FP32
+// costs ~1e-13).  A warp per column, the column in shared memory as FP32; D
+// (Hermitian, column-major) is read through L1, lanes along its rows.
+enum { FS_COLS = 8 };
+
+__global__ void __launch_bounds__(32 * FS_COLS) k_fold_small(const float2* __restrict__ Dbase,
+                                                             const Dims* __restrict__ dims,
+                                                             const ProbPtr* __restrict__ ptrs, int Lc, int jk) {
+  __shared__ float2 xs[FS_COLS][QF_MAXL_BIG];
+  const int z = blockIdx.y;
+  const Dims Dm = dims[z];
+  if (!Dm.active) return;
+  const int L = Dm.l, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.x * FS_COLS + warp;
+  if (c >= (jk ? Dm.k : L)) return;  // warps work alone
+  cplx* x = (jk ? ptrs[z].Jk : ptrs[z].R) + (size_t)c * L;
+  const float2* D = Dbase + (size_t)z * Lc * Lc;
+  for (int r = lane; r < L; r += 32) {
+    const cplx v = x[r];
+    xs[warp][r] = make_float2((float)v.x, (float)v.y);
+  }
+  __syncwarp();
+  for (int r = lane; r < L; r += 32) {
+    float sx = 0.f, sy = 0.f;
+    for (int k = 0; k < L; ++k) {
+      const float2 d = __ldg(&D[(size_t)k * L + r]), v = xs[warp][k];
+      sx = fmaf(d.x, v.x, fmaf(-d.y, v.y, sx));
+      sy = fmaf(d.x, v.y, fmaf(d.y, v.x, sy));
+    }
+    const cplx v = x[r];
+    x[r] = cmk(v.x + (double)sx, v.y + (double)sy);
+  }
+}
+
+cudaError_t launch_fold_small(const float2* Dbuf, const Dims* dims, const ProbPtr* ptrs, int l, int k, int batch,
+                              int jk, cudaStream_t st) {
+  ProfScope ps("k_fold[small]", st);
+  k_fold_small<<<dim3(((jk ? k : l) + FS_COLS - 1) / FS_COLS, batch), 32 * FS_COLS, 0, st>>>(Dbuf, dims, ptrs, l, jk);
+  return cudaGetLastError();
 }
 
 }  // namespace tg

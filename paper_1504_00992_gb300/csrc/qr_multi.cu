@@ -161,9 +161,10 @@ template <int QS>
 struct QmSrc64 {
   const Dims* dims;
   const ProbPtr* ptrs;
+  int which;  // QRS_*: the problems to factor
   __device__ __forceinline__ bool get(int p, QmView<double2>& v) const {
     const Dims D = dims[p];
-    if (!D.active) return false;
+    if (!D.active || !qr_takes(D, which)) return false;
     const ProbPtr P = ptrs[p];
     v.M = (QS == QR_Y) ? D.m : D.n;
     v.L = D.l;
@@ -536,9 +537,9 @@ __global__ void qm_qinit(Src src) {
 // X = Rb^H into R (as k_qr): element (r, c) is conj(Rb[c][r]); Rb above the
 // diagonal of the factored B^H, alpha on it.  After the Q formation (R held
 // the partial products until then).
-__global__ void qm_rextract(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs) {
+__global__ void qm_rextract(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs, int which) {
   const Dims D = dims[blockIdx.y];
-  if (!D.active) return;
+  if (!D.active || !qr_takes(D, which)) return;
   const ProbPtr P = ptrs[blockIdx.y];
   const int M = D.n, L = D.l;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < L * L; e += gridDim.x * blockDim.x) {
@@ -585,20 +586,30 @@ bool qr_multi_chosen(int stage, const Caps& cap, int batch, int force) {
   return force == 2 ? qr_multi_fits(M, cap.l, 1) : (force == 0 && qr_multi_fits(M, cap.l, batch));
 }
 
+cudaError_t launch_qr_rest(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
+                           cudaStream_t st, int which) {
+  // the one-CTA kernel runs at ~8 GFLOP/s: from ~0.3 s per matrix on the ~100
+  // launches of the many-CTA form are the smaller cost, also when none needs it
+  const int M = (stage == QR_Y) ? cap.m : cap.n;
+  const bool large = (double)M * cap.l * cap.l >= 1e8 && qr_multi_fits(M, cap.l, 1);
+  return large ? launch_qr_sized(stage, dims, ptrs, batch, cap, st, 2, which)
+               : launch_qr(stage, dims, ptrs, batch, st, which);
+}
+
 cudaError_t launch_qr_sized(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
-                            cudaStream_t st, int force) {
+                            cudaStream_t st, int force, int which) {
   const int M = (stage == QR_Y) ? cap.m : cap.n;
   const bool multi = force == 2 ? qr_multi_fits(M, cap.l, 1) : (force == 0 && qr_multi_fits(M, cap.l, batch));
-  if (!multi) return launch_qr(stage, dims, ptrs, batch, st);
+  if (!multi) return launch_qr(stage, dims, ptrs, batch, st, which);
   ProfScope ps("k_qr[multi]", st);
   cudaError_t e;
   switch (stage) {
-    case QR_Y: e = qm_run<double2, QmSrc64<QR_Y>, false>(QmSrc64<QR_Y>{dims, ptrs}, batch, M, cap.l, st); break;
-    case QR_YT: e = qm_run<double2, QmSrc64<QR_YT>, false>(QmSrc64<QR_YT>{dims, ptrs}, batch, M, cap.l, st); break;
+    case QR_Y: e = qm_run<double2, QmSrc64<QR_Y>, false>(QmSrc64<QR_Y>{dims, ptrs, which}, batch, M, cap.l, st); break;
+    case QR_YT: e = qm_run<double2, QmSrc64<QR_YT>, false>(QmSrc64<QR_YT>{dims, ptrs, which}, batch, M, cap.l, st); break;
     case QR_BH:
-      e = qm_run<double2, QmSrc64<QR_BH>, false>(QmSrc64<QR_BH>{dims, ptrs}, batch, M, cap.l, st);
+      e = qm_run<double2, QmSrc64<QR_BH>, false>(QmSrc64<QR_BH>{dims, ptrs, which}, batch, M, cap.l, st);
       if (e == cudaSuccess) {
-        qm_rextract<<<dim3((cap.l * cap.l + 255) / 256, batch), 256, 0, st>>>(dims, ptrs);
+        qm_rextract<<<dim3((cap.l * cap.l + 255) / 256, batch), 256, 0, st>>>(dims, ptrs, which);
         e = cudaGetLastError();
       }
       break;

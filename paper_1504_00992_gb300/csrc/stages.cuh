@@ -69,6 +69,20 @@ __device__ __forceinline__ GemmOp gemm_of(const Dims& D, const ProbPtr& P) {
     g.A = L; g.ars = D.n; g.acs = 1;             // op(A)(i, k) = conj(L[k][i])
     g.B = Rt; g.brs = 1; g.bcs = D.n;
     g.C = P.R; g.crs = 1; g.ccs = D.l;
+  } else if (STAGE == G_CYG || STAGE == G_CQG || STAGE == G_CTG || STAGE == G_CRG) {  // X^H X of a basis
+    const bool y = (STAGE == G_CYG || STAGE == G_CQG);
+    const cplx* X = (STAGE == G_CYG) ? P.Y : (STAGE == G_CQG) ? P.Q : (STAGE == G_CTG) ? P.Yt : P.Qt;
+    g.M = D.l; g.N = D.l; g.K = y ? D.m : D.n;
+    g.A = X; g.ars = g.K; g.acs = 1;
+    g.B = X; g.brs = 1; g.bcs = g.K;
+    g.C = P.R; g.crs = 1; g.ccs = D.l;
+  } else if (STAGE == G_CYQ || STAGE == G_CQQ || STAGE == G_CTQ || STAGE == G_CRQ) {  // (X S) J
+    const bool y = (STAGE == G_CYQ || STAGE == G_CQQ);
+    const cplx* X = (STAGE == G_CYQ) ? P.Y : (STAGE == G_CQQ) ? P.Q : (STAGE == G_CTQ) ? P.Yt : P.Qt;
+    g.M = y ? D.m : D.n; g.N = D.l; g.K = D.l;
+    g.A = X; g.ars = 1; g.acs = g.M;
+    g.B = P.J; g.brs = 1; g.bcs = D.l;
+    g.C = y ? P.Q : P.Qt; g.crs = 1; g.ccs = g.M;
   } else {  // G_Q1 = Yt J, G_QB = omega J: n x l times the l x l inverse factor
     g.M = D.n; g.N = D.l; g.K = D.l;
     g.A = (STAGE == G_Q1) ? P.Yt : P.omega; g.ars = 1; g.acs = D.n;
@@ -81,7 +95,10 @@ __device__ __forceinline__ GemmOp gemm_of(const Dims& D, const ProbPtr& P) {
 template <int STAGE>
 struct StageFlags {
   static constexpr bool conjA =
-      (STAGE == G_YT || STAGE == G_BH || STAGE == G_PQ || STAGE == G_G1 || STAGE == G_G2 || STAGE == G_X);
+      (STAGE == G_YT || STAGE == G_BH || STAGE == G_PQ || STAGE == G_G1 || STAGE == G_G2 || STAGE == G_X ||
+       STAGE == G_CYG || STAGE == G_CQG || STAGE == G_CTG || STAGE == G_CRG);
+  // the left operand's column k is scaled by sigma[k] (a power of two)
+  static constexpr bool scaleA = (STAGE == G_CYQ || STAGE == G_CQQ || STAGE == G_CTQ || STAGE == G_CRQ);
   static constexpr bool conjC = (STAGE == G_V);
 };
 
@@ -385,7 +402,7 @@ __device__ __forceinline__ void jacobi_finish(const Dims& D, const ProbPtr& P, d
 // the rebuild after truncation (tebd_kernels.cu documents each).
 // ---------------------------------------------------------------------------
 // Sizes of one bond from its current bond dimensions (see k_plan).
-__device__ __forceinline__ Dims plan_dev(const ProbPtr& P, int p) {
+__device__ __forceinline__ Dims plan_dev(const ProbPtr& P, int p, int digits) {
   Dims D;
   D.dl = P.dl_s;
   D.dr = P.dr_s;
@@ -403,6 +420,9 @@ __device__ __forceinline__ Dims plan_dev(const ProbPtr& P, int p) {
   D.r = 0;
   D.chk = 0;
   D.qflag = 0;
+  D.dig = (digits && dp_rule(D.m, D.n, D.l)) ? 1 : 0;
+  D.cq = 0;
+  D.cf = 0;
   return D;
 }
 

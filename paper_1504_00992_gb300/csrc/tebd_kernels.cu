@@ -16,15 +16,15 @@ namespace tg {
 //   l = min(k + p, m, n)   (sketch width; exact when it reaches min(m, n)).
 // Bonds of one parity share no site, so their updates are independent.
 // ---------------------------------------------------------------------------
-__global__ void k_plan(const ProbPtr* __restrict__ ptrs, Dims* dims, int batch, int p) {
+__global__ void k_plan(const ProbPtr* __restrict__ ptrs, Dims* dims, int batch, int p, int digits) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= batch) return;
-  dims[t] = plan_dev(ptrs[t], p);
+  dims[t] = plan_dev(ptrs[t], p, digits);
 }
 
-cudaError_t launch_plan(const ProbPtr* ptrs, Dims* dims, int batch, int p, cudaStream_t st) {
+cudaError_t launch_plan(const ProbPtr* ptrs, Dims* dims, int batch, int p, cudaStream_t st, int digits) {
   ProfScope ps("k_plan", st);
-  k_plan<<<(batch + 127) / 128, 128, 0, st>>>(ptrs, dims, batch, p);
+  k_plan<<<(batch + 127) / 128, 128, 0, st>>>(ptrs, dims, batch, p, digits);
   return cudaGetLastError();
 }
 

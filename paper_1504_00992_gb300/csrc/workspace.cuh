@@ -38,10 +38,11 @@ __host__ __device__ inline void fill_ptrs(ProbPtr& P, char* base, const WsLayout
 // Descriptors of a standalone batch (api.cu): instance p reads theta at
 // theta + p * theta_stride and writes U / V^H into the caller's arrays (or its
 // own block when NULL); with dims_m > 0 the Dims of every instance are also
-// written (m, n, k, l, active) and *status is cleared.
+// written (m, n, k, l, active, dig), and *status is cleared unless status is null.
 __global__ void k_rrsvd_bind(ProbPtr* ptrs, int batch, char* ws, size_t per, WsLayout lay, const cplx* theta,
                              size_t theta_stride, cplx* U, size_t U_stride, cplx* Vh, size_t V_stride, Dims* dims,
-                             int dims_m, int dims_n, int dims_k, int dims_l, int* status);
+                             int dims_m, int dims_n, int dims_k, int dims_l, int dig,
+                             int* status);
 
 // Host-side fault injection (test hook, tebd_fault_inject): true once for
 // each armed fault of `kind` (a one-shot flag; thread-safe).
