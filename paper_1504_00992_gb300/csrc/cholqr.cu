@@ -318,9 +318,9 @@ static cudaError_t chol_inv(Dims* dims, const ProbPtr* ptrs, int batch, int lcap
   } while (0)
 
 cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
-                          const OzScratch* oz, int* err) {
+                          const OzScratch* oz, int* err, bool phases) {
   if (oz) {
-    CQ_TRY(run_cholqr(1, 2, CQ_LOWDIN, CQ_MIN_PIVOT, dims, ptrs, batch, cap, *oz, batch, 0, err, st));
+    CQ_TRY(run_cholqr(1, 2, phases ? CQ_PHASES : CQ_LOWDIN, CQ_MIN_PIVOT, dims, ptrs, batch, cap, *oz, batch, 0, err, st));
     CQ_TRY(launch_oz_stage(G_X, dims, ptrs, batch, cap, *oz, err, st, DPC_OK));  // X = B Qb = Rb^H
     return launch_qr_rest(QR_BH, dims, ptrs, batch, cap, st, QRS_CF);
   }

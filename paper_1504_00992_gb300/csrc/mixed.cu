@@ -687,12 +687,16 @@ cudaError_t mixed_prepare(const Caps& cap) {
 
 // The QR of B^H where no choice is set.  On the tensor cores the Cholesky QR
 // (with Householder per ill-conditioned instance) also takes the few tall
-// matrices the many-CTA FP64 Householder ran before: 8 x 2000 x 120 in 1.3 ms
-// against 21 ms, 16 x 7700 x 262 in 5 ms against 28 ms.
+// matrices of the many-CTA FP64 Householder: 8 x 2000 x 120 in 1.3 ms against
+// 21 ms, 16 x 7700 x 262 in 5 ms against 28 ms.  Those keep that QR's column
+// phases, and with them the singular vectors' and the next truncations'
+// samples (without them a spin-boson chain's Schmidt values moved by 2e-5 to
+// 7e-5 over three waves, with them by 1e-6).
 int mixed_qrbh(const MixedKnobs& kn, const Caps& cap, int batch) {
   if (kn.qrbh) return kn.qrbh;
   const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));
-  return tc || !qr_multi_chosen(QR_BH, cap, batch, 0) ? 3 : 2;
+  if (!qr_multi_chosen(QR_BH, cap, batch, 0)) return 3;
+  return tc ? 4 : 2;
 }
 
 // The Jacobi SVD where no choice is set: double-float on one CTA, or for a few
@@ -788,10 +792,11 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   // QR of it (mixed_qrbh); then Rb^H of B^H = A^H Q_f (I + D) is (I + D) times what it gives (folding
   // I + D into the n x l and m x l matrices instead took 6.3 ms of the 92 ms
   // step of 152 x 2000 x 2000, folding it into the small ones 0.2 ms)
-  if (mixed_qrbh(kn, cap, batch) == 3)
-    MX_TRY(run_cholqr_bh(const_cast<Dims*>(dims), ptrs, batch, cap, st, tc ? &oz : nullptr, err));
+  const int qrbh = mixed_qrbh(kn, cap, batch);
+  if (qrbh >= 3)
+    MX_TRY(run_cholqr_bh(const_cast<Dims*>(dims), ptrs, batch, cap, st, tc ? &oz : nullptr, err, qrbh == 4));
   else
-    MX_TRY(launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st, mixed_qrbh(kn, cap, batch)));
+    MX_TRY(launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st, qrbh));
   MX_TRY(launch_fold_small(mp.Df, dims, ptrs, l, k, batch, 0, st));
   // Jacobi SVD: double-float one-CTA kernel unless the cluster form is chosen
   const int jac = mixed_jac(kn, cap, batch);

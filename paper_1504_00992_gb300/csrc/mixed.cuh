@@ -177,9 +177,9 @@ cudaError_t launch_oz_range(int stage, const Dims* dims, const ProbPtr* ptrs, in
 // Cholesky QR (two passes) of B^H for well-conditioned instances, Householder
 // for the others (cholqr.cu); writes dims[p].qflag.  oz: the products on the
 // tensor cores (raising *err on a pipeline stall), or null for double-float
-// GEMMs.
+// GEMMs.  phases: with the column phases of the Householder QR (with oz only).
 cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
-                          const OzScratch* oz, int* err);
+                          const OzScratch* oz, int* err, bool phases);
 cudaError_t cholqr_prepare();
 cudaError_t launch_oz_digits_theta(const Dims* dims, const ProbPtr* ptrs, uint16_t* Bd, int* Bs, int m, int n,
                                    int batch, cudaStream_t st);
@@ -213,7 +213,8 @@ struct MixedKnobs {
 };
 
 // The choices a launch on `batch` problems of capacities cap makes (a set knob,
-// or the size rule): the QR of B^H (1, 2 or 3) and the Jacobi SVD.
+// or the size rule): the QR of B^H (1, 2 or 3; 4 is 3 with Householder's column
+// phases) and the Jacobi SVD.
 int mixed_qrbh(const MixedKnobs& kn, const Caps& cap, int batch);
 int mixed_jac(const MixedKnobs& kn, const Caps& cap, int batch);
 
