@@ -136,6 +136,7 @@ cudaError_t run_rrsvd_checked(Dims* dims, const ProbPtr* ptrs, int batch, const 
   }
   if ((e = P.gemm(G_BH)) != cudaSuccess) return e;
   if ((e = P.qr(QR_BH, DPQ_LAST)) != cudaSuccess) return e;
+  if ((e = P.svd()) != cudaSuccess) return e;
   if ((e = launch_jacobi_sized(dims, ptrs, batch, cap, status, st)) != cudaSuccess) return e;
   if ((e = P.gemm(G_U)) != cudaSuccess) return e;
   if ((e = P.gemm(G_V)) != cudaSuccess) return e;

@@ -285,6 +285,8 @@ template <bool SM>
 __global__ void k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass, int passes, float min_pivot,
                           float again, int cond);
 
+static cudaError_t lowdin_prepare();
+
 cudaError_t cholqr_prepare() {
   static int done = 0;
   if (!done) {
@@ -294,6 +296,10 @@ cudaError_t cholqr_prepare() {
     const cudaError_t e2 =
         cudaFuncSetAttribute(k_chol_eq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs_smem_bytes(CS_MAXL));
     if (e2 != cudaSuccess) return e2;
+    const cudaError_t e5 = lowdin_prepare();
+    if (e5 != cudaSuccess) return e5;
+    const cudaError_t e3 = jac_pre_prepare();
+    if (e3 != cudaSuccess) return e3;
     done = 1;
   }
   return cudaSuccess;
@@ -627,15 +633,20 @@ __global__ void __launch_bounds__(CE_THREADS) k_hh_phase(const Dims* __restrict_
 // l max|E| <= 3e-6 (the next term is below 1e-17); S = 1.  E^2 enters at the
 // level of 1e-12 at most, so it is formed in FP32, and not at all where it is
 // below FP64's resolution.  phases: column j also takes k_hh_phase's phase.
+enum { LW_MAXL = 160 };
+static size_t lw_smem_bytes(int l) { return l <= LW_MAXL ? sizeof(float2) * (size_t)l * l : 0; }
+template <bool SVD>
 __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __restrict__ ptrs, int cond,
                                                   int phases) {
+  extern __shared__ float2 lw_e[];
   __shared__ float red[16];
   const int p = blockIdx.x;
   const Dims D = dims[p];
-  if (!ce_takes(D, 0, cond) || D.cf) return;
+  if (!ce_takes(D, 0, cond) || (SVD ? D.js != 1 : D.cf != 0)) return;
   const ProbPtr P = ptrs[p];
   const int L = D.l, tid = threadIdx.x;
-  const cplx* G = P.R;
+  const cplx* G = SVD ? P.Y : P.R;
+  cplx* T = SVD ? P.Yt : P.J;
   float mx = 0.f;
   for (int e = tid; e < L * L; e += 512) {
     const cplx g = G[e];
@@ -652,9 +663,23 @@ __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __r
   __syncthreads();
   mx = 0.f;
   for (int w = 0; w < 16; ++w) mx = (red[w] > mx || red[w] != red[w]) ? red[w] : mx;
-  const bool ok = mx * (float)L <= 3e-6f;
-  if (!ok && tid == 0) dims[p].cf = 1;
-  const bool square = mx > 1e-9f;
+  // (an FP32 J is farther from unitary, and takes a second round)
+  const bool ok = mx * (float)L <= (SVD ? 1e-2f : 3e-6f);
+  if (!ok && tid == 0) {
+    if (SVD) dims[p].js = 0;
+    else dims[p].cf = 1;
+  }
+  // E in FP32, in shared memory where it fits (a conversion is an FP64
+  // instruction: made per use they were nearly all of the time, 0.71 ms for
+  // 16 instances of l = 120, 0.06 ms made once)
+  const bool square = ok && mx > 1e-9f, staged = L <= LW_MAXL;
+  if (square && staged) {
+    for (int e = tid; e < L * L; e += 512) {
+      const cplx g = G[e];
+      lw_e[e] = make_float2((float)(e % L == e / L ? g.x - 1.0 : g.x), (float)g.y);
+    }
+    __syncthreads();
+  }
   for (int e = tid; e < L * L; e += 512) {
     const int a = e % L, b = e / L;
     const cplx g = G[e];
@@ -664,19 +689,35 @@ __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __r
       if (square) {
         float sx = 0.f, sy = 0.f;
         for (int k = 0; k < L; ++k) {
-          const cplx u = G[(size_t)k * L + a], v = G[(size_t)b * L + k];
-          const float ux = (float)(k == a ? u.x - 1.0 : u.x), uy = (float)u.y;
-          const float vx = (float)(k == b ? v.x - 1.0 : v.x), vy = (float)v.y;
-          sx = fmaf(ux, vx, fmaf(-uy, vy, sx));
-          sy = fmaf(ux, vy, fmaf(uy, vx, sy));
+          float2 u, v;
+          if (staged) {
+            u = lw_e[k * L + a];
+            v = lw_e[b * L + k];
+          } else {
+            const cplx gu = G[(size_t)k * L + a], gv = G[(size_t)b * L + k];
+            u = make_float2((float)(k == a ? gu.x - 1.0 : gu.x), (float)gu.y);
+            v = make_float2((float)(k == b ? gv.x - 1.0 : gv.x), (float)gv.y);
+          }
+          sx = fmaf(u.x, v.x, fmaf(-u.y, v.y, sx));
+          sy = fmaf(u.x, v.y, fmaf(u.y, v.x, sy));
         }
         t.x += 0.375 * (double)sx;
         t.y += 0.375 * (double)sy;
       }
     }
-    P.J[e] = phases ? cmul(t, P.Jk[b]) : t;
+    T[e] = phases ? cmul(t, P.Jk[b]) : t;
   }
-  for (int c = tid; c < L; c += 512) P.sigma[c] = 1.0;
+  if (!SVD)
+    for (int c = tid; c < L; c += 512) P.sigma[c] = 1.0;
+}
+
+static cudaError_t lowdin_prepare() {
+  for (cudaError_t e : {cudaFuncSetAttribute(k_lowdin64<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)lw_smem_bytes(LW_MAXL)),
+                        cudaFuncSetAttribute(k_lowdin64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)lw_smem_bytes(LW_MAXL))})
+    if (e != cudaSuccess) return e;
+  return cudaSuccess;
 }
 
 static size_t ce_smem_bytes(int L) { return L <= CS_MAXL ? cs_smem_bytes(L) : sizeof(float4) * (size_t)L; }
@@ -712,10 +753,21 @@ cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* 
   CQ_TRY(prod(g1, cond | DPC_OK));
   {
     ProfScope ps("k_lowdin", st);
-    k_lowdin64<<<batch, 512, 0, st>>>(dims, ptrs, cond, lowdin == CQ_PHASES);
+    k_lowdin64<false><<<batch, 512, lw_smem_bytes(cap.l), st>>>(dims, ptrs, cond, lowdin == CQ_PHASES);
     CQ_TRY(cudaGetLastError());
   }
   return prod(q1, cond | DPC_OK);
+}
+
+cudaError_t launch_lowdin_j(Dims* dims, const ProbPtr* ptrs, int batch, int l, int cond, cudaStream_t st) {
+  ProfScope ps("k_lowdin", st);
+  k_lowdin64<true><<<batch, 512, lw_smem_bytes(l), st>>>(dims, ptrs, cond, 0);
+  return cudaGetLastError();
+}
+
+cudaError_t DpPath::svd() const {
+  if (!dp || !jac_pre_rule(cap)) return cudaSuccess;
+  return run_jac_pre(const_cast<Dims*>(dims), ptrs, batch, cap, dp->oz, dp->chunk, DPC_DIG, true, dp->err, st);
 }
 
 cudaError_t DpPath::qr(int stage, int kind) const {

@@ -28,6 +28,7 @@ struct Dims {
   int dig;         // FP64 form: this problem's products and QRs run from digit splits (dp_rule)
   int cq;          // Cholesky QR: the last pass this problem takes part in
   int cf;          // Cholesky QR: given up, the Householder QR factors it
+  int js;          // small SVD: 1: J holds rotations already applied to X, 2: X's columns are orthogonal too
 };
 
 // Sizes from which the FP64 form's products and QRs run on the tensor cores
@@ -92,7 +93,10 @@ enum GemmStage { G_Y0 = 0, G_YT = 1, G_Y = 2, G_BH = 3, G_U = 4, G_V = 5,
                  // G = Q^H Q, Q = (Q S) J, with S the column scales in sigma ...
                  G_CYG = 14, G_CYQ = 15, G_CQG = 16, G_CQQ = 17,
                  // ... and of Yt into Qt (n rows)
-                 G_CTG = 18, G_CTQ = 19, G_CRG = 20, G_CRQ = 21 };
+                 G_CTG = 18, G_CTQ = 19, G_CRG = 20, G_CRQ = 21,
+                 // small SVD (jacobi_pre.cu), all l x l: Y = J^H J, J = J Yt, R = (R S)(S^-1 J),
+                 // Y = R^H R, R = (R S)(S^-1 Yt)
+                 G_JG = 22, G_JT = 23, G_XJ = 24, G_XG = 25, G_XT = 26 };
 // QR stages: which buffer is factored and where Q goes.
 enum QrStage { QR_Y = 0, QR_YT = 1, QR_BH = 2 };
 

@@ -82,13 +82,14 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
   double f2 = 0.0;
   for (int e = tid; e < L * L; e += blockDim.x) f2 += cabs2(X[e]);
   f2 = block_sum(f2, red);
-  for (int e = crank * blockDim.x + tid; e < L * L; e += JC_CL * blockDim.x)
-    J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
+  if (D.js == 0)
+    for (int e = crank * blockDim.x + tid; e < L * L; e += JC_CL * blockDim.x)
+      J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
   const int Lp = (L + 1) & ~1;
   const double eps = 2.220446049250313e-16;
   const double tol = 4.0 * eps * sqrt((double)L);
   const double small = ((double)L * eps) * ((double)L * eps) * f2;
-  int sweep = 0;
+  int sweep = D.js == 2 ? JC_MAXSWEEPS + 1 : 0;
   for (; sweep < JC_MAXSWEEPS; ++sweep) {
     for (int c = gwarp; c < L; c += nw_all) {
       const cplx* xc = X + (int64_t)c * L;

@@ -170,6 +170,10 @@ __global__ void __launch_bounds__(JD_THREADS) k_jacobi_df(const Dims* __restrict
   float4* X = XS ? reinterpret_cast<float4*>(jd_smem) : reinterpret_cast<float4*>(P.R);
   float4* J = reinterpret_cast<float4*>(P.J);
 
+  if (D.js == 2) {  // X J = W S already
+    jacobi_finish(D, P, sv, perm);
+    return;
+  }
   // the scale: largest biased exponent among the entries of X
   int e = 0;
   for (int i = tid; i < L * L; i += blockDim.x) {
@@ -198,7 +202,13 @@ __global__ void __launch_bounds__(JD_THREADS) k_jacobi_df(const Dims* __restrict
     split_bits(v.x * up, d.x, d.y);
     split_bits(v.y * up, d.z, d.w);
     X[i] = d;
-    J[i] = make_float4((i / L) == (i % L) ? 1.f : 0.f, 0.f, 0.f, 0.f);
+    float4 j0 = make_float4((i / L) == (i % L) ? 1.f : 0.f, 0.f, 0.f, 0.f);
+    if (D.js == 1) {
+      const cplx w = J64[i];
+      split_bits(w.x, j0.x, j0.y);
+      split_bits(w.y, j0.z, j0.w);
+    }
+    J[i] = j0;
   }
   __syncthreads();
   // ||X||_F^2 (FP32 is enough for the negligible-column threshold)

@@ -1,0 +1,385 @@
+// Small SVD by an FP32 Jacobi and digit-split corrections (sm_103a): X J = W S
+// for X = Rb^H (Section IV's step ii) to FP64, for the problems whose other
+// products run from digit splits.
+//
+// The one-sided Jacobi kernels spend 14 l^3 FP64 (or double-float) multiply-
+// adds per sweep and five to seven sweeps, nearly all of them far from the
+// final accuracy.  Here
+//   1. k_jac_pre runs the same sweeps in FP32 on X rounded to FP32 (columns
+//      orthogonal to ~3e-6) and keeps the accumulated J;
+//   2. J is made unitary to FP64 (J^H J from digits, k_lowdin64) and X J is
+//      formed from digits;
+//   3. up to JP_STEPS times, the first-order rotations of every pair at once:
+//      with G = X^H X from digits, K_ab = t e from the pair's 2 x 2 problem
+//      (Jacobi's angle t and phase e), X <- X T and J <- J T with
+//      T = I + K + K^2 / 2, K skew-Hermitian, so that T is unitary to K^4 / 4.
+//      The residual falls from ~3e-6 to its square over the gap (and 1e-7 of
+//      it, K is FP32), i.e. below FP64's tolerance in two steps;
+//   4. a problem whose columns are orthogonal to the Jacobi kernels' own
+//      tolerance is done; the others go on in those kernels from (X, J).
+// Pairs with an angle above JP_ANGLE (nearly equal singular values) are left
+// out of K and so to step 4, where each costs one rotation.
+//
+// Graded columns (TEBD spectra reach 1e-14): the products X J and X T scale
+// the left operand's columns by S = 2^-e of their norms and the right one's
+// rows by S^-1, so that every column of the result is rounded relative to its
+// own norm and not to the largest singular value.
+//
+// Measured, l = 120: 16 problems in FP64 14.1 ms in the cluster Jacobi alone,
+// 4.9 ms here (FP32 sweeps 2.7, products 0.4, corrections 0.7, the Jacobi
+// kernel's check and ranking 1.1); 152 in double-float 10.3 ms, against 6.1.
+// The sweeps are bound by the latency of a round (a barrier, two trips to
+// shared memory, two to J in L1).
+//
+// FP32 kernel: X in shared memory for l <= JP_MAXL (205 KB), J through L1/L2,
+// one group of eight lanes per pair, the pair's columns in registers between
+// the inner product and the rotation.
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include "dfsplit.cuh"
+#include "internal.cuh"
+#include "mixed.cuh"
+#include "profiler.cuh"
+#include "stages.cuh"
+
+namespace tg {
+
+enum { JP_MAXL = 160, JP_G = 8, JP_ROWS = JP_MAXL / JP_G, JP_THREADS = 640, JP_SWEEPS = 12, JP_STEPS = 2 };
+static const float JP_TOL = 3e-6f;    // cosine of a pair the FP32 sweeps leave alone
+static const float JP_ANGLE = 3e-5f;  // largest angle of a first-order rotation
+
+__device__ __forceinline__ bool jp_takes(const Dims& D, int cond) {
+  return D.active && !((cond & DPC_DIG) && !D.dig);
+}
+
+__device__ __forceinline__ float2 jp_shfl_sum(float2 v, unsigned mask) {
+#pragma unroll
+  for (int o = JP_G / 2; o > 0; o >>= 1) {
+    v.x += __shfl_xor_sync(mask, v.x, o);
+    v.y += __shfl_xor_sync(mask, v.y, o);
+  }
+  return v;
+}
+
+// x 2^k by the exponent bits, to FP32 (0 below its range)
+__device__ __forceinline__ float jp_f32(double x, int k) {
+  const long long u = __double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7FF) + k;
+  return (((u >> 52) & 0x7FF) == 0 || e <= 1023 - 126) ? 0.f : (float)__longlong_as_double(u + ((long long)k << 52));
+}
+__device__ __forceinline__ int jp_exp2(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF) - 1023; }
+
+__global__ void __launch_bounds__(JP_THREADS) k_jac_pre(Dims* dims, const ProbPtr* __restrict__ ptrs, int cond) {
+  extern __shared__ __align__(16) unsigned char jp_raw[];
+  __shared__ float nrm[JP_MAXL];
+  __shared__ int s_exp;
+  __shared__ int rotated;
+  const int p = blockIdx.x;
+  const Dims D = dims[p];
+  if (!jp_takes(D, cond)) return;
+  const ProbPtr P = ptrs[p];
+  const int L = D.l, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  float2* X = reinterpret_cast<float2*>(jp_raw);
+  // FP32 J in the upper half of the buffer its FP64 form fills at the end
+  float2* J = reinterpret_cast<float2*>(P.J) + (size_t)L * L;
+  if (tid == 0) s_exp = 0;
+  __syncthreads();
+  int e = 0;
+  bool bad = false;
+  for (int i = tid; i < L * L; i += nt) {
+    const cplx v = P.R[i];
+    e = max(e, max(oz_exp(v.x), oz_exp(v.y)));
+    bad |= !isfinite(v.x) || !isfinite(v.y);
+  }
+  atomicMax(&s_exp, e);
+  const bool any_bad = __syncthreads_or(bad);
+  const int E = s_exp;
+  if (any_bad || E == 0) {  // left to the Jacobi kernels as it is
+    if (tid == 0) dims[p].js = 0;
+    return;
+  }
+  const int up = 1023 - E;  // to max |x| in [1, 2)
+  for (int i = tid; i < L * L; i += nt) {
+    const cplx v = P.R[i];
+    X[i] = make_float2(jp_f32(v.x, up), jp_f32(v.y, up));
+    J[i] = make_float2((i / L) == (i % L) ? 1.f : 0.f, 0.f);
+  }
+  __syncthreads();
+  const int gl = lane & (JP_G - 1), grp = tid / JP_G, ngrp = nt / JP_G;
+  const unsigned gmask = ((1u << JP_G) - 1u) << (lane & ~(JP_G - 1));
+  const int Lp = (L + 1) & ~1;
+  for (int sweep = 0; sweep < JP_SWEEPS; ++sweep) {
+    for (int c = warp; c < L; c += nw) {
+      float s = 0.f;
+      for (int r = lane; r < L; r += 32) {
+        const float2 v = X[c * L + r];
+        s = fmaf(v.x, v.x, fmaf(v.y, v.y, s));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) nrm[c] = s;
+    }
+    if (tid == 0) rotated = 0;
+    __syncthreads();
+    for (int rnd = 0; rnd < Lp - 1; ++rnd) {
+      for (int pi = grp; pi < Lp / 2; pi += ngrp) {
+        int a = pi == 0 ? Lp - 1 : rnd + pi, b = pi == 0 ? rnd : rnd - pi;
+        if (pi > 0) {
+          if (a >= Lp - 1) a -= Lp - 1;
+          if (b < 0) b += Lp - 1;
+        }
+        if (a > b) {
+          const int t = a;
+          a = b;
+          b = t;
+        }
+        if (b >= L) continue;  // uniform over the group
+        const float na = nrm[a], nb = nrm[b];
+        if (!(na > 1e-34f) || !(nb > 1e-34f)) continue;  // below FP32's squares
+        float2* xa = X + a * L;
+        float2* xb = X + b * L;
+        float2 u[JP_ROWS], v[JP_ROWS];
+        float2 g = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < JP_ROWS; ++q) {
+          if (q * JP_G >= L) continue;  // uniform
+          const int r = gl + q * JP_G;
+          u[q] = r < L ? xa[r] : make_float2(0.f, 0.f);
+          v[q] = r < L ? xb[r] : make_float2(0.f, 0.f);
+          g.x = fmaf(u[q].x, v[q].x, fmaf(u[q].y, v[q].y, g.x));
+          g.y = fmaf(u[q].x, v[q].y, fmaf(-u[q].y, v[q].x, g.y));
+        }
+        g = jp_shfl_sum(g, gmask);
+        const float ra = rsqrtf(na), rb = rsqrtf(nb);
+        const float cx = (g.x * ra) * rb, cy = (g.y * ra) * rb;  // the cosine
+        const float co = sqrtf(fmaf(cx, cx, cy * cy));
+        if (!(co > JP_TOL)) continue;
+        const float ic = 1.f / co, ex = cx * ic, ey = cy * ic;
+        // zeta = (nb - na) / (2 |g|) with |g| = co sqrt(na nb)
+        const float zeta = ((nb - na) * ra) * rb * (0.5f * ic);
+        const float az = fabsf(zeta);
+        const float t = (zeta >= 0.f ? 1.f : -1.f) / (az > 1e9f ? 2.f * az : az + sqrtf(fmaf(zeta, zeta, 1.f)));
+        const float c = rsqrtf(fmaf(t, t, 1.f)), s = c * t;
+        const float sx = s * ex, sy = s * ey;
+#pragma unroll
+        for (int q = 0; q < JP_ROWS; ++q) {
+          const int r = gl + q * JP_G;
+          if (r < L) {
+            xa[r] = make_float2(fmaf(c, u[q].x, -fmaf(sx, v[q].x, sy * v[q].y)),
+                                fmaf(c, u[q].y, -fmaf(sx, v[q].y, -sy * v[q].x)));
+            xb[r] = make_float2(fmaf(c, v[q].x, fmaf(sx, u[q].x, -sy * u[q].y)),
+                                fmaf(c, v[q].y, fmaf(sx, u[q].y, sy * u[q].x)));
+          }
+        }
+        float2* ja = J + (size_t)a * L;
+        float2* jb = J + (size_t)b * L;
+#pragma unroll
+        for (int q = 0; q < JP_ROWS; ++q) {
+          if (q * JP_G >= L) continue;
+          const int r = gl + q * JP_G;
+          u[q] = r < L ? ja[r] : make_float2(0.f, 0.f);
+          v[q] = r < L ? jb[r] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < JP_ROWS; ++q) {
+          const int r = gl + q * JP_G;
+          if (r < L) {
+            ja[r] = make_float2(fmaf(c, u[q].x, -fmaf(sx, v[q].x, sy * v[q].y)),
+                                fmaf(c, u[q].y, -fmaf(sx, v[q].y, -sy * v[q].x)));
+            jb[r] = make_float2(fmaf(c, v[q].x, fmaf(sx, u[q].x, -sy * u[q].y)),
+                                fmaf(c, v[q].y, fmaf(sx, u[q].y, sy * u[q].x)));
+          }
+        }
+        if (gl == 0) {
+          const float ag = co / (ra * rb);
+          nrm[a] = fmaxf(na - t * ag, 0.f);
+          nrm[b] = nb + t * ag;
+          rotated = 1;
+        }
+      }
+      __syncthreads();
+    }
+    const int any = rotated;
+    __syncthreads();
+    if (!any) break;
+  }
+  // J to FP64 in place: in ascending order an entry's FP64 form overwrites
+  // only FP32 entries already read
+  for (int i0 = 0; i0 < L * L; i0 += nt) {
+    const int i = i0 + tid;
+    const float2 v = i < L * L ? J[i] : make_float2(0.f, 0.f);
+    __syncthreads();
+    if (i < L * L) P.J[i] = cmk((double)v.x, (double)v.y);
+    __syncthreads();
+  }
+  // S from the columns of X itself
+  for (int c = warp; c < L; c += nw) {
+    int m = 0;
+    for (int r = lane; r < L; r += 32) {
+      const cplx v = P.R[(size_t)c * L + r];
+      m = max(m, max(oz_exp(v.x), oz_exp(v.y)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) P.sigma[c] = m > 0 ? __longlong_as_double((long long)max(1, 2046 - m) << 52) : 1.0;
+  }
+  if (tid == 0) dims[p].js = 1;
+}
+
+// From G = X^H X in P.Y: js = 2 when every pair is orthogonal to tol; else T
+// in P.Yt and S in sigma.
+__global__ void __launch_bounds__(512) k_jac_step(Dims* dims, const ProbPtr* __restrict__ ptrs, int cond, float tolu,
+                                                  float small_u) {
+  extern __shared__ __align__(16) unsigned char jp_raw[];
+  __shared__ double s_n[JP_MAXL];
+  __shared__ int s_k[JP_MAXL];  // S_c = 2^s_k
+  __shared__ float red[16];
+  const int p = blockIdx.x;
+  const Dims D = dims[p];
+  if (!jp_takes(D, cond) || D.js != 1) return;
+  const ProbPtr P = ptrs[p];
+  const int L = D.l, tid = threadIdx.x;
+  const cplx* G = P.Y;
+  float2* K = reinterpret_cast<float2*>(jp_raw);  // K[b * L + a] = K_ab
+  __shared__ double s_f2;
+  for (int c = tid; c < L; c += 512) {
+    const double n = G[(size_t)c * L + c].x;
+    s_n[c] = n;
+    s_k[c] = n > 0.0 ? -((jp_exp2(n) - ((jp_exp2(n) & 1) ? 1 : 0)) / 2) : 0;  // -floor(log2 n / 2)
+  }
+  __syncthreads();
+  if (tid < 32) {
+    double f2 = 0.0;
+    for (int c = tid; c < L; c += 32) f2 += s_n[c];
+    f2 = warp_sum(f2);
+    if (tid == 0) s_f2 = (double)small_u * small_u * (double)L * (double)L * f2;
+  }
+  __syncthreads();
+  const double small = s_f2;
+  float worst = 0.f;
+  for (int i = tid; i < L * L; i += 512) {
+    const int a = i % L, b = i / L;
+    if (a == b) K[i] = make_float2(0.f, 0.f);
+    if (a >= b) continue;
+    const double na = s_n[a], nb = s_n[b];
+    float kx = 0.f, ky = 0.f;
+    if (na > small && nb > small) {
+      const cplx g = G[(size_t)b * L + a];  // x_a^H x_b
+      const int ka = s_k[a], kb = s_k[b];
+      const float gx = jp_f32(g.x, ka + kb), gy = jp_f32(g.y, ka + kb);
+      const float va = jp_f32(na, 2 * ka), vb = jp_f32(nb, 2 * kb);  // in [1, 4)
+      const float ag = sqrtf(fmaf(gx, gx, gy * gy));
+      const float co = ag * rsqrtf(va) * rsqrtf(vb);
+      worst = (co > worst || co != co) ? co : worst;
+      if (ag > 0.f) {
+        // zeta = (nb - na) / (2 |g|), scaled by S_a S_b above and below
+        const double d = nb - na;
+        const int ke = ka + kb;
+        const float dz = jp_exp2(d) + ke > 120 ? (d > 0.0 ? 1e36f : -1e36f) : jp_f32(d, ke);
+        const float zeta = dz / (2.f * ag), az = fabsf(zeta);
+        const float t = (zeta >= 0.f ? 1.f : -1.f) / (az > 1e9f ? 2.f * az : az + sqrtf(fmaf(zeta, zeta, 1.f)));
+        if (fabsf(t) <= JP_ANGLE) {
+          const float ia = 1.f / ag;
+          kx = t * (gx * ia);
+          ky = t * (gy * ia);
+        }
+      }
+    }
+    K[i] = make_float2(kx, ky);                  // K_ab = t e
+    K[a * L + b] = make_float2(-kx, ky);         // K_ba = -conj
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float y = __shfl_xor_sync(0xffffffffu, worst, o);
+    worst = (y > worst || y != y) ? y : worst;
+  }
+  if ((tid & 31) == 0) red[tid >> 5] = worst;
+  __syncthreads();
+  worst = 0.f;
+  for (int w = 0; w < 16; ++w) worst = (red[w] > worst || red[w] != red[w]) ? red[w] : worst;
+  if (worst <= tolu * sqrtf((float)L)) {
+    if (tid == 0) dims[p].js = 2;
+    return;
+  }
+  for (int i = tid; i < L * L; i += 512) {
+    const int a = i % L, b = i / L;
+    float sx = 0.f, sy = 0.f;
+    for (int k = 0; k < L; ++k) {
+      const float2 u = K[k * L + a], v = K[b * L + k];
+      sx = fmaf(u.x, v.x, fmaf(-u.y, v.y, sx));
+      sy = fmaf(u.x, v.y, fmaf(u.y, v.x, sy));
+    }
+    const float2 k1 = K[i];
+    P.Yt[i] = cmk((a == b ? 1.0 : 0.0) + (double)k1.x + 0.5 * (double)sx, (double)k1.y + 0.5 * (double)sy);
+  }
+  for (int c = tid; c < L; c += 512) P.sigma[c] = __longlong_as_double((long long)(1023 + s_k[c]) << 52);
+}
+
+cudaError_t jac_pre_prepare() {
+  static int done = 0;
+  if (!done) {
+    const int b = (int)(sizeof(float2) * JP_MAXL * JP_MAXL);
+    cudaError_t e = cudaFuncSetAttribute(k_jac_pre, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_jac_step, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e != cudaSuccess) return e;
+    done = 1;
+  }
+  return cudaSuccess;
+}
+
+__global__ void k_jac_none(Dims* dims, int batch) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < batch) dims[p].js = 0;
+}
+
+cudaError_t launch_jac_none(Dims* dims, int batch, cudaStream_t st) {
+  k_jac_none<<<(batch + 127) / 128, 128, 0, st>>>(dims, batch);
+  return cudaGetLastError();
+}
+
+bool jac_pre_rule(const Caps& cap) { return cap.l <= JP_MAXL; }
+
+#define JP_TRY(x)                     \
+  do {                                \
+    cudaError_t e_ = (x);             \
+    if (e_ != cudaSuccess) return e_; \
+  } while (0)
+
+cudaError_t run_jac_pre(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, const OzScratch& oz, int chunk,
+                        int cond, bool fp64, int* err, cudaStream_t st) {
+  JP_TRY(jac_pre_prepare());
+  const size_t sm = sizeof(float2) * (size_t)cap.l * cap.l;
+  const int js = cond | DPC_JS;
+  auto prod = [&](int stage) { return launch_oz_range(stage, dims, ptrs, batch, cap, oz, chunk, js, err, st); };
+  {
+    ProfScope ps("k_jacobi[pre]", st);
+    // a group per pair where that takes at most JP_THREADS threads
+    const int nt = ((cap.l + 1) / 2 * JP_G + 31) / 32 * 32;
+    k_jac_pre<<<batch, nt < 128 ? 128 : (nt > JP_THREADS ? JP_THREADS : nt), sm, st>>>(dims, ptrs, cond);
+    JP_TRY(cudaGetLastError());
+  }
+  for (int it = 0; it < 2; ++it) {  // |E| ~ 1e-6, then its cube
+    JP_TRY(prod(G_JG));                                    // J^H J = I + E
+    JP_TRY(launch_lowdin_j(dims, ptrs, batch, cap.l, cond, st));  // T = (J^H J)^-1/2
+    JP_TRY(prod(G_JT));                                    // J <- J T
+  }
+  JP_TRY(prod(G_XJ));  // X <- X J
+  // tolerances of the kernels that would go on: 4 eps sqrt(l) and L eps in
+  // FP64, 8 2^-48 sqrt(l) and L 2^-48 in double-float
+  const float tolu = fp64 ? 8.8817842e-16f : 2.8421709e-14f, small_u = fp64 ? 2.220446e-16f : 3.5527137e-15f;
+  for (int it = 0; it <= JP_STEPS; ++it) {
+    JP_TRY(prod(G_XG));
+    {
+      ProfScope ps("k_jacobi[step]", st);
+      k_jac_step<<<batch, 512, sm, st>>>(dims, ptrs, cond, tolu, small_u);
+      JP_TRY(cudaGetLastError());
+    }
+    if (it == JP_STEPS) break;
+    JP_TRY(prod(G_XT));
+    JP_TRY(prod(G_JT));
+  }
+  return cudaSuccess;
+}
+
+}  // namespace tg

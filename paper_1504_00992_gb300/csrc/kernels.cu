@@ -453,7 +453,8 @@ cudaError_t run_rrsvd(const Dims* dims, const ProbPtr* ptrs, int batch, const Ca
   }
   TG_TRY(P.gemm(G_BH));                              // B^H = A^H Q
   TG_TRY(P.qr(QR_BH, DPQ_LAST));                     // B^H = Qb Rb
-  TG_TRY(launch_jacobi_sized(dims, ptrs, batch, cap, status, st));  // Rb^H J = W S
+  TG_TRY(P.svd());                                   // Rb^H J = W S, but for what the Jacobi kernel leaves
+  TG_TRY(launch_jacobi_sized(dims, ptrs, batch, cap, status, st));
   TG_TRY(P.gemm(G_U));                               // U = Q J_k
   TG_TRY(P.gemm(G_V));                               // V = Qb W_k  (stored as V^H)
   TG_TRY(launch_frob2(dims, ptrs, batch, st));

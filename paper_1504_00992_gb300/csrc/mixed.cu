@@ -798,8 +798,13 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   else
     MX_TRY(launch_qr_sized(QR_BH, dims, ptrs, batch, cap, st, qrbh));
   MX_TRY(launch_fold_small(mp.Df, dims, ptrs, l, k, batch, 0, st));
-  // Jacobi SVD: double-float one-CTA kernel unless the cluster form is chosen
+  // Jacobi SVD: double-float one-CTA kernel, after an FP32 one and digit-split
+  // corrections, unless another form is chosen
   const int jac = mixed_jac(kn, cap, batch);
+  if (jac == 3 && tc && jac_pre_rule(cap))
+    MX_TRY(run_jac_pre(const_cast<Dims*>(dims), ptrs, batch, cap, oz, batch, 0, false, err, st));
+  else
+    MX_TRY(launch_jac_none(const_cast<Dims*>(dims), batch, st));
   if (jac == 3)
     MX_TRY(launch_jacobi_df(dims, ptrs, batch, cap.l, status, st));
   else

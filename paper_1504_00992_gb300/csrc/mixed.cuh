@@ -157,11 +157,12 @@ struct DpPath {
   const int* tiles;
   cudaError_t gemm(int stage) const;
   cudaError_t qr(int stage, int kind) const;
+  cudaError_t svd() const;  // run_jac_pre where it applies; a Jacobi kernel follows
 };
 cudaError_t dp_begin(const DpPath& p);  // theta's digits, when they are kept
 // one digit-split product of the problems selected by cond: bits, and from
 // bit 8 up the pass of a Cholesky QR (the problems that take part in it)
-enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_PASS = 8 };
+enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_JS = 16, DPC_PASS = 8 };
 cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
 // Cholesky QR of Y into Q (side 0) or Yt into Qt (side 1) (cholqr.cu): up to
 // `passes` passes, then, with lowdin, the symmetric orthonormalisation to
@@ -171,6 +172,17 @@ cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
 enum { CQ_LOWDIN = 1, CQ_PHASES = 2 };
 cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* dims, const ProbPtr* ptrs, int batch,
                        const Caps& cap, const OzScratch& oz, int chunk, int cond, int* err, cudaStream_t st);
+// The small SVD X J = W S (X in R) of the problems selected by cond, up to the
+// tolerance of the Jacobi kernels (Dims::js says how far; jacobi_pre.cu), for
+// capacities of jac_pre_rule.  fp64: the FP64 kernels' tolerance, else the
+// double-float one's.
+bool jac_pre_rule(const Caps& cap);
+cudaError_t jac_pre_prepare();
+cudaError_t run_jac_pre(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, const OzScratch& oz, int chunk,
+                        int cond, bool fp64, int* err, cudaStream_t st);
+cudaError_t launch_jac_none(Dims* dims, int batch, cudaStream_t st);  // js = 0
+// T = (J^H J)^-1/2 in Yt from J^H J in Y; js = 0 where J is too far from unitary
+cudaError_t launch_lowdin_j(Dims* dims, const ProbPtr* ptrs, int batch, int l, int cond, cudaStream_t st);
 cudaError_t launch_oz_range(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
                             const OzScratch& sc, int chunk, int cond, int* err, cudaStream_t st);
 

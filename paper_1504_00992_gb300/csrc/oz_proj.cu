@@ -234,6 +234,7 @@ __device__ __forceinline__ bool oz_takes(const Dims& D, int cond) {
   if ((cond & DPC_QFLAG) && !D.qflag) return false;
   if ((cond & DPC_DIG) && !D.dig) return false;
   if ((cond & DPC_CHK) && !D.chk) return false;
+  if ((cond & DPC_JS) && D.js != 1) return false;
   return true;
 }
 
@@ -251,6 +252,11 @@ __device__ __forceinline__ void oz_store(const Dims& D, const ProbPtr& P, const 
     if (ST == OZ_GRAM && i == j) re -= 1.0;  // E = Q_f^H Q_f - I
     op.C[(int64_t)i * op.crs + (int64_t)j * op.ccs] = cmk(re, OzConj<ST>::C ? -im : im);
   }
+}
+
+// 1 / x of a power of two
+__device__ __forceinline__ double oz_pow2_inv(double x) {
+  return __longlong_as_double((2046ll << 52) - __double_as_longlong(x));
 }
 
 // Operand sources of k_oz_digits_op in their K-major views: element (row, k)
@@ -274,6 +280,7 @@ struct OzSrc {  // a GemmStage: strided operand of the stage table
   __device__ cplx at(int r, int k) const {
     const cplx v = X[(int64_t)r * rs + (int64_t)k * ks];
     if constexpr (SIDE == 0 && StageFlags<ST>::scaleA) return cscale(v, scale[k]);
+    if constexpr (SIDE == 1 && StageFlags<ST>::scaleB) return cscale(v, oz_pow2_inv(scale[k]));
     return v;
   }
 };
@@ -862,7 +869,8 @@ cudaError_t oz_prepare() {
         oz_attr<G_U>(),     oz_attr<G_V>(),     oz_attr<G_Y0>(),     oz_attr<G_Y>(),     oz_attr<G_YT>(),
         oz_attr<G_BH>(),    oz_attr<G_PR>(),    oz_attr<G_PQ>(),     oz_attr<G_PD>(),    oz_attr<G_CYG>(),
         oz_attr<G_CYQ>(),   oz_attr<G_CQG>(),   oz_attr<G_CQQ>(),    oz_attr<G_CTG>(),   oz_attr<G_CTQ>(),
-        oz_attr<G_CRG>(),   oz_attr<G_CRQ>()};
+        oz_attr<G_CRG>(),   oz_attr<G_CRQ>(),   oz_attr<G_JG>(),     oz_attr<G_JT>(),    oz_attr<G_XJ>(),
+        oz_attr<G_XG>(),    oz_attr<G_XT>()};
     for (cudaError_t e : es)
       if (e != cudaSuccess) return e;
     done = 1;
@@ -882,6 +890,7 @@ static void oz_stage_caps(int stage, const Caps& c, int& Mc, int& Nc, int& Kc) {
     case G_CYQ: case G_CQQ: Mc = c.m; Nc = c.l; Kc = c.l; break;
     case G_CTG: case G_CRG: case G_X: Mc = c.l; Nc = c.l; Kc = c.n; break;
     case G_CTQ: case G_CRQ: Mc = c.n; Nc = c.l; Kc = c.l; break;
+    case G_JG: case G_JT: case G_XJ: case G_XG: case G_XT: Mc = c.l; Nc = c.l; Kc = c.l; break;
     case G_U: Mc = c.m; Nc = c.k; Kc = c.l; break;
     case OZ_THETA: Mc = c.m; Nc = c.n; Kc = c.cm; break;  // K = chi_m, at most its bond's capacity
     case OZ_GATE: Mc = c.dl * c.dr; Nc = c.cl * c.cr; Kc = c.dl * c.dr; break;
@@ -942,7 +951,8 @@ static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch
                                 const uint16_t* pre = nullptr, const int* pre_es = nullptr) {
   const int Kp = oz_kpad(Kc);
   // an operand times its own adjoint: one set of digits
-  constexpr bool same = ST == G_G1 || ST == G_G2 || ST == G_CYG || ST == G_CQG || ST == G_CTG || ST == G_CRG;
+  constexpr bool same = ST == G_G1 || ST == G_G2 || ST == G_CYG || ST == G_CQG || ST == G_CTG || ST == G_CRG ||
+                        ST == G_JG || ST == G_XG;
   cudaError_t e = cudaSuccess;
   if (!same && !pre && Kp <= OZ_SELF_K) {
     if constexpr (!same) {
@@ -973,6 +983,7 @@ static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch
   ProfScope ps(ST == G_U || ST == G_V ? "k_oz_gemm[uv]"
                : ST == OZ_THETA          ? "k_oz_gemm[theta]"
                : ST == OZ_GATE           ? "k_oz_gemm[gate]"
+               : ST >= G_JG && ST <= G_XT ? "k_oz_gemm[svd]"
                : ST <= G_BH || (ST >= G_PR && ST <= G_PD) ? "k_oz_gemm[sketch]"
                                          : "k_oz_gemm[cholqr]",
                st);
@@ -1006,6 +1017,11 @@ cudaError_t launch_oz_stage(int stage, const Dims* dims, const ProbPtr* ptrs, in
     OZ_CASE(G_CTQ);
     OZ_CASE(G_CRG);
     OZ_CASE(G_CRQ);
+    OZ_CASE(G_JG);
+    OZ_CASE(G_JT);
+    OZ_CASE(G_XJ);
+    OZ_CASE(G_XG);
+    OZ_CASE(G_XT);
     default: return cudaErrorInvalidValue;
   }
 #undef OZ_CASE

@@ -69,6 +69,14 @@ __device__ __forceinline__ GemmOp gemm_of(const Dims& D, const ProbPtr& P) {
     g.A = L; g.ars = D.n; g.acs = 1;             // op(A)(i, k) = conj(L[k][i])
     g.B = Rt; g.brs = 1; g.bcs = D.n;
     g.C = P.R; g.crs = 1; g.ccs = D.l;
+  } else if (STAGE == G_JG || STAGE == G_JT || STAGE == G_XJ || STAGE == G_XG || STAGE == G_XT) {
+    const cplx* L = (STAGE == G_JG || STAGE == G_JT) ? P.J : P.R;
+    const cplx* Rt = (STAGE == G_JG || STAGE == G_XJ) ? P.J : (STAGE == G_XG ? P.R : P.Yt);
+    const bool gram = STAGE == G_JG || STAGE == G_XG;
+    g.M = g.N = g.K = D.l;
+    g.A = L; g.ars = gram ? D.l : 1; g.acs = gram ? 1 : D.l;
+    g.B = Rt; g.brs = 1; g.bcs = D.l;
+    g.C = gram ? P.Y : (STAGE == G_JT ? P.J : P.R); g.crs = 1; g.ccs = D.l;
   } else if (STAGE == G_CYG || STAGE == G_CQG || STAGE == G_CTG || STAGE == G_CRG) {  // X^H X of a basis
     const bool y = (STAGE == G_CYG || STAGE == G_CQG);
     const cplx* X = (STAGE == G_CYG) ? P.Y : (STAGE == G_CQG) ? P.Q : (STAGE == G_CTG) ? P.Yt : P.Qt;
@@ -96,9 +104,12 @@ template <int STAGE>
 struct StageFlags {
   static constexpr bool conjA =
       (STAGE == G_YT || STAGE == G_BH || STAGE == G_PQ || STAGE == G_G1 || STAGE == G_G2 || STAGE == G_X ||
-       STAGE == G_CYG || STAGE == G_CQG || STAGE == G_CTG || STAGE == G_CRG);
+       STAGE == G_CYG || STAGE == G_CQG || STAGE == G_CTG || STAGE == G_CRG || STAGE == G_JG || STAGE == G_XG);
   // the left operand's column k is scaled by sigma[k] (a power of two)
-  static constexpr bool scaleA = (STAGE == G_CYQ || STAGE == G_CQQ || STAGE == G_CTQ || STAGE == G_CRQ);
+  // (scaleB: and the right operand's row k by its inverse)
+  static constexpr bool scaleB = (STAGE == G_XJ || STAGE == G_XT);
+  static constexpr bool scaleA =
+      (STAGE == G_CYQ || STAGE == G_CQQ || STAGE == G_CTQ || STAGE == G_CRQ || scaleB);
   static constexpr bool conjC = (STAGE == G_V);
 };
 
@@ -287,7 +298,8 @@ __device__ __forceinline__ void jacobi_dev(const Dims& D, const ProbPtr& P, int*
   const int grp = tid / JAC_G, ngrp = blockDim.x / JAC_G;  // group index, groups per CTA
   const unsigned gmask = ((1u << JAC_G) - 1u) << (lane & ~(JAC_G - 1));
   double f2 = 0.0;
-  for (int e = tid; e < L * L; e += blockDim.x) J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
+  if (D.js == 0)
+    for (int e = tid; e < L * L; e += blockDim.x) J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
   if (tid < RED_LANES)
     for (int e = tid; e < L * L; e += RED_LANES) f2 += cabs2(X[e]);
   f2 = block_sum(f2, red);
@@ -295,7 +307,7 @@ __device__ __forceinline__ void jacobi_dev(const Dims& D, const ProbPtr& P, int*
   const double eps = 2.220446049250313e-16;
   const double tol = 4.0 * eps * sqrt((double)L);
   const double small = ((double)L * eps) * ((double)L * eps) * f2;
-  int sweep = 0;
+  int sweep = D.js == 2 ? JAC_MAXSWEEPS + 1 : 0;
   for (; sweep < JAC_MAXSWEEPS; ++sweep) {
     // exact squared column norms at the start of every sweep; within the sweep
     // they follow each rotation: |x_a'|^2 = |x_a|^2 - t|g|, |x_b'|^2 = |x_b|^2 + t|g|
@@ -423,6 +435,7 @@ __device__ __forceinline__ Dims plan_dev(const ProbPtr& P, int p, int digits) {
   D.dig = (digits && dp_rule(D.m, D.n, D.l)) ? 1 : 0;
   D.cq = 0;
   D.cf = 0;
+  D.js = 0;
   return D;
 }
 
