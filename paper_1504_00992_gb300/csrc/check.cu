@@ -109,7 +109,7 @@ cudaError_t run_accuracy_check(const Dims* dims_mut, const ProbPtr* ptrs, int ba
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // [Q | Br] = Q' R' (a basis no power round follows stays with Householder)
-    e = (dp && !final_basis) ? P.qr(QR_Y, DPQ_CHECK) : launch_qr(QR_Y, dims, ptrs, batch, st, QRS_QFLAG);
+    e = (dp && !final_basis) ? P.qr(QR_Y, DPQ_CHECK) : launch_qr(QR_Y, dims, ptrs, batch, cap, st, QRS_QFLAG);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

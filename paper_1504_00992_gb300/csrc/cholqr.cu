@@ -298,6 +298,8 @@ cudaError_t cholqr_prepare() {
     if (e2 != cudaSuccess) return e2;
     const cudaError_t e5 = lowdin_prepare();
     if (e5 != cudaSuccess) return e5;
+    const cudaError_t e4 = qr_small_prepare();
+    if (e4 != cudaSuccess) return e4;
     const cudaError_t e3 = jac_pre_prepare();
     if (e3 != cudaSuccess) return e3;
     done = 1;
@@ -339,7 +341,7 @@ cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps
   CQ_TRY(gemm(G_QB));                          // Qb = Q1 R2^-1
   CQ_TRY(gemm(G_X));                           // X = B Qb = Rb^H
   // ill-conditioned instances: Householder QR of B^H (overwrites X and Qb)
-  return launch_qr(QR_BH, dims, ptrs, batch, st, QRS_QFLAG);
+  return launch_qr(QR_BH, dims, ptrs, batch, cap, st, QRS_QFLAG);
 }
 
 // ---------------------------------------------------------------------------

@@ -142,18 +142,18 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2) k_bond_fused(const ProbPtr* 
     }
     __syncthreads();
     gemm_all<G_Y0>(D, P, sm);  // Y0 = A Omega
-    qr_dev<QR_Y>(D, P, sm.red, sm.u.qr.tau, sm.u.qr.alph);
+    qr_dev<QR_Y>(D, P, sm.u.qr.tau, sm.u.qr.alph);
     __syncthreads();
     for (int j = 0; j < q; ++j) {
       gemm_all<G_YT>(D, P, sm);  // Y~ = A^H Q
-      qr_dev<QR_YT>(D, P, sm.red, sm.u.qr.tau, sm.u.qr.alph);
+      qr_dev<QR_YT>(D, P, sm.u.qr.tau, sm.u.qr.alph);
       __syncthreads();
       gemm_all<G_Y>(D, P, sm);  // Y = A Q~
-      qr_dev<QR_Y>(D, P, sm.red, sm.u.qr.tau, sm.u.qr.alph);
+      qr_dev<QR_Y>(D, P, sm.u.qr.tau, sm.u.qr.alph);
       __syncthreads();
     }
     gemm_all<G_BH>(D, P, sm);  // B^H = A^H Q
-    qr_dev<QR_BH>(D, P, sm.red, sm.u.qr.tau, sm.u.qr.alph);
+    qr_dev<QR_BH>(D, P, sm.u.qr.tau, sm.u.qr.alph);
     __syncthreads();
     jacobi_dev(D, P, status, sm.u.jac.sv, sm.u.jac.nrm, sm.u.jac.perm, &sm.rotated, sm.red);
     __syncthreads();

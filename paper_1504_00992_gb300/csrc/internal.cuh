@@ -124,8 +124,13 @@ __host__ __device__ inline bool qr_takes(const Dims& D, int which) {
   if ((which & QRS_REST) && D.dig && !D.cf) return false;
   return !((which & QRS_CF) && !D.cf);
 }
-cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, cudaStream_t st,
+cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
                       int which = QRS_ALL);
+// the same on a cluster of CTAs per matrix, the matrix in shared memory (qr_small.cu)
+bool qr_small_fits(int stage, const Caps& cap);
+cudaError_t launch_qr_small(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
+                            cudaStream_t st, int which);
+cudaError_t qr_small_prepare();
 // the same, spread over many CTAs per instance (qr_multi.cu) when the batch
 // is a few tall matrices (cap.m or cap.n rows, cap.l columns); every
 // instance's R and J buffers must hold at least qr_multi_scratch_r(l) and

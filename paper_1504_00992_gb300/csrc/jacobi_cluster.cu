@@ -18,13 +18,14 @@
 
 #include "internal.cuh"
 #include "profiler.cuh"
+#include "stages.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace tg {
 
 enum { JC_CL = 8, JC_THREADS = 256, JC_G = 8, JC_U = 4, JC_MAXSWEEPS = 60, JC_MAXL = 512 };
-enum { JC_MIN_L = 64, JC_MAX_BATCH = 40 };
+enum { JC_MIN_L = 64, JC_MAX_BATCH = 40, JC_SMALL_L = 24, JC_SMALL_BATCH = 19 };
 
 __device__ __forceinline__ double jc_grp_sum(double v, unsigned mask) {
 #pragma unroll
@@ -120,7 +121,7 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
         cplx* xb = X + (int64_t)b * L;
         const double aa = __ldcg(nrm + a), bb = __ldcg(nrm + b);
         if (aa <= small || bb <= small) continue;
-        cplx g = cmk(0.0, 0.0);
+        double rx = 0.0, ry = 0.0, ix = 0.0, iy = 0.0;
         for (int r0 = gl; r0 < L; r0 += JC_G * JC_U) {
           cplx u[JC_U], v[JC_U];
 #pragma unroll
@@ -130,23 +131,27 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
             v[q] = (r < L) ? __ldcg(xb + r) : cmk(0.0, 0.0);
           }
 #pragma unroll
-          for (int q = 0; q < JC_U; ++q) cfma_conj(g, u[q], v[q]);
+          for (int q = 0; q < JC_U; ++q) {
+            if (r0 + q * JC_G < L) {
+              rx = fma(u[q].x, v[q].x, rx);
+              ry = fma(u[q].y, v[q].y, ry);
+              ix = fma(u[q].x, v[q].y, ix);
+              iy = fma(-u[q].y, v[q].x, iy);
+            }
+          }
         }
-        g.x = jc_grp_sum(g.x, gmask);
-        g.y = jc_grp_sum(g.y, gmask);
+        const cplx g = cmk(jc_grp_sum(rx + ry, gmask), jc_grp_sum(ix + iy, gmask));
         const double ag2 = cabs2(g);
-        if (!(ag2 > tol * tol * (aa * bb)) || ag2 == 0.0) continue;
-        const double ag = sqrt(ag2);
-        const cplx e = cscale(g, 1.0 / ag);
-        const double zeta = (bb - aa) / (2.0 * ag);
-        const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-        const cplx se = cscale(e, s), sec = cconj(se);
+        if (!(ag2 > tol * tol * (aa * bb)) || ag2 < 2.2250738585072014e-308) continue;
+        double c, tg;
+        cplx se;
+        jac_rotation(aa, bb, g, ag2, c, se, tg);
+        const cplx sec = cconj(se);
         jc_rotate(xa, xb, L, gl, c, se, sec);
         jc_rotate(J + (int64_t)a * L, J + (int64_t)b * L, L, gl, c, se, sec);
         if (gl == 0) {
-          nrm[a] = aa - t * ag;
-          nrm[b] = bb + t * ag;
+          nrm[a] = aa - tg;
+          nrm[b] = bb + tg;
           rotated = 1;
         }
       }
@@ -189,7 +194,10 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
 }
 
 bool jacobi_cluster_chosen(const Caps& cap, int batch, int force) {
+  // a few matrices of any width from JC_SMALL_L on (a cluster's SMs would idle
+  // otherwise), up to JC_MAX_BATCH wide ones
   const bool fits = cap.l >= JC_MIN_L && cap.l <= JC_MAXL;
+  if (force == 0 && cap.l >= JC_SMALL_L && cap.l <= JC_MAXL && batch <= JC_SMALL_BATCH) return true;
   return force == 2 ? fits : (force == 0 && fits && batch <= JC_MAX_BATCH);
 }
 

@@ -278,19 +278,19 @@ cudaError_t launch_zgemm(int stage, const Dims* dims, const ProbPtr* ptrs, int b
 template <int QS>
 __global__ void __launch_bounds__(QR_THREADS) k_qr(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
                                             int which) {
-  __shared__ double red[32];
   __shared__ double tau[QR_MAXL];
   __shared__ cplx alph[QR_MAXL];
   const int p = blockIdx.x;
   const Dims D = dims[p];
   if (!D.active) return;
   if (!qr_takes(D, which)) return;
-  qr_dev<QS>(D, ptrs[p], red, tau, alph);
+  qr_dev<QS>(D, ptrs[p], tau, alph);
 }
 
-cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, cudaStream_t st,
+cudaError_t launch_qr(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
                       int which) {
   ProfScope ps("k_qr", st);
+  if (qr_small_fits(stage, cap)) return launch_qr_small(stage, dims, ptrs, batch, cap, st, which);
   // batches of four matrices per SM or more: 256-thread CTAs, four per SM,
   // so that one matrix's per-column barriers overlap with the others' work
   const int nt = batch >= 4 * 152 ? 256 : QR_THREADS;

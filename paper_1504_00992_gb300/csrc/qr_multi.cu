@@ -593,14 +593,14 @@ cudaError_t launch_qr_rest(int stage, const Dims* dims, const ProbPtr* ptrs, int
   const int M = (stage == QR_Y) ? cap.m : cap.n;
   const bool large = (double)M * cap.l * cap.l >= 1e8 && qr_multi_fits(M, cap.l, 1);
   return large ? launch_qr_sized(stage, dims, ptrs, batch, cap, st, 2, which)
-               : launch_qr(stage, dims, ptrs, batch, st, which);
+               : launch_qr(stage, dims, ptrs, batch, cap, st, which);
 }
 
 cudaError_t launch_qr_sized(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
                             cudaStream_t st, int force, int which) {
   const int M = (stage == QR_Y) ? cap.m : cap.n;
   const bool multi = force == 2 ? qr_multi_fits(M, cap.l, 1) : (force == 0 && qr_multi_fits(M, cap.l, batch));
-  if (!multi) return launch_qr(stage, dims, ptrs, batch, st, which);
+  if (!multi) return launch_qr(stage, dims, ptrs, batch, cap, st, which);
   ProfScope ps("k_qr[multi]", st);
   cudaError_t e;
   switch (stage) {

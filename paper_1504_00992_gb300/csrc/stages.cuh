@@ -189,55 +189,276 @@ enum { QR_MAXL = 512 };
 
 enum { QR_THREADS = 1024, JAC_THREADS = 512 };
 
-// Householder QR with explicit Q of one problem (stage QS) by the whole CTA
-// (any multiple of 32 threads); red >= 32 doubles, tau / alph >= l entries of
-// shared memory.
+// ---------------------------------------------------------------------------
+// Householder QR.  FP64 runs at half a multiply-add per clock on each quarter
+// of an SM: a warp's FP64 instruction takes 64 clocks there, whether the next
+// one depends on it or not and however many lanes take part (measured: 65
+// clocks a step for a dependent chain, 64 for eight independent ones; 128 with
+// two warps on the quarter).  So what counts is the number of warp
+// instructions on the fullest quarter, and for the chain of reflectors that
+// its warp has a quarter for itself:
+//   - warp 0 alone applies H_j to column j + 1 and forms the next reflector,
+//     one row per lane at a time (qr_next: ~50 instructions for 64 rows), while
+//     the others apply H_j to the columns right of it, 16 lanes per column
+//     (qr_apply: ~36 instructions for two columns); one barrier per column;
+//   - the others' work is dealt out to the other quarters first (qr_slot);
+//   - re and im sums of an inner product share the additions of the reduction
+//     (qr_csum), square roots and reciprocals are one third-order step from an
+//     FP32 seed, powers of two go into the exponent bits;
+//   - Q's columns are independent: one warp each, in registers.
+// The sums and their order are fixed by the column's role alone, so the
+// one-CTA kernel, the cluster kernel (qr_small.cu) and the fused kernel give
+// the same results bit for bit.
+// ---------------------------------------------------------------------------
+enum { QR_G = 16 };
+
+// sums of re and im over the G lanes of a group, to all of them
+template <int G>
+__device__ __forceinline__ cplx qr_csum(double re, double im, int lane, unsigned mask) {
+  const bool odd = lane & 1;
+  double v = odd ? im : re;
+  v += __shfl_xor_sync(mask, odd ? re : im, 1);
+#pragma unroll
+  for (int o = G / 2; o > 1; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  const double w = __shfl_xor_sync(mask, v, 1);
+  return odd ? cmk(w, v) : cmk(v, w);
+}
+// biased exponent, and x 2^k by the exponent bits (0 where that leaves the normal range below)
+__device__ __forceinline__ int qr_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
+__device__ __forceinline__ double qr_scale(double x, int k) {
+  const int e = qr_exp(x);
+  return (e == 0 || e + k <= 0) ? 0.0 : __longlong_as_double(__double_as_longlong(x) + ((long long)k << 52));
+}
+__device__ __forceinline__ double qr_pow2(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
+// a positive normal double of FP32's range to FP32 (cut off) and back, by the bits
+__device__ __forceinline__ float qr_f32(double x) {
+  const long long u = __double_as_longlong(x);
+  return __uint_as_float((unsigned)((u >> 29) - (896ll << 23)));
+}
+__device__ __forceinline__ double qr_f64(float x) {
+  return __longlong_as_double(((long long)__float_as_uint(x) << 29) + (896ll << 52));
+}
+// y = 1 / sqrt(v) and q = sqrt(v), v in [1, 8)
+__device__ __forceinline__ void qr_roots(double v, double& y, double& q) {
+  const double y0 = qr_f64(rsqrtf(qr_f32(v)));
+  const double t = v * y0, r = fma(-t, y0, 1.0), p = fma(0.375, r, 0.5);
+  y = fma(y0 * r, p, y0);
+  q = fma(t * r, p, t);
+}
+// 1 / v, v a normal number with a normal reciprocal
+__device__ __forceinline__ double qr_rcp(double v) {
+  const int e = qr_exp(v) - 1023;
+  const double m = qr_scale(v, -e);  // [1, 2)
+  const double y0 = qr_f64(1.f / qr_f32(m)), r = fma(-m, y0, 1.0);
+  return qr_scale(fma(y0, fma(r, r, r), y0), -e);
+}
+
+// Reflector of column j from s = sum of |x|^2 over its rows from j on, by a
+// whole warp: v_0 = x_0 - alpha into a[j], tau and (ALPHA) alpha.
+template <bool ALPHA>
+__device__ __forceinline__ void qr_reflect(cplx* a, int j, double s, int lane, double* tau, cplx* alph) {
+  const cplx x0 = a[j];
+  double t = 0.0;
+  cplx al = cmk(0.0, 0.0), v0 = x0;
+  // zero column, or one so small that tau would overflow (||x|| < 1e-150)
+  if (!(s < INFINITY)) {
+    al = cmk(-s, 0.0);
+  } else if (s >= 1e-300) {
+    // ||x|| and |x_0| by lanes of the same instructions: both scaled to [1, 8)
+    const int e2 = (qr_exp(s) - 1023) & ~1;
+    const int ex = max(qr_exp(x0.x), qr_exp(x0.y)) - 1023;
+    const bool has = ex > -1023 + 60;
+    const double ux = has ? qr_scale(x0.x, -ex) : 1.0, uy = has ? qr_scale(x0.y, -ex) : 0.0;
+    const double a2 = fma(ux, ux, uy * uy);
+    double y, q;
+    qr_roots((lane & 1) ? a2 : qr_scale(s, -e2), y, q);
+    const double ys = __shfl_xor_sync(0xffffffffu, y, 1), qs = __shfl_xor_sync(0xffffffffu, q, 1);
+    const double nx = qr_scale((lane & 1) ? qs : q, e2 / 2);
+    const double ya = (lane & 1) ? y : ys;
+    const double ax0 = has ? qr_scale((lane & 1) ? q : qs, ex) : 0.0;
+    // the phase of a leading entry negligible against ||x|| is not used
+    const cplx ph = (ax0 > 1e-15 * nx) ? cmk(ux * ya, uy * ya) : cmk(1.0, 0.0);
+    const double d = ax0 + nx;
+    if (ALPHA) al = cscale(ph, -nx);
+    v0 = cscale(ph, d);  // x_0 - alpha
+    t = qr_rcp(nx * d);
+  }
+  __syncwarp();  // every lane has read x_0
+  if (lane == 0) {
+    a[j] = v0;
+    *tau = t;
+    if (ALPHA) *alph = al;
+  }
+}
+
+// sum of |x|^2 over the rows from j on, by a whole warp
+__device__ __forceinline__ double qr_norm2(const cplx* a, int j, int M, int lane) {
+  double s = 0.0;
+  for (int r = (j & ~31) + lane; r < M; r += 32)
+    if (r >= j) s = fma(a[r].x, a[r].x, fma(a[r].y, a[r].y, s));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// a = column j + 1 <- H_j a with reflector v, then its reflector, by a whole warp
+template <bool ALPHA>
+__device__ __forceinline__ void qr_next(const cplx* v, cplx* a, int j, int M, const double t, int lane, double* tau,
+                                        cplx* alph) {
+  double s = 0.0;
+  if (t != 0.0) {
+    double re = 0.0, im = 0.0;
+    for (int r = (j & ~31) + lane; r < M; r += 32) {
+      if (r < j) continue;
+      const cplx x = v[r], y = a[r];
+      re = fma(x.x, y.x, fma(x.y, y.y, re));
+      im = fma(x.x, y.y, fma(-x.y, y.x, im));
+    }
+    const cplx g = qr_csum<32>(re, im, lane, 0xffffffffu);
+    const double sr = t * g.x, si = t * g.y;
+    for (int r = (j & ~31) + lane; r < M; r += 32) {
+      if (r < j) continue;
+      const cplx x = v[r];
+      cplx y = a[r];
+      y.x = fma(-x.x, sr, fma(x.y, si, y.x));
+      y.y = fma(-x.x, si, fma(-x.y, sr, y.y));
+      a[r] = y;
+      if (r > j) s = fma(y.x, y.x, fma(y.y, y.y, s));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  } else {
+    s = qr_norm2(a, j + 1, M, lane);
+  }
+  __syncwarp();
+  qr_reflect<ALPHA>(a, j + 1, s, lane, tau, alph);
+}
+
+// c <- H c, H = I - t v v^H, over the rows from j on, by a group of QR_G lanes
+__device__ __forceinline__ void qr_apply(const cplx* v, cplx* c, int j, int M, double t, int gl, unsigned mask) {
+  double re = 0.0, im = 0.0;
+  for (int r = (j & ~(QR_G - 1)) + gl; r < M; r += QR_G) {
+    if (r < j) continue;
+    const cplx x = v[r], y = c[r];
+    re = fma(x.x, y.x, fma(x.y, y.y, re));
+    im = fma(x.x, y.y, fma(-x.y, y.x, im));
+  }
+  const cplx g = qr_csum<QR_G>(re, im, gl, mask);
+  const double sr = t * g.x, si = t * g.y;
+  for (int r = (j & ~(QR_G - 1)) + gl; r < M; r += QR_G) {
+    if (r < j) continue;
+    const cplx x = v[r];
+    cplx y = c[r];
+    y.x = fma(-x.x, sr, fma(x.y, si, y.x));
+    y.y = fma(-x.x, si, fma(-x.y, sr, y.y));
+    c[r] = y;
+  }
+}
+
+// Column c of Q = H_0 ... H_{L-1} [I; 0], i.e. H_c, ..., H_0 applied to e_c
+// (H_j leaves e_c alone for j > c), by a whole warp: the column in registers,
+// row lane + 32 k in x[k], for M <= 32 R.  The reflectors that start in row
+// block s are one loop whose blocks are known at compile time: blocks left out
+// by a condition at run time would be predicated FP64 instructions, which take
+// the pipe's time all the same (at eight blocks for 64 rows 1.5 ms for 256
+// 64 x 42 matrices, against 0.6).
+template <int R>
+__device__ __forceinline__ void qr_qcol_r(const cplx* V, const double* tau, cplx* q, int c, int M, int lane) {
+  cplx x[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) x[k] = cmk(lane + 32 * k == c ? 1.0 : 0.0, 0.0);
+#pragma unroll
+  for (int s = R - 1; s >= 0; --s) {
+    for (int j = min(c, 32 * s + 31); j >= 32 * s; --j) {
+      const double t = tau[j];
+      if (t == 0.0) continue;
+      const cplx* v = V + (int64_t)j * M;
+      cplx y[R];
+      double re = 0.0, im = 0.0;
+#pragma unroll
+      for (int k = s; k < R; ++k) {
+        const int r = lane + 32 * k;
+        y[k] = (r >= j && r < M) ? v[r] : cmk(0.0, 0.0);
+        re = fma(y[k].x, x[k].x, fma(y[k].y, x[k].y, re));
+        im = fma(y[k].x, x[k].y, fma(-y[k].y, x[k].x, im));
+      }
+      const cplx g = qr_csum<32>(re, im, lane, 0xffffffffu);
+      const double sr = t * g.x, si = t * g.y;
+#pragma unroll
+      for (int k = s; k < R; ++k) {
+        x[k].x = fma(-y[k].x, sr, fma(y[k].y, si, x[k].x));
+        x[k].y = fma(-y[k].x, si, fma(-y[k].y, sr, x[k].y));
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k)
+    if (lane + 32 * k < M) q[lane + 32 * k] = x[k];
+}
+
+__device__ __forceinline__ void qr_qcol(const cplx* V, const double* tau, cplx* q, int c, int M, int lane) {
+  switch ((M + 31) / 32) {
+    case 1: return qr_qcol_r<1>(V, tau, q, c, M, lane);
+    case 2: return qr_qcol_r<2>(V, tau, q, c, M, lane);
+    case 3: return qr_qcol_r<3>(V, tau, q, c, M, lane);
+    case 4: return qr_qcol_r<4>(V, tau, q, c, M, lane);
+    default: break;
+  }
+  for (int r = lane; r < M; r += 32) q[r] = cmk(r == c ? 1.0 : 0.0, 0.0);
+  for (int j = c; j >= 0; --j) {
+    const double t = tau[j];
+    if (t == 0.0) continue;
+    const cplx* v = V + (int64_t)j * M;
+    double re = 0.0, im = 0.0;
+    for (int r = (j & ~31) + lane; r < M; r += 32) {
+      if (r < j) continue;
+      const cplx y = v[r], x = q[r];
+      re = fma(y.x, x.x, fma(y.y, x.y, re));
+      im = fma(y.x, x.y, fma(-y.y, x.x, im));
+    }
+    const cplx g = qr_csum<32>(re, im, lane, 0xffffffffu);
+    const double sr = t * g.x, si = t * g.y;
+    for (int r = (j & ~31) + lane; r < M; r += 32) {
+      if (r < j) continue;
+      const cplx y = v[r];
+      cplx x = q[r];
+      x.x = fma(-y.x, sr, fma(y.y, si, x.x));
+      x.y = fma(-y.x, si, fma(-y.y, sr, x.y));
+      q[r] = x;
+    }
+  }
+}
+
+// Order in which warp w >= 1 of a CTA takes the columns right of the next one:
+// two rounds over the quarters without warp 0, then all quarters in turn (the
+// chain is worth one to two of a quarter's tasks).
+__device__ __forceinline__ int qr_slot(int w) {
+  const int s = w & 3, q = w >> 2;
+  if (s == 0) return 6 + (q - 1) * 4;
+  return q < 2 ? q * 3 + s - 1 : 6 + (q - 2) * 4 + s;
+}
+
+// QR with explicit Q of one problem (stage QS) by the whole CTA (a multiple of
+// 128 threads); tau / alph >= l entries of shared memory.
 template <int QS>
-__device__ __forceinline__ void qr_dev(const Dims& D, const ProbPtr& P, double* red, double* tau, cplx* alph) {
+__device__ __forceinline__ void qr_dev(const Dims& D, const ProbPtr& P, double* tau, cplx* alph) {
   const int M = (QS == QR_Y) ? D.m : D.n;
   const int L = D.l;
   cplx* A = (QS == QR_Y) ? P.Y : P.Yt;
   cplx* Qo = (QS == QR_Y) ? P.Q : P.Qt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-
-  for (int j = 0; j < L; ++j) {
-    cplx* aj = A + (int64_t)j * M;
-    double s = 0.0;
-    // a fixed decomposition over RED_LANES partial sums, whatever the CTA
-    // size: the result does not depend on the launch configuration
-    if (tid < RED_LANES)
-      for (int r = j + tid; r < M; r += RED_LANES) s += cabs2(aj[r]);
-    s = block_sum(s, red);
-    if (tid == 0) {
-      const cplx x0 = aj[j];
-      // |x0| by hypot: the phase x0/|x0| must stay on the unit circle for H to be unitary
-      const double ax0 = hypot(x0.x, x0.y);
-      const double nx = sqrt(s);
-      if (!(nx >= 1e-150)) {  // zero column, or one so small that tau would overflow
-        tau[j] = 0.0;
-        alph[j] = cmk(0.0, 0.0);
-      } else {
-        // the phase of a leading entry negligible against ||x|| is not used
-        const cplx ph = (ax0 > 1e-15 * nx) ? cscale(x0, 1.0 / ax0) : cmk(1.0, 0.0);
-        alph[j] = cscale(ph, -nx);
-        aj[j] = cscale(ph, ax0 + nx);  // v_0 = x_0 - alpha
-        tau[j] = 1.0 / (nx * (nx + ax0));
-      }
-    }
-    __syncthreads();
+  const int gl = lane & (QR_G - 1), half = lane / QR_G;
+  const unsigned gmask = ((1u << QR_G) - 1u) << (lane & ~(QR_G - 1));
+  const int slot = qr_slot(warp);
+  if (warp == 0) qr_reflect<QS == QR_BH>(A, 0, qr_norm2(A, 0, M, lane), lane, tau, alph);
+  __syncthreads();
+  for (int j = 0; j + 1 < L; ++j) {
     const double t = tau[j];
-    if (t != 0.0) {
-      for (int c = j + 1 + warp; c < L; c += nw) {
-        cplx* ac = A + (int64_t)c * M;
-        cplx sd = cmk(0.0, 0.0);
-        for (int r = j + lane; r < M; r += 32) cfma_conj(sd, aj[r], ac[r]);
-        sd = cscale(warp_sum(sd), t);
-        for (int r = j + lane; r < M; r += 32) {
-          const cplx v = aj[r];
-          ac[r] = csub(ac[r], cmul(v, sd));
-        }
-      }
-    }
+    const cplx* v = A + (int64_t)j * M;
+    if (warp == 0)
+      qr_next<QS == QR_BH>(v, A + (int64_t)(j + 1) * M, j, M, t, lane, tau + j + 1, alph + j + 1);
+    else if (t != 0.0)
+      for (int c = j + 2 + 2 * slot + half; c < L; c += 2 * (nw - 1)) qr_apply(v, A + (int64_t)c * M, j, M, t, gl, gmask);
     __syncthreads();
   }
   // X = Rb^H (lower triangle, column-major L x L) for the SVD of B: element
@@ -252,25 +473,8 @@ __device__ __forceinline__ void qr_dev(const Dims& D, const ProbPtr& P, double* 
       P.R[(int64_t)c * L + r] = v;
     }
   }
-  // Q = [I; 0], then Q <- H_j Q for j = L-1 .. 0 (only columns c >= j change)
-  for (int64_t e = tid; e < (int64_t)M * L; e += blockDim.x) {
-    const int c = (int)(e / M), r = (int)(e % M);
-    Qo[e] = cmk(r == c ? 1.0 : 0.0, 0.0);
-  }
+  for (int c = L - 1 - warp; c >= 0; c -= nw) qr_qcol(A, tau, Qo + (int64_t)c * M, c, M, lane);
   __syncthreads();
-  for (int j = L - 1; j >= 0; --j) {
-    const double t = tau[j];
-    if (t == 0.0) continue;  // uniform across the block
-    const cplx* aj = A + (int64_t)j * M;
-    for (int c = j + warp; c < L; c += nw) {
-      cplx* qc = Qo + (int64_t)c * M;
-      cplx sd = cmk(0.0, 0.0);
-      for (int r = j + lane; r < M; r += 32) cfma_conj(sd, aj[r], qc[r]);
-      sd = cscale(warp_sum(sd), t);
-      for (int r = j + lane; r < M; r += 32) qc[r] = csub(qc[r], cmul(aj[r], sd));
-    }
-    __syncthreads();
-  }
 }
 
 enum { JAC_MAXSWEEPS = 60, JAC_G = 8 };
@@ -283,6 +487,34 @@ __device__ __forceinline__ double grp_sum(double v, unsigned mask) {
 }
 
 __device__ __forceinline__ void jacobi_finish(const Dims& D, const ProbPtr& P, double* sv, int* perm);
+
+// Rotation of a pair: x_a' = c x_a - conj(se) x_b, x_b' = se x_a + c x_b that
+// makes them orthogonal, from aa = |x_a|^2, bb = |x_b|^2, g = x_a^H x_b and
+// ag2 = |g|^2; tg = t |g|, what the squared norms change by.  About 30 FP64
+// operations: |g| and 1 / |g| from one Newton reciprocal root, the tangent t
+// from FP32 and one Newton step of t^2 + 2 zeta t - 1 = 0 (relative error
+// ~1e-14; c and s = c t are unitary to FP64 whatever t is).  Eight lanes
+// repeat them, so the ~140 operations of the library's roots and divisions
+// were as much FP64 work as the rows of a 40-row pair.
+__device__ __forceinline__ void jac_rotation(double aa, double bb, cplx g, double ag2, double& c, cplx& se, double& tg) {
+  // |g|^2 = w 2^e2, w in [1, 4)
+  const int e2 = (qr_exp(ag2) - 1023) & ~1;
+  const double w = ag2 * qr_pow2(-e2);
+  double y, q;
+  qr_roots(w, y, q);
+  const double inv = y * qr_pow2(-(e2 / 2)), ag = q * qr_pow2(e2 / 2);
+  const cplx e = cscale(g, inv);
+  const double zeta = (0.5 * (bb - aa)) * inv;
+  const float zf = fabsf((float)zeta);
+  const float tf = zf > 1e9f ? 0.5f / zf : 1.f / (zf + sqrtf(fmaf(zf, zf, 1.f)));
+  const double t0 = (double)tf, az = fabs(zeta);
+  const double res = fma(t0, t0 + 2.0 * az, -1.0);
+  const double t1 = t0 - (double)((float)res / (2.f * (tf + zf)));
+  const double t = zeta >= 0.0 ? t1 : -t1;
+  qr_roots(fma(t, t, 1.0), c, q);
+  se = cscale(e, c * t);
+  tg = t * ag;
+}
 
 // One-sided Jacobi SVD of one problem by the whole CTA (any multiple of
 // JAC_G threads, at least 32); sv, nrm, perm >= l entries and red >= 32
@@ -331,19 +563,21 @@ __device__ __forceinline__ void jacobi_dev(const Dims& D, const ProbPtr& P, int*
         cplx* xb = X + (int64_t)b * L;
         const double aa = nrm[a], bb = nrm[b];
         if (aa <= small || bb <= small) continue;
-        cplx g = cmk(0.0, 0.0);
-        for (int r = gl; r < L; r += JAC_G) cfma_conj(g, xa[r], xb[r]);
-        g.x = grp_sum(g.x, gmask);
-        g.y = grp_sum(g.y, gmask);
+        double rx = 0.0, ry = 0.0, ix = 0.0, iy = 0.0;
+        for (int r = gl; r < L; r += JAC_G) {
+          const cplx u = xa[r], v = xb[r];
+          rx = fma(u.x, v.x, rx);
+          ry = fma(u.y, v.y, ry);
+          ix = fma(u.x, v.y, ix);
+          iy = fma(-u.y, v.x, iy);
+        }
+        const cplx g = cmk(grp_sum(rx + ry, gmask), grp_sum(ix + iy, gmask));
         const double ag2 = cabs2(g);
-        if (!(ag2 > tol * tol * (aa * bb)) || ag2 == 0.0) continue;
-        const double ag = sqrt(ag2);
-        // rotation: x_a' = c x_a - s e* x_b, x_b' = s e x_a + c x_b, e = g/|g|
-        const cplx e = cscale(g, 1.0 / ag);
-        const double zeta = (bb - aa) / (2.0 * ag);
-        const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-        const cplx se = cscale(e, s), sec = cconj(se);
+        if (!(ag2 > tol * tol * (aa * bb)) || ag2 < 2.2250738585072014e-308) continue;  // (below normal numbers)
+        double c, tg;
+        cplx se;
+        jac_rotation(aa, bb, g, ag2, c, se, tg);
+        const cplx sec = cconj(se);
         for (int r = gl; r < L; r += JAC_G) {
           const cplx u = xa[r], v = xb[r];
           xa[r] = csub(cscale(u, c), cmul(sec, v));
@@ -357,8 +591,8 @@ __device__ __forceinline__ void jacobi_dev(const Dims& D, const ProbPtr& P, int*
           jb[r] = cadd(cmul(se, u), cscale(v, c));
         }
         if (gl == 0) {
-          nrm[a] = aa - t * ag;
-          nrm[b] = bb + t * ag;
+          nrm[a] = aa - tg;
+          nrm[b] = bb + tg;
           rotated = 1;
         }
       }
