@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_inv_sm(Dims* dims, const Pr
 // the kernel of the digit-split form below
 template <bool SM>
 __global__ void k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass, int passes, float min_pivot,
-                          float again, int cond);
+                          float again, int cond, int f32);
 
 static cudaError_t lowdin_prepare();
 
@@ -374,6 +374,8 @@ static const float CE_AGAIN = 1.4901161193847656e-08f;  // 2^-26: below it anoth
 static const float CE_AGAIN_LD = 6.103515625e-05f;      // 2^-14: the same before the symmetric correction
 
 enum { CE_THREADS = 512, CE_MAXL = 512 };
+static const float CE_F32_LAST = 16.f, CE_F32_MID = 1e4f;  // bounds of the FP32 form's R^-1 column sums
+enum { CE_F32_EXP = 96 };  // column norms 2^+-96 leave S R^-1 inside FP32's range
 
 // x 2^k by the exponent bits (x = 0 and results below the normal range: 0)
 __device__ __forceinline__ double ce_scale(double x, int k) {
@@ -395,13 +397,15 @@ __device__ __forceinline__ bool ce_takes(const Dims& D, int pass, int cond) {
 // for a second attempt with the shift).
 template <bool SM>
 __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass,
-                                                        int passes, float min_pivot, float again, int cond) {
+                                                        int passes, float min_pivot, float again, int cond,
+                                                        int f32) {
   extern __shared__ __align__(16) unsigned char ce_raw[];
   __shared__ double s_diag[CE_MAXL];
   __shared__ int s_exp[CE_MAXL];
   __shared__ float2 s_inv;
   __shared__ int s_state;  // 0 factored, 1 a pivot below the bound, 2 not a Gram matrix
   __shared__ float s_min;
+  __shared__ int s_sum;  // bits of a non-negative float
   const int p = blockIdx.x;
   const Dims D = dims[p];
   if (!ce_takes(D, pass, cond)) return;
@@ -413,12 +417,16 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
   float4* Ts = reinterpret_cast<float4*>(ce_raw);
   float4* tmp = SM ? Ts + (size_t)L * (L + 1) / 2 : Ts;  // L
   auto T = [&](int r, int c) -> float4& { return SM ? Ts[cs_at(r, c)] : Tg[(size_t)c * L + r]; };
-  if (tid == 0) s_state = 0;
+  if (tid == 0) {
+    s_state = 0;
+    s_sum = 0;
+  }
   __syncthreads();
   for (int c = tid; c < L; c += CE_THREADS) {
     const double d = G[(size_t)c * L + c].x;
     const int e = (int)(((unsigned long long)__double_as_longlong(d) >> 52) & 0x7FF);
     if (!(d > 0.0) || e == 0 || e == 0x7FF) s_state = 2;
+    if (f32 && abs(e - 1023) > 2 * CE_F32_EXP) s_state = 2;
     s_diag[c] = d;
     s_exp[c] = -((e - 1023) >> 1);
   }
@@ -501,7 +509,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     if (!retry) break;
   }
   const bool fail = s_state != 0 || (shifted && pass + 1 == passes);
-  const bool more = !fail && (shifted || (s_min < again && pass + 1 < passes));
+  const bool more = !fail && (shifted || (!f32 && s_min < again && pass + 1 < passes));
   if (tid == 0) {
     dims[p].cf = fail ? 1 : 0;
     dims[p].cq = more ? pass + 1 : pass;
@@ -551,6 +559,38 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
       }
     }
     __syncthreads();
+  }
+  if (f32) {  // S R^-1 in FP32 (k_trmm_f32)
+    float2* J32 = reinterpret_cast<float2*>(P.J);
+    for (int e = tid; e < L * L; e += CE_THREADS) {
+      const int r = e % L, c = e / L;
+      float2 v = make_float2(0.f, 0.f);
+      if (r <= c) {
+        const float4 t = T(r, c);
+        const float s = __uint_as_float((unsigned)(127 + s_exp[r]) << 23);
+        v = make_float2(t.x * s, t.z * s);
+      }
+      J32[e] = v;
+    }
+    // Column c of the product is rounded to 6e-8 of sum_r |R^-1_rc| (the
+    // pivots say little about it): another pass where that is above `again`,
+    // none left: given up
+    float worst = 0.f;
+    for (int c = tid; c < L; c += CE_THREADS) {
+      float sum = 0.f;
+      for (int r = 0; r <= c; ++r) {
+        const float4 t = T(r, c);
+        sum += fabsf(t.x) + fabsf(t.z);
+      }
+      worst = (sum > worst || sum != sum) ? sum : worst;
+    }
+    if (tid < L) atomicMax(&s_sum, __float_as_int(worst) & 0x7FFFFFFF);
+    __syncthreads();
+    if (tid == 0 && !more && !(__int_as_float(s_sum) <= again)) {
+      if (pass + 1 < passes) dims[p].cq = pass + 1;
+      else dims[p].cf = 1;
+    }
+    return;
   }
   for (int e = tid; e < L * L; e += CE_THREADS) {
     const int r = e % L, c = e / L;
@@ -739,9 +779,9 @@ cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* 
       ProfScope ps("k_chol_inv", st);
       const float mp = pass == 0 ? min_pivot : 0.f, again = lowdin ? CE_AGAIN_LD : CE_AGAIN;
       if (cap.l <= CS_MAXL)
-        k_chol_eq<true><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond);
+        k_chol_eq<true><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
       else
-        k_chol_eq<false><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond);
+        k_chol_eq<false><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
       CQ_TRY(cudaGetLastError());
     }
     CQ_TRY(prod(pass ? q1 : q0, in_pass | DPC_OK));
@@ -759,6 +799,28 @@ cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* 
     CQ_TRY(cudaGetLastError());
   }
   return prod(q1, cond | DPC_OK);
+}
+
+cudaError_t run_cholqr_f32(float2* A, float2* Q, int M, int l, int use_n, bool last, Dims* dims, const ProbPtr* ptrs,
+                           int batch, const OzScratch& oz, int* err, cudaStream_t st) {
+  CQ_TRY(cholqr_prepare());
+  enum { PASSES = 4 };
+  for (int pass = 0; pass < PASSES; ++pass) {
+    const float2* X = pass ? Q : A;
+    const int cond = pass ? (pass << DPC_PASS) | DPC_OK : 0;
+    CQ_TRY(launch_oz_gram_f32(dims, ptrs, X, oz.ad, oz.as, M, l, use_n, batch, cond, err, st));
+    {
+      ProfScope ps("k_chol_inv", st);
+      const float again = last ? CE_F32_LAST : CE_F32_MID;
+      if (l <= CS_MAXL)
+        k_chol_eq<true><<<batch, CE_THREADS, ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
+      else
+        k_chol_eq<false><<<batch, CE_THREADS, ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
+      CQ_TRY(cudaGetLastError());
+    }
+    CQ_TRY(launch_trmm_f32(X, Q, dims, ptrs, M, l, use_n, pass, batch, st));
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_lowdin_j(Dims* dims, const ProbPtr* ptrs, int batch, int l, int cond, cudaStream_t st) {

@@ -2,17 +2,17 @@
 // cores, then the FP64 projection and small SVD of Section IV.
 //
 //   Y0 = A Omega and power rounds 1..q-1  : TF32 tensor-core products (FP32
-//                                           accumulation), FP32 Householder QR
-//                                           (blocked when it fits in shared memory);
+//                                           accumulation), FP32 QR (qr_f32);
 //   power round q (Y0 if q = 0)            : the refinement pass, 3xTF32 split
 //                                           products (FP32-level accuracy);
-//   last QR                                : FP32 blocked Householder and an
-//                                           FP64-accurate re-orthonormalisation
-//                                           (qr_blocked.cu; l <= 512);
-//   B^H = A^H Q, U = Q J_k, V = Qb W_k      : double-float products on the FP32
-//                                           pipes (df_proj.cu for B^H, k_zgemm_df
-//                                           for U and V; ~1e-14 relative);
-//   QR of B^H, Jacobi SVD                   : FP64 (the existing kernels).
+//   last QR                                : FP32, and an FP64-accurate
+//                                           re-orthonormalisation (l <= 512);
+//   B^H = A^H Q, its QR, U = Q J_k, V = Qb W_k : products of exact digit splits
+//                                           on the tensor cores (oz_proj.cu,
+//                                           cholqr.cu), or in double-float;
+//   small SVD                              : FP32 sweeps and digit-split
+//                                           corrections (jacobi_pre.cu), then
+//                                           double-float or FP64 Jacobi.
 //
 // Complex products use the real embedding: A (M x K complex) becomes the
 // M x 2K real matrix of interleaved (Re, Im) entries, and X (K x l complex)
@@ -309,12 +309,14 @@ __device__ __forceinline__ float fwarp_sum(float v) {
   return v;
 }
 
-__global__ void __launch_bounds__(1024) k_qr_f32(float2* Abase, float2* Qbase, int M, int L) {
+__global__ void __launch_bounds__(1024) k_qr_f32(float2* Abase, float2* Qbase, int M, int L,
+                                                 const Dims* __restrict__ dims, int rest) {
   __shared__ float red[32];
   __shared__ float2 vscale;
   __shared__ float vnorm;
   __shared__ float tau[512];
   const int z = blockIdx.x;
+  if (rest && (!dims[z].active || !dims[z].cf)) return;
   float2* A = Abase + (size_t)z * M * L;
   float2* Qo = Qbase + (size_t)z * M * L;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -650,13 +652,22 @@ static cudaError_t tc_product(const void* A0, const void* A1, const void* B0, co
   return cudaGetLastError();
 }
 
+// QR of an FP32 sketch.  At the sizes of oz_stage_rule by the Cholesky QR from
+// digits (chol), then Householder for the instances it gives
+// up; elsewhere, and where the CTA size of the Householder kernels is chosen,
+// by those alone.  Householder on one CTA, or on many CTAs, per instance
+// against the Cholesky QR: 152 x 2000 x 120 4.9 against 2.9 ms, 8 x 2000 x 120
+// 4.1 against 0.7 ms, 15 x 7700 x 262 8 against 6.5 ms.
 static cudaError_t qr_f32(float2* A, float2* Q, int M, int L, int batch, const MixedPtrs& mp, const MixedSizes& s,
-                          const Dims* dims, int use_n, cudaStream_t st, int threads) {
+                          Dims* dims, const ProbPtr* ptrs, int use_n, bool chol, bool last, const OzScratch& oz,
+                          int* err, cudaStream_t st, int threads) {
+  chol = chol && threads == 0;
+  if (chol) MX_TRY(run_cholqr_f32(A, Q, M, L, use_n, last, dims, ptrs, batch, oz, err, st));
   if (!qr_blk_f32_fits(M, L) && mp.qscr && qr_multi_f32_fits(M, L))
-    return launch_qr_multi_f32(A, Q, mp.qscr, s.qs / sizeof(float2), M, L, batch, st, dims, use_n);
+    return launch_qr_multi_f32(A, Q, mp.qscr, s.qs / sizeof(float2), M, L, batch, st, dims, use_n, chol);
   ProfScope ps("k_qr_f32", st);
-  if (qr_blk_f32_fits(M, L)) return launch_qr_blk_f32(A, Q, M, L, batch, st, dims, use_n, threads);
-  k_qr_f32<<<batch, 1024, 0, st>>>(A, Q, M, L);
+  if (qr_blk_f32_fits(M, L)) return launch_qr_blk_f32(A, Q, M, L, batch, st, dims, use_n, threads, chol);
+  k_qr_f32<<<batch, 1024, 0, st>>>(A, Q, M, L, dims, chol);
   return cudaGetLastError();
 }
 
@@ -719,6 +730,14 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   // BF16 products: every one before the refinement round (the last power
   // round; Y0 itself when q = 0, which then stays 3xTF32)
   const bool bf = bf16_form && mp.thf_b && q > 0;
+  // the FP64-accurate products after the projection: tensor cores from digit
+  // splits, or double-float GEMMs on the CUDA cores
+  const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));
+  const OzScratch oz{mp.gad, mp.gas, mp.gbd, mp.gbs};
+  auto qr = [&](float2* A, float2* Q, int M, int use_n, bool last) {
+    return qr_f32(A, Q, M, l, batch, mp, s, const_cast<Dims*>(dims), ptrs, use_n, oz_stage_rule(cap), last, oz, err, st,
+                  kn.qr_threads);
+  };
   {
     ProfScope ps("k_conv_theta", st);
     // padded extents (>= n, >= m) of every copy written
@@ -753,7 +772,7 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   for (int j = 1; j <= q; ++j) {
     const int np = (j == q) ? 3 : 1;
     const bool b16 = bf && np == 1;  // BF16 for the rounds before the refinement round
-    MX_TRY(qr_f32(mp.Yf, mp.Qf, m, l, batch, mp, s, dims, 0, st, kn.qr_threads));    // Y = Q R
+    MX_TRY(qr(mp.Yf, mp.Qf, m, 0, false));  // Y = Q R
     if (b16) {
       MX_TRY(conv_bt_bf16(mp.Qf, dims, mp, m, l, s.K2b, s, batch, st));
       MX_TRY(tc_product(mp.tha_b, nullptr, mp.bt_b, nullptr, n, s.K2b, s, l, 1, mp.Ytf, batch, err, st, kn.tc_half,
@@ -763,7 +782,7 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
       MX_TRY(tc_product(mp.tha_hi, mp.tha_lo, mp.bt_hi, mp.bt_lo, n, s.K2, s, l, np, mp.Ytf, batch, err, st,
                         kn.tc_half));  // A^H Q
     }
-    MX_TRY(qr_f32(mp.Ytf, mp.Qtf, n, l, batch, mp, s, dims, 1, st, kn.qr_threads));  // = Q~ R~
+    MX_TRY(qr(mp.Ytf, mp.Qtf, n, 1, false));  // = Q~ R~
     if (b16) {
       MX_TRY(conv_bt_bf16(mp.Qtf, dims, mp, n, l, s.K1b, s, batch, st));
       MX_TRY(tc_product(mp.thf_b, nullptr, mp.bt_b, nullptr, m, s.K1b, s, l, 1, mp.Yf, batch, err, st, kn.tc_half,
@@ -774,15 +793,11 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
                         kn.tc_half));  // A Q~
     }
   }
-  // last QR: FP32 Householder, then the FP64-accurate re-orthonormalisation.
+  // last QR in FP32, then the FP64-accurate re-orthonormalisation.
   // Plans and handles refuse sketches wider than 512 columns, and l <= m, so
   // every basis they pass fits it.
   if (!reorth_fits(m, l)) return cudaErrorInvalidValue;
-  MX_TRY(qr_f32(mp.Yf, mp.Qf, m, l, batch, mp, s, dims, 0, st, kn.qr_threads));
-  // the FP64-accurate products after the projection: tensor cores from digit
-  // splits, or double-float GEMMs on the CUDA cores
-  const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));
-  const OzScratch oz{mp.gad, mp.gas, mp.gbd, mp.gbs};
+  MX_TRY(qr(mp.Yf, mp.Qf, m, 0, true));
   // digits of Q_f once: the Gram of the re-orthonormalisation and the
   // projection A^H Q_f both take them
   MX_TRY(launch_oz_digits_qf(dims, ptrs, mp.Qf, mp.ad, mp.asc, m, l, batch, st));

@@ -64,9 +64,9 @@ MixedPtrs mixed_carve(char* base, const MixedSizes& s, int batch);
 // D.l columns of the zero-padded M x L layout.
 bool qr_blk_f32_fits(int M, int L);
 // threads: 0 picks the CTA size by batch; 128, 256 or 512 force it (when its
-// shared memory fits)
+// shared memory fits).  rest: only the instances the Cholesky QR gave up (cf)
 cudaError_t launch_qr_blk_f32(float2* A, float2* Q, int M, int L, int batch, cudaStream_t st,
-                              const Dims* dims = nullptr, int use_n = 0, int threads = 0);
+                              const Dims* dims = nullptr, int use_n = 0, int threads = 0, int rest = 0);
 // The same QR spread over many CTAs per instance (qr_multi.cu), for matrices
 // too tall for the blocked kernel's shared memory; scr holds
 // qr_multi_f32_scratch(M, L) float2 per instance at the given stride; with
@@ -74,7 +74,7 @@ cudaError_t launch_qr_blk_f32(float2* A, float2* Q, int M, int L, int batch, cud
 bool qr_multi_f32_fits(int M, int L);
 size_t qr_multi_f32_scratch(int M, int L);
 cudaError_t launch_qr_multi_f32(float2* A, float2* Q, float2* scr, size_t stride, int M, int L, int batch,
-                                cudaStream_t st, const Dims* dims = nullptr, int use_n = 0);
+                                cudaStream_t st, const Dims* dims = nullptr, int use_n = 0, int rest = 0);
 // The correction D of the re-orthonormalisation Q = Q_f (I + D) (FP64
 // orthonormal to ~1e-13, spanning range(Q_f)) from E = Q_f^H Q_f - I already in
 // ptrs[z].R (launch_oz_gram); with fold, Q itself into ptrs[z].Q; usable when
@@ -172,6 +172,18 @@ cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
 enum { CQ_LOWDIN = 1, CQ_PHASES = 2 };
 cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* dims, const ProbPtr* ptrs, int batch,
                        const Caps& cap, const OzScratch& oz, int chunk, int cond, int* err, cudaStream_t st);
+// Cholesky QR of an FP32 sketch A (M x l capacities, m or, with use_n, n rows
+// per instance) into Q (cholqr.cu): Gram matrices from the digits of A, the
+// product in FP32.  last: the basis the FP64 re-orthonormalisation takes.
+// Instances given up have cf set (and A as it was).
+cudaError_t run_cholqr_f32(float2* A, float2* Q, int M, int l, int use_n, bool last, Dims* dims, const ProbPtr* ptrs,
+                           int batch, const OzScratch& oz, int* err, cudaStream_t st);
+// Q = A S R^-1 (S R^-1 in FP32 in ptrs[z].J) of the instances of a pass
+cudaError_t launch_trmm_f32(const float2* src, float2* dst, const Dims* dims, const ProbPtr* ptrs, int Mc, int Lc,
+                            int use_n, int pass, int batch, cudaStream_t st);
+// Gram matrix of an FP32 sketch into ptrs[z].R, its digits in Ad / As
+cudaError_t launch_oz_gram_f32(const Dims* dims, const ProbPtr* ptrs, const float2* X, uint16_t* Ad, int* As, int M,
+                               int l, int use_n, int batch, int cond, int* err, cudaStream_t st);
 // The small SVD X J = W S (X in R) of the problems selected by cond, up to the
 // tolerance of the Jacobi kernels (Dims::js says how far; jacobi_pre.cu), for
 // capacities of jac_pre_rule.  fp64: the FP64 kernels' tolerance, else the

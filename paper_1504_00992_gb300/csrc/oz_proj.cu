@@ -171,7 +171,13 @@ __device__ __forceinline__ double oz_scale(int E) {
 // OZ_THETA, OZ_GATE: the contraction and the gate of bonds whose gate is a
 // GEMM (d_l d_r >= GATE_GEMM_MIN), the mixed forms' counterparts of
 // k_cgemm_df<DgTheta> / <DgGate> (df_gemm.cu documents the operands).
-enum { OZ_PROJ = 100, OZ_GRAM = 101, OZ_THETA = 102, OZ_GATE = 103 };
+// OZ_GRAMY, OZ_GRAMT: Gram matrices of FP32 sketches (m or n rows), as OZ_GRAM
+// but without subtracting the identity.
+enum { OZ_PROJ = 100, OZ_GRAM = 101, OZ_THETA = 102, OZ_GATE = 103, OZ_GRAMY = 104, OZ_GRAMT = 105 };
+template <int ST>
+struct OzFp32Gram {
+  static constexpr bool yes = ST == OZ_GRAM || ST == OZ_GRAMY || ST == OZ_GRAMT;
+};
 static_assert(OZ_THETA == OZ_THETA_STAGE && OZ_GATE == OZ_GATE_STAGE, "stage ids of mixed.cuh");
 
 struct OzOp {
@@ -186,9 +192,9 @@ __device__ __forceinline__ OzOp oz_op(const Dims& D, const ProbPtr& P) {
   if constexpr (ST == OZ_PROJ) {
     o.M = D.l; o.N = D.n; o.K = D.m;
     o.C = P.Yt; o.crs = D.n; o.ccs = 1;  // element (j, i) of the n x l column-major B^H
-  } else if constexpr (ST == OZ_GRAM) {
-    o.M = D.l; o.N = D.l; o.K = D.m;
-    o.C = P.R; o.crs = 1; o.ccs = D.l;  // E = Q_f^H Q_f - I, l x l column-major
+  } else if constexpr (OzFp32Gram<ST>::yes) {
+    o.M = D.l; o.N = D.l; o.K = ST == OZ_GRAMT ? D.n : D.m;
+    o.C = P.R; o.crs = 1; o.ccs = D.l;  // OZ_GRAM: E = Q_f^H Q_f - I; l x l column-major
   } else if constexpr (ST == OZ_THETA) {
     o.M = D.dl * D.cl; o.N = D.dr * D.cr; o.K = D.cm;  // into the pre-gate buffer (oz_store)
     o.C = P.Cpre; o.crs = D.n; o.ccs = 1;
@@ -206,15 +212,15 @@ __device__ __forceinline__ OzOp oz_op(const Dims& D, const ProbPtr& P) {
 template <int ST>
 struct OzConj {
   static constexpr bool own = ST < OZ_PROJ;  // a GemmStage of stages.cuh
-  static constexpr bool A = ST == OZ_PROJ || ST == OZ_GRAM || (own && StageFlags<ST>::conjA);  // Q_f^H
+  static constexpr bool A = ST == OZ_PROJ || OzFp32Gram<ST>::yes || (own && StageFlags<ST>::conjA);  // Q_f^H
   static constexpr bool C = ST == OZ_PROJ || (own && StageFlags<ST>::conjC);
 };
 
 // Digits of each operand and the ring of stages of a product.
 template <int ST>
 struct OzGeo {
-  static constexpr int SA = (ST == OZ_PROJ || ST == OZ_GRAM) ? OZ_SQ : OZ_S;
-  static constexpr int SB = ST == OZ_GRAM ? OZ_SQ : OZ_S;
+  static constexpr int SA = (ST == OZ_PROJ || OzFp32Gram<ST>::yes) ? OZ_SQ : OZ_S;
+  static constexpr int SB = OzFp32Gram<ST>::yes ? OZ_SQ : OZ_S;
   static constexpr uint32_t A_STAGE = 2 * SA * OZ_A_TILE, B_STAGE = 2 * SB * OZ_B_TILE;
   static constexpr int STAGES = SA == OZ_S ? 3 : 4;
   static constexpr size_t smem = 1024 + (size_t)STAGES * (A_STAGE + B_STAGE) + (2 * STAGES + 3) * 8 + 16;
@@ -480,16 +486,19 @@ __global__ void __launch_bounds__(256) k_oz_digits_two(const Dims* __restrict__ 
 // keep all their 24 bits).  Against seven digits the projection loads 47 KB
 // instead of 72 KB per k step and runs 22 digit pairs instead of 28.  The same
 // numbers go to P.Q in FP64, the left operand of U = Q_f (I + D) J_k.
+// ROUND false: the digits alone, of a sketch with m or (use_n) n rows.
+template <bool ROUND>
 __global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ dims,
                                                      const ProbPtr* __restrict__ ptrs, float2* __restrict__ Qf,
-                                                     uint16_t* Ad, int* Es, int mc, int lc, int Kp) {
+                                                     uint16_t* Ad, int* Es, int mc, int lc, int Kp, int use_n,
+                                                     int cond) {
   const int z = blockIdx.y;
   const Dims D = dims[z];
-  if (!D.active) return;
+  if (!D.active || !oz_takes(D, cond)) return;
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= lc) return;
-  const int K = i < D.l ? D.m : 0;
+  const int Mi = use_n ? D.n : D.m, K = i < D.l ? Mi : 0;
   float2* q = Qf + (size_t)z * mc * lc + (size_t)i * mc;
   cplx* Qd = ptrs[z].Q + (size_t)i * D.m;  // (i < D.l where it is written)
   int E = 0;
@@ -503,7 +512,7 @@ __global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ di
   // x = N 2^(E - 1023 - 30), the scale as an FP32 number (a Q_f column has unit norm: E far from its ends)
   const float unit = __uint_as_float((unsigned)max(1, min(254, E - 1023 - 30 + 127)) << 23);
   uint16_t* base = Ad + (size_t)z * 2 * OZ_SQ * lc * Kp;
-  const int kend = min(Kp, ((D.m + OZ_KB - 1) / OZ_KB) * OZ_KB);
+  const int kend = min(Kp, ((Mi + OZ_KB - 1) / OZ_KB) * OZ_KB);
   for (int k = 4 * lane; k < kend; k += 128) {
     int64_t nr[4], ni[4];
 #pragma unroll
@@ -511,7 +520,7 @@ __global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ di
       const float2 v = (k + u < K) ? q[k + u] : make_float2(0.f, 0.f);
       nr[u] = oz_fix31(v.x, E);
       ni[u] = oz_fix31(v.y, E);
-      if (k + u < K) {
+      if (ROUND && k + u < K) {
         const float2 r = make_float2((float)(int)nr[u] * unit, (float)(int)ni[u] * unit);
         q[k + u] = r;
         Qd[k + u] = cmk((double)r.x, (double)r.y);
@@ -865,6 +874,7 @@ cudaError_t oz_prepare() {
   static int done = 0;
   if (!done) {
     const cudaError_t es[] = {
+        oz_attr<OZ_GRAMY>(), oz_attr<OZ_GRAMT>(),
         oz_attr<OZ_PROJ>(), oz_attr<OZ_GRAM>(), oz_attr<OZ_THETA>(), oz_attr<OZ_GATE>(), oz_attr<G_X>(),
         oz_attr<G_U>(),     oz_attr<G_V>(),     oz_attr<G_Y0>(),     oz_attr<G_Y>(),     oz_attr<G_YT>(),
         oz_attr<G_BH>(),    oz_attr<G_PR>(),    oz_attr<G_PQ>(),     oz_attr<G_PD>(),    oz_attr<G_CYG>(),
@@ -916,6 +926,7 @@ OzStageBytes oz_stage_bytes(int m, int n, int k, int l, const Caps* gate) {
   Caps c{};
   c.m = m; c.n = n; c.k = k; c.l = l;
   for (int stage : OZ_STAGE_LIST) oz_grow(b, stage, c);
+  b.ad = std::max(b.ad, oz_digits_q_bytes(l, std::max(m, n)));  // of the FP32 sketches
   if (gate && gate->dl * gate->dr >= GATE_GEMM_MIN) {
     oz_grow(b, OZ_THETA, *gate);
     oz_grow(b, OZ_GATE, *gate);
@@ -1171,7 +1182,7 @@ cudaError_t launch_oz_digits_qf(const Dims* dims, const ProbPtr* ptrs, float2* Q
                                 cudaStream_t st) {
   const int Kp = oz_kpad(m);
   ProfScope ps("k_oz_digits[q]", st);
-  k_oz_digits_q<<<dim3((l + 7) / 8, batch), 256, 0, st>>>(dims, ptrs, Qf, Ad, As, m, l, Kp);
+  k_oz_digits_q<true><<<dim3((l + 7) / 8, batch), 256, 0, st>>>(dims, ptrs, Qf, Ad, As, m, l, Kp, 0, 0);
   return cudaGetLastError();
 }
 
@@ -1193,6 +1204,31 @@ cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t
   oa.cond = 0;
   ProfScope ps("k_oz_gemm[gram]", st);
   return oz_launch<OZ_GRAM>(l, l, batch, dims, ptrs, oa, st);
+}
+
+cudaError_t launch_oz_gram_f32(const Dims* dims, const ProbPtr* ptrs, const float2* X, uint16_t* Ad, int* As, int M,
+                               int l, int use_n, int batch, int cond, int* err, cudaStream_t st) {
+  const cudaError_t e = oz_prepare();
+  if (e != cudaSuccess) return e;
+  const int Kp = oz_kpad(M);
+  {
+    ProfScope ps("k_oz_digits[q]", st);
+    k_oz_digits_q<false><<<dim3((l + 7) / 8, batch), 256, 0, st>>>(dims, ptrs, const_cast<float2*>(X), Ad, As, M, l,
+                                                                   Kp, use_n, cond);
+    const cudaError_t e2 = cudaGetLastError();
+    if (e2 != cudaSuccess) return e2;
+  }
+  OzArgs oa;
+  oa.Ad = oa.Bd = Ad;
+  oa.lc = oa.nc = l;
+  oa.Kp = Kp;
+  oa.As = oa.Bs = As;
+  oa.err = err;
+  oa.poll_limit = 1u << 24;
+  oa.stall = 0;
+  oa.cond = cond;
+  ProfScope ps("k_oz_gemm[gram]", st);
+  return use_n ? oz_launch<OZ_GRAMT>(l, l, batch, dims, ptrs, oa, st) : oz_launch<OZ_GRAMY>(l, l, batch, dims, ptrs, oa, st);
 }
 
 cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const int* As, const uint16_t* Bd, const int* Bs, int m, int n, int l, int batch,

@@ -200,7 +200,7 @@ __device__ void qb_apply(float2* C, int ldc, int M, int j0, int jb, int c0, int 
 // qb_smem_bytes(Mc, Lc) of dynamic shared memory.
 template <int NT>
 __global__ void __launch_bounds__(NT) k_qr_blk_f32(float2* Abase, float2* Qbase, int Mc, int Lc,
-                                                  const Dims* __restrict__ dims, int use_n) {
+                                                  const Dims* __restrict__ dims, int use_n, int rest) {
   constexpr int NW = NT / 32;
   extern __shared__ __align__(16) unsigned char qb_raw[];
   __shared__ float2 vscale;
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(NT) k_qr_blk_f32(float2* Abase, float2* Qbase,
   int M = Mc, L = Lc;  // this instance's rows and columns
   if (dims) {
     const Dims D = dims[z];
-    if (!D.active) return;  // uniform over the block
+    if (!D.active || (rest && !D.cf)) return;  // uniform over the block
     M = use_n ? D.n : D.m;
     L = D.l;
   }
@@ -469,27 +469,27 @@ static size_t g_attr_qr = 0, g_attr_qr256 = 0, g_attr_ld = 0, g_attr_fold[2] = {
 static size_t g_attr_qr128 = 0;
 
 cudaError_t launch_qr_blk_f32(float2* A, float2* Q, int M, int L, int batch, cudaStream_t st, const Dims* dims,
-                              int use_n, int threads) {
+                              int use_n, int threads, int rest) {
   const bool t128 = threads == 128 || (threads == 0 && batch >= 4 * 152);
   const bool t256 = threads == 256 || (threads == 0 && batch >= 2 * 152);
   if (t128 && qb_smem_bytes(M, L, 4) <= 56 * 1024) {
     const size_t sm = qb_smem_bytes(M, L, 4);
     cudaError_t e = ensure_smem(k_qr_blk_f32<128>, sm, &g_attr_qr128);
     if (e != cudaSuccess) return e;
-    k_qr_blk_f32<128><<<batch, 128, sm, st>>>(A, Q, M, L, dims, use_n);
+    k_qr_blk_f32<128><<<batch, 128, sm, st>>>(A, Q, M, L, dims, use_n, rest);
     return cudaGetLastError();
   }
   if ((t128 || t256) && qb_smem_bytes(M, L, 8) <= 112 * 1024) {
     const size_t sm = qb_smem_bytes(M, L, 8);
     cudaError_t e = ensure_smem(k_qr_blk_f32<256>, sm, &g_attr_qr256);
     if (e != cudaSuccess) return e;
-    k_qr_blk_f32<256><<<batch, 256, sm, st>>>(A, Q, M, L, dims, use_n);
+    k_qr_blk_f32<256><<<batch, 256, sm, st>>>(A, Q, M, L, dims, use_n, rest);
     return cudaGetLastError();
   }
   const size_t sm = qb_smem_bytes(M, L);
   cudaError_t e = ensure_smem(k_qr_blk_f32<QB_THREADS>, sm, &g_attr_qr);
   if (e != cudaSuccess) return e;
-  k_qr_blk_f32<QB_THREADS><<<batch, QB_THREADS, sm, st>>>(A, Q, M, L, dims, use_n);
+  k_qr_blk_f32<QB_THREADS><<<batch, QB_THREADS, sm, st>>>(A, Q, M, L, dims, use_n, rest);
   return cudaGetLastError();
 }
 

@@ -191,13 +191,13 @@ struct QmSrc32 {
   size_t stride;  // float2 elements of scratch per instance
   int M, L;
   const Dims* dims;
-  int use_n;
+  int use_n, rest;
   __device__ __forceinline__ bool get(int p, QmView<float2>& v) const {
     v.M = M;
     v.L = L;
     if (dims) {
       const Dims D = dims[p];
-      if (!D.active) return false;
+      if (!D.active || (rest && !D.cf)) return false;
       v.M = use_n ? D.n : D.m;
       v.L = D.l;
     }
@@ -634,10 +634,10 @@ size_t qr_multi_f32_scratch(int M, int L) {
 }
 
 cudaError_t launch_qr_multi_f32(float2* A, float2* Q, float2* scr, size_t stride, int M, int L, int batch,
-                                cudaStream_t st, const Dims* dims, int use_n) {
+                                cudaStream_t st, const Dims* dims, int use_n, int rest) {
   if (stride < qr_multi_f32_scratch(M, L)) return cudaErrorInvalidValue;
   ProfScope ps("k_qr_f32[multi]", st);
-  return qm_run<float2, QmSrc32, true>(QmSrc32{A, Q, scr, stride, M, L, dims, use_n}, batch, M, L, st);
+  return qm_run<float2, QmSrc32, true>(QmSrc32{A, Q, scr, stride, M, L, dims, use_n, rest}, batch, M, L, st);
 }
 
 }  // namespace tg
