@@ -679,7 +679,7 @@ enum { LW_MAXL = 160 };
 static size_t lw_smem_bytes(int l) { return l <= LW_MAXL ? sizeof(float2) * (size_t)l * l : 0; }
 template <bool SVD>
 __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __restrict__ ptrs, int cond,
-                                                  int phases) {
+                                                  int phases, int cap_l) {
   extern __shared__ float2 lw_e[];
   __shared__ float red[16];
   const int p = blockIdx.x;
@@ -689,33 +689,43 @@ __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __r
   const int L = D.l, tid = threadIdx.x;
   const cplx* G = SVD ? P.Y : P.R;
   cplx* T = SVD ? P.Yt : P.J;
+  // SVD: |E|^2 summed (an FP32 J of l = 262 has columns off by 4e-5, whose
+  // bound l max|E| says nothing), else max|E|
   float mx = 0.f;
   for (int e = tid; e < L * L; e += 512) {
     const cplx g = G[e];
-    const double re = (e / L == e % L) ? g.x - 1.0 : g.x;
-    const float m = fmaxf(fabsf((float)re), fabsf((float)g.y));
-    mx = (m > mx || m != m) ? m : mx;  // NaN sticks
+    const float re = (float)((e / L == e % L) ? g.x - 1.0 : g.x), im = (float)g.y;
+    if (SVD) {
+      mx += fmaf(re, re, im * im);
+    } else {
+      const float m = fmaxf(fabsf(re), fabsf(im));
+      mx = (m > mx || m != m) ? m : mx;  // NaN sticks
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float y = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = (y > mx || y != y) ? y : mx;
+    mx = SVD ? mx + y : ((y > mx || y != y) ? y : mx);
   }
   if ((tid & 31) == 0) red[tid >> 5] = mx;
   __syncthreads();
   mx = 0.f;
-  for (int w = 0; w < 16; ++w) mx = (red[w] > mx || red[w] != red[w]) ? red[w] : mx;
-  // (an FP32 J is farther from unitary, and takes a second round)
-  const bool ok = mx * (float)L <= (SVD ? 1e-2f : 3e-6f);
+  for (int w = 0; w < 16; ++w) mx = SVD ? mx + red[w] : ((red[w] > mx || red[w] != red[w]) ? red[w] : mx);
+  // (an FP32 J is farther from unitary, and takes a second round: 0.3 |E|^3
+  // of the first is below 3e-6, of the second below FP64)
+  const bool ok = SVD ? mx <= 4e-4f : mx * (float)L <= 3e-6f;
   if (!ok && tid == 0) {
     if (SVD) dims[p].js = 0;
     else dims[p].cf = 1;
   }
-  // E in FP32, in shared memory where it fits (a conversion is an FP64
+  if (!SVD)
+    for (int c = tid; c < L; c += 512) P.sigma[c] = 1.0;
+  // E in FP32 in shared memory (a conversion is an FP64
   // instruction: made per use they were nearly all of the time, 0.71 ms for
   // 16 instances of l = 120, 0.06 ms made once)
-  const bool square = ok && mx > 1e-9f, staged = L <= LW_MAXL;
-  if (square && staged) {
+  if (cap_l > LW_MAXL) return;  // k_lowdin64_tile does the rest
+  const bool square = ok && mx > (SVD ? 1e-18f : 1e-9f);
+  if (square) {
     for (int e = tid; e < L * L; e += 512) {
       const cplx g = G[e];
       lw_e[e] = make_float2((float)(e % L == e / L ? g.x - 1.0 : g.x), (float)g.y);
@@ -732,14 +742,8 @@ __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __r
         float sx = 0.f, sy = 0.f;
         for (int k = 0; k < L; ++k) {
           float2 u, v;
-          if (staged) {
-            u = lw_e[k * L + a];
-            v = lw_e[b * L + k];
-          } else {
-            const cplx gu = G[(size_t)k * L + a], gv = G[(size_t)b * L + k];
-            u = make_float2((float)(k == a ? gu.x - 1.0 : gu.x), (float)gu.y);
-            v = make_float2((float)(k == b ? gv.x - 1.0 : gv.x), (float)gv.y);
-          }
+          u = lw_e[k * L + a];
+          v = lw_e[b * L + k];
           sx = fmaf(u.x, v.x, fmaf(-u.y, v.y, sx));
           sy = fmaf(u.x, v.y, fmaf(u.y, v.x, sy));
         }
@@ -749,8 +753,71 @@ __global__ void __launch_bounds__(512) k_lowdin64(Dims* dims, const ProbPtr* __r
     }
     T[e] = phases ? cmul(t, P.Jk[b]) : t;
   }
-  if (!SVD)
-    for (int c = tid; c < L; c += 512) P.sigma[c] = 1.0;
+}
+
+// The same J for l above LW_MAXL (k_lowdin64 has checked max|E|), 32 x 32 per
+// CTA: l = 262 on one CTA without the shared copy took 12 ms.
+template <bool SVD>
+__global__ void __launch_bounds__(256) k_lowdin64_tile(const Dims* __restrict__ dims,
+                                                       const ProbPtr* __restrict__ ptrs, int cond, int phases) {
+  __shared__ float2 A[32][33], Bt[32][33];  // E in FP32: [k][a], [b][k]
+  const int p = blockIdx.z;
+  const Dims D = dims[p];
+  const int L = D.l, a0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
+  if (!ce_takes(D, 0, cond) || (SVD ? D.js != 1 : D.cf != 0) || a0 >= L || b0 >= L) return;
+  const ProbPtr P = ptrs[p];
+  const cplx* G = SVD ? P.Y : P.R;
+  cplx* T = SVD ? P.Yt : P.J;
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  auto at = [&](int r, int c) {
+    const cplx g = G[(size_t)c * L + r];
+    return make_float2((float)(r == c ? g.x - 1.0 : g.x), (float)g.y);
+  };
+  float2 acc[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) acc[q] = make_float2(0.f, 0.f);
+  for (int k0 = 0; k0 < L; k0 += 32) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int y = ty + 8 * q;
+      A[y][lane] = (k0 + y < L && a0 + lane < L) ? at(a0 + lane, k0 + y) : make_float2(0.f, 0.f);
+      Bt[y][lane] = (b0 + y < L && k0 + lane < L) ? at(k0 + lane, b0 + y) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < 32; ++k) {
+      const float2 u = A[k][lane];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 v = Bt[ty + 8 * q][k];
+        acc[q].x = fmaf(u.x, v.x, fmaf(-u.y, v.y, acc[q].x));
+        acc[q].y = fmaf(u.x, v.y, fmaf(u.y, v.x, acc[q].y));
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int a = a0 + lane, b = b0 + ty + 8 * q;
+    if (a < L && b < L) {
+      const cplx g = G[(size_t)b * L + a];
+      const cplx t = cmk((a == b ? 1.0 - 0.5 * (g.x - 1.0) : -0.5 * g.x) + 0.375 * (double)acc[q].x,
+                         -0.5 * g.y + 0.375 * (double)acc[q].y);
+      T[(size_t)b * L + a] = phases ? cmul(t, P.Jk[b]) : t;
+    }
+  }
+}
+
+template <bool SVD>
+static cudaError_t launch_lowdin64(Dims* dims, const ProbPtr* ptrs, int batch, int l, int cond, int phases,
+                                   cudaStream_t st) {
+  ProfScope ps("k_lowdin", st);
+  k_lowdin64<SVD><<<batch, 512, lw_smem_bytes(l), st>>>(dims, ptrs, cond, phases, l);
+  if (l > LW_MAXL) {
+    const int nb = (l + 31) / 32;
+    k_lowdin64_tile<SVD><<<dim3(nb, nb, batch), 256, 0, st>>>(dims, ptrs, cond, phases);
+  }
+  return cudaGetLastError();
 }
 
 static cudaError_t lowdin_prepare() {
@@ -793,11 +860,7 @@ cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* 
     CQ_TRY(cudaGetLastError());
   }
   CQ_TRY(prod(g1, cond | DPC_OK));
-  {
-    ProfScope ps("k_lowdin", st);
-    k_lowdin64<false><<<batch, 512, lw_smem_bytes(cap.l), st>>>(dims, ptrs, cond, lowdin == CQ_PHASES);
-    CQ_TRY(cudaGetLastError());
-  }
+  CQ_TRY(launch_lowdin64<false>(dims, ptrs, batch, cap.l, cond, lowdin == CQ_PHASES, st));
   return prod(q1, cond | DPC_OK);
 }
 
@@ -824,13 +887,11 @@ cudaError_t run_cholqr_f32(float2* A, float2* Q, int M, int l, int use_n, bool l
 }
 
 cudaError_t launch_lowdin_j(Dims* dims, const ProbPtr* ptrs, int batch, int l, int cond, cudaStream_t st) {
-  ProfScope ps("k_lowdin", st);
-  k_lowdin64<true><<<batch, 512, lw_smem_bytes(l), st>>>(dims, ptrs, cond, 0);
-  return cudaGetLastError();
+  return launch_lowdin64<true>(dims, ptrs, batch, l, cond, 0, st);
 }
 
 cudaError_t DpPath::svd() const {
-  if (!dp || !jac_pre_rule(cap)) return cudaSuccess;
+  if (!dp || !jac_pre_rule(cap, dp->chunk >= batch)) return cudaSuccess;
   return run_jac_pre(const_cast<Dims*>(dims), ptrs, batch, cap, dp->oz, dp->chunk, DPC_DIG, true, dp->err, st);
 }
 

@@ -816,7 +816,7 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   // Jacobi SVD: double-float one-CTA kernel, after an FP32 one and digit-split
   // corrections, unless another form is chosen
   const int jac = mixed_jac(kn, cap, batch);
-  if (jac == 3 && tc && jac_pre_rule(cap))
+  if ((jac == 3 || (jac == 2 && cap.l > 160)) && tc && jac_pre_rule(cap, true))
     MX_TRY(run_jac_pre(const_cast<Dims*>(dims), ptrs, batch, cap, oz, batch, 0, false, err, st));
   else
     MX_TRY(launch_jac_none(const_cast<Dims*>(dims), batch, st));

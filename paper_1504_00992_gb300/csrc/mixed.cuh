@@ -186,9 +186,9 @@ cudaError_t launch_oz_gram_f32(const Dims* dims, const ProbPtr* ptrs, const floa
                                int l, int use_n, int batch, int cond, int* err, cudaStream_t st);
 // The small SVD X J = W S (X in R) of the problems selected by cond, up to the
 // tolerance of the Jacobi kernels (Dims::js says how far; jacobi_pre.cu), for
-// capacities of jac_pre_rule.  fp64: the FP64 kernels' tolerance, else the
+// capacities of jac_pre_rule (whole: the products' scratch holds the whole batch).  fp64: the FP64 kernels' tolerance, else the
 // double-float one's.
-bool jac_pre_rule(const Caps& cap);
+bool jac_pre_rule(const Caps& cap, bool whole);
 cudaError_t jac_pre_prepare();
 cudaError_t run_jac_pre(Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, const OzScratch& oz, int chunk,
                         int cond, bool fp64, int* err, cudaStream_t st);
