@@ -1132,7 +1132,7 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
     } else if ((e = wave_rrsvd(h, w, dims, ptrs, h->stream)) != cudaSuccess) {
       return e;
     }
-    if ((e = launch_rebuild(dims, ptrs, w.count, h->cutoff, h->wout + w.first, h->status, h->stream)) != cudaSuccess)
+    if ((e = launch_rebuild(dims, ptrs, w.count, w.cap, h->cutoff, h->wout + w.first, h->status, h->stream)) != cudaSuccess)
       return e;
     if ((e = launch_wacc(dims, ptrs, h->wout + w.first, w.count, h->wacc, h->stream)) != cudaSuccess) return e;
   }
@@ -1467,7 +1467,7 @@ extern "C" int tebd_backward(tebd_t h, int site, const double* op, double* dgate
             launch_theta(dims, ptrs, w.count, w.cap, st) != cudaSuccess ||
             launch_gate_gemm(dims, ptrs, w.count, w.cap, st) != cudaSuccess ||
             wave_rrsvd(h, w, dims, ptrs, st) != cudaSuccess ||
-            launch_rebuild(dims, ptrs, w.count, h->cutoff, h->wout + w.first, h->status, st) != cudaSuccess ||
+            launch_rebuild(dims, ptrs, w.count, w.cap, h->cutoff, h->wout + w.first, h->status, st) != cudaSuccess ||
             launch_adj_bond(dims, ptrs, adj, w.count, region, region + rbytes, ck.buf, h->cutoff, 1e-24, 1e-24,
                             st) != cudaSuccess ||
             launch_adj_accum(dims, adj, w.count, st) != cudaSuccess) { rc = TEBD_ECUDA; break; }

@@ -228,8 +228,8 @@ struct ChainDev {
 // (digits: bonds of the sizes of dp_rule get Dims::dig)
 cudaError_t launch_plan(const ProbPtr* ptrs, Dims* dims, int batch, int p, cudaStream_t st, int digits = 0);
 // truncation, renormalisation and Gamma rebuild; w of problem i goes to wout[i]
-cudaError_t launch_rebuild(const Dims* dims, const ProbPtr* ptrs, int batch, double cutoff, double* wout,
-                           int* status, cudaStream_t st);
+cudaError_t launch_rebuild(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, double cutoff,
+                           double* wout, int* status, cudaStream_t st);
 // adds the w of a wave into the per-slot accumulators (2 doubles per chain slot)
 cudaError_t launch_wacc(const Dims* dims, const ProbPtr* ptrs, const double* wout, int batch, double* wacc,
                         cudaStream_t st);

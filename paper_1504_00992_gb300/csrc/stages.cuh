@@ -759,9 +759,12 @@ __device__ __forceinline__ void theta_tile_dev(const Dims& D, const ProbPtr& P, 
 }
 
 // Truncation, renormalisation and Gamma rebuild of one bond by the whole CTA
-// (see k_rebuild); s_rank_p / s_inv_p point at shared scratch.
+// (see k_rebuild), or by `parts` CTAs of which this is `part`: each finds the
+// rank itself and the first one writes what there is once per bond.
+// s_rank_p / s_inv_p point at shared scratch.
 __device__ __forceinline__ void rebuild_dev(const Dims& D, const ProbPtr& P, double cutoff, double* wout_p,
-                                            int* status, int* s_rank_p, double* s_inv_p) {
+                                            int* status, int* s_rank_p, double* s_inv_p, int part = 0,
+                                            int parts = 1) {
   if (threadIdx.x == 0) {
     double nf = 0.0;
     for (int i = 0; i < NPART; ++i) nf += P.part[i];
@@ -776,23 +779,25 @@ __device__ __forceinline__ void rebuild_dev(const Dims& D, const ProbPtr& P, dou
       }
     }
     if (!finite || r == 0 || !isfinite(kept)) {
-      atomicOr(status, 1);
+      if (part == 0) atomicOr(status, 1);
       r = 0;
     }
     (*s_rank_p) = r;
     (*s_inv_p) = (r > 0) ? 1.0 / sqrt(kept) : 0.0;
-    *wout_p = (r > 0 && nf > 0.0) ? 1.0 - kept / nf : 0.0;
+    if (part == 0) *wout_p = (r > 0 && nf > 0.0) ? 1.0 - kept / nf : 0.0;
   }
   __syncthreads();
   const int r = (*s_rank_p);
   if (r == 0) return;
   double* lam = const_cast<double*>(P.lamm);
   const int capm = P.cap_m;
-  for (int i = threadIdx.x; i < capm; i += blockDim.x) lam[i] = (i < r) ? P.sigma[i] * (*s_inv_p) : 0.0;
+  if (part == 0)
+    for (int i = threadIdx.x; i < capm; i += blockDim.x) lam[i] = (i < r) ? P.sigma[i] * (*s_inv_p) : 0.0;
+  const int64_t e0 = (int64_t)part * blockDim.x + threadIdx.x, es = (int64_t)parts * blockDim.x;
   cplx* gl = const_cast<cplx*>(P.gl);
   cplx* gr = const_cast<cplx*>(P.gr);
   const int dl = D.dl, dr = D.dr, cl = D.cl, cr = D.cr, K = D.k;
-  for (int64_t e = threadIdx.x; e < (int64_t)dl * cl * r; e += blockDim.x) {
+  for (int64_t e = e0; e < (int64_t)dl * cl * r; e += es) {
     const int g = (int)(e % r);
     const int row = (int)(e / r);  // i*cl + a
     const int a = row % cl, i = row / cl;
@@ -800,7 +805,7 @@ __device__ __forceinline__ void rebuild_dev(const Dims& D, const ProbPtr& P, dou
     const cplx u = P.U[(int64_t)row * K + g];
     gl[((int64_t)i * P.cap_l + a) * capm + g] = (ll > 0.0) ? cscale(u, 1.0 / ll) : cmk(0.0, 0.0);
   }
-  for (int64_t e = threadIdx.x; e < (int64_t)dr * r * cr; e += blockDim.x) {
+  for (int64_t e = e0; e < (int64_t)dr * r * cr; e += es) {
     const int c = (int)(e % cr);
     const int rest = (int)(e / cr);
     const int g = rest % r, j = rest / r;
@@ -809,7 +814,7 @@ __device__ __forceinline__ void rebuild_dev(const Dims& D, const ProbPtr& P, dou
     gr[((int64_t)j * capm + g) * P.cap_r + c] = (lr > 0.0) ? cscale(v, 1.0 / lr) : cmk(0.0, 0.0);
   }
   __syncthreads();
-  if (threadIdx.x == 0) *P.chi_m = r;
+  if (part == 0 && threadIdx.x == 0) *P.chi_m = r;
 }
 
 }  // namespace tg

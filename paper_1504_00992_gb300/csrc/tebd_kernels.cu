@@ -147,8 +147,10 @@ cudaError_t launch_theta(const Dims* dims, const ProbPtr* ptrs, int batch, const
 //   w = 1 - sum_kept s^2 / ||theta~||_F^2,
 //   Gamma'[b]^i[a][g]   = U[(i*cl + a)][g] / lam_l[a],
 //   Gamma'[b+1]^j[g][c] = Vh[g][(j*cr + c)] / lam_r[c]   (divide only if lam > 0).
-// One CTA per bond.  A zero or non-finite theta~ leaves the bond unchanged
-// and raises status bit 1.
+// A zero or non-finite theta~ leaves the bond unchanged and raises status bit
+// 1.  Memory-bound on many CTAs per bond (one per RB_ELEMS elements of the
+// larger Gamma, four waves of CTAs at most); on one CTA per bond the 15 bonds
+// of a spin-boson wave of local dimension 32 and chi 256 took 7 ms.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_rebuild(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
                                                  double cutoff, double* wout, int* status) {
@@ -157,13 +159,19 @@ __global__ void __launch_bounds__(256) k_rebuild(const Dims* __restrict__ dims, 
   const int p = blockIdx.x;
   const Dims D = dims[p];
   if (!D.active) return;
-  rebuild_dev(D, ptrs[p], cutoff, wout + p, status, &s_rank, &s_inv);
+  rebuild_dev(D, ptrs[p], cutoff, wout + p, status, &s_rank, &s_inv, blockIdx.y, gridDim.y);
 }
 
-cudaError_t launch_rebuild(const Dims* dims, const ProbPtr* ptrs, int batch, double cutoff, double* wout,
-                           int* status, cudaStream_t st) {
+enum { RB_ELEMS = 4096 };
+
+cudaError_t launch_rebuild(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, double cutoff,
+                           double* wout, int* status, cudaStream_t st) {
   ProfScope ps("k_rebuild", st);
-  k_rebuild<<<batch, 256, 0, st>>>(dims, ptrs, cutoff, wout, status);
+  const size_t elems = (size_t)(cap.m > cap.n ? cap.m : cap.n) * cap.k;
+  size_t parts = (elems + RB_ELEMS - 1) / RB_ELEMS;
+  const size_t most = (4 * 152 * 8 + batch - 1) / batch;
+  parts = parts > most ? most : parts;
+  k_rebuild<<<dim3(batch, (unsigned)parts), 256, 0, st>>>(dims, ptrs, cutoff, wout, status);
   return cudaGetLastError();
 }
 
