@@ -1108,10 +1108,16 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
     if (prec_mixed(h->precision)) {
       // bonds of large local dimensions: contraction and gate as GEMMs, on
       // the tensor cores from digit splits or in double-float arithmetic
-      if ((e = launch_theta(dims, ptrs, w.count, w.cap, h->stream, 0, 1)) != cudaSuccess) return e;
+      const bool cont = theta_digits_rule(w.cap.m, w.cap.n, w.cap.cm) && w.mk.dfg != 2;
+      if ((e = launch_theta(dims, ptrs, w.count, w.cap, h->stream, 0, 1, cont ? 2 : 0)) != cudaSuccess) return e;
+      const MixedPtrs mp = mixed_carve(h->mixed, w.ms, w.count);
+      const OzScratch oz{mp.gad, mp.gas, mp.gbd, mp.gbs};
+      if (cont) {
+        if ((e = launch_oz_stage(OZ_CONT_STAGE, dims, ptrs, w.count, w.cap, oz, h->tcerr, h->stream)) != cudaSuccess)
+          return e;
+        if ((e = launch_gate_small(dims, ptrs, w.count, w.cap, 0, h->stream)) != cudaSuccess) return e;
+      }
       if (oz_gate_rule(w.cap) && w.mk.dfg != 2) {
-        const MixedPtrs mp = mixed_carve(h->mixed, w.ms, w.count);
-        const OzScratch oz{mp.gad, mp.gas, mp.gbd, mp.gbs};
         if ((e = launch_oz_stage(OZ_THETA_STAGE, dims, ptrs, w.count, w.cap, oz, h->tcerr, h->stream)) != cudaSuccess)
           return e;
         if ((e = launch_oz_stage(OZ_GATE_STAGE, dims, ptrs, w.count, w.cap, oz, h->tcerr, h->stream)) != cudaSuccess)
@@ -1121,7 +1127,15 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
         if ((e = launch_gate_gemm_df(dims, ptrs, w.count, w.cap, h->stream)) != cudaSuccess) return e;
       }
     } else {
-      if ((e = launch_theta(dims, ptrs, w.count, w.cap, h->stream)) != cudaSuccess) return e;
+      const bool cont = w.dp > 0 && theta_digits_rule(w.cap.m, w.cap.n, w.cap.cm);
+      if ((e = launch_theta(dims, ptrs, w.count, w.cap, h->stream, 0, 0, cont ? 1 : 0)) != cudaSuccess) return e;
+      if (cont) {
+        const DpScratch dp = dp_carve(h->mixed, w.cap, w.count, h->plan.dp_limit, h->tcerr);
+        if ((e = launch_oz_range(OZ_CONT_STAGE, dims, ptrs, w.count, w.cap, dp.oz, dp.chunk, DPC_DIG, h->tcerr,
+                                 h->stream)) != cudaSuccess)
+          return e;
+        if ((e = launch_gate_small(dims, ptrs, w.count, w.cap, 1, h->stream)) != cudaSuccess) return e;
+      }
       if ((e = launch_gate_gemm(dims, ptrs, w.count, w.cap, h->stream)) != cudaSuccess) return e;
     }
     if (prec_mixed(h->precision)) {

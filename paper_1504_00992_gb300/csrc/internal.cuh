@@ -38,6 +38,12 @@ __host__ __device__ inline bool dp_rule(int m, int n, int l) { return l >= 40 &&
 // size (its smaller bonds of dp_rule's sizes then take them too): the ~80
 // launches of a wave cost ~0.2 ms also while the bonds are still small.
 inline bool dp_handle_rule(int m, int n, int l) { return dp_rule(m, n, l) && (long long)m * n >= 192 * 192; }
+// Bonds whose theta is contracted from digit splits (their gate, too small for a
+// GEMM, is then applied in place): FP64 bonds of dp_rule, and in the mixed
+// forms (whose Dims::dig is 0) those of these sizes.  The contraction is
+// d_l d_r chi^3 multiply-adds on the FP64 pipe otherwise; below 128 rows the
+// digits' tiles of 128 x 32 are mostly padding.
+__host__ __device__ inline bool theta_digits_rule(int m, int n, int cm) { return m >= 128 && n >= 128 && cm >= 32; }
 
 struct ProbPtr {
   // operands of the theta contraction (TEBD only)
@@ -164,9 +170,13 @@ cudaError_t launch_frob2(const Dims* dims, const ProbPtr* ptrs, int batch, cudaS
 // identity_gate = 1 writes the pre-gate theta (reverse pass).  Otherwise a
 // bond with ptrs[p].Cpre set gets its pre-gate theta written there, and
 // launch_gate_gemm applies its gate; skip_pre = 1 leaves those bonds to
-// launch_theta_df.
+// launch_theta_df.  skip_dig: the bonds of theta_digits_rule are left out (1: with
+// Dims::dig, 2: any).
 cudaError_t launch_theta(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
-                         int identity_gate = 0, int skip_pre = 0);
+                         int identity_gate = 0, int skip_pre = 0, int skip_dig = 0);
+// the gate of the bonds contracted from digit splits, in place; need_dig: those with Dims::dig
+cudaError_t launch_gate_small(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int need_dig,
+                              cudaStream_t st);
 // theta~ = G C for the bonds with Cpre set (a complex GEMM over the physical
 // indices, FP64): local dimensions with d_l d_r >= GATE_GEMM_MIN take this path.
 enum { GATE_GEMM_MIN = 32 };

@@ -114,7 +114,7 @@ OzStageBytes oz_stage_bytes(int m, int n, int k, int l, const Caps* gate = nullp
 // the contraction and gate GEMMs of a wave on the tensor cores: stages
 // OZ_THETA (into the pre-gate buffers) and OZ_GATE (into theta) of
 // launch_oz_stage; the wave's bonds without a pre-gate buffer are skipped
-enum { OZ_THETA_STAGE = 102, OZ_GATE_STAGE = 103 };
+enum { OZ_THETA_STAGE = 102, OZ_GATE_STAGE = 103, OZ_CONT_STAGE = 106 };
 bool oz_gate_rule(const Caps& cap);
 cudaError_t launch_oz_stage(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
                             const OzScratch& sc, int* err, cudaStream_t st, int cond = 0);

@@ -173,12 +173,14 @@ __device__ __forceinline__ double oz_scale(int E) {
 // k_cgemm_df<DgTheta> / <DgGate> (df_gemm.cu documents the operands).
 // OZ_GRAMY, OZ_GRAMT: Gram matrices of FP32 sketches (m or n rows), as OZ_GRAM
 // but without subtracting the identity.
-enum { OZ_PROJ = 100, OZ_GRAM = 101, OZ_THETA = 102, OZ_GATE = 103, OZ_GRAMY = 104, OZ_GRAMT = 105 };
+enum { OZ_PROJ = 100, OZ_GRAM = 101, OZ_THETA = 102, OZ_GATE = 103, OZ_GRAMY = 104, OZ_GRAMT = 105,
+       OZ_CONT = 106 };  // OZ_THETA for the bonds of theta_digits_rule without a pre-gate buffer, into theta
 template <int ST>
 struct OzFp32Gram {
   static constexpr bool yes = ST == OZ_GRAM || ST == OZ_GRAMY || ST == OZ_GRAMT;
 };
-static_assert(OZ_THETA == OZ_THETA_STAGE && OZ_GATE == OZ_GATE_STAGE, "stage ids of mixed.cuh");
+static_assert(OZ_THETA == OZ_THETA_STAGE && OZ_GATE == OZ_GATE_STAGE && OZ_CONT == OZ_CONT_STAGE,
+              "stage ids of mixed.cuh");
 
 struct OzOp {
   int M, N, K;  // rows and columns of C, depth
@@ -195,9 +197,9 @@ __device__ __forceinline__ OzOp oz_op(const Dims& D, const ProbPtr& P) {
   } else if constexpr (OzFp32Gram<ST>::yes) {
     o.M = D.l; o.N = D.l; o.K = ST == OZ_GRAMT ? D.n : D.m;
     o.C = P.R; o.crs = 1; o.ccs = D.l;  // OZ_GRAM: E = Q_f^H Q_f - I; l x l column-major
-  } else if constexpr (ST == OZ_THETA) {
-    o.M = D.dl * D.cl; o.N = D.dr * D.cr; o.K = D.cm;  // into the pre-gate buffer (oz_store)
-    o.C = P.Cpre; o.crs = D.n; o.ccs = 1;
+  } else if constexpr (ST == OZ_THETA || ST == OZ_CONT) {
+    o.M = D.dl * D.cl; o.N = D.dr * D.cr; o.K = D.cm;  // into the pre-gate buffer or theta (oz_store)
+    o.C = ST == OZ_THETA ? P.Cpre : const_cast<cplx*>(P.theta); o.crs = D.n; o.ccs = 1;
   } else if constexpr (ST == OZ_GATE) {
     o.M = D.dl * D.dr; o.N = D.cl * D.cr; o.K = D.dl * D.dr;  // into theta (oz_store)
     o.C = const_cast<cplx*>(P.theta); o.crs = 0; o.ccs = 0;
@@ -229,7 +231,8 @@ struct OzGeo {
 // The stages that skip a bond: the contraction and gate GEMMs run only for
 // bonds with a pre-gate buffer.
 template <int ST>
-__device__ __forceinline__ bool oz_skip(const ProbPtr& P) {
+__device__ __forceinline__ bool oz_skip(const Dims& D, const ProbPtr& P) {
+  if (ST == OZ_CONT) return P.Cpre != nullptr || !theta_digits_rule(D.m, D.n, D.cm);
   return (ST == OZ_THETA || ST == OZ_GATE) && P.Cpre == nullptr;
 }
 
@@ -248,7 +251,7 @@ __device__ __forceinline__ bool oz_takes(const Dims& D, int cond) {
 template <int ST>
 __device__ __forceinline__ void oz_store(const Dims& D, const ProbPtr& P, const OzOp& op, int i, int j, double re,
                                          double im) {
-  if constexpr (ST == OZ_THETA) {
+  if constexpr (ST == OZ_THETA || ST == OZ_CONT) {
     // lam_l[alpha] lam_r[beta] scale the contraction (rows (i, alpha), columns (j, beta))
     op.C[(int64_t)i * D.n + j] = cscale(cmk(re, im), P.laml[i % D.cl] * P.lamr[j % D.cr]);
   } else if constexpr (ST == OZ_GATE) {
@@ -318,6 +321,10 @@ struct OzSrc<OZ_THETA, SIDE> {  // A = Gamma_l (rows (i, alpha)), B = lam_m Gamm
   }
 };
 template <int SIDE>
+struct OzSrc<OZ_CONT, SIDE> : OzSrc<OZ_THETA, SIDE> {
+  __device__ OzSrc(const Dims& d, const ProbPtr& p) : OzSrc<OZ_THETA, SIDE>(d, p) {}
+};
+template <int SIDE>
 struct OzSrc<OZ_GATE, SIDE> {  // A = the gate (rows (i, j)), B = the (i', j') x (alpha, beta) gather of C
   Dims D;
   const ProbPtr* P;
@@ -345,7 +352,7 @@ __global__ void __launch_bounds__(256) k_oz_max(const Dims* __restrict__ dims, c
   __shared__ int emax[16];
   const int z = blockIdx.z;
   const Dims D = dims[z];
-  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(ptrs[z])) return;
+  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(D, ptrs[z])) return;
   const OzSrc<ST, SIDE> src(D, ptrs[z]);
   const int r0 = blockIdx.x * 16, k0 = blockIdx.y * OZ_MAX_K, k1 = min(src.K, k0 + OZ_MAX_K);
   if (r0 >= src.rows || k0 >= src.K) return;  // uniform over the block
@@ -395,7 +402,7 @@ __device__ __forceinline__ void oz_digits_block(const Dims* __restrict__ dims, c
   auto& emax = sm.emax;
   const int z = blockIdx.z;
   const Dims D = dims[z];
-  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(ptrs[z])) return;
+  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(D, ptrs[z])) return;
   const OzSrc<ST, SIDE> src(D, ptrs[z]);
   const int rows = src.rows, K = src.K;
   const bool rowc = src.rows_contig();
@@ -636,7 +643,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   const int z = blockIdx.z;
   const Dims D = dims[z];
   const int i0 = blockIdx.y * OZ_BM, j0 = blockIdx.x * OZ_BN;
-  if (!D.active || !oz_takes(D, a.cond) || oz_skip<ST>(ptrs[z])) return;
+  if (!D.active || !oz_takes(D, a.cond) || oz_skip<ST>(D, ptrs[z])) return;
   const OzOp op = oz_op<ST>(D, ptrs[z]);
   if (i0 >= op.M || j0 >= op.N) return;  // uniform: before any barrier or allocation
   uint8_t* smem = (uint8_t*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
@@ -874,7 +881,7 @@ cudaError_t oz_prepare() {
   static int done = 0;
   if (!done) {
     const cudaError_t es[] = {
-        oz_attr<OZ_GRAMY>(), oz_attr<OZ_GRAMT>(),
+        oz_attr<OZ_CONT>(), oz_attr<OZ_GRAMY>(), oz_attr<OZ_GRAMT>(),
         oz_attr<OZ_PROJ>(), oz_attr<OZ_GRAM>(), oz_attr<OZ_THETA>(), oz_attr<OZ_GATE>(), oz_attr<G_X>(),
         oz_attr<G_U>(),     oz_attr<G_V>(),     oz_attr<G_Y0>(),     oz_attr<G_Y>(),     oz_attr<G_YT>(),
         oz_attr<G_BH>(),    oz_attr<G_PR>(),    oz_attr<G_PQ>(),     oz_attr<G_PD>(),    oz_attr<G_CYG>(),
@@ -902,7 +909,7 @@ static void oz_stage_caps(int stage, const Caps& c, int& Mc, int& Nc, int& Kc) {
     case G_CTQ: case G_CRQ: Mc = c.n; Nc = c.l; Kc = c.l; break;
     case G_JG: case G_JT: case G_XJ: case G_XG: case G_XT: Mc = c.l; Nc = c.l; Kc = c.l; break;
     case G_U: Mc = c.m; Nc = c.k; Kc = c.l; break;
-    case OZ_THETA: Mc = c.m; Nc = c.n; Kc = c.cm; break;  // K = chi_m, at most its bond's capacity
+    case OZ_THETA: case OZ_CONT: Mc = c.m; Nc = c.n; Kc = c.cm; break;  // K = chi_m, at most its bond's capacity
     case OZ_GATE: Mc = c.dl * c.dr; Nc = c.cl * c.cr; Kc = c.dl * c.dr; break;
     default: Mc = c.n; Nc = c.k; Kc = c.l; break;  // G_V
   }
@@ -927,6 +934,7 @@ OzStageBytes oz_stage_bytes(int m, int n, int k, int l, const Caps* gate) {
   c.m = m; c.n = n; c.k = k; c.l = l;
   for (int stage : OZ_STAGE_LIST) oz_grow(b, stage, c);
   b.ad = std::max(b.ad, oz_digits_q_bytes(l, std::max(m, n)));  // of the FP32 sketches
+  if (gate && theta_digits_rule(gate->m, gate->n, gate->cm)) oz_grow(b, OZ_CONT, *gate);
   if (gate && gate->dl * gate->dr >= GATE_GEMM_MIN) {
     oz_grow(b, OZ_THETA, *gate);
     oz_grow(b, OZ_GATE, *gate);
@@ -992,7 +1000,7 @@ static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch
   oa.stall = 0;
   oa.cond = cond;
   ProfScope ps(ST == G_U || ST == G_V ? "k_oz_gemm[uv]"
-               : ST == OZ_THETA          ? "k_oz_gemm[theta]"
+               : ST == OZ_THETA || ST == OZ_CONT ? "k_oz_gemm[theta]"
                : ST == OZ_GATE           ? "k_oz_gemm[gate]"
                : ST >= G_JG && ST <= G_XT ? "k_oz_gemm[svd]"
                : ST <= G_BH || (ST >= G_PR && ST <= G_PD) ? "k_oz_gemm[sketch]"
@@ -1015,6 +1023,7 @@ cudaError_t launch_oz_stage(int stage, const Dims* dims, const ProbPtr* ptrs, in
       if (!oz_gate_rule(cap)) return cudaSuccess;
       return stage == OZ_THETA ? oz_stage_run<OZ_THETA>(dims, ptrs, batch, Mc, Nc, Kc, sc, cond, err, st)
                                : oz_stage_run<OZ_GATE>(dims, ptrs, batch, Mc, Nc, Kc, sc, cond, err, st);
+    OZ_CASE(OZ_CONT);
     OZ_CASE(G_X);
     OZ_CASE(G_U);
     OZ_CASE(G_V);
@@ -1068,6 +1077,11 @@ static DpLayout dp_layout(const Caps& c) {
   d.as = oz_scales_bytes(std::max(mx, c.l));
   d.bd = std::max(oz_digits_bytes(w, mx), oz_digits_bytes(w, c.l));
   d.bs = oz_scales_bytes(w);
+  if (theta_digits_rule(c.m, c.n, c.cm)) {  // a handle's contraction
+    d.ad = std::max(d.ad, oz_digits_bytes(c.m, c.cm));
+    d.bd = std::max(d.bd, oz_digits_bytes(c.n, c.cm));
+    d.bs = std::max(d.bs, oz_scales_bytes(c.n));
+  }
   return d;
 }
 

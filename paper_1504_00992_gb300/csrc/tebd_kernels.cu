@@ -37,14 +37,71 @@ cudaError_t launch_plan(const ProbPtr* ptrs, Dims* dims, int batch, int p, cudaS
 // the contraction.  Tile: dl*TA <= 32 rows (TA >= 1), dr*TB <= 32 columns.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_theta(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
-                                               int identity_gate, int skip_pre) {
+                                               int identity_gate, int skip_pre, int skip_dig) {
   extern __shared__ cplx th_sm[];
   const int p = blockIdx.z;
   const Dims D = dims[p];
   if (!D.active) return;
   const ProbPtr P = ptrs[p];
   if (skip_pre && !identity_gate && P.Cpre) return;  // contracted by launch_theta_df
+  if (skip_dig && !P.Cpre && (D.dig || skip_dig == 2) && theta_digits_rule(D.m, D.n, D.cm)) return;  // k_gate_small's
   theta_tile_dev(D, P, blockIdx.y, blockIdx.x, identity_gate, th_sm);
+}
+
+// theta <- gate applied to the contraction in theta, in place, for the bonds
+// k_theta leaves to the digit-split contraction: a thread takes the d_l d_r
+// entries (i, j) of one (alpha, beta), which no other thread touches, through
+// shared memory.  Bound by the FP64
+// pipe, (d_l d_r)^2 complex multiply-adds per (alpha, beta): 12 chains' bonds
+// of chi up to 128, contraction and gate: 8.3 ms on the FP64 pipe alone, 2.1 ms
+// with this and the digits (0.6 the contraction, 1.1 both kernels' rest).
+enum { GS_T = 128 };
+
+__global__ void __launch_bounds__(GS_T) k_gate_small(const Dims* __restrict__ dims,
+                                                     const ProbPtr* __restrict__ ptrs, int need_dig) {
+  extern __shared__ cplx gs_sm[];  // [dd][GS_T], then the gate
+  const int p = blockIdx.y;
+  const Dims D = dims[p];
+  if (!D.active || (need_dig && !D.dig) || !theta_digits_rule(D.m, D.n, D.cm)) return;
+  const ProbPtr P = ptrs[p];
+  if (P.Cpre) return;
+  const int dl = D.dl, dr = D.dr, cl = D.cl, cr = D.cr, dd = dl * dr, tid = threadIdx.x;
+  cplx* g = gs_sm + (size_t)dd * GS_T;
+  for (int e = tid; e < dd * dd; e += GS_T) g[e] = P.gate[e];
+  __syncthreads();
+  const int64_t n = (int64_t)cl * cr;
+  cplx* th = const_cast<cplx*>(P.theta);
+  for (int64_t e = (int64_t)blockIdx.x * GS_T + tid; e < n; e += (int64_t)gridDim.x * GS_T) {
+    const int al = (int)(e / cr), be = (int)(e % cr);
+    cplx* t0 = th + (int64_t)al * D.n + be;
+    for (int k = 0; k < dd; ++k) gs_sm[k * GS_T + tid] = t0[(int64_t)(k / dr) * cl * D.n + (k % dr) * cr];
+    for (int r = 0; r < dd; ++r) {
+      cplx v = cmk(0.0, 0.0);
+      for (int k = 0; k < dd; ++k) cfma(v, g[r * dd + k], gs_sm[k * GS_T + tid]);
+      t0[(int64_t)(r / dr) * cl * D.n + (r % dr) * cr] = v;
+    }
+  }
+}
+
+static size_t gs_smem(int dd) { return sizeof(cplx) * ((size_t)dd * GS_T + (size_t)dd * dd); }
+
+cudaError_t launch_gate_small(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int need_dig,
+                              cudaStream_t st) {
+  // (cap.dl cap.dr may come from different bonds; those of GATE_GEMM_MIN and more have their own path)
+  const int dd = cap.dl * cap.dr < GATE_GEMM_MIN ? cap.dl * cap.dr : GATE_GEMM_MIN - 1;
+  static bool attr_set = false;
+  if (!attr_set) {
+    const cudaError_t e = cudaFuncSetAttribute(k_gate_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)gs_smem(GATE_GEMM_MIN - 1));
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  ProfScope ps("k_theta", st);
+  size_t gx = ((size_t)cap.cl * cap.cr + GS_T - 1) / GS_T;
+  const size_t most = (8 * 152 * 8 + batch - 1) / batch;
+  gx = gx > most ? most : gx;
+  k_gate_small<<<dim3((unsigned)gx, batch), GS_T, gs_smem(dd), st>>>(dims, ptrs, need_dig);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -126,7 +183,7 @@ cudaError_t launch_gate_gemm(const Dims* dims, const ProbPtr* ptrs, int batch, c
 }
 
 cudaError_t launch_theta(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
-                         int identity_gate, int skip_pre) {
+                         int identity_gate, int skip_pre, int skip_dig) {
   const int TA = (cap.dl >= 32) ? 1 : 32 / cap.dl;
   const int TB = (cap.dr >= 32) ? 1 : 32 / cap.dr;
   dim3 grid((cap.cr + TB - 1) / TB, (cap.cl + TA - 1) / TA, batch);
@@ -137,7 +194,7 @@ cudaError_t launch_theta(const Dims* dims, const ProbPtr* ptrs, int batch, const
     attr_set = true;
   }
   ProfScope ps("k_theta", st);
-  k_theta<<<grid, 256, smem, st>>>(dims, ptrs, identity_gate, skip_pre);
+  k_theta<<<grid, 256, smem, st>>>(dims, ptrs, identity_gate, skip_pre, skip_dig);
   return cudaGetLastError();
 }
 
