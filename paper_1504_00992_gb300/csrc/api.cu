@@ -218,6 +218,8 @@ struct tebd_s {
   double* one_lam = nullptr;
   bool use_graph = false;
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  // pinned host memory (and its device address) of the queries' answers: three ints, then doubles from offset 16
+  char *rep = nullptr, *rep_dev = nullptr;
   cudaStream_t own_stream = nullptr;  // used for graphs when the caller gives the legacy stream 0
   // reverse pass: checkpoints of the chain's state before every recorded sweep
   bool recording = false;
@@ -242,11 +244,31 @@ static void free_ckpts(tebd_s* h) {
   h->ckpts.clear();
 }
 
-static int tebd_check_status(tebd_t h) {
-  int st = 0, te = 0;
-  CU_OR(h, cudaMemcpyAsync(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  if (h->tcerr) CU_OR(h, cudaMemcpyAsync(&te, h->tcerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+// Pinned memory for the answers of every chain's queries.
+static bool report_alloc(tebd_s* h) {
+  size_t n = 2;
+  for (const ChainH& C : h->ch) {
+    n = std::max(n, (size_t)C.N);
+    for (int c : C.cap_ext) n = std::max(n, (size_t)c);
+  }
+  if (cudaHostAlloc((void**)&h->rep, 16 + sizeof(double) * n, cudaHostAllocMapped) == cudaSuccess &&
+      cudaHostGetDevicePointer((void**)&h->rep_dev, h->rep, 0) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
+// Waits for the handle's work and returns its error state; src: n doubles into
+// out first, and chi into *chi_out.
+static int tebd_check_status(tebd_t h, const double* src = nullptr, int n = 0, double* out = nullptr,
+                             const int* chi = nullptr, int* chi_out = nullptr) {
+  CU_OR(h, launch_report(h->status, h->tcerr, src, n, chi, (int*)h->rep_dev, (double*)(h->rep_dev + 16), h->stream));
   CU_OR(h, cudaStreamSynchronize(h->stream));
+  int head[3];
+  memcpy(head, h->rep, sizeof head);
+  if (n) memcpy(out, h->rep + 16, sizeof(double) * n);
+  if (chi) *chi_out = head[2];
+  const int st = head[0], te = head[1];
   if (te) h->err.set(TEBD_ETIMEOUT, "a tensor-core pipeline wait timed out");
   else if (st & 4)
     h->err.set(TEBD_ENUMERIC, "the re-orthonormalisation of an FP32 basis met a non-finite or far from orthonormal "
@@ -265,6 +287,7 @@ static void tebd_free(tebd_s* h) {
     if (h->gexec[i]) cudaGraphExecDestroy(h->gexec[i]);
   h->alloc.put(h->arena);
   if (h->own_stream) cudaStreamDestroy(h->own_stream);
+  if (h->rep) cudaFreeHost(h->rep);
   delete h;
 }
 
@@ -741,12 +764,17 @@ extern "C" int tebd_create_multi(int n_chains, const tebd_desc_t* descs, tebd_t*
     }
     h->arena = (char*)blk;
   }
+  if (!report_alloc(h)) { tebd_free(h); return TEBD_ENOMEM; }
   if (cudaMemset(h->arena, 0, h->plan.ws_off) != cudaSuccess) { tebd_free(h); return TEBD_ECUDA; }
-  if (prec_mixed(h->precision))
+  if (prec_mixed(h->precision)) {
     for (int par = 0; par < 2; ++par)
       for (const Wave& w : h->par[par].waves)
         if (mixed_prepare(w.cap) != cudaSuccess) { cudaGetLastError(); tebd_free(h); return TEBD_ECUDA; }
-  else if (oz_prepare() != cudaSuccess || cholqr_prepare() != cudaSuccess) { cudaGetLastError(); tebd_free(h); return TEBD_ECUDA; }
+  } else if (oz_prepare() != cudaSuccess || cholqr_prepare() != cudaSuccess) {
+    cudaGetLastError();
+    tebd_free(h);
+    return TEBD_ECUDA;
+  }
   if (fused_prepare() != cudaSuccess) { cudaGetLastError(); tebd_free(h); return TEBD_ECUDA; }
   if (!bind_arena(h)) { tebd_free(h); return TEBD_ECUDA; }
   // every chain starts in |0...0>
@@ -1213,8 +1241,7 @@ extern "C" int tebd_expect(tebd_t h, int site, const double* op, double* out) {
   CU_OR(h, cudaMemcpyAsync(h->op_dev, op, sizeof(cplx) * d * d, cudaMemcpyHostToDevice, h->stream));
   CU_OR(h, launch_expect(C.dev, site, (int64_t)C.cap_ext[site] * C.cap_ext[site + 1], h->op_dev, d,
                          h->out_dev + 1, h->out_dev, h->stream));
-  CU_OR(h, cudaMemcpyAsync(out, h->out_dev, sizeof(cplx), cudaMemcpyDeviceToHost, h->stream));
-  return tebd_check_status(h);
+  return tebd_check_status(h, (const double*)h->out_dev, 2, out);
 }
 
 extern "C" int tebd_get_lambda(tebd_t h, int bond, double* out, int* chi) {
@@ -1223,10 +1250,7 @@ extern "C" int tebd_get_lambda(tebd_t h, int bond, double* out, int* chi) {
   ChainH& C = h->ch[h->cur];
   if (bond < 0 || bond >= C.N - 1 || !out) { h->err.set(TEBD_EINVAL, "bad bond or NULL pointer"); return h->err.code; }
   int c = 0;
-  CU_OR(h, cudaMemcpyAsync(&c, C.chi_ext + bond + 1, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CU_OR(h, cudaMemcpyAsync(out, C.lam_ptr[bond + 1], sizeof(double) * C.cap_ext[bond + 1], cudaMemcpyDeviceToHost,
-                           h->stream));
-  if (tebd_check_status(h)) return h->err.code;
+  if (tebd_check_status(h, C.lam_ptr[bond + 1], C.cap_ext[bond + 1], out, C.chi_ext + bond + 1, &c)) return h->err.code;
   if (chi) *chi = c;
   return TEBD_OK;
 }
@@ -1235,8 +1259,7 @@ extern "C" int tebd_discarded_weight(tebd_t h, double* out) {
   if (!h) return TEBD_EINVAL;
   if (h->err.code) return h->err.code;
   if (!out) { h->err.set(TEBD_EINVAL, "NULL pointer"); return h->err.code; }
-  CU_OR(h, cudaMemcpyAsync(out, h->wacc + 2 * h->cur, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  return tebd_check_status(h);
+  return tebd_check_status(h, h->wacc + 2 * h->cur, 2, out);
 }
 
 extern "C" int tebd_sweep_count(tebd_t h, int64_t* out) {
@@ -1261,8 +1284,7 @@ extern "C" int tebd_bond_weights(tebd_t h, double* out) {
   if (h->err.code) return h->err.code;
   if (!out) { h->err.set(TEBD_EINVAL, "NULL pointer"); return h->err.code; }
   const ChainH& C = h->ch[h->cur];
-  CU_OR(h, cudaMemcpyAsync(out, C.wbond, sizeof(double) * (C.N - 1), cudaMemcpyDeviceToHost, h->stream));
-  return tebd_check_status(h);
+  return tebd_check_status(h, C.wbond, C.N - 1, out);
 }
 
 extern "C" int tebd_wave_info(tebd_t h, int parity, int wave, int* info, double* ms) {

@@ -373,7 +373,9 @@ static const float CE_SHIFT = 2.9103830456733704e-11f;  // 2^-35
 static const float CE_AGAIN = 1.4901161193847656e-08f;  // 2^-26: below it another pass, where one is left
 static const float CE_AGAIN_LD = 6.103515625e-05f;      // 2^-14: the same before the symmetric correction
 
-enum { CE_THREADS = 512, CE_MAXL = 512 };
+// (k_chol_eq: twice the warps from CE_WIDE columns on, whose updates have work for them)
+enum { CE_THREADS = 512, CE_THREADS_BIG = 1024, CE_WIDE = 64, CE_MAXL = 512 };
+static int ce_threads(int l) { return l > CE_WIDE ? CE_THREADS_BIG : CE_THREADS; }
 static const float CE_F32_LAST = 16.f, CE_F32_MID = 1e4f;  // bounds of the FP32 form's R^-1 column sums
 enum { CE_F32_EXP = 96 };  // column norms 2^+-96 leave S R^-1 inside FP32's range
 
@@ -396,7 +398,7 @@ __device__ __forceinline__ bool ce_takes(const Dims& D, int pass, int cond) {
 // shared memory (SM), or in place in P.R's upper half (the lower half keeps G
 // for a second attempt with the shift).
 template <bool SM>
-__global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass,
+__global__ void __launch_bounds__(CE_THREADS_BIG) k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass,
                                                         int passes, float min_pivot, float again, int cond,
                                                         int f32) {
   extern __shared__ __align__(16) unsigned char ce_raw[];
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
   const Dims D = dims[p];
   if (!ce_takes(D, pass, cond)) return;
   const ProbPtr P = ptrs[p];
-  const int L = D.l, tid = threadIdx.x;
+  const int L = D.l, tid = threadIdx.x, nt = blockDim.x;
   cplx* G = P.R;
   cplx* J = P.J;
   float4* Tg = reinterpret_cast<float4*>(P.R);
@@ -422,7 +424,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     s_sum = 0;
   }
   __syncthreads();
-  for (int c = tid; c < L; c += CE_THREADS) {
+  for (int c = tid; c < L; c += nt) {
     const double d = G[(size_t)c * L + c].x;
     const int e = (int)(((unsigned long long)__double_as_longlong(d) >> 52) & 0x7FF);
     if (!(d > 0.0) || e == 0 || e == 0x7FF) s_state = 2;
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
   bool shifted = false;
   for (int attempt = 0; s_state != 2 && attempt < 2; ++attempt) {
     shifted = attempt == 1;
-    for (int e = tid; e < L * L; e += CE_THREADS) {
+    for (int e = tid; e < L * L; e += nt) {
       const int r = e % L, c = e / L;
       if (r > c) continue;
       const int k = s_exp[r] + s_exp[c];
@@ -479,14 +481,14 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
       __syncthreads();
       if (s_state) break;
       const dfl inv{s_inv.x, s_inv.y};
-      for (int c = j + 1 + tid; c < L; c += CE_THREADS) {
+      for (int c = j + 1 + tid; c < L; c += nt) {
         const float4 v = T(j, c);
         const dfl re = dmul(dfl{v.x, v.y}, inv), im = dmul(dfl{v.z, v.w}, inv);
         T(j, c) = make_float4(re.h, re.l, im.h, im.l);
       }
       __syncthreads();
       const int w = L - j - 1, j1 = j + 1;
-      for (int e = tid; e < w * (w + 1) / 2; e += CE_THREADS) {
+      for (int e = tid; e < w * (w + 1) / 2; e += nt) {
         int a, b;
         cs_pair(e, a, b);
         const int c1 = j1 + a, c2 = j1 + b;
@@ -515,15 +517,15 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     dims[p].cq = more ? pass + 1 : pass;
   }
   if (fail) {  // an identity factor: the products in between stay finite
-    for (int e = tid; e < L * L; e += CE_THREADS) J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
-    for (int c = tid; c < L; c += CE_THREADS) P.sigma[c] = 1.0;
+    for (int e = tid; e < L * L; e += nt) J[e] = cmk((e / L) == (e % L) ? 1.0 : 0.0, 0.0);
+    for (int c = tid; c < L; c += nt) P.sigma[c] = 1.0;
     return;
   }
   // R^-1 in place, column by column: X[0:j, j] = -X[j][j] X[0:j, 0:j] R[0:j, j].
   // Four lanes per row: the dot products of a column are up to j long.
   const int quad = tid >> 2, ql = tid & 3;
   for (int j = 0; j < L; ++j) {
-    for (int r0 = 0; r0 < j; r0 += CE_THREADS / 4) {
+    for (int r0 = 0; r0 < j; r0 += nt / 4) {
       const int r = r0 + quad;
       float sh = 0.f, sl = 0.f, th = 0.f, tl = 0.f;
       if (r < j)
@@ -549,7 +551,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     const float4 djj = T(j, j);
     const dfl dj = drecip(dfl{djj.x, djj.y});
     __syncthreads();
-    for (int r = tid; r <= j; r += CE_THREADS) {
+    for (int r = tid; r <= j; r += nt) {
       if (r == j) {
         T(j, j) = make_float4(dj.h, dj.l, 0.f, 0.f);
       } else {
@@ -562,7 +564,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
   }
   if (f32) {  // S R^-1 in FP32 (k_trmm_f32)
     float2* J32 = reinterpret_cast<float2*>(P.J);
-    for (int e = tid; e < L * L; e += CE_THREADS) {
+    for (int e = tid; e < L * L; e += nt) {
       const int r = e % L, c = e / L;
       float2 v = make_float2(0.f, 0.f);
       if (r <= c) {
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     // pivots say little about it): another pass where that is above `again`,
     // none left: given up
     float worst = 0.f;
-    for (int c = tid; c < L; c += CE_THREADS) {
+    for (int c = tid; c < L; c += nt) {
       float sum = 0.f;
       for (int r = 0; r <= c; ++r) {
         const float4 t = T(r, c);
@@ -592,7 +594,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     }
     return;
   }
-  for (int e = tid; e < L * L; e += CE_THREADS) {
+  for (int e = tid; e < L * L; e += nt) {
     const int r = e % L, c = e / L;
     cplx v = cmk(0.0, 0.0);
     if (r <= c) {
@@ -601,7 +603,7 @@ __global__ void __launch_bounds__(CE_THREADS) k_chol_eq(Dims* dims, const ProbPt
     }
     J[e] = v;
   }
-  for (int c = tid; c < L; c += CE_THREADS) P.sigma[c] = ce_scale(1.0, s_exp[c]);
+  for (int c = tid; c < L; c += nt) P.sigma[c] = ce_scale(1.0, s_exp[c]);
 }
 
 // Column phases of the Householder QR.  The Cholesky QR has a positive
@@ -846,9 +848,9 @@ cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* 
       ProfScope ps("k_chol_inv", st);
       const float mp = pass == 0 ? min_pivot : 0.f, again = lowdin ? CE_AGAIN_LD : CE_AGAIN;
       if (cap.l <= CS_MAXL)
-        k_chol_eq<true><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
+        k_chol_eq<true><<<batch, ce_threads(cap.l), ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
       else
-        k_chol_eq<false><<<batch, CE_THREADS, ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
+        k_chol_eq<false><<<batch, ce_threads(cap.l), ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
       CQ_TRY(cudaGetLastError());
     }
     CQ_TRY(prod(pass ? q1 : q0, in_pass | DPC_OK));
@@ -876,9 +878,9 @@ cudaError_t run_cholqr_f32(float2* A, float2* Q, int M, int l, int use_n, bool l
       ProfScope ps("k_chol_inv", st);
       const float again = last ? CE_F32_LAST : CE_F32_MID;
       if (l <= CS_MAXL)
-        k_chol_eq<true><<<batch, CE_THREADS, ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
+        k_chol_eq<true><<<batch, ce_threads(l), ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
       else
-        k_chol_eq<false><<<batch, CE_THREADS, ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
+        k_chol_eq<false><<<batch, ce_threads(l), ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
       CQ_TRY(cudaGetLastError());
     }
     CQ_TRY(launch_trmm_f32(X, Q, dims, ptrs, M, l, use_n, pass, batch, st));

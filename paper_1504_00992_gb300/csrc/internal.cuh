@@ -246,6 +246,8 @@ cudaError_t launch_wacc(const Dims* dims, const ProbPtr* ptrs, const double* wou
 cudaError_t launch_sweep_tick(uint64_t* sweep_dev, cudaStream_t st);
 // elems: the capacity of the site's bond pair; part: scratch of EX_PARTS numbers
 enum { EX_PARTS = 304 };
+cudaError_t launch_report(const int* status, const int* tcerr, const double* src, int n, const int* chi, int* head,
+                          double* out, cudaStream_t st);
 cudaError_t launch_expect(const ChainDev& ch, int site, int64_t elems, const cplx* op, int d, cplx* part, cplx* out,
                           cudaStream_t st);
 
