@@ -27,15 +27,9 @@ namespace tg {
 enum { JC_CL = 8, JC_THREADS = 256, JC_G = 8, JC_U = 4, JC_MAXSWEEPS = 60, JC_MAXL = 512 };
 enum { JC_MIN_L = 64, JC_MAX_BATCH = 40, JC_SMALL_L = 24, JC_SMALL_BATCH = 19 };
 
-__device__ __forceinline__ double jc_grp_sum(double v, unsigned mask) {
-#pragma unroll
-  for (int o = JC_G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-  return v;
-}
-
 // x_a' = c x_a - s e* x_b, x_b' = s e x_a + c x_b on the rows of this lane,
 // JC_U rows loaded before any is written
-__device__ __forceinline__ void jc_rotate(cplx* xa, cplx* xb, int L, int gl, double c, cplx se, cplx sec) {
+__device__ __forceinline__ void jc_rotate(cplx* xa, cplx* xb, int L, int gl, double c, cplx se) {
   for (int r0 = gl; r0 < L; r0 += JC_G * JC_U) {
     cplx u[JC_U], v[JC_U];
 #pragma unroll
@@ -47,14 +41,12 @@ __device__ __forceinline__ void jc_rotate(cplx* xa, cplx* xb, int L, int gl, dou
 #pragma unroll
     for (int q = 0; q < JC_U; ++q) {
       const int r = r0 + q * JC_G;
-      if (r < L) {
-        xa[r] = csub(cscale(u[q], c), cmul(sec, v[q]));
-        xb[r] = cadd(cmul(se, u[q]), cscale(v[q], c));
-      }
+      if (r < L) jac_rotate(c, se, u[q], v[q], xa[r], xb[r]);
     }
   }
 }
 
+template <int R>
 __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
     k_jacobi_cl(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs, int* status) {
   __shared__ double sv[JC_MAXL];
@@ -102,7 +94,7 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
     if (tid == 0) rotated = 0;
     cluster.sync();  // norms and J visible to the cluster
     for (int rnd = 0; rnd < Lp - 1; ++rnd) {
-      for (int pi = grp; pi < Lp / 2; pi += ngrp_all) {
+      for (int pi = R ? gwarp : grp; pi < Lp / 2; pi += R ? nw_all : ngrp_all) {
         int a, b;
         if (pi == 0) {
           a = Lp - 1;
@@ -116,12 +108,54 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
           a = b;
           b = t;
         }
-        if (b >= L) continue;  // uniform over the group
+        if (b >= L) continue;  // uniform over the group or warp
         cplx* xa = X + (int64_t)a * L;
         cplx* xb = X + (int64_t)b * L;
         const double aa = __ldcg(nrm + a), bb = __ldcg(nrm + b);
         if (aa <= small || bb <= small) continue;
-        double rx = 0.0, ry = 0.0, ix = 0.0, iy = 0.0;
+        if constexpr (R > 0) {  // a warp per pair, the columns in registers
+          cplx* ja = J + (int64_t)a * L;
+          cplx* jb = J + (int64_t)b * L;
+          cplx u[R], v[R], w[R], x[R];
+#pragma unroll
+          for (int k = 0; k < R; ++k) {
+            const int r = lane + 32 * k;
+            u[k] = (r < L) ? __ldcg(xa + r) : cmk(0.0, 0.0);
+            v[k] = (r < L) ? __ldcg(xb + r) : cmk(0.0, 0.0);
+          }
+#pragma unroll
+          for (int k = 0; k < R; ++k) {
+            const int r = lane + 32 * k;
+            w[k] = (r < L) ? __ldcg(ja + r) : cmk(0.0, 0.0);
+            x[k] = (r < L) ? __ldcg(jb + r) : cmk(0.0, 0.0);
+          }
+          JacDot dot;
+#pragma unroll
+          for (int k = 0; k < R; ++k) dot.add(u[k], v[k]);
+          const cplx g = jac_gram_warp(dot, lane);
+          const double ag2 = fma(g.x, g.x, __dmul_rn(g.y, g.y));
+          if (!(ag2 > tol * tol * (aa * bb)) || ag2 < 2.2250738585072014e-308) continue;
+          double c, tg;
+          cplx se;
+          jac_rotation(aa, bb, g, ag2, c, se, tg);
+#pragma unroll
+          for (int k = 0; k < R; ++k) {
+            const int r = lane + 32 * k;
+            if (r < L) jac_rotate(c, se, u[k], v[k], xa[r], xb[r]);
+          }
+#pragma unroll
+          for (int k = 0; k < R; ++k) {
+            const int r = lane + 32 * k;
+            if (r < L) jac_rotate(c, se, w[k], x[k], ja[r], jb[r]);
+          }
+          if (lane == 0) {
+            nrm[a] = aa - tg;
+            nrm[b] = bb + tg;
+            rotated = 1;
+          }
+          continue;
+        }
+        JacDot dot[JC_U];  // rows gl + 8 q + 32 k in dot[q]
         for (int r0 = gl; r0 < L; r0 += JC_G * JC_U) {
           cplx u[JC_U], v[JC_U];
 #pragma unroll
@@ -131,24 +165,16 @@ __global__ void __cluster_dims__(JC_CL, 1, 1) __launch_bounds__(JC_THREADS)
             v[q] = (r < L) ? __ldcg(xb + r) : cmk(0.0, 0.0);
           }
 #pragma unroll
-          for (int q = 0; q < JC_U; ++q) {
-            if (r0 + q * JC_G < L) {
-              rx = fma(u[q].x, v[q].x, rx);
-              ry = fma(u[q].y, v[q].y, ry);
-              ix = fma(u[q].x, v[q].y, ix);
-              iy = fma(-u[q].y, v[q].x, iy);
-            }
-          }
+          for (int q = 0; q < JC_U; ++q) dot[q].add(u[q], v[q]);
         }
-        const cplx g = cmk(jc_grp_sum(rx + ry, gmask), jc_grp_sum(ix + iy, gmask));
-        const double ag2 = cabs2(g);
+        const cplx g = jac_gram(dot, lane, gmask);
+        const double ag2 = fma(g.x, g.x, __dmul_rn(g.y, g.y));
         if (!(ag2 > tol * tol * (aa * bb)) || ag2 < 2.2250738585072014e-308) continue;
         double c, tg;
         cplx se;
         jac_rotation(aa, bb, g, ag2, c, se, tg);
-        const cplx sec = cconj(se);
-        jc_rotate(xa, xb, L, gl, c, se, sec);
-        jc_rotate(J + (int64_t)a * L, J + (int64_t)b * L, L, gl, c, se, sec);
+        jc_rotate(xa, xb, L, gl, c, se);
+        jc_rotate(J + (int64_t)a * L, J + (int64_t)b * L, L, gl, c, se);
         if (gl == 0) {
           nrm[a] = aa - tg;
           nrm[b] = bb + tg;
@@ -205,7 +231,13 @@ cudaError_t launch_jacobi_sized(const Dims* dims, const ProbPtr* ptrs, int batch
                                 cudaStream_t st, int force) {
   if (!jacobi_cluster_chosen(cap, batch, force)) return launch_jacobi(dims, ptrs, batch, status, st);
   ProfScope ps("k_jacobi[cluster]", st);
-  k_jacobi_cl<<<batch * JC_CL, JC_THREADS, 0, st>>>(dims, ptrs, status);
+  // a warp per pair while the cluster's warps are as many as the pairs
+  auto go = [&](auto kernel) { kernel<<<batch * JC_CL, JC_THREADS, 0, st>>>(dims, ptrs, status); };
+  if (cap.l <= 32) go(k_jacobi_cl<1>);
+  else if (cap.l <= 64) go(k_jacobi_cl<2>);
+  else if (cap.l <= 96) go(k_jacobi_cl<3>);
+  else if (cap.l <= 128) go(k_jacobi_cl<4>);
+  else go(k_jacobi_cl<0>);
   return cudaGetLastError();
 }
 

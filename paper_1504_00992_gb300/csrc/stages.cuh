@@ -479,11 +479,33 @@ __device__ __forceinline__ void qr_dev(const Dims& D, const ProbPtr& P, double* 
 
 enum { JAC_MAXSWEEPS = 60, JAC_G = 8 };
 
-// sum over the JAC_G lanes of this lane's group (the group's lanes all call it)
-__device__ __forceinline__ double grp_sum(double v, unsigned mask) {
+// x_a' = c u - conj(se) v, x_b' = se u + c v, each part three operations in a
+// fixed order (every Jacobi kernel gives the same bits)
+__device__ __forceinline__ void jac_rotate(double c, cplx se, cplx u, cplx v, cplx& xa, cplx& xb) {
+  xa = cmk(fma(-se.y, v.y, fma(-se.x, v.x, __dmul_rn(c, u.x))), fma(se.y, v.x, fma(-se.x, v.y, __dmul_rn(c, u.y))));
+  xb = cmk(fma(-se.y, u.y, fma(se.x, u.x, __dmul_rn(c, v.x))), fma(se.y, u.x, fma(se.x, u.y, __dmul_rn(c, v.y))));
+}
+
+// One lane's part of x_a^H x_b
+struct JacDot {
+  double re = 0.0, im = 0.0;
+  __device__ __forceinline__ void add(cplx u, cplx v) {
+    re = fma(u.x, v.x, fma(u.y, v.y, re));
+    im = fma(u.x, v.y, fma(-u.y, v.x, im));
+  }
+};
+// x_a^H x_b from the four parts each of the JAC_G lanes of a group holds
+__device__ __forceinline__ cplx jac_gram(const JacDot* d, int lane, unsigned mask) {
+  return qr_csum<8>((d[0].re + d[2].re) + (d[1].re + d[3].re), (d[0].im + d[2].im) + (d[1].im + d[3].im), lane, mask);
+}
+// the same from the one part of each lane of a warp (part m in lanes 8 m .. 8 m + 7)
+__device__ __forceinline__ cplx jac_gram_warp(JacDot d, int lane) {
 #pragma unroll
-  for (int o = JAC_G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-  return v;
+  for (int o = 16; o >= 8; o >>= 1) {
+    d.re += __shfl_xor_sync(0xffffffffu, d.re, o);
+    d.im += __shfl_xor_sync(0xffffffffu, d.im, o);
+  }
+  return qr_csum<8>(d.re, d.im, lane, 0xffffffffu);
 }
 
 __device__ __forceinline__ void jacobi_finish(const Dims& D, const ProbPtr& P, double* sv, int* perm);
@@ -513,7 +535,7 @@ __device__ __forceinline__ void jac_rotation(double aa, double bb, cplx g, doubl
   const double t = zeta >= 0.0 ? t1 : -t1;
   qr_roots(fma(t, t, 1.0), c, q);
   se = cscale(e, c * t);
-  tg = t * ag;
+  tg = __dmul_rn(t, ag);  // (a product of its own: the callers' sums must not contract with it)
 }
 
 // One-sided Jacobi SVD of one problem by the whole CTA (any multiple of
@@ -563,33 +585,25 @@ __device__ __forceinline__ void jacobi_dev(const Dims& D, const ProbPtr& P, int*
         cplx* xb = X + (int64_t)b * L;
         const double aa = nrm[a], bb = nrm[b];
         if (aa <= small || bb <= small) continue;
-        double rx = 0.0, ry = 0.0, ix = 0.0, iy = 0.0;
-        for (int r = gl; r < L; r += JAC_G) {
-          const cplx u = xa[r], v = xb[r];
-          rx = fma(u.x, v.x, rx);
-          ry = fma(u.y, v.y, ry);
-          ix = fma(u.x, v.y, ix);
-          iy = fma(-u.y, v.x, iy);
+        JacDot dot[4];  // rows gl + 8 m + 32 k in dot[m], as the lanes of k_jacobi_cl's warps take them
+        int r = gl;
+        for (; r + 24 < L; r += 32) {
+#pragma unroll
+          for (int m = 0; m < 4; ++m) dot[m].add(xa[r + 8 * m], xb[r + 8 * m]);
         }
-        const cplx g = cmk(grp_sum(rx + ry, gmask), grp_sum(ix + iy, gmask));
-        const double ag2 = cabs2(g);
+        if (r < L) dot[0].add(xa[r], xb[r]);
+        if (r + 8 < L) dot[1].add(xa[r + 8], xb[r + 8]);
+        if (r + 16 < L) dot[2].add(xa[r + 16], xb[r + 16]);
+        const cplx g = jac_gram(dot, lane, gmask);
+        const double ag2 = fma(g.x, g.x, __dmul_rn(g.y, g.y));
         if (!(ag2 > tol * tol * (aa * bb)) || ag2 < 2.2250738585072014e-308) continue;  // (below normal numbers)
         double c, tg;
         cplx se;
         jac_rotation(aa, bb, g, ag2, c, se, tg);
-        const cplx sec = cconj(se);
-        for (int r = gl; r < L; r += JAC_G) {
-          const cplx u = xa[r], v = xb[r];
-          xa[r] = csub(cscale(u, c), cmul(sec, v));
-          xb[r] = cadd(cmul(se, u), cscale(v, c));
-        }
+        for (r = gl; r < L; r += JAC_G) jac_rotate(c, se, xa[r], xb[r], xa[r], xb[r]);
         cplx* ja = J + (int64_t)a * L;
         cplx* jb = J + (int64_t)b * L;
-        for (int r = gl; r < L; r += JAC_G) {
-          const cplx u = ja[r], v = jb[r];
-          ja[r] = csub(cscale(u, c), cmul(sec, v));
-          jb[r] = cadd(cmul(se, u), cscale(v, c));
-        }
+        for (r = gl; r < L; r += JAC_G) jac_rotate(c, se, ja[r], jb[r], ja[r], jb[r]);
         if (gl == 0) {
           nrm[a] = aa - tg;
           nrm[b] = bb + tg;
