@@ -9,7 +9,13 @@
 // too (the instance's sigma buffer until the final values are written); the
 // cluster barrier (release/acquire at cluster scope) separates the rounds,
 // and columns and norms written by other CTAs are read through L2
-// (ld.global.cg), JC_U rows per lane at a time so that the loads overlap.  A
+// (ld.global.cg), JC_U rows per lane at a time so that the loads overlap.  Up to
+// 128 columns a round has no more pairs than the cluster has warps: a warp then
+// takes a pair, its columns in registers (R rows per lane), with a quarter of
+// the FP64 instructions per round, since what a warp's instruction costs (64
+// clocks of its quarter of the SM) does not depend on the lanes that take part:
+// 10 x l = 42 in 0.59 ms instead of 1.08; the latency of L2 and the cluster
+// barrier are a third of what is left.  A
 // round's pairs are disjoint, so no two groups touch the same column within a
 // round; the arithmetic of every pair is that of k_jacobi.
 #include <cooperative_groups.h>
