@@ -390,6 +390,7 @@ __device__ __forceinline__ bool ce_takes(const Dims& D, int pass, int cond) {
   if (!D.active) return false;
   if ((cond & DPC_QFLAG) && !D.qflag) return false;
   if ((cond & DPC_DIG) && !D.dig) return false;
+  if ((cond & DPC_WIDE) && D.l < DP_WIDE_L) return false;
   return pass == 0 || (D.cq >= pass && !D.cf);
 }
 
@@ -410,7 +411,10 @@ __global__ void __launch_bounds__(CE_THREADS_BIG) k_chol_eq(Dims* dims, const Pr
   __shared__ int s_sum;  // bits of a non-negative float
   const int p = blockIdx.x;
   const Dims D = dims[p];
-  if (!ce_takes(D, pass, cond)) return;
+  if (!ce_takes(D, pass, cond)) {
+    if (f32 && pass == 0 && threadIdx.x == 0) dims[p].cf = 1;  // too narrow: Householder's
+    return;
+  }
   const ProbPtr P = ptrs[p];
   const int L = D.l, tid = threadIdx.x, nt = blockDim.x;
   cplx* G = P.R;
@@ -872,15 +876,15 @@ cudaError_t run_cholqr_f32(float2* A, float2* Q, int M, int l, int use_n, bool l
   enum { PASSES = 4 };
   for (int pass = 0; pass < PASSES; ++pass) {
     const float2* X = pass ? Q : A;
-    const int cond = pass ? (pass << DPC_PASS) | DPC_OK : 0;
+    const int cond = DPC_WIDE | (pass ? (pass << DPC_PASS) | DPC_OK : 0);
     CQ_TRY(launch_oz_gram_f32(dims, ptrs, X, oz.ad, oz.as, M, l, use_n, batch, cond, err, st));
     {
       ProfScope ps("k_chol_inv", st);
       const float again = last ? CE_F32_LAST : CE_F32_MID;
       if (l <= CS_MAXL)
-        k_chol_eq<true><<<batch, ce_threads(l), ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
+        k_chol_eq<true><<<batch, ce_threads(l), ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, DPC_WIDE, 1);
       else
-        k_chol_eq<false><<<batch, ce_threads(l), ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, 0, 1);
+        k_chol_eq<false><<<batch, ce_threads(l), ce_smem_bytes(l), st>>>(dims, ptrs, pass, PASSES, 0.f, again, DPC_WIDE, 1);
       CQ_TRY(cudaGetLastError());
     }
     CQ_TRY(launch_trmm_f32(X, Q, dims, ptrs, M, l, use_n, pass, batch, st));

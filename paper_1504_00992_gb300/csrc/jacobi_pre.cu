@@ -53,7 +53,7 @@ static const float JP_TOL = 3e-6f;    // cosine of a pair the FP32 sweeps leave 
 static const float JP_ANGLE = 3e-5f;  // largest angle of a first-order rotation
 
 __device__ __forceinline__ bool jp_takes(const Dims& D, int cond) {
-  return D.active && !((cond & DPC_DIG) && !D.dig);
+  return D.active && !((cond & DPC_DIG) && !D.dig) && !((cond & DPC_WIDE) && D.l < DP_WIDE_L);
 }
 
 __device__ __forceinline__ float2 jp_shfl_sum(float2 v, unsigned mask) {
@@ -107,7 +107,10 @@ __global__ void __launch_bounds__(JP_THREADS) k_jac_pre(Dims* dims, const ProbPt
   __shared__ int rotated;
   const int p = blockIdx.x;
   const Dims D = dims[p];
-  if (!jp_takes(D, cond)) return;
+  if (!jp_takes(D, cond)) {
+    if ((cond & DPC_WIDE) && threadIdx.x == 0) dims[p].js = 0;
+    return;
+  }
   const ProbPtr P = ptrs[p];
   const int L = D.l, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   float2* X = reinterpret_cast<float2*>(jp_raw);
@@ -349,7 +352,10 @@ __global__ void __cluster_dims__(JB_CL, 1, 1) __launch_bounds__(JB_THREADS)
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank(), p = blockIdx.x / JB_CL;
   const Dims D = dims[p];
-  if (!jp_takes(D, cond)) return;  // uniform over the cluster
+  if (!jp_takes(D, cond)) {  // uniform over the cluster
+    if ((cond & DPC_WIDE) && crank == 0 && threadIdx.x == 0) dims[p].js = 0;
+    return;
+  }
   const ProbPtr P = ptrs[p];
   const int L = D.l, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   float2* X = scr + (size_t)p * stride;

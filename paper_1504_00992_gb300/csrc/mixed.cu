@@ -652,12 +652,23 @@ static cudaError_t tc_product(const void* A0, const void* A1, const void* B0, co
   return cudaGetLastError();
 }
 
-// QR of an FP32 sketch.  At the sizes of oz_stage_rule by the Cholesky QR from
-// digits (chol), then Householder for the instances it gives
-// up; elsewhere, and where the CTA size of the Householder kernels is chosen,
-// by those alone.  Householder on one CTA, or on many CTAs, per instance
-// against the Cholesky QR: 152 x 2000 x 120 4.9 against 2.9 ms, 8 x 2000 x 120
-// 4.1 against 0.7 ms, 15 x 7700 x 262 8 against 6.5 ms.
+// Whether the FP32 QRs of M-row sketches go by the Cholesky QR first.  A chain
+// handle's bonds (cap.cm > 0) grow from product states: their sketches are
+// singular to FP32 for many steps, take every pass and then the Householder QR
+// after all (256 XXZ chains from Neel states, fourth step: 0.98 s against 0.68
+// by Householder alone; 12 chains at their caps 121 ms, or 160 with unlucky
+// inputs, against 107), so there only bonds
+// too tall for the one-CTA Householder kernel do.
+static bool qr_f32_chol(const Caps& cap, int M) {
+  return oz_stage_rule(cap) && (cap.cm == 0 || !qr_blk_f32_fits(M, cap.l));
+}
+
+// QR of an FP32 sketch: with chol by the Cholesky QR from digits, then
+// Householder for the instances it gives up; else, and where the CTA size of
+// the Householder kernels is chosen, by those alone.  Householder on one CTA,
+// or on many CTAs, per instance against the Cholesky QR: 152 x 2000 x 120 4.9
+// against 2.9 ms, 8 x 2000 x 120 4.1 against 0.7 ms, 15 x 7700 x 262 8 against
+// 6.5 ms.
 static cudaError_t qr_f32(float2* A, float2* Q, int M, int L, int batch, const MixedPtrs& mp, const MixedSizes& s,
                           Dims* dims, const ProbPtr* ptrs, int use_n, bool chol, bool last, const OzScratch& oz,
                           int* err, cudaStream_t st, int threads) {
@@ -735,7 +746,7 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));
   const OzScratch oz{mp.gad, mp.gas, mp.gbd, mp.gbs};
   auto qr = [&](float2* A, float2* Q, int M, int use_n, bool last) {
-    return qr_f32(A, Q, M, l, batch, mp, s, const_cast<Dims*>(dims), ptrs, use_n, oz_stage_rule(cap), last, oz, err, st,
+    return qr_f32(A, Q, M, l, batch, mp, s, const_cast<Dims*>(dims), ptrs, use_n, qr_f32_chol(cap, M), last, oz, err, st,
                   kn.qr_threads);
   };
   {
@@ -817,7 +828,7 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   // corrections, unless another form is chosen
   const int jac = mixed_jac(kn, cap, batch);
   if ((jac == 3 || (jac == 2 && cap.l > 160)) && tc && jac_pre_rule(cap, true))
-    MX_TRY(run_jac_pre(const_cast<Dims*>(dims), ptrs, batch, cap, oz, batch, 0, false, err, st));
+    MX_TRY(run_jac_pre(const_cast<Dims*>(dims), ptrs, batch, cap, oz, batch, DPC_WIDE, false, err, st));
   else
     MX_TRY(launch_jac_none(const_cast<Dims*>(dims), batch, st));
   if (jac == 3)

@@ -162,7 +162,11 @@ struct DpPath {
 cudaError_t dp_begin(const DpPath& p);  // theta's digits, when they are kept
 // one digit-split product of the problems selected by cond: bits, and from
 // bit 8 up the pass of a Cholesky QR (the problems that take part in it)
-enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_JS = 16, DPC_PASS = 8 };
+// (DPC_WIDE: those of at least DP_WIDE_L columns; a handle's wave also holds bonds
+// far below its capacities, whose Householder QR and double-float Jacobi are
+// cheaper than the passes and products of the digit forms)
+enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_JS = 16, DPC_WIDE = 32, DPC_PASS = 8 };
+enum { DP_WIDE_L = 40 };
 cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
 // Cholesky QR of Y into Q (side 0) or Yt into Qt (side 1) (cholqr.cu): up to
 // `passes` passes, then, with lowdin, the symmetric orthonormalisation to

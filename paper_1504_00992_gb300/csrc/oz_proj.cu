@@ -244,6 +244,7 @@ __device__ __forceinline__ bool oz_takes(const Dims& D, int cond) {
   if ((cond & DPC_DIG) && !D.dig) return false;
   if ((cond & DPC_CHK) && !D.chk) return false;
   if ((cond & DPC_JS) && D.js != 1) return false;
+  if ((cond & DPC_WIDE) && D.l < DP_WIDE_L) return false;
   return true;
 }
 
