@@ -46,12 +46,13 @@ CLOCK_QUERY = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.ac
 
 
 # arithmetic of each form of the single-bond measurement
-DTYPES = {"fp64": "f64", "tf32": "tf32+f32+bf16x6+df64+f64", "bf16": "bf16+tf32+f32+bf16x6+df64+f64"}
-_MIXED_TAIL = ("3xTF32 refinement round, FP32 Householder QRs, FP64-accurate re-orthonormalisation of the last "
-               "Q, projection B = Q^H theta on the tensor cores from exact BF16 digit splits (FP64-accurate), "
-               "two Cholesky QR passes of B^H and U, V on the same digit-split tensor-core products, "
-               "double-float Jacobi SVD")
-FORMS = {"fp64": "plain path, every step in FP64",
+DTYPES = {"fp64": "bf16x7+df64+f64", "tf32": "tf32+f32+bf16x7+df64+f64", "bf16": "bf16+tf32+f32+bf16x7+df64+f64"}
+_MIXED_TAIL = ("3xTF32 refinement round, FP32 QRs (Cholesky QR from exact digits), FP64-accurate re-orthonormalisation of "
+               "the last Q, projection B = Q^H A on the tensor cores from exact BF16 digit splits (FP64-accurate), "
+               "Cholesky QR of B^H and U, V on the same digit-split tensor-core products, FP32 Jacobi sweeps with "
+               "digit-split corrections and a double-float Jacobi SVD")
+FORMS = {"fp64": "plain path, every result to FP64 (products, Cholesky QRs and the SVD's corrections from exact "
+                 "seven-digit BF16 splits on the tensor cores)",
          "tf32": "TF32 sketch and power rounds before the last, " + _MIXED_TAIL,
          "bf16": "BF16 sketch and power rounds before the last, " + _MIXED_TAIL}
 
@@ -381,10 +382,10 @@ def _src_hash(name):
     return hashlib.sha256(src).hexdigest()[:16]
 
 
-# The tensor-core projection forms each complex multiply-add of C = Q_f^H A
-# from 21 pairs of BF16 digits (six 8-bit digits per operand, pairs t + u <=
-# 7) x 4 real products: 168 BF16 flop per 8 FP64-equivalent flop, so its
-# FP64-equivalent ceiling is the measured BF16 rate x 8 / 168.
+# An FP64-accurate complex multiply-add takes at least 21 pairs of BF16 digits
+# (48 bits: six 8-bit digits per operand, pairs t + u <= 7) x 4 real products:
+# 168 BF16 flop per 8 FP64-equivalent flop, a ceiling of the measured BF16 rate
+# x 8 / 168.  The kernel runs 28 pairs (seven digits), the projection 22.
 OZ_BF16_FLOP_PER_CMAC = 21 * 4 * 2
 # FP32 CUDA-core peak of GB300: 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2.07 GHz
 FP32_PEAK_GFLOPS = 152 * 128 * 2 * 2.07
@@ -434,6 +435,10 @@ def roofline(res, batch):
         # the mixed form's Jacobi in double-float arithmetic: the same
         # algorithmic flops against the double-float ceiling
         "k_jacobi[df]": (60.0 * l ** 3 * batch, "alu", df_peak, df_src, "jacobi_df.cu"),
+        # the FP32 sweeps of the small SVD
+        "k_jacobi[pre]": (60.0 * l ** 3 * batch, "alu", fp32_peak, fp32_src, "jacobi_pre.cu"),
+        # the FP64 form's products with theta
+        "k_oz_gemm[sketch]": (8.0 * M * N_ * l * batch, "tensor", oz_peak, oz_src, "oz_proj.cu"),
         # the FP32 Householder QRs of the sketch rounds (R and explicit Q of an
         # m x l complex matrix, m = n here)
         "k_qr_f32": ((16.0 * M * l * l - 16.0 * l ** 3 / 3) * batch, "alu", fp32_peak, fp32_src, "qr_blocked.cu"),
@@ -479,6 +484,12 @@ def roofline(res, batch):
         # with the Cholesky QR of B^H, k_qr factors only the instances it
         # flags as ill-conditioned (usually none): no fixed flop count
         if kk == "k_qr" and cholqr:
+            continue
+        # the same for the FP32 QRs (and the Gram matrices: later passes mostly
+        # find nothing to do), and for the Jacobi kernel after the FP32 sweeps
+        if kk in ("k_qr_f32", "k_oz_gemm[gram]") and "k_trmm_f32" in prof:
+            continue
+        if kk.startswith("k_jacobi") and kk != "k_jacobi[pre]" and "k_jacobi[pre]" in prof:
             continue
         if kk in prof and prof[kk][1] > 0:
             a = flk / (prof[kk][0] / prof[kk][1] / 1e3) / 1e12

@@ -62,18 +62,24 @@ enum {
 };
 
 /* Arithmetic of the RRSVD (Alg. 1 and the steps after it).
- *   TEBD_PREC_FP64: the plain path, every step in FP64.
+ *   TEBD_PREC_FP64: the plain path, every result to FP64.  Large problems
+ *     (plans with m, n >= 128 and k + p >= 40; bonds of those sizes of handles
+ *     with fused = 0 and a bond of m n >= 192^2) run their products and QRs on
+ *     the tensor cores: operands cut exactly into seven 8-bit digits (56 bits
+ *     relative to the largest entry of each row or column), integer sums,
+ *     Cholesky QR with column scaling (Householder for what it gives up), an
+ *     FP32 Jacobi with corrections to FP64.  The others, and plans with forced
+ *     GEMM tiles, run on the FP64 pipe.
  *   TEBD_PREC_TF32: the mixed form.  Y0 = A Omega and power rounds 1..q-1
  *     on the tensor cores in TF32 with FP32 accumulation and FP32 QR;
  *     power round q (Y0 when q = 0) as the refinement pass in split 3xTF32
  *     products (FP32-level accuracy); the last basis re-orthonormalised
- *     FP64-accurately (FP32 QR and a double-float Loewdin correction);
+ *     FP64-accurately (FP32 QR and a Loewdin correction);
  *     B = Q^H A on the tensor cores from exact BF16 digit splits of Q and
- *     A (products exact in FP32, digit levels summed in double-float:
- *     FP64-level accuracy); the QR of B^H by two Cholesky QR passes in
- *     double-float arithmetic (Householder QR in FP64 for an instance whose
- *     Gram matrix is too ill-conditioned); the Jacobi SVD, U, V and lambda
- *     FP64-accurate.  Omega comes from the same Philox words by an FP32
+ *     A (products and digit levels exact: FP64-level accuracy); the QR of
+ *     B^H by Cholesky QR passes from digits (Householder QR in FP64 for an
+ *     instance whose Gram matrix is too ill-conditioned); the Jacobi SVD, U,
+ *     V and lambda FP64-accurate.  Omega comes from the same Philox words by an FP32
  *     Box-Muller.
  *   TEBD_PREC_BF16: the mixed form with the products before the refinement
  *     round (Y0 and power rounds 1..q-1) in BF16 with FP32 accumulation,
@@ -134,8 +140,9 @@ typedef struct {
                               persistent launch, for waves whose bonds have
                               d_l d_r < 32 and m, n <= 512.  0: where the autotuner
                               finds it faster (never without autotune); 1: wherever
-                              it fits; -1: never.  Same results as the staged launches,
-                              bit for bit */
+                              it fits; -1: never.  1 gives the results of -1, bit for
+                              bit; the staged launches of 0 may also take the tensor
+                              cores for large FP64 bonds (TEBD_PREC_FP64) */
 } tebd_desc_t;
 
 /* Section II (Eq. defmps, deftheta, defupdatetheta) with the RRSVD of
