@@ -36,15 +36,14 @@ __device__ __forceinline__ void split_bits(double x, float& hi, float& lo) {
   lo = sign ? -l : l;
 }
 
-// Biased FP64 exponent of x; 0 for zero, subnormal and non-finite values
-// (the last are flagged elsewhere).  The digit splits scale rows by its maximum.
-__device__ __forceinline__ int oz_exp(double x) {
-  const int e = (int)(((uint64_t)__double_as_longlong(x) >> 52) & 0x7FF);
-  return e == 0x7FF ? 0 : e;
-}
+// Biased FP64 exponent of x; 0 for zero and subnormal values, OZ_NONFINITE
+// for Inf and NaN.  The digit splits scale rows by its maximum, so a row with
+// a non-finite entry has that as its exponent, and its products are NaN.
+enum { OZ_NONFINITE = 0x7FF };
+__device__ __forceinline__ int oz_exp(double x) { return (int)(((uint64_t)__double_as_longlong(x) >> 52) & 0x7FF); }
 __device__ __forceinline__ int oz_exp(float x) {
   const int e = (int)((__float_as_uint(x) >> 23) & 0xFF);
-  return (e == 0 || e == 0xFF) ? 0 : e - 127 + 1023;
+  return e == 0xFF ? OZ_NONFINITE : (e == 0 ? 0 : e - 127 + 1023);
 }
 
 // (s, e) with s + e = a + b exactly (Knuth's TwoSum)

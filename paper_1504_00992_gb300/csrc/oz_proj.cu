@@ -157,8 +157,11 @@ __device__ __forceinline__ size_t oz_at(int ks, int plane, int row, int ch, int 
   return (((size_t)ks * (2 * NS) + plane) * rc + row) * OZ_KS + 8 * (ch ^ ((row >> 2) & 1));
 }
 
-// Scale of a row in the product: 2^(E - 1023 - 22); zero for a zero row.
+// Scale of a row in the product: 2^(E - 1023 - 22); zero for a zero row, NaN
+// for a row with a non-finite entry (whose digits are zero): the row or column
+// of the result is NaN then, as a sum of FP64 multiply-adds would make it.
 __device__ __forceinline__ double oz_scale(int E) {
+  if (E == OZ_NONFINITE) return __longlong_as_double(0x7FF8ll << 48);
   return E > 22 ? __longlong_as_double((long long)(E - 22) << 52) : 0.0;
 }
 
