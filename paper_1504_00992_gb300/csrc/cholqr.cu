@@ -330,7 +330,7 @@ cudaError_t run_cholqr_bh(Dims* dims, const ProbPtr* ptrs, int batch, const Caps
   if (oz) {
     CQ_TRY(run_cholqr(1, 2, phases ? CQ_PHASES : CQ_LOWDIN, CQ_MIN_PIVOT, dims, ptrs, batch, cap, *oz, batch, 0, err, st));
     CQ_TRY(launch_oz_stage(G_X, dims, ptrs, batch, cap, *oz, err, st, DPC_OK));  // X = B Qb = Rb^H
-    return launch_qr_rest(QR_BH, dims, ptrs, batch, cap, st, QRS_CF);
+    return launch_qr_rest(QR_BH, dims, ptrs, batch, cap, st, QRS_CF, true);
   }
   auto gemm = [&](int stage) { return launch_zgemm_df(stage, dims, ptrs, batch, cap, st); };
   CQ_TRY(gemm(G_G1));                          // G1 = B B^H
@@ -912,7 +912,7 @@ cudaError_t DpPath::qr(int stage, int kind) const {
   CQ_TRY(run_cholqr(side, passes, lowdin, min_pivot, const_cast<Dims*>(dims), ptrs, batch, cap, dp->oz, dp->chunk,
                     DPC_DIG | check, dp->err, st));
   if (stage == QR_BH) CQ_TRY(launch_dp_stage(G_X, *this, DPC_DIG | DPC_OK));  // X = B Qb = Rb^H
-  return launch_qr_rest(stage, dims, ptrs, batch, cap, st, check ? QRS_QFLAG_REST : QRS_REST);
+  return launch_qr_rest(stage, dims, ptrs, batch, cap, st, check ? QRS_QFLAG_REST : QRS_REST, kind == DPQ_LAST);
 }
 
 }  // namespace tg

@@ -145,9 +145,10 @@ cudaError_t qr_small_prepare();
 // its structure allows (the autotuner's choices)
 cudaError_t launch_qr_sized(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
                            cudaStream_t st, int force = 0, int which = QRS_ALL);
-// the problems the Cholesky QR left: one CTA each, or the many-CTA form for large ones
+// the problems the Cholesky QR left: one CTA each, or the many-CTA form for
+// large ones and (last: the last basis or B^H) for few tall ones
 cudaError_t launch_qr_rest(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
-                           cudaStream_t st, int which);
+                           cudaStream_t st, int which, bool last);
 // true when launch_qr_sized(stage, ..., force) runs the many-CTA form
 bool qr_multi_chosen(int stage, const Caps& cap, int batch, int force);
 size_t qr_multi_scratch_r(int l);

@@ -587,13 +587,19 @@ bool qr_multi_chosen(int stage, const Caps& cap, int batch, int force) {
 }
 
 cudaError_t launch_qr_rest(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
-                           cudaStream_t st, int which) {
-  // the one-CTA kernel runs at ~8 GFLOP/s: from ~0.3 s per matrix on the ~100
-  // launches of the many-CTA form are the smaller cost, also when none needs it
+                           cudaStream_t st, int which, bool last) {
+  // The one-CTA kernel runs at ~8 GFLOP/s: from ~0.2 s per matrix on the 42
+  // (l = 120) or more launches of the many-CTA form are the smaller cost, also
+  // when none needs it.  The two QRs that ask for a well-conditioned basis
+  // (the last basis, B^H) give up every steep spectrum, so there the few tall
+  // matrices of the many-CTA form's own size rule take it too: 2000 x 120 is
+  // 58 ms on one CTA; a mixed plan of 1 or 16 matrices whose spectrum falls as
+  // exp(-j / 4) took 67 or 72 ms with it, 15 or 30 ms this way, and where no
+  // matrix needs them the launches cost 0.16 ms (16 x 2000 x 120).
   const int M = (stage == QR_Y) ? cap.m : cap.n;
   const bool large = (double)M * cap.l * cap.l >= 1e8 && qr_multi_fits(M, cap.l, 1);
-  return large ? launch_qr_sized(stage, dims, ptrs, batch, cap, st, 2, which)
-               : launch_qr(stage, dims, ptrs, batch, cap, st, which);
+  return large || last ? launch_qr_sized(stage, dims, ptrs, batch, cap, st, large ? 2 : 0, which)
+                       : launch_qr(stage, dims, ptrs, batch, cap, st, which);
 }
 
 cudaError_t launch_qr_sized(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,
