@@ -839,6 +839,8 @@ static size_t ce_smem_bytes(int L) { return L <= CS_MAXL ? cs_smem_bytes(L) : si
 
 cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* dims, const ProbPtr* ptrs, int batch,
                        const Caps& cap, const OzScratch& oz, int chunk, int cond, int* err, cudaStream_t st) {
+  const float again = (lowdin & CQ_SHIFTED) ? 0.f : (lowdin ? CE_AGAIN_LD : CE_AGAIN);
+  lowdin &= ~CQ_SHIFTED;
   auto prod = [&](int stage, int c) {
     return launch_oz_range(stage, dims, ptrs, batch, cap, oz, chunk, c, err, st);
   };
@@ -850,7 +852,7 @@ cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* 
     CQ_TRY(prod(pass ? g1 : g0, in_pass | (pass ? DPC_OK : 0)));
     {
       ProfScope ps("k_chol_inv", st);
-      const float mp = pass == 0 ? min_pivot : 0.f, again = lowdin ? CE_AGAIN_LD : CE_AGAIN;
+      const float mp = pass == 0 ? min_pivot : 0.f;
       if (cap.l <= CS_MAXL)
         k_chol_eq<true><<<batch, ce_threads(cap.l), ce_smem_bytes(cap.l), st>>>(dims, ptrs, pass, passes, mp, again, cond, 0);
       else
@@ -906,9 +908,19 @@ cudaError_t DpPath::qr(int stage, int kind) const {
   const int side = stage == QR_Y ? 0 : 1;
   const int check = kind == DPQ_CHECK ? DPC_QFLAG : 0;
   const bool first = kind == DPQ_FIRST || kind == DPQ_FIRST_LD;
-  const int passes = first ? 3 : (kind == DPQ_CHECK ? 2 : 1);
-  const int lowdin = kind == DPQ_LAST ? CQ_PHASES : (kind == DPQ_CHECK || kind == DPQ_FIRST_LD ? CQ_LOWDIN : 0);
-  const float min_pivot = first ? 0.f : (kind == DPQ_LAST ? CE_AGAIN_LD : CE_PIVOT);
+  // A middle basis is well-conditioned once its columns are scaled, unless
+  // theta's rank is below l to rounding: A^H q of the directions past it is
+  // what q has left of the leading singular vectors, the same direction for
+  // all.  Those take shifted passes as the first basis does (one 2000 x 2000
+  // of spectrum exp(-j / 2), l = 120, q = 1: 76 ms with the Householder QR on
+  // one CTA instead, 19 ms so; where none needs them the launches cost 0.08 ms
+  // a basis of 16 x 2000 x 120).
+  const bool mid = kind == DPQ_MID;
+  const int passes = first || mid ? 3 : (kind == DPQ_CHECK ? 2 : 1);
+  const int lowdin = kind == DPQ_LAST ? CQ_PHASES
+                     : mid            ? CQ_SHIFTED
+                                      : (kind == DPQ_CHECK || kind == DPQ_FIRST_LD ? CQ_LOWDIN : 0);
+  const float min_pivot = first || mid ? 0.f : (kind == DPQ_LAST ? CE_AGAIN_LD : CE_PIVOT);
   CQ_TRY(run_cholqr(side, passes, lowdin, min_pivot, const_cast<Dims*>(dims), ptrs, batch, cap, dp->oz, dp->chunk,
                     DPC_DIG | check, dp->err, st));
   if (stage == QR_BH) CQ_TRY(launch_dp_stage(G_X, *this, DPC_DIG | DPC_OK));  // X = B Qb = Rb^H

@@ -170,10 +170,11 @@ enum { DP_WIDE_L = 40 };
 cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
 // Cholesky QR of Y into Q (side 0) or Yt into Qt (side 1) (cholqr.cu): up to
 // `passes` passes, then, with lowdin, the symmetric orthonormalisation to
-// FP64 (CQ_PHASES: with the column phases of the Householder QR);
+// FP64 (CQ_PHASES: with the column phases of the Householder QR; CQ_SHIFTED:
+// without it, further passes only for the problems a pass shifted);
 // min_pivot: the smallest pivot of the scaled Gram matrix accepted in a first
 // pass (0: any, by shifted passes).  Problems given up have cf set.
-enum { CQ_LOWDIN = 1, CQ_PHASES = 2 };
+enum { CQ_LOWDIN = 1, CQ_PHASES = 2, CQ_SHIFTED = 4 };
 cudaError_t run_cholqr(int side, int passes, int lowdin, float min_pivot, Dims* dims, const ProbPtr* ptrs, int batch,
                        const Caps& cap, const OzScratch& oz, int chunk, int cond, int* err, cudaStream_t st);
 // Cholesky QR of an FP32 sketch A (M x l capacities, m or, with use_n, n rows

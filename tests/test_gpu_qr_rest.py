@@ -32,7 +32,9 @@ def _run(B, theta, k, p, q, prec, tuning=None, profile=False):
             try:
                 B.tebd_profiler_reset()
                 rrsvd_device(B, plan, theta)
-                out["kernels"] = {name: rec[1] for name, rec in B.tebd_profiler_read().items()}
+                prof = B.tebd_profiler_read()
+                out["kernels"] = {name: rec[1] for name, rec in prof.items()}
+                out["ms"] = {name: rec[0] for name, rec in prof.items()}
             finally:
                 B.tebd_profiler_enable(False)
         return out
@@ -62,6 +64,9 @@ def test_fp64_form_agrees_with_the_fp64_pipe(lib, m, n, k, p, q, batch):
     a = _run(B, theta, k, p, q, B.TEBD_PREC_FP64, profile=True)
     b = _run(B, theta, k, p, q, B.TEBD_PREC_FP64, {"tiles": [32] * 6})
     assert a["kernels"].get("k_qr[multi]") == 2  # the last basis and B^H
+    # no first or middle basis is left to one CTA: M l^2 16 flop at 8 GFLOP/s
+    # would be 5 ms or more each, an empty launch is a few microseconds
+    assert a["ms"]["k_qr"] < 0.2 * a["kernels"]["k_qr"]
     for t in range(batch):
         s1, nrm = b["sigma"][t][0], np.linalg.norm(theta[t])
         assert np.abs(a["sigma"][t] - b["sigma"][t]).max() <= 1e-12 * s1
