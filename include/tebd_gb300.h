@@ -125,9 +125,11 @@ typedef struct {
                            runs on a blocking stream of its own */
   int autotune;         /* nonzero: at creation, time each wave's launch choices at its
                            capacity sizes and keep the fastest (tebd_wave_info): FP64 --
-                           the 16x16 or 32x32 GEMM tiles of every stage and (with
-                           fused = 0) the staged sequence against the fused persistent
-                           launch; TF32 -- the mixed form's choices as for
+                           the 16x16 or 32x32 GEMM tiles of every stage (of bonds on the
+                           FP64 pipe) and, with fused = 0, the staged sequence against
+                           the fused persistent launch (for waves without bonds on the
+                           tensor cores: the choices of an FP64 handle leave every bit
+                           as it is); TF32 -- the mixed form's choices as for
                            rrsvd_plan_autotune */
   size_t workspace_budget; /* bytes of per-bond workspace one wave may use (0 = all bonds
                               of a parity in one wave); larger batches run in waves */
@@ -139,8 +141,9 @@ typedef struct {
                               every bond of a wave updated whole by one CTA of one
                               persistent launch, for waves whose bonds have
                               d_l d_r < 32 and m, n <= 512.  0: where the autotuner
-                              finds it faster (never without autotune); 1: wherever
-                              it fits; -1: never.  1 gives the results of -1, bit for
+                              finds it faster (never without autotune, nor for a wave
+                              with bonds on the tensor cores); 1: wherever it fits;
+                              -1: never.  1 gives the results of -1, bit for
                               bit; the staged launches of 0 may also take the tensor
                               cores for large FP64 bonds (TEBD_PREC_FP64) */
 } tebd_desc_t;

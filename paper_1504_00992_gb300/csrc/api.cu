@@ -345,14 +345,10 @@ static int tune_wave(tebd_s* h, const ParitySet& ps, Wave& w, cudaStream_t st, D
   }
   // the whole RRSVD of the wave, staged (tuned tiles) against the persistent
   // fused kernel, on synthetic theta at the capacity sizes (the two give the
-  // same results; the data only sets the QR and Jacobi work)
-  if (fused_mode == 0 && fused_fits(w.cap)) {
-    DpScratch dp;
-    if (w.dp) {  // the staged launches as enqueue_sweep makes them
-      dp = dp_carve(h->mixed, w.cap, w.count, h->plan.dp_limit, h->tcerr);
-      for (Dims& D : hd) D.dig = dp_rule(D.m, D.n, D.l) ? 1 : 0;
-      if (cudaMemcpy(scratch_dims, hd.data(), sizeof(Dims) * w.count, cudaMemcpyHostToDevice) != cudaSuccess) return -1;
-    }
+  // same bits; the data only sets the QR and Jacobi work).  A wave with
+  // digit-split bonds stays staged: its bits differ from the fused kernel's,
+  // and a stopwatch must not choose between them.
+  if (fused_mode == 0 && fused_fits(w.cap) && !w.dp) {
     if (launch_tune_theta(scratch_dims, ps.ptrs + w.first, w.count, st) != cudaSuccess) return -1;
     float ms[2] = {1e30f, 1e30f};
     for (int variant = 0; variant < 2; ++variant)
@@ -360,7 +356,7 @@ static int tune_wave(tebd_s* h, const ParitySet& ps, Wave& w, cudaStream_t st, D
         cudaEventRecord(e0, st);
         const cudaError_t e =
             variant == 0 ? run_rrsvd(scratch_dims, ps.ptrs + w.first, w.count, w.cap, h->q, h->seed, 0, 0, -1,
-                                     h->status, st, h->sweep_dev, w.tiles, w.dp ? &dp : nullptr)
+                                     h->status, st, h->sweep_dev, w.tiles)
                          : launch_bond_fused(ps.ptrs + w.first, nullptr, scratch_dims, w.count, p_os, h->q, h->seed,
                                              h->sweep_dev, h->cutoff, nullptr, h->status, h->queue, st);
         if (e != cudaSuccess) return -1;

@@ -13,8 +13,9 @@
 // only: no CTA waits on another.
 //
 // The stages run the code of the staged kernels (stages.cuh) with the same
-// per-element summation orders, so the fused and the staged paths give
-// bit-identical states.  Bonds whose gate takes the GEMM path (d_l d_r >= 32)
+// per-element summation orders, so the fused and the staged launches on the
+// FP64 pipe give bit-identical states (waves with bonds on the tensor cores
+// are never fused).  Bonds whose gate takes the GEMM path (d_l d_r >= 32)
 // and sketches wider than QR_MAXL stay on the staged path (fused_fits).
 #include <cuda_runtime.h>
 
