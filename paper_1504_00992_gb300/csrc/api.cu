@@ -1104,6 +1104,22 @@ extern "C" int tebd_set_gates(tebd_t h, int parity, const double* gates) {
   return TEBD_OK;
 }
 
+// theta~ of one wave of an FP64 handle, as every sweep and its recomputation
+// in the reverse pass form it: large bonds contracted from digit splits.
+static cudaError_t wave_theta(tebd_t h, const Wave& w, const Dims* dims, const ProbPtr* ptrs, cudaStream_t st) {
+  cudaError_t e;
+  const bool cont = w.dp > 0 && theta_digits_rule(w.cap.m, w.cap.n, w.cap.cm);
+  if ((e = launch_theta(dims, ptrs, w.count, w.cap, st, 0, 0, cont ? 1 : 0)) != cudaSuccess) return e;
+  if (cont) {
+    const DpScratch dp = dp_carve(h->mixed, w.cap, w.count, h->plan.dp_limit, h->tcerr);
+    if ((e = launch_oz_range(OZ_CONT_STAGE, dims, ptrs, w.count, w.cap, dp.oz, dp.chunk, DPC_DIG, h->tcerr, st)) !=
+        cudaSuccess)
+      return e;
+    if ((e = launch_gate_small(dims, ptrs, w.count, w.cap, 1, st)) != cudaSuccess) return e;
+  }
+  return launch_gate_gemm(dims, ptrs, w.count, w.cap, st);
+}
+
 // The staged RRSVD of one wave of an FP64 handle.
 static cudaError_t wave_rrsvd(tebd_t h, const Wave& w, const Dims* dims, const ProbPtr* ptrs, cudaStream_t st) {
   DpScratch dp;
@@ -1150,17 +1166,8 @@ static cudaError_t enqueue_sweep(tebd_t h, int parity) {
         if ((e = launch_theta_df(dims, ptrs, w.count, w.cap, h->stream)) != cudaSuccess) return e;
         if ((e = launch_gate_gemm_df(dims, ptrs, w.count, w.cap, h->stream)) != cudaSuccess) return e;
       }
-    } else {
-      const bool cont = w.dp > 0 && theta_digits_rule(w.cap.m, w.cap.n, w.cap.cm);
-      if ((e = launch_theta(dims, ptrs, w.count, w.cap, h->stream, 0, 0, cont ? 1 : 0)) != cudaSuccess) return e;
-      if (cont) {
-        const DpScratch dp = dp_carve(h->mixed, w.cap, w.count, h->plan.dp_limit, h->tcerr);
-        if ((e = launch_oz_range(OZ_CONT_STAGE, dims, ptrs, w.count, w.cap, dp.oz, dp.chunk, DPC_DIG, h->tcerr,
-                                 h->stream)) != cudaSuccess)
-          return e;
-        if ((e = launch_gate_small(dims, ptrs, w.count, w.cap, 1, h->stream)) != cudaSuccess) return e;
-      }
-      if ((e = launch_gate_gemm(dims, ptrs, w.count, w.cap, h->stream)) != cudaSuccess) return e;
+    } else if ((e = wave_theta(h, w, dims, ptrs, h->stream)) != cudaSuccess) {
+      return e;
     }
     if (prec_mixed(h->precision)) {
       const MixedPtrs mp = mixed_carve(h->mixed, w.ms, w.count);
@@ -1496,8 +1503,7 @@ extern "C" int tebd_backward(tebd_t h, int site, const double* op, double* dgate
         if (launch_plan(ptrs, dims, w.count, h->p, st, w.dp > 0) != cudaSuccess ||
             launch_theta(dims, ptrs, w.count, w.cap, st, 1) != cudaSuccess ||
             launch_adj_keep_theta(dims, ptrs, adj, w.count, st) != cudaSuccess ||
-            launch_theta(dims, ptrs, w.count, w.cap, st) != cudaSuccess ||
-            launch_gate_gemm(dims, ptrs, w.count, w.cap, st) != cudaSuccess ||
+            wave_theta(h, w, dims, ptrs, st) != cudaSuccess ||  // the forward sweep's own bits: its gauge
             wave_rrsvd(h, w, dims, ptrs, st) != cudaSuccess ||
             launch_rebuild(dims, ptrs, w.count, w.cap, h->cutoff, h->wout + w.first, h->status, st) != cudaSuccess ||
             launch_adj_bond(dims, ptrs, adj, w.count, region, region + rbytes, ck.buf, h->cutoff, 1e-24, 1e-24,
