@@ -23,6 +23,7 @@
 #include "dfsplit.cuh"
 #include "internal.cuh"
 #include "mixed.cuh"
+#include "once.cuh"
 #include "profiler.cuh"
 
 namespace tg {
@@ -288,23 +289,16 @@ __global__ void k_chol_eq(Dims* dims, const ProbPtr* __restrict__ ptrs, int pass
 static cudaError_t lowdin_prepare();
 
 cudaError_t cholqr_prepare() {
-  static int done = 0;
-  if (!done) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_chol_inv_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs_smem_bytes(CS_MAXL));
-    if (e != cudaSuccess) return e;
-    const cudaError_t e2 =
-        cudaFuncSetAttribute(k_chol_eq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs_smem_bytes(CS_MAXL));
-    if (e2 != cudaSuccess) return e2;
-    const cudaError_t e5 = lowdin_prepare();
-    if (e5 != cudaSuccess) return e5;
-    const cudaError_t e4 = qr_small_prepare();
-    if (e4 != cudaSuccess) return e4;
-    const cudaError_t e3 = jac_pre_prepare();
-    if (e3 != cudaSuccess) return e3;
-    done = 1;
-  }
-  return cudaSuccess;
+  static DeviceOnce once;
+  return once([] {
+    const int sm = (int)cs_smem_bytes(CS_MAXL);
+    cudaError_t e = cudaFuncSetAttribute(k_chol_inv_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chol_eq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e == cudaSuccess) e = lowdin_prepare();
+    if (e == cudaSuccess) e = qr_small_prepare();
+    if (e == cudaSuccess) e = jac_pre_prepare();
+    return e;
+  });
 }
 
 static cudaError_t chol_inv(Dims* dims, const ProbPtr* ptrs, int batch, int lcap, int pass, cudaStream_t st) {

@@ -173,6 +173,7 @@ cudaError_t launch_frob2(const Dims* dims, const ProbPtr* ptrs, int batch, cudaS
 // launch_gate_gemm applies its gate; skip_pre = 1 leaves those bonds to
 // launch_theta_df.  skip_dig: the bonds of theta_digits_rule are left out (1: with
 // Dims::dig, 2: any).
+cudaError_t theta_prepare();  // kernel attributes, once per device
 cudaError_t launch_theta(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, cudaStream_t st,
                          int identity_gate = 0, int skip_pre = 0, int skip_dig = 0);
 // the gate of the bonds contracted from digit splits, in place; need_dig: those with Dims::dig

@@ -41,6 +41,7 @@
 #include "dfsplit.cuh"
 #include "internal.cuh"
 #include "mixed.cuh"
+#include "once.cuh"
 #include "profiler.cuh"
 #include "stages.cuh"
 
@@ -574,15 +575,12 @@ __global__ void __launch_bounds__(256) k_jac_t(const Dims* __restrict__ dims, co
 }
 
 cudaError_t jac_pre_prepare() {
-  static int done = 0;
-  if (!done) {
+  static DeviceOnce once;
+  return once([] {
     const int b = (int)(sizeof(float2) * JP_MAXL * JP_MAXL);
-    cudaError_t e = cudaFuncSetAttribute(k_jac_pre, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_jac_step, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e != cudaSuccess) return e;
-    done = 1;
-  }
-  return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(k_jac_pre, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_jac_step, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  });
 }
 
 __global__ void k_jac_none(Dims* dims, int batch) {

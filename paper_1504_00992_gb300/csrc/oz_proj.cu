@@ -73,6 +73,7 @@
 #include "dfsplit.cuh"
 #include "internal.cuh"
 #include "mixed.cuh"
+#include "once.cuh"
 #include "profiler.cuh"
 #include "stages.cuh"
 #include "tc_sync.cuh"
@@ -882,8 +883,8 @@ static cudaError_t oz_attr() {
 }
 
 cudaError_t oz_prepare() {
-  static int done = 0;
-  if (!done) {
+  static DeviceOnce once;
+  return once([] {
     const cudaError_t es[] = {
         oz_attr<OZ_CONT>(), oz_attr<OZ_GRAMY>(), oz_attr<OZ_GRAMT>(),
         oz_attr<OZ_PROJ>(), oz_attr<OZ_GRAM>(), oz_attr<OZ_THETA>(), oz_attr<OZ_GATE>(), oz_attr<G_X>(),
@@ -894,9 +895,8 @@ cudaError_t oz_prepare() {
         oz_attr<G_XG>(),    oz_attr<G_XT>()};
     for (cudaError_t e : es)
       if (e != cudaSuccess) return e;
-    done = 1;
-  }
-  return cudaSuccess;
+    return cudaSuccess;
+  });
 }
 
 // Capacities (rows of C, columns of C, depth) of a stage's product.

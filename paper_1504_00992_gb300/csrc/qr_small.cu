@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "once.cuh"
 #include "profiler.cuh"
 #include "stages.cuh"
 
@@ -105,13 +106,12 @@ static cudaError_t qs_attr() {
 }
 
 cudaError_t qr_small_prepare() {
-  static int done = 0;
-  if (!done) {
+  static DeviceOnce once;
+  return once([] {
     for (cudaError_t e : {qs_attr<QR_Y>(), qs_attr<QR_YT>(), qs_attr<QR_BH>()})
       if (e != cudaSuccess) return e;
-    done = 1;
-  }
-  return cudaSuccess;
+    return cudaSuccess;
+  });
 }
 
 cudaError_t launch_qr_small(int stage, const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap,

@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include "internal.cuh"
+#include "once.cuh"
 #include "profiler.cuh"
 #include "stages.cuh"
 
@@ -85,17 +86,24 @@ __global__ void __launch_bounds__(GS_T) k_gate_small(const Dims* __restrict__ di
 
 static size_t gs_smem(int dd) { return sizeof(cplx) * ((size_t)dd * GS_T + (size_t)dd * dd); }
 
+static const size_t TH_SMEM = sizeof(cplx) * (2 * TH_TK * TH_MAXR + TH_MAXR * TH_MAXR);
+
+cudaError_t theta_prepare() {
+  static DeviceOnce once;
+  return once([] {
+    const cudaError_t e = cudaFuncSetAttribute(k_gate_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)gs_smem(GATE_GEMM_MIN - 1));
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_theta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TH_SMEM);
+  });
+}
+
 cudaError_t launch_gate_small(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int need_dig,
                               cudaStream_t st) {
   // (cap.dl cap.dr may come from different bonds; those of GATE_GEMM_MIN and more have their own path)
   const int dd = cap.dl * cap.dr < GATE_GEMM_MIN ? cap.dl * cap.dr : GATE_GEMM_MIN - 1;
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_gate_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)gs_smem(GATE_GEMM_MIN - 1));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  const cudaError_t e = theta_prepare();
+  if (e != cudaSuccess) return e;
   ProfScope ps("k_theta", st);
   size_t gx = ((size_t)cap.cl * cap.cr + GS_T - 1) / GS_T;
   const size_t most = (8 * 152 * 8 + batch - 1) / batch;
@@ -187,14 +195,10 @@ cudaError_t launch_theta(const Dims* dims, const ProbPtr* ptrs, int batch, const
   const int TA = (cap.dl >= 32) ? 1 : 32 / cap.dl;
   const int TB = (cap.dr >= 32) ? 1 : 32 / cap.dr;
   dim3 grid((cap.cr + TB - 1) / TB, (cap.cl + TA - 1) / TA, batch);
-  const size_t smem = sizeof(cplx) * (2 * TH_TK * TH_MAXR + TH_MAXR * TH_MAXR);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_theta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  const cudaError_t e = theta_prepare();
+  if (e != cudaSuccess) return e;
   ProfScope ps("k_theta", st);
-  k_theta<<<grid, 256, smem, st>>>(dims, ptrs, identity_gate, skip_pre, skip_dig);
+  k_theta<<<grid, 256, TH_SMEM, st>>>(dims, ptrs, identity_gate, skip_pre, skip_dig);
   return cudaGetLastError();
 }
 
