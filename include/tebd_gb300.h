@@ -131,8 +131,12 @@ typedef struct {
                            tensor cores: the choices of an FP64 handle leave every bit
                            as it is); TF32 -- the mixed form's choices as for
                            rrsvd_plan_autotune */
-  size_t workspace_budget; /* bytes of per-bond workspace one wave may use (0 = all bonds
-                              of a parity in one wave); larger batches run in waves */
+  size_t workspace_budget; /* bytes of workspace one wave may use (0 = all bonds of a
+                              parity in one wave); larger batches run in waves.  It
+                              covers the per-bond workspace, a mixed form's FP32 arrays
+                              and the operand digits of FP64 bonds on the tensor cores
+                              (those at most a quarter of it, 6 GiB without a budget);
+                              one bond's needs are granted whatever the budget */
   tebd_alloc_fn alloc;     /* optional: allocator of every device block of the handle
                               (read from descs[0]); with release, or both NULL */
   tebd_release_fn release;
@@ -330,8 +334,13 @@ typedef struct rrsvd_plan_s* rrsvd_plan_t;
  * iterations.  Instance t of a call uses Philox counter chain = chain0 + t,
  * bond 0, sweep 0.  precision: TEBD_PREC_FP64, TEBD_PREC_TF32 or
  * TEBD_PREC_BF16 (the workspace then also holds FP32 copies of theta, about
- * 4 m n 8 bytes per instance, and with BF16 half as much again).  Errors: TEBD_EINVAL (m, n, batch < 1, k_max < 1, p < 0,
- * q < 0), TEBD_ENOTIMPL (precision, or l > 512). */
+ * 4 m n 8 bytes per instance, and with BF16 half as much again).  The
+ * workspace of an FP64 plan on the tensor cores (TEBD_PREC_FP64) also holds
+ * operand digits: 28 bytes per entry of theta for each of its two
+ * directions, and of the bases, for all instances where that is at most
+ * 6 GiB, else for as many as fit 6 GiB (one at least), by turns.
+ * Errors: TEBD_EINVAL (m, n, batch < 1, k_max < 1, p < 0, q < 0),
+ * TEBD_ENOTIMPL (precision, or l > 512). */
 int rrsvd_plan_create(int m, int n, int k_max, int p, int q, int batch, int precision, uint64_t seed,
                       rrsvd_plan_t* out);
 int rrsvd_plan_destroy(rrsvd_plan_t plan);

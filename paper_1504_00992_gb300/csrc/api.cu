@@ -576,7 +576,11 @@ static int plan_handle(tebd_s* h, int n_chains, const tebd_desc_t* descs, Handle
       cp.cl = std::max(cp.cl, C.cap_ext[b]); cp.cr = std::max(cp.cr, C.cap_ext[b + 2]);
       cp.cm = std::max(cp.cm, C.cap_ext[b + 1]);
       cp.dl = std::max(cp.dl, C.d[b]); cp.dr = std::max(cp.dr, C.d[b + 1]);
-      const size_t mix = tf32 ? mixed_bytes(mixed_sizes(cp.m, cp.n, cp.k, cp.l, bf16, &cp), w.count + 1) : 0;
+      // the wave's arrays besides the per-bond workspace: a mixed form's FP32
+      // arrays, or an FP64 wave's digits (one rule for both: inside the budget)
+      const size_t mix = tf32 ? mixed_bytes(mixed_sizes(cp.m, cp.n, cp.k, cp.l, bf16, &cp), w.count + 1)
+                         : digits && dp_rule(cp.m, cp.n, cp.l) ? dp_bytes(cp, w.count + 1, lay_plan.dp_limit)
+                                                               : 0;
       if (w.count > 0 && budget > 0 && acc + pbytes[par][i] + mix > budget) {
         ps.waves.push_back(w);
         ws_max = std::max(ws_max, acc);

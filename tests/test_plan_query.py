@@ -123,3 +123,20 @@ def test_a_handle_larger_than_any_device_reports_enomem():
     with pytest.raises(B.TebdError) as e:
         B.tebd_create_multi(chains, 10, 2, 0)
     assert e.value.code == B.TEBD_ENOMEM
+
+
+@pytest.mark.parametrize("gb", [0.25, 0.5, 1, 2, 4])
+@pytest.mark.parametrize("spec", [(40, 2, 128), (60, 2, 100), (30, 3, 96)])
+def test_an_fp64_handle_keeps_its_digits_inside_the_budget(spec, gb):
+    """The budget bounds what a wave may use: its bonds' workspace and, for
+    bonds on the tensor cores, their digits.  An arena is the state and the
+    descriptors (what a one-byte budget's arena holds besides its largest
+    bond) plus the largest wave, so it stays below that arena plus the
+    budget wherever one bond fits it."""
+    budget = int(gb * (1 << 30))
+    chains = [_chain(*spec)] * 8
+    state, _, _ = B.tebd_plan_query(chains, 10, 2, 0, workspace_budget=1)
+    arena, we, wo = B.tebd_plan_query(chains, 10, 2, 0, workspace_budget=budget)
+    full, _, _ = B.tebd_plan_query(chains, 10, 2, 0)
+    assert arena <= state + budget
+    assert arena <= full
