@@ -29,6 +29,7 @@ struct Dims {
   int cq;          // Cholesky QR: the last pass this problem takes part in
   int cf;          // Cholesky QR: given up, the Householder QR factors it
   int js;          // small SVD: 1: J holds rotations already applied to X, 2: X's columns are orthogonal too
+  int gr;          // mixed forms: theta's rows are graded (k_graded), its basis takes seven digits
 };
 
 // Sizes from which the FP64 form's products and QRs run on the tensor cores

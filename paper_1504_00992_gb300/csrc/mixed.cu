@@ -65,6 +65,44 @@ __device__ __forceinline__ float tf32_rna(float x) {
 //   152 x 2000 x 2000 step).
 // The tiles cover the zero padding of every copy.
 // ---------------------------------------------------------------------------
+// Whether theta's rows are graded: a row (other than a zero one) whose largest
+// entry in the last sketch Y = A Q~ is below 2^-GR_SPAN of Y's.  The FP32 chain
+// forms a row of the basis with errors relative to the row's own size (a few
+// 1e-6); the basis's four digits round its entries at 2^-32 of the largest of
+// a column, which is below that while the rows are alike, but takes a small
+// row's bits away (rows of U at 2^-30 were off by half of themselves): such an
+// instance takes seven (its projection and Gram matrix cost 1.27 times the
+// digit pairs).  span[z]: the largest exponent and 0x7FF minus the smallest
+// one of a row; zero before.  Bound by reading Y; with the launches of the
+// seven-digit kernels that find nothing 0.4 of the 71 ms of a step of
+// 152 x 2000 x 2000 whose rows are alike.
+enum { GR_SPAN = 13 };
+__global__ void __launch_bounds__(256) k_row_span(const Dims* __restrict__ dims, const float2* __restrict__ Yf,
+                                                  int2* span, int mc, int lc) {
+  const int z = blockIdx.y, r = blockIdx.x * 256 + threadIdx.x;
+  const Dims D = dims[z];
+  if (!D.active) return;
+  int e = 0;
+  if (r < D.m) {
+    const float2* y = Yf + (size_t)z * mc * lc + r;
+#pragma unroll 8
+    for (int i = 0; i < D.l; ++i) {
+      const float2 v = y[(size_t)i * mc];
+      e = max(e, max(oz_exp(v.x), oz_exp(v.y)));
+    }
+  }
+  const int hi = __reduce_max_sync(0xffffffffu, e);
+  const int lo = __reduce_max_sync(0xffffffffu, e > 0 ? 0x7FF - e : 0);
+  if ((threadIdx.x & 31) == 0 && hi > 0) {
+    atomicMax(&span[z].x, hi);
+    atomicMax(&span[z].y, lo);
+  }
+}
+__global__ void k_graded(Dims* dims, const int2* __restrict__ span, int batch) {
+  const int z = blockIdx.x * blockDim.x + threadIdx.x;
+  if (z < batch) dims[z].gr = (0x7FF - span[z].y) + GR_SPAN < span[z].x ? 1 : 0;
+}
+
 // double-float pair sum (Knuth's TwoSum on the high words)
 __device__ __forceinline__ void df_add2(float& h, float& l, float oh, float ol) {
   const float s = h + oh;
@@ -486,8 +524,9 @@ MixedSizes mixed_sizes(int m, int n, int k, int l, int bf16, const Caps* gate) {
   // the projection runs on the tensor cores from BF16 digits (oz_proj.cu)
   s.bd = oz_digits_bytes(n, m);
   s.bsc = oz_scales_bytes(n);
-  s.ad = oz_digits_q_bytes(l, m);
+  s.ad = oz_digits_bytes(l, m);  // (of a graded basis; others use four of the seven)
   s.asc = oz_scales_bytes(l);
+  s.span = sizeof(int2);
   s.thfb = s.bf16 ? (size_t)m * s.K1b * 2 : 0;
   s.thab = s.bf16 ? (size_t)n * s.K2b * 2 : 0;
   s.btb = s.bf16 ? (size_t)s.Np * (s.K1b > s.K2b ? s.K1b : s.K2b) * 2 : 0;
@@ -516,7 +555,7 @@ size_t mixed_bytes(const MixedSizes& s, int batch) {
   return 2 * up256(s.thf * batch) + 2 * up256(s.tha * batch) + 2 * up256(s.bt * batch) + 2 * up256(s.yf * batch) +
          2 * up256(s.ytf * batch) + up256(s.df * batch) +
          up256((size_t)s.ntile * sizeof(double) * batch) + up256(s.qs * batch) + up256(s.bd * batch) +
-         up256(s.bsc * batch) + up256(s.ad * batch) + up256(s.asc * batch) + up256(s.thfb * batch) +
+         up256(s.bsc * batch) + up256(s.ad * batch) + up256(s.asc * batch) + up256(s.span * batch) + up256(s.thfb * batch) +
          up256(s.thab * batch) + up256(s.btb * batch) + up256(s.gad * batch) + up256(s.gas * batch) +
          up256(s.gbd * batch) + up256(s.gbs * batch);
 }
@@ -543,6 +582,7 @@ MixedPtrs mixed_carve(char* base, const MixedSizes& s, int batch) {
   p.bsc = (int*)(base + o); o += up256(s.bsc * batch);
   p.ad = (uint16_t*)(base + o); o += up256(s.ad * batch);
   p.asc = (int*)(base + o); o += up256(s.asc * batch);
+  p.span = (int2*)(base + o); o += up256(s.span * batch);
   p.thf_b = s.bf16 ? (uint16_t*)(base + o) : nullptr; o += up256(s.thfb * batch);
   p.tha_b = s.bf16 ? (uint16_t*)(base + o) : nullptr; o += up256(s.thab * batch);
   p.bt_b = s.bf16 ? (uint16_t*)(base + o) : nullptr; o += up256(s.btb * batch);
@@ -574,6 +614,7 @@ MixedPtrs mixed_offset(const MixedPtrs& p, const MixedSizes& s, int z0) {
   o.bsc = adv(p.bsc, s.bsc);
   o.ad = adv(p.ad, s.ad);
   o.asc = adv(p.asc, s.asc);
+  o.span = adv(p.span, s.span);
   o.thf_b = adv(p.thf_b, s.thfb);
   o.tha_b = adv(p.tha_b, s.thab);
   o.bt_b = adv(p.bt_b, s.btb);
@@ -808,6 +849,13 @@ cudaError_t run_rrsvd_mixed(const Dims* dims, const ProbPtr* ptrs, int batch, co
   // Plans and handles refuse sketches wider than 512 columns, and l <= m, so
   // every basis they pass fits it.
   if (!reorth_fits(m, l)) return cudaErrorInvalidValue;
+  {
+    ProfScope ps("k_row_span", st);
+    MX_TRY(cudaMemsetAsync(mp.span, 0, s.span * batch, st));
+    k_row_span<<<dim3((m + 255) / 256, batch), 256, 0, st>>>(dims, mp.Yf, mp.span, m, l);
+    k_graded<<<(batch + 127) / 128, 128, 0, st>>>(const_cast<Dims*>(dims), mp.span, batch);
+    MX_TRY(cudaGetLastError());
+  }
   MX_TRY(qr(mp.Yf, mp.Qf, m, 0, true));
   // digits of Q_f once: the Gram of the re-orthonormalisation and the
   // projection A^H Q_f both take them

@@ -17,6 +17,7 @@ struct MixedSizes {
   int BN;        // tensor-core tile width, min(Np, 256)
   size_t thf, tha, bt, yf, ytf, df;  // bytes per instance
   size_t bd, bsc, ad, asc;  // BF16 digits and row exponents of theta and of Q_f^H (tensor-core projection)
+  size_t span;              // exponent range of the last sketch's rows (k_row_span)
   size_t thfb, thab, btb;   // BF16 copies of theta, theta^H and Bt (bf16 only)
   size_t gad, gas, gbd, gbs;  // digit scratch of the other tensor-core products (oz_stage_bytes)
   size_t qs;     // bytes per instance of the many-CTA FP32 QR's scratch (0: not used)
@@ -40,6 +41,7 @@ struct MixedPtrs {
   int* bsc;       // their rows' largest exponents
   uint16_t* ad;   // digits of Q_f^H
   int* asc;
+  int2* span;
   uint16_t* thf_b;  // m x K1b BF16 theta (bf16 form), or null
   uint16_t* tha_b;  // n x K2b BF16 theta^H
   uint16_t* bt_b;   // Np x max(K1b, K2b) BF16 right operand
@@ -165,7 +167,9 @@ cudaError_t dp_begin(const DpPath& p);  // theta's digits, when they are kept
 // (DPC_WIDE: those of at least DP_WIDE_L columns; a handle's wave also holds bonds
 // far below its capacities, whose Householder QR and double-float Jacobi are
 // cheaper than the passes and products of the digit forms)
-enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_JS = 16, DPC_WIDE = 32, DPC_PASS = 8 };
+// (DPC_GRADED, DPC_FLAT: by Dims::gr)
+enum { DPC_OK = 1, DPC_QFLAG = 2, DPC_DIG = 4, DPC_CHK = 8, DPC_JS = 16, DPC_WIDE = 32, DPC_GRADED = 64, DPC_FLAT = 128,
+       DPC_PASS = 8 };
 enum { DP_WIDE_L = 40 };
 cudaError_t launch_dp_stage(int stage, const DpPath& p, int cond);
 // Cholesky QR of Y into Q (side 0) or Yt into Qt (side 1) (cholqr.cu): up to
@@ -217,7 +221,8 @@ cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const uint16_t
                            const uint16_t* Bd, const int* Bs, int m, int n, int l, int batch, int* err,
                            cudaStream_t st);
 // Digits of Q_f (the projection's left operand, conjugated by the MMAs; Q_f's
-// entries are rounded to what its four digits hold) into Ad / As, and the
+// entries are rounded to what its four digits hold, or where theta's rows are
+// graded take seven as they are) into Ad (room for seven) / As, and the
 // Gram matrix E = Q_f^H Q_f - I of the re-orthonormalisation from them into
 // ptrs[z].R (l x l column-major), FP64-accurate, on the tensor cores.
 cudaError_t launch_oz_digits_qf(const Dims* dims, const ProbPtr* ptrs, float2* Qf, uint16_t* Ad, int* As, int m, int l, int batch,

@@ -88,7 +88,7 @@ enum {
   OZ_BM = 128,     // rows of C per CTA (TMEM lanes)
   OZ_BN = 32,      // columns of C per CTA
   OZ_DRAIN = 64,   // k per exact accumulation (the accumulators are read and cleared after each)
-  OZ_SQ = 4,       // digits of the FP32 basis Q_f
+  OZ_SQ = 4,       // digits of the FP32 basis Q_f (of a theta whose rows are not graded)
   OZ_EPI_WARPS = 16,  // four per TMEM lane quadrant, 8 columns each
   OZ_THREADS = 64 + 32 * OZ_EPI_WARPS,
   OZ_NGRP = OZ_S,  // accumulators per part: levels 2 .. 8
@@ -115,14 +115,21 @@ __device__ __forceinline__ int64_t oz_fix(double x, int E) {
   const int64_t n = sh <= 0 ? (m << (-sh)) : (sh >= 56 ? 0 : ((m + (1ll << (sh - 1))) >> sh));
   return (u >> 63) ? -n : n;
 }
-// N = rint(x 2^(30 - (E - 1023))) of an FP32 value, |N| < 2^31 (E the row's largest exponent)
-__device__ __forceinline__ int64_t oz_fix31(float x, int E) {
+// The same of an FP32 value for NS = 7 digits; for four, N = rint(x 2^(30 - (E - 1023))),
+// |N| < 2^31 (E the row's largest exponent)
+template <int NS>
+__device__ __forceinline__ int64_t oz_fix_f32(float x, int E) {
   const unsigned u = __float_as_uint(x);
   const int e = (int)((u >> 23) & 0xFF);
   if (e == 0 || e == 0xFF) return 0;
   const int m = (int)((u & 0x7FFFFFu) | 0x800000u);
-  const int sh = E - (e - 127 + 1023) - 7;  // x = m 2^(e - 150), N = m 2^-sh; sh >= -7
-  const int n = sh <= 0 ? (m << (-sh)) : (sh >= 26 ? 0 : ((m + (1 << (sh - 1))) >> sh));
+  if constexpr (NS == OZ_SQ) {
+    const int sh = E - (e - 127 + 1023) - 7;  // x = m 2^(e - 150), N = m 2^-sh; sh >= -7
+    const int n = sh <= 0 ? (m << (-sh)) : (sh >= 26 ? 0 : ((m + (1 << (sh - 1))) >> sh));
+    return (u >> 31) ? -n : n;
+  }
+  const int sh = E - (e - 127 + 1023) - 31;  // sh >= -31
+  const int64_t n = sh <= 0 ? ((int64_t)m << (-sh)) : (sh >= 26 ? 0 : ((m + (1 << (sh - 1))) >> sh));
   return (u >> 31) ? -n : n;
 }
 
@@ -177,11 +184,18 @@ __device__ __forceinline__ double oz_scale(int E) {
 // k_cgemm_df<DgTheta> / <DgGate> (df_gemm.cu documents the operands).
 // OZ_GRAMY, OZ_GRAMT: Gram matrices of FP32 sketches (m or n rows), as OZ_GRAM
 // but without subtracting the identity.
+// OZ_PROJ7, OZ_GRAM7: OZ_PROJ and OZ_GRAM of the instances whose Q_f takes seven
+// digits (Dims::gr).
 enum { OZ_PROJ = 100, OZ_GRAM = 101, OZ_THETA = 102, OZ_GATE = 103, OZ_GRAMY = 104, OZ_GRAMT = 105,
+       OZ_PROJ7 = 107, OZ_GRAM7 = 108,
        OZ_CONT = 106 };  // OZ_THETA for the bonds of theta_digits_rule without a pre-gate buffer, into theta
 template <int ST>
 struct OzFp32Gram {
-  static constexpr bool yes = ST == OZ_GRAM || ST == OZ_GRAMY || ST == OZ_GRAMT;
+  static constexpr bool yes = ST == OZ_GRAM || ST == OZ_GRAM7 || ST == OZ_GRAMY || ST == OZ_GRAMT;
+};
+template <int ST>
+struct OzProj {
+  static constexpr bool yes = ST == OZ_PROJ || ST == OZ_PROJ7;
 };
 static_assert(OZ_THETA == OZ_THETA_STAGE && OZ_GATE == OZ_GATE_STAGE && OZ_CONT == OZ_CONT_STAGE,
               "stage ids of mixed.cuh");
@@ -195,7 +209,7 @@ struct OzOp {
 template <int ST>
 __device__ __forceinline__ OzOp oz_op(const Dims& D, const ProbPtr& P) {
   OzOp o;
-  if constexpr (ST == OZ_PROJ) {
+  if constexpr (OzProj<ST>::yes) {
     o.M = D.l; o.N = D.n; o.K = D.m;
     o.C = P.Yt; o.crs = D.n; o.ccs = 1;  // element (j, i) of the n x l column-major B^H
   } else if constexpr (OzFp32Gram<ST>::yes) {
@@ -218,15 +232,16 @@ __device__ __forceinline__ OzOp oz_op(const Dims& D, const ProbPtr& P) {
 template <int ST>
 struct OzConj {
   static constexpr bool own = ST < OZ_PROJ;  // a GemmStage of stages.cuh
-  static constexpr bool A = ST == OZ_PROJ || OzFp32Gram<ST>::yes || (own && StageFlags<ST>::conjA);  // Q_f^H
-  static constexpr bool C = ST == OZ_PROJ || (own && StageFlags<ST>::conjC);
+  static constexpr bool A = OzProj<ST>::yes || OzFp32Gram<ST>::yes || (own && StageFlags<ST>::conjA);  // Q_f^H
+  static constexpr bool C = OzProj<ST>::yes || (own && StageFlags<ST>::conjC);
 };
 
 // Digits of each operand and the ring of stages of a product.
 template <int ST>
 struct OzGeo {
-  static constexpr int SA = (ST == OZ_PROJ || OzFp32Gram<ST>::yes) ? OZ_SQ : OZ_S;
-  static constexpr int SB = OzFp32Gram<ST>::yes ? OZ_SQ : OZ_S;
+  static constexpr bool four = OzFp32Gram<ST>::yes && ST != OZ_GRAM7;
+  static constexpr int SA = (ST == OZ_PROJ || four) ? OZ_SQ : OZ_S;
+  static constexpr int SB = four ? OZ_SQ : OZ_S;
   static constexpr uint32_t A_STAGE = 2 * SA * OZ_A_TILE, B_STAGE = 2 * SB * OZ_B_TILE;
   static constexpr int STAGES = SA == OZ_S ? 3 : 4;
   static constexpr size_t smem = 1024 + (size_t)STAGES * (A_STAGE + B_STAGE) + (2 * STAGES + 3) * 8 + 16;
@@ -249,6 +264,8 @@ __device__ __forceinline__ bool oz_takes(const Dims& D, int cond) {
   if ((cond & DPC_CHK) && !D.chk) return false;
   if ((cond & DPC_JS) && D.js != 1) return false;
   if ((cond & DPC_WIDE) && D.l < DP_WIDE_L) return false;
+  if ((cond & DPC_GRADED) && !D.gr) return false;
+  if ((cond & DPC_FLAT) && D.gr) return false;
   return true;
 }
 
@@ -263,7 +280,7 @@ __device__ __forceinline__ void oz_store(const Dims& D, const ProbPtr& P, const 
     const int a = i / D.dr, b = i - a * D.dr, al = j / D.cr, be = j - al * D.cr;  // rows (i, j), columns (alpha, beta)
     op.C[(int64_t)(a * D.cl + al) * D.n + b * D.cr + be] = cmk(re, im);
   } else {
-    if (ST == OZ_GRAM && i == j) re -= 1.0;  // E = Q_f^H Q_f - I
+    if ((ST == OZ_GRAM || ST == OZ_GRAM7) && i == j) re -= 1.0;  // E = Q_f^H Q_f - I
     op.C[(int64_t)i * op.crs + (int64_t)j * op.ccs] = cmk(re, OzConj<ST>::C ? -im : im);
   }
 }
@@ -497,13 +514,16 @@ __global__ void __launch_bounds__(256) k_oz_digits_two(const Dims* __restrict__ 
 // the numbers the digits hold exactly (entries above 2^-8 of the largest one
 // keep all their 24 bits).  Against seven digits the projection loads 47 KB
 // instead of 72 KB per k step and runs 22 digit pairs instead of 28.  The same
-// numbers go to P.Q in FP64, the left operand of U = Q_f (I + D) J_k.
-// ROUND false: the digits alone, of a sketch with m or (use_n) n rows.
-template <bool ROUND>
+// numbers go to P.Q in FP64, the left operand of U = Q_f (I + D) J_k.  Where
+// theta's rows are graded (NS = OZ_S) it is seven digits, exact down to 2^-31 of
+// the largest entry, and nothing is rounded.
+// BASIS false: the digits alone, of a sketch with m or (use_n) n rows.
+// (zs: digits of Ad per instance)
+template <bool BASIS, int NS>
 __global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ dims,
                                                      const ProbPtr* __restrict__ ptrs, float2* __restrict__ Qf,
-                                                     uint16_t* Ad, int* Es, int mc, int lc, int Kp, int use_n,
-                                                     int cond) {
+                                                     uint16_t* Ad, size_t zs, int* Es, int mc, int lc, int Kp,
+                                                     int use_n, int cond) {
   const int z = blockIdx.y;
   const Dims D = dims[z];
   if (!D.active || !oz_takes(D, cond)) return;
@@ -523,29 +543,32 @@ __global__ void __launch_bounds__(256) k_oz_digits_q(const Dims* __restrict__ di
   if (lane == 0) Es[(size_t)z * lc + i] = E;
   // x = N 2^(E - 1023 - 30), the scale as an FP32 number (a Q_f column has unit norm: E far from its ends)
   const float unit = __uint_as_float((unsigned)max(1, min(254, E - 1023 - 30 + 127)) << 23);
-  uint16_t* base = Ad + (size_t)z * 2 * OZ_SQ * lc * Kp;
+  uint16_t* base = Ad + z * zs;
   const int kend = min(Kp, ((Mi + OZ_KB - 1) / OZ_KB) * OZ_KB);
   for (int k = 4 * lane; k < kend; k += 128) {
     int64_t nr[4], ni[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const float2 v = (k + u < K) ? q[k + u] : make_float2(0.f, 0.f);
-      nr[u] = oz_fix31(v.x, E);
-      ni[u] = oz_fix31(v.y, E);
-      if (ROUND && k + u < K) {
-        const float2 r = make_float2((float)(int)nr[u] * unit, (float)(int)ni[u] * unit);
-        q[k + u] = r;
+      nr[u] = oz_fix_f32<NS>(v.x, E);
+      ni[u] = oz_fix_f32<NS>(v.y, E);
+      if (BASIS && k + u < K) {
+        float2 r = v;
+        if (NS == OZ_SQ) {
+          r = make_float2((float)(int)nr[u] * unit, (float)(int)ni[u] * unit);
+          q[k + u] = r;
+        }
         Qd[k + u] = cmk((double)r.x, (double)r.y);
       }
     }
-    uint2 d[OZ_SQ];
-    uint16_t* at = base + oz_at<OZ_SQ>(k >> 4, 0, i, (k >> 3) & 1, lc) + (k & 4);
-    oz_digits4<OZ_SQ>(nr, d);
+    uint2 d[NS];
+    uint16_t* at = base + oz_at<NS>(k >> 4, 0, i, (k >> 3) & 1, lc) + (k & 4);
+    oz_digits4<NS>(nr, d);
 #pragma unroll
-    for (int t = 0; t < OZ_SQ; ++t) *reinterpret_cast<uint2*>(at + (size_t)t * lc * OZ_KS) = d[t];
-    oz_digits4<OZ_SQ>(ni, d);
+    for (int t = 0; t < NS; ++t) *reinterpret_cast<uint2*>(at + (size_t)t * lc * OZ_KS) = d[t];
+    oz_digits4<NS>(ni, d);
 #pragma unroll
-    for (int t = 0; t < OZ_SQ; ++t) *reinterpret_cast<uint2*>(at + (size_t)(OZ_SQ + t) * lc * OZ_KS) = d[t];
+    for (int t = 0; t < NS; ++t) *reinterpret_cast<uint2*>(at + (size_t)(NS + t) * lc * OZ_KS) = d[t];
   }
 }
 
@@ -556,6 +579,7 @@ struct OzArgs {
   const uint16_t* Ad;  // digits of both operands (oz_at)
   const uint16_t* Bd;
   int lc, nc, Kp;      // capacities: rows of C, columns of C, padded k
+  size_t az, bz;       // digits per instance
   const int* As;       // [z][i] largest biased exponents of the left operand's rows
   const int* Bs;       // [z][j]
   int* err;
@@ -697,7 +721,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int plane = isA ? lane : lane - 2 * SA, row0 = isA ? i0 : j0, rc = isA ? a.lc : a.nc;
     const int na = min((int)OZ_BM, a.lc - i0), nb = min((int)OZ_BN, a.nc - j0);  // rows copied
     const uint32_t bytes = (uint32_t)(isA ? na : nb) * (OZ_KS * 2);
-    const uint16_t* src = (isA ? a.Ad : a.Bd) + (size_t)z * (isA ? 2 * SA : 2 * SB) * rc * a.Kp + ((size_t)plane * rc + row0) * OZ_KS;
+    const uint16_t* src = (isA ? a.Ad : a.Bd) + z * (isA ? a.az : a.bz) + ((size_t)plane * rc + row0) * OZ_KS;
     const size_t step = (size_t)(isA ? 2 * SA : 2 * SB) * rc * OZ_KS;
     uint8_t* dst = (isA ? sA : sB) + (size_t)plane * (isA ? OZ_A_TILE : OZ_B_TILE);
     const uint32_t stage = isA ? Geo::A_STAGE : Geo::B_STAGE;
@@ -887,6 +911,7 @@ cudaError_t oz_prepare() {
   return once([] {
     const cudaError_t es[] = {
         oz_attr<OZ_CONT>(), oz_attr<OZ_GRAMY>(), oz_attr<OZ_GRAMT>(),
+        oz_attr<OZ_PROJ7>(), oz_attr<OZ_GRAM7>(),
         oz_attr<OZ_PROJ>(), oz_attr<OZ_GRAM>(), oz_attr<OZ_THETA>(), oz_attr<OZ_GATE>(), oz_attr<G_X>(),
         oz_attr<G_U>(),     oz_attr<G_V>(),     oz_attr<G_Y0>(),     oz_attr<G_Y>(),     oz_attr<G_YT>(),
         oz_attr<G_BH>(),    oz_attr<G_PR>(),    oz_attr<G_PQ>(),     oz_attr<G_PD>(),    oz_attr<G_CYG>(),
@@ -997,6 +1022,8 @@ static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch
   oa.lc = Mc;
   oa.nc = Nc;
   oa.Kp = Kp;
+  oa.az = (size_t)2 * OZ_S * Mc * Kp;
+  oa.bz = (size_t)2 * OZ_S * Nc * Kp;
   oa.As = pre ? pre_es : sc.as;
   oa.Bs = same ? oa.As : sc.bs;
   oa.err = err;
@@ -1196,17 +1223,21 @@ cudaError_t launch_oz_digits_theta(const Dims* dims, const ProbPtr* ptrs, uint16
   return cudaGetLastError();
 }
 
+// The digits of Q_f: per instance four or seven of the seven planes' room.
 cudaError_t launch_oz_digits_qf(const Dims* dims, const ProbPtr* ptrs, float2* Qf, uint16_t* Ad, int* As, int m, int l, int batch,
                                 cudaStream_t st) {
   const int Kp = oz_kpad(m);
+  const size_t zs = (size_t)2 * OZ_S * l * Kp;
+  const dim3 grid((l + 7) / 8, batch);
   ProfScope ps("k_oz_digits[q]", st);
-  k_oz_digits_q<true><<<dim3((l + 7) / 8, batch), 256, 0, st>>>(dims, ptrs, Qf, Ad, As, m, l, Kp, 0, 0);
+  k_oz_digits_q<true, OZ_SQ><<<grid, 256, 0, st>>>(dims, ptrs, Qf, Ad, zs, As, m, l, Kp, 0, DPC_FLAT);
+  k_oz_digits_q<true, OZ_S><<<grid, 256, 0, st>>>(dims, ptrs, Qf, Ad, zs, As, m, l, Kp, 0, DPC_GRADED);
   return cudaGetLastError();
 }
 
 cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t* Ad, const int* As, int m, int l,
                            int batch, int* err, cudaStream_t st) {
-  const cudaError_t e = oz_prepare();
+  cudaError_t e = oz_prepare();
   if (e != cudaSuccess) return e;
   const int Kp = oz_kpad(m);
   OzArgs oa;
@@ -1214,14 +1245,17 @@ cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t
   oa.lc = l;
   oa.nc = l;
   oa.Kp = Kp;
+  oa.az = oa.bz = (size_t)2 * OZ_S * l * Kp;
   oa.As = As;
   oa.Bs = As;
   oa.err = err;
   oa.poll_limit = 1u << 24;
   oa.stall = 0;
-  oa.cond = 0;
+  oa.cond = DPC_FLAT;
   ProfScope ps("k_oz_gemm[gram]", st);
-  return oz_launch<OZ_GRAM>(l, l, batch, dims, ptrs, oa, st);
+  if ((e = oz_launch<OZ_GRAM>(l, l, batch, dims, ptrs, oa, st)) != cudaSuccess) return e;
+  oa.cond = DPC_GRADED;
+  return oz_launch<OZ_GRAM7>(l, l, batch, dims, ptrs, oa, st);
 }
 
 cudaError_t launch_oz_gram_f32(const Dims* dims, const ProbPtr* ptrs, const float2* X, uint16_t* Ad, int* As, int M,
@@ -1231,8 +1265,8 @@ cudaError_t launch_oz_gram_f32(const Dims* dims, const ProbPtr* ptrs, const floa
   const int Kp = oz_kpad(M);
   {
     ProfScope ps("k_oz_digits[q]", st);
-    k_oz_digits_q<false><<<dim3((l + 7) / 8, batch), 256, 0, st>>>(dims, ptrs, const_cast<float2*>(X), Ad, As, M, l,
-                                                                   Kp, use_n, cond);
+    k_oz_digits_q<false, OZ_SQ><<<dim3((l + 7) / 8, batch), 256, 0, st>>>(
+        dims, ptrs, const_cast<float2*>(X), Ad, (size_t)2 * OZ_SQ * l * Kp, As, M, l, Kp, use_n, cond);
     const cudaError_t e2 = cudaGetLastError();
     if (e2 != cudaSuccess) return e2;
   }
@@ -1240,6 +1274,7 @@ cudaError_t launch_oz_gram_f32(const Dims* dims, const ProbPtr* ptrs, const floa
   oa.Ad = oa.Bd = Ad;
   oa.lc = oa.nc = l;
   oa.Kp = Kp;
+  oa.az = oa.bz = (size_t)2 * OZ_SQ * l * Kp;
   oa.As = oa.Bs = As;
   oa.err = err;
   oa.poll_limit = 1u << 24;
@@ -1261,6 +1296,8 @@ cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const uint16_t
     oa.lc = l;
     oa.nc = n;
     oa.Kp = Kp;
+    oa.az = (size_t)2 * OZ_S * l * Kp;
+    oa.bz = (size_t)2 * OZ_S * n * Kp;
     oa.As = As;
     oa.Bs = Bs;
     oa.err = err;
@@ -1270,10 +1307,11 @@ cudaError_t launch_proj_oz(const Dims* dims, const ProbPtr* ptrs, const uint16_t
     const bool stall = cap_st == cudaStreamCaptureStatusNone && fault_take(TEBD_FAULT_TC_STALL);
     oa.poll_limit = stall ? (1u << 12) : (1u << 24);
     oa.stall = stall ? 1 : 0;
-    oa.cond = 0;
+    oa.cond = DPC_FLAT;
     ProfScope ps("k_oz_proj[project]", st);
-    e = oz_launch<OZ_PROJ>(l, n, batch, dims, ptrs, oa, st);
-    return e;
+    if ((e = oz_launch<OZ_PROJ>(l, n, batch, dims, ptrs, oa, st)) != cudaSuccess) return e;
+    oa.cond = DPC_GRADED;
+    return oz_launch<OZ_PROJ7>(l, n, batch, dims, ptrs, oa, st);
   }
 }
 

@@ -684,6 +684,7 @@ __device__ __forceinline__ Dims plan_dev(const ProbPtr& P, int p, int digits) {
   D.cq = 0;
   D.cf = 0;
   D.js = 0;
+  D.gr = 0;
   return D;
 }
 
