@@ -106,12 +106,13 @@ static const uint32_t OZ_B_TILE = OZ_BN * OZ_KS * 2;  // one digit tile of the r
 // runs at 1/64 of the FP32 rate), then balanced base-256 digits: adding 128
 // to each of the six lower digits makes them plain bytes.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int64_t oz_fix(double x, int E) {
+// (shift: of x 2^shift)
+__device__ __forceinline__ int64_t oz_fix(double x, int E, int shift) {
   const uint64_t u = (uint64_t)__double_as_longlong(x);
   const int e = (int)((u >> 52) & 0x7FF);
   if (e == 0 || e == 0x7FF) return 0;
   const int64_t m = (int64_t)((u & 0xFFFFFFFFFFFFFull) | (1ull << 52));
-  const int sh = E - e - 2;  // x = m 2^(e - 1075), N = m 2^-sh; sh >= -2
+  const int sh = E - (e + shift) - 2;  // x = m 2^(e - 1075), N = m 2^-sh; sh >= -2
   const int64_t n = sh <= 0 ? (m << (-sh)) : (sh >= 56 ? 0 : ((m + (1ll << (sh - 1))) >> sh));
   return (u >> 63) ? -n : n;
 }
@@ -308,6 +309,7 @@ struct OzSrc {  // a GemmStage: strided operand of the stage table
     ks = SIDE == 0 ? g.acs : g.brs;
   }
   __device__ bool rows_contig() const { return rs == 1; }
+  __device__ int shift(int) const { return 0; }
   __device__ cplx at(int r, int k) const {
     const cplx v = X[(int64_t)r * rs + (int64_t)k * ks];
     if constexpr (SIDE == 0 && StageFlags<ST>::scaleA) return cscale(v, scale[k]);
@@ -321,18 +323,28 @@ struct OzSrc<OZ_PROJ, 1> {  // the columns of theta
   int rows, K;
   __device__ OzSrc(const Dims& D, const ProbPtr& P) : X(P.theta), rows(D.n), K(D.m) {}
   __device__ bool rows_contig() const { return true; }
+  __device__ int shift(int) const { return 0; }
   __device__ cplx at(int r, int k) const { return X[(int64_t)k * rows + r]; }
 };
+// The shifts of a bond's contraction (k_oz_balance), in the sketch matrix's
+// buffer, which the truncation fills later; null for a bond whose buffer is
+// shorter than chi_m.
+__device__ __forceinline__ int* oz_shifts(const Dims& D, const ProbPtr& P) {
+  return (int64_t)D.cm <= 4ll * D.n * D.l ? reinterpret_cast<int*>(P.omega) : nullptr;
+}
+
 template <int SIDE>
 struct OzSrc<OZ_THETA, SIDE> {  // A = Gamma_l (rows (i, alpha)), B = lam_m Gamma_r (columns (j, beta))
   Dims D;
   const ProbPtr* P;
+  const int* sh;
   int rows, K;
-  __device__ OzSrc(const Dims& d, const ProbPtr& p) : D(d), P(&p) {
+  __device__ OzSrc(const Dims& d, const ProbPtr& p) : D(d), P(&p), sh(oz_shifts(d, p)) {
     rows = SIDE == 0 ? d.dl * d.cl : d.dr * d.cr;
     K = d.cm;
   }
   __device__ bool rows_contig() const { return SIDE == 1; }
+  __device__ int shift(int g) const { return (sh && g < K) ? (SIDE == 0 ? sh[g] : -sh[g]) : 0; }
   __device__ cplx at(int r, int g) const {
     if (SIDE == 0) {
       const int i = r / D.cl, al = r - i * D.cl;
@@ -356,12 +368,67 @@ struct OzSrc<OZ_GATE, SIDE> {  // A = the gate (rows (i, j)), B = the (i', j') x
     K = d.dl * d.dr;
   }
   __device__ bool rows_contig() const { return SIDE == 1; }
+  __device__ int shift(int) const { return 0; }
   __device__ cplx at(int r, int k) const {
     if (SIDE == 0) return P->gate[(int64_t)r * (D.dl * D.dr) + k];
     const int ip = k / D.dr, jp = k - ip * D.dr, al = r / D.cr, be = r - al * D.cr;
     return P->Cpre[(int64_t)(ip * D.cl + al) * D.n + jp * D.cr + be];
   }
 };
+
+// Exponent of an entry times 2^shift.
+__device__ __forceinline__ int oz_exp(cplx v, int shift) {
+  const int e = max(oz_exp(v.x), oz_exp(v.y));
+  return (e == 0 || e == OZ_NONFINITE) ? e : max(e + shift, 0);
+}
+
+// The contraction sum_g Gamma_l[., g] (lam_m[g] Gamma_r[g, .]) does not see a
+// factor moved between the two sides of a term g, but digits relative to a
+// row's largest entry do: a column of Gamma_l that is large where lam_m is
+// small (1e14 at lam_m = 1e-14 in a gauge that is not canonical) left ten bits
+// of the others.  So both sides of every term are brought to the same largest
+// entry by a power of two: shift[g] is half the difference of the exponents,
+// and only the exponents the digits are cut at change.  A CTA takes 32 terms,
+// one read of both Gammas.
+template <int ST>
+__global__ void __launch_bounds__(256) k_oz_balance(const Dims* __restrict__ dims, const ProbPtr* __restrict__ ptrs,
+                                                    int cond) {
+  __shared__ int ea[32], eb[32];
+  const int z = blockIdx.y;
+  const Dims D = dims[z];
+  if (!D.active || !oz_takes(D, cond) || oz_skip<ST>(D, ptrs[z])) return;
+  const ProbPtr& P = ptrs[z];
+  int* sh = oz_shifts(D, P);
+  const int g0 = blockIdx.x * 32;
+  if (!sh || g0 >= D.cm) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < 32) ea[tid] = eb[tid] = 0;
+  __syncthreads();
+  int e = 0;
+  if (g0 + lane < D.cm)
+    for (int i = 0; i < D.dl; ++i) {
+      const cplx* row = P.gl + (int64_t)i * P.cap_l * P.cap_m + g0 + lane;
+#pragma unroll 4
+      for (int al = warp; al < D.cl; al += 8) e = max(e, oz_exp(row[(int64_t)al * P.cap_m], 0));
+    }
+  atomicMax(&ea[lane], e);
+  for (int q = warp; q < 32 && g0 + q < D.cm; q += 8) {
+    e = 0;
+    for (int j = 0; j < D.dr; ++j) {
+      const cplx* row = P.gr + ((int64_t)j * P.cap_m + g0 + q) * P.cap_r;
+#pragma unroll 4
+      for (int be = lane; be < D.cr; be += 32) e = max(e, oz_exp(row[be], 0));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) eb[q] = e;
+  }
+  __syncthreads();
+  if (tid < 32 && g0 + tid < D.cm) {
+    const int a = ea[tid], b = eb[tid], l = oz_exp(P.lamm[g0 + tid]);
+    const bool any = a > 0 && b > 0 && l > 0 && a < OZ_NONFINITE && b < OZ_NONFINITE && l < OZ_NONFINITE;
+    sh[g0 + tid] = any ? (b + l - 1023 - a) >> 1 : 0;
+  }
+}
 
 // Largest biased exponent of every row of a stage operand into Es[z][row]
 // (zero before the launch; a maximum does not depend on the order of the
@@ -387,17 +454,11 @@ __global__ void __launch_bounds__(256) k_oz_max(const Dims* __restrict__ dims, c
   if (rowc) {
     r = tid & 15;
     if (r0 + r < src.rows)
-      for (int k = k0 + (tid >> 4); k < k1; k += 16) {
-        const cplx v = src.at(r0 + r, k);
-        E = max(E, max(oz_exp(v.x), oz_exp(v.y)));
-      }
+      for (int k = k0 + (tid >> 4); k < k1; k += 16) E = max(E, oz_exp(src.at(r0 + r, k), src.shift(k)));
   } else {
     r = tid >> 4;
     if (r0 + r < src.rows)
-      for (int k = k0 + (tid & 15); k < k1; k += 16) {
-        const cplx v = src.at(r0 + r, k);
-        E = max(E, max(oz_exp(v.x), oz_exp(v.y)));
-      }
+      for (int k = k0 + (tid & 15); k < k1; k += 16) E = max(E, oz_exp(src.at(r0 + r, k), src.shift(k)));
   }
   atomicMax(&emax[r], E);
   __syncthreads();
@@ -438,10 +499,7 @@ __device__ __forceinline__ void oz_digits_block(const Dims* __restrict__ dims, c
     const int lr = rowc ? (tid & 15) : (tid >> 4);
     int e = 0;
     if (r0 + lr < rows)
-      for (int k = rowc ? (tid >> 4) : (tid & 15); k < K; k += 16) {
-        const cplx v = src.at(r0 + lr, k);
-        e = max(e, max(oz_exp(v.x), oz_exp(v.y)));
-      }
+      for (int k = rowc ? (tid >> 4) : (tid & 15); k < K; k += 16) e = max(e, oz_exp(src.at(r0 + lr, k), src.shift(k)));
     atomicMax(&emax[lr], e);
     __syncthreads();
     E = emax[r];
@@ -464,8 +522,9 @@ __device__ __forceinline__ void oz_digits_block(const Dims* __restrict__ dims, c
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const cplx v = tile[r][pq * 4 + q];
-      nr[q] = oz_fix(v.x, E);
-      ni[q] = oz_fix(v.y, E);
+      const int sh = src.shift(k0 + pq * 4 + q);
+      nr[q] = oz_fix(v.x, E, sh);
+      ni[q] = oz_fix(v.y, E, sh);
     }
     uint2 d[OZ_S];
     oz_digits4<OZ_S>(nr, d);
@@ -1002,6 +1061,11 @@ static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch
   constexpr bool same = ST == G_G1 || ST == G_G2 || ST == G_CYG || ST == G_CQG || ST == G_CTG || ST == G_CRG ||
                         ST == G_JG || ST == G_XG;
   cudaError_t e = cudaSuccess;
+  if constexpr (ST == OZ_THETA || ST == OZ_CONT) {
+    ProfScope ps("k_oz_balance", st);
+    k_oz_balance<ST><<<dim3((Kc + 31) / 32, batch), 256, 0, st>>>(dims, ptrs, cond);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   if (!same && !pre && Kp <= OZ_SELF_K) {
     if constexpr (!same) {
       ProfScope ps("k_oz_digits[op]", st);
