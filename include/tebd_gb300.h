@@ -65,9 +65,10 @@ enum {
  *   TEBD_PREC_FP64: the plain path, every result to FP64.  Large problems
  *     (plans with m, n >= 128 and k + p >= 40; bonds of those sizes of handles
  *     with fused = 0 and a bond of m n >= 192^2) run their products and QRs on
- *     the tensor cores: operands cut exactly into seven 8-bit digits (56 bits
- *     relative to the largest entry of each row or column), integer sums,
- *     Cholesky QR with column scaling (Householder for what it gives up), an
+ *     the tensor cores: operands cut into seven 8-bit digits (56 bits relative
+ *     to the largest entry of each row or column), products of digits exact,
+ *     their sums exact to 2^-36 of the leading digits' and in FP32 below
+ *     (errors of an FP64 sum's size), Cholesky QR with column scaling (Householder for what it gives up), an
  *     FP32 Jacobi with corrections to FP64.  The others, and plans with forced
  *     GEMM tiles, run on the FP64 pipe.
  *   TEBD_PREC_TF32: the mixed form.  Y0 = A Omega and power rounds 1..q-1
@@ -75,9 +76,9 @@ enum {
  *     power round q (Y0 when q = 0) as the refinement pass in split 3xTF32
  *     products (FP32-level accuracy); the last basis re-orthonormalised
  *     FP64-accurately (FP32 QR and a Loewdin correction);
- *     B = Q^H A on the tensor cores from exact BF16 digit splits of Q and
- *     A (products and digit levels exact: FP64-level accuracy); the QR of
- *     B^H by Cholesky QR passes from digits (Householder QR in FP64 for an
+ *     B = Q^H A on the tensor cores from BF16 digit splits of Q and A, as in
+ *     the FP64 form (Q's FP32 entries in four digits, in seven where A's rows
+ *     are graded); the QR of B^H by Cholesky QR passes from digits (Householder QR in FP64 for an
  *     instance whose Gram matrix is too ill-conditioned); the Jacobi SVD, U,
  *     V and lambda FP64-accurate.  Omega comes from the same Philox words by an FP32
  *     Box-Muller.
@@ -188,7 +189,8 @@ int tebd_workspace_info(tebd_t h, size_t* arena_bytes, int* waves_even, int* wav
 /* Plan and tuning of wave `wave` of a parity (0 <= wave < its count from
  * tebd_workspace_info).  info (20 ints): [0] bonds in the wave, [1..4] its
  * capacities m, n, k, l, [5] 1 if it runs as the persistent fused launch,
- * [6..11] the GEMM tile of stages Y0, Y~, Y, B^H, U, V (0: by grid size),
+ * [6..11] the GEMM tile of stages Y0, Y~, Y, B^H, U, V (0: by grid size;
+ * for the bonds on the FP64 pipe: those on the tensor cores stay there),
  * [12..15] the mixed form's launch choices of mixed-form handles (as
  * rrsvd_plan_tuning's [6..9]), [16] as rrsvd_plan_tuning's [11], [17..19]
  * zero.  ms (2 doubles): the autotuner's timings on
@@ -377,8 +379,9 @@ int rrsvd_plan_dims(rrsvd_plan_t plan, int* k, int* l);
  * using `workspace` (device, >= rrsvd_workspace_size bytes, 256-byte
  * aligned).  theta is only read.  Asynchronous on `stream`.
  * Errors: TEBD_EINVAL (NULL theta/sigma/workspace, small workspace, chain0 < 0),
- * TEBD_ECUDA.  A bounded tensor-core pipeline wait that expires (TF32 plans)
- * is reported by the next rrsvd_execute_host as TEBD_ETIMEOUT. */
+ * TEBD_ECUDA.  A bounded tensor-core pipeline wait that expires (mixed-form
+ * plans, FP64 plans on the tensor cores) is reported by the next
+ * rrsvd_execute_host as TEBD_ETIMEOUT. */
 int rrsvd_execute(rrsvd_plan_t plan, const double* theta, int64_t chain0, double* sigma, double* U, double* Vh,
                   double* w, int* rank, void* workspace, size_t workspace_bytes, void* stream);
 
@@ -426,7 +429,9 @@ const char* rrsvd_last_error(rrsvd_plan_t plan);
 /* Autotuner of a plan (the batched launches of Section IV's steps): times
  * the launch choices on the caller's theta (device, as for rrsvd_execute) and
  * keeps the fastest for later executes.  FP64 plans: the GEMM tile of every
- * stage; mixed-form plans: the mixed form's choices (tensor-core tile width,
+ * stage on the FP64 pipe and, where the plan's sizes are on the tensor cores,
+ * the whole truncation with those tiles against the digit splits (all tiles
+ * 0 where the digits are as fast); mixed-form plans: the mixed form's choices (tensor-core tile width,
  * CTA size of the FP32 QRs, one-CTA or many-CTA QR of B^H, one-CTA or
  * cluster Jacobi, the products after the projection on the tensor cores or
  * the CUDA cores), one at a time, each kept only for a clear gain.  Results of a
@@ -436,7 +441,8 @@ int rrsvd_plan_autotune(rrsvd_plan_t plan, const double* theta, void* workspace,
                         void* stream);
 
 /* What the autotuner chose: info (16 ints): [0..5] the FP64 GEMM tile of
- * stages Y0, Y~, Y, B^H, U, V (0: by grid size), [6..9] the mixed form's
+ * stages Y0, Y~, Y, B^H, U, V (0: by grid size; a tuned plan with any tile
+ * set runs on the FP64 pipe whatever its sizes), [6..9] the mixed form's
  * choices (tile split, FP32 QR threads, QR of B^H, Jacobi; 0: the size rule;
  * Jacobi 1: one CTA in FP64, 2: a cluster per instance in FP64, 3: one CTA
  * in double-float arithmetic),
@@ -449,7 +455,9 @@ int rrsvd_plan_tuning(rrsvd_plan_t plan, int* info, double* ms);
 /* Sets a plan's launch choices (info: 16 ints laid out as rrsvd_plan_tuning
  * gives them; [10] and [12..15] are ignored), e.g. to restore choices tuned
  * in another process or to compare two of them.  The plan counts as tuned
- * afterwards.  Results agree with those of any other choice to rounding.
+ * afterwards.  A nonzero tile keeps an FP64 plan off the tensor cores, many
+ * times slower at large sizes: choices saved by a version without the digit
+ * splits are better left out or tuned again.  Results agree with those of any other choice to rounding.
  * Errors: TEBD_EINVAL (NULL, a tile other than 0, 16 or 32, a choice out of
  * range: [6] 0..1, [7] 0, 128, 256 or 512, [8] 0..3, [9] 0..3, [11] 0..2). */
 int rrsvd_plan_set_tuning(rrsvd_plan_t plan, const int* info);
@@ -535,7 +543,9 @@ int rrsvd_sketch_omega(int n, int l, uint64_t seed, int64_t bond, int64_t sweep,
  * budget -- and so can neither create an rrsvd plan nor supply a workspace.
  *
  * Same truncation, Omega and outputs as rrsvd_execute on a plan created
- * with (m, n, k_max, p, q, batch, TEBD_PREC_FP64, seed); theta, sigma, U,
+ * with (m, n, k_max, p, q, batch, TEBD_PREC_FP64, seed), bit for bit where that
+ * plan runs on the FP64 pipe and to rounding where it takes the tensor cores
+ * (this call never does: its scratch has no room for the digits); theta, sigma, U,
  * Vh, w and rank are caller device buffers with the shapes given there (U,
  * Vh, w, rank may be NULL).  All scratch is one static 16 MiB device array
  * inside the library, held by every GPU that loads it until the process

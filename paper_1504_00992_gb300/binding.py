@@ -542,7 +542,8 @@ def rrsvd_host_wait(plan):
 def rrsvd_execute_noalloc(m, n, k_max, p, q, batch, seed, chain0, theta_ptr, sigma_ptr, U_ptr=0, Vh_ptr=0,
                           w_ptr=0, rank_ptr=0, stream_ptr=0):
     """No-allocation truncation on device buffers (integers, 0 for NULL):
-    same results as rrsvd_execute with a plan of the same sizes; scratch is a
+    same results as rrsvd_execute with a plan of the same sizes (to rounding
+    for sizes that plan runs on the tensor cores); scratch is a
     fixed 16 MiB array inside the library shared by every call."""
     def vp(x):
         return _vp(int(x)) if x else None

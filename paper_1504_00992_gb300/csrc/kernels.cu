@@ -437,9 +437,9 @@ cudaError_t launch_rrsvd_finalize(const Dims* dims, const ProbPtr* ptrs, int bat
 cudaError_t run_rrsvd(const Dims* dims, const ProbPtr* ptrs, int batch, const Caps& cap, int q, uint64_t seed,
                       uint64_t sweep, int64_t chain0, int chain_stride, int* status, cudaStream_t st,
                       const uint64_t* sweep_dev, const int* tiles, const DpScratch* dp) {
-  // with scratch for them, the problems of dp_rule's sizes take every product
-  // and QR from digit splits (a forced GEMM tile keeps all on the FP64 pipe);
-  // the launches of the others skip them
+  // with scratch for them, the problems with Dims::dig take every product and
+  // QR from digit splits, whatever the tiles say; the launches of the others
+  // skip them.  (A plan whose tiles are set passes no scratch: plan_digits.)
   const DpPath P{dims, ptrs, batch, cap, dp, st, tiles};
   TG_TRY(launch_omega(dims, ptrs, batch, cap, seed, sweep, chain0, chain_stride, st, sweep_dev));
   TG_TRY(dp_begin(P));

@@ -754,7 +754,8 @@ cudaError_t mixed_prepare(const Caps& cap) {
 // 21 ms, 16 x 7700 x 262 in 5 ms against 28 ms.  Those keep that QR's column
 // phases, and with them the singular vectors' and the next truncations'
 // samples (without them a spin-boson chain's Schmidt values moved by 2e-5 to
-// 7e-5 over three waves, with them by 1e-6).
+// 7e-5 over three waves, with them by 1e-8 to 2e-6 over 13 chains and two
+// seeds).
 int mixed_qrbh(const MixedKnobs& kn, const Caps& cap, int batch) {
   if (kn.qrbh) return kn.qrbh;
   const bool tc = kn.dfg == 1 || (kn.dfg == 0 && oz_stage_rule(cap));

@@ -232,16 +232,13 @@ cudaError_t launch_oz_gram(const Dims* dims, const ProbPtr* ptrs, const uint16_t
 
 // Launch choices of the mixed form that the autotuner may override (0 keeps
 // each size rule): tc_half = 1 splits the tensor-core products' columns over
-// two CTAs; qr_threads sets the CTA size of the blocked FP32 QRs (128, 256,
-// 512); qrbh forces the QR of B^H (1 one-CTA Householder, 2 many-CTA
-// Householder, 3 Cholesky QR with Householder for ill-conditioned instances;
-// the size rule takes the Cholesky QR wherever it would run the one-CTA
-// kernel); jac forces the Jacobi SVD as in launch_jacobi_sized.
-// Launch choices of the mixed form (0: the size rule).  jac: 1 the one-CTA
-// FP64 Jacobi, 2 the cluster form, 3 the one-CTA double-float one.  dfg: the
-// Cholesky QR
-// and U / V products on the tensor cores (digit splits, 0 by rule / 1) or as
-// double-float CUDA-core GEMMs (2).
+// two CTAs; qr_threads sets the CTA size of the blocked FP32 Householder QRs
+// (128, 256, 512) and takes them in place of the Cholesky QR; qrbh forces the
+// QR of B^H (1 one-CTA Householder, 2 many-CTA Householder, 3 Cholesky QR with
+// Householder for ill-conditioned instances, mixed_qrbh's rule); jac the
+// Jacobi SVD (1 the one-CTA FP64 kernel, 2 the cluster form, 3 the one-CTA
+// double-float one); dfg the products after the projection: on the tensor
+// cores from digit splits (0 by size, 1) or as double-float CUDA-core GEMMs (2).
 struct MixedKnobs {
   int tc_half, qr_threads, qrbh, jac, dfg;
 };

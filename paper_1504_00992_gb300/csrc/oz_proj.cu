@@ -16,11 +16,13 @@
 // OZ_DRAIN = 64 k every level up to 8 stays below 128 * 7 * 2^14 < 2^24: the
 // tensor core's FP32 sums are exact integers.  The epilogue reads the
 // fourteen accumulators (C_r and C_i at levels 2 .. 8) after every 64 k and
-// adds them exactly: levels 2 .. 6 into one 64-bit integer, levels 7 and 8
-// (2^-40 and 2^-48 of the leading level) into one FP32 number.  The scales
-// are applied once at the end.  What is lost is the rounding of the operands
-// (2^-56 of a row's largest entry) and the digit pairs with t + u > 8
-// (2^-56 of the largest product, random signs): on a CPU emulation 1.8e-16
+// adds levels 2 .. 6 exactly, in one 64-bit integer (moved to FP64 every 2^14
+// k), and levels 7 and 8 (2^-40 and 2^-48 of the leading level) in one FP32
+// number.  The scales are applied once at the end.  What is lost, in units of
+// max|a| max|b| over the row and column: the rounding of the operands and the
+// digit pairs with t + u > 8 (2^-56 each per k, random signs), and the FP32
+// additions, K / 64 of them at 2^-24 of a sum below 2^-36 K: at most
+// K^2 2^-67 (2^-56 K at K = 2000, 2^-54 K at K = 8000).  On a CPU emulation 1.8e-16
 // relative at K = 64 and 3e-16 at K = 2000 for Gaussian or orthonormal
 // operands, against 3e-16 and 1.5e-15 of FP64 multiply-adds in order; rows
 // graded over 2^-46 give 1.4e-15 against 2e-15.  Six digits would give
@@ -1058,7 +1060,7 @@ static cudaError_t oz_stage_run(const Dims* dims, const ProbPtr* ptrs, int batch
                                 const uint16_t* pre = nullptr, const int* pre_es = nullptr) {
   const int Kp = oz_kpad(Kc);
   // an operand times its own adjoint: one set of digits
-  constexpr bool same = ST == G_G1 || ST == G_G2 || ST == G_CYG || ST == G_CQG || ST == G_CTG || ST == G_CRG ||
+  constexpr bool same = ST == G_CYG || ST == G_CQG || ST == G_CTG || ST == G_CRG ||
                         ST == G_JG || ST == G_XG;
   cudaError_t e = cudaSuccess;
   if constexpr (ST == OZ_THETA || ST == OZ_CONT) {

@@ -238,14 +238,16 @@ __device__ __forceinline__ float qr_f32(double x) {
 __device__ __forceinline__ double qr_f64(float x) {
   return __longlong_as_double(((long long)__float_as_uint(x) << 29) + (896ll << 52));
 }
-// y = 1 / sqrt(v) and q = sqrt(v), v in [1, 8)
+// y = 1 / sqrt(v) and q = sqrt(v), v in [1, 8), from an FP32 seed y0 by the
+// binomial series (1 - r)^-1/2 = 1 + r / 2 + 3 r^2 / 8 of r = 1 - v y0^2
 __device__ __forceinline__ void qr_roots(double v, double& y, double& q) {
   const double y0 = qr_f64(rsqrtf(qr_f32(v)));
   const double t = v * y0, r = fma(-t, y0, 1.0), p = fma(0.375, r, 0.5);
   y = fma(y0 * r, p, y0);
   q = fma(t * r, p, t);
 }
-// 1 / v, v a normal number with a normal reciprocal
+// 1 / v, v a normal number with a normal reciprocal: the geometric series
+// 1 / (1 - r) = 1 + r + r^2 of r = 1 - m y0 on an FP32 seed y0
 __device__ __forceinline__ double qr_rcp(double v) {
   const int e = qr_exp(v) - 1023;
   const double m = qr_scale(v, -e);  // [1, 2)
